@@ -66,7 +66,7 @@ typedef enum {
 typedef enum {
     TP_FP64 = 0,  /* pair arithmetic in FP64 */
     TP_FP32 = 1,  /* pair arithmetic in FP32, per-tile partial sums folded into FP64 */
-    TP_MIXED = 2  /* FP32 pairs on double-float positions, FP64 for pairs closer than near_cutoff */
+    TP_MIXED = 2  /* FP32 pairs on double-float positions, double-float for pairs closer than near_cutoff */
 } tp_precision;
 
 typedef enum {
@@ -497,36 +497,35 @@ TPE_API tp_status tp_gnn_train_step(tp_ctx *ctx, const double *gamma, int n, con
 /* Autotuner of the pair passes (not in the paper).  For TP_MIXED contexts with the specialised
  * powers ((alpha, beta) = (2, 4.5)) it times, on the curve gamma, every candidate number of target
  * edges per thread of the energy (1, 2, 4), differential (1, 2) and apply / diag (1, 2, 4) gather
- * passes, and the symmetric energy, differential and apply passes (each unordered pair evaluated once, 1 or 2
- * targets per thread, when their partial sums fit in 32 GB and in half the free device memory), one
+ * passes, and the variants of the symmetric energy, differential and apply passes (each unordered pair
+ * evaluated once; when their partial sums fit in 32 GB and in half the free device memory), one
  * warm-up and three timed passes each
  * (CUDA events on `stream`), and keeps the fastest, rebuilding that op's work queue; other contexts
  * keep their defaults and are left unchanged.
  *   tpt (HOST int32 [6], may be NULL): the chosen targets per thread of the energy, differential and
- *       apply gather passes, then of the symmetric apply and energy, then the symmetric differential's
- *       variant (tp_set_diff_variant; 0: gather pass).
+ *       apply gather passes, then the variants of the symmetric apply, energy and differential (tp_set_*_variant; 0: gather
+ *       pass).
  *   ms  (HOST double [17], may be NULL): ms per pass for 1, 2, 4 targets per thread of the energy
- *       [0..2], differential [3..5] and apply [6..8] gather passes, then the symmetric apply [9..10],
- *       energy [11..12] with 1, 2, and the symmetric differential variants 1, 2 [13..14] and 3, 4
- *       [15..16] (0 where not a candidate).
+ *       [0..2], differential [3..5] and apply [6..8] gather passes, then the variants 1, 2 of the symmetric
+ *       apply [9..10] and energy [11..12] and the variants 1, 2 [13..14] and 3, 4 [15..16] of the symmetric
+ *       differential (0 where not a candidate).
  * May reallocate the context's partial-sum buffer (the only allocation after tp_create).
  * Synchronises the stream.  Errors: TP_ERR_INVALID_ARG, TP_ERR_CUDA, TP_ERR_DEGENERATE_EDGE. */
 TPE_API tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms, tp_stream stream);
 
-/* Select the apply pass: symmetric_tpt = 0 the gather pass (every ordered pair, the default), 1 or 2
- * the symmetric pass (every unordered pair evaluated once; both rows receive their terms; TP_MIXED with
- * (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED) with that many target edges per thread.  Both
- * are deterministic and differ only in summation order.  May grow the partial-sum buffer. */
+/* Select the apply pass: symmetric_tpt = 0 the gather pass (every ordered pair), 1 or 2 the symmetric pass
+ * (every unordered pair evaluated once, two targets per thread in packed arithmetic; both rows receive their
+ * terms; TP_MIXED with (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED), its registers held to three
+ * (1) or two (2) resident CTAs per SM.  Both are deterministic and differ only in summation order.  May grow the partial-sum buffer. */
 TPE_API tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt);
 
-/* The same choice for the energy pass (0: gather, 1 or 2: symmetric; the rows E_I are the same
- * sums in another order). */
+/* The same choice for the energy pass (0: gather, 1 or 2: symmetric at three or four resident CTAs per SM; the
+ * rows E_I are the same sums in another order). */
 TPE_API tp_status tp_set_energy_variant(tp_ctx *ctx, int symmetric_tpt);
 
-/* The same choice for the differential pass (0: gather; 1 or 2: symmetric with that many targets per
- * thread; 3: symmetric, one target per thread with registers held to 4 resident CTAs per SM; 4: two
- * targets per thread held to 3 CTAs per SM.  Row J's terms of a pair are the mirror of row I's; near
- * pairs are FP64 on both sides). */
+/* The same choice for the differential pass (0: gather; 1 or 2: symmetric at two resident CTAs per SM, 3 or 4
+ * at three, with spilled registers).  Row J's terms of a pair are the mirror of row I's; near pairs are
+ * double-float on both sides). */
 TPE_API tp_status tp_set_diff_variant(tp_ctx *ctx, int symmetric_tpt);
 
 /* Throughput microbenchmarks on the current device (no context needed): FP32 FMA FLOP/s, MUFU

@@ -42,7 +42,7 @@ def _stale(out, deps):
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
-    headers = [os.path.join(CSRC, h) for h in ("tpe_internal.cuh", "pair_device.cuh", "df.cuh", "coarse.cuh")]
+    headers = [os.path.join(CSRC, h) for h in ("tpe_internal.cuh", "pair_device.cuh", "pair_lanes.cuh", "df.cuh", "coarse.cuh")]
     headers.append(os.path.join(HERE, "..", "include", "tpe.h"))
     jobs = []
     for src in SOURCES:

@@ -1424,6 +1424,11 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         return pair_apply(c, gamma, 0, gamma, c.d_t2, s);  // any u times the same
     };
     cudaError_t err = cudaSuccess;
+    if (c.prm.precision == TP_MIXED && c.kp.fast) {  // the gather passes are timed first
+        CK(sym_select(c, 0));
+        CK(sym_select_energy(c, 0));
+        CK(sym_select_diff(c, 0));
+    }
     // a symmetric variant is a candidate while its partial sums fit in 32 GB and in half the free memory
     // (on top of what the partial buffer already holds); the buffer is shrunk to the winners' need below
     size_t free_b = 0, total_b = 0;
@@ -1462,8 +1467,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 1 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 4 && err == cudaSuccess; ++t) {
-                const int tpt_t = (t == 2 || t == 4) ? 2 : 1;
-                if (!fits(sym_slots(c, tpt_t) * (size_t)c.nE * 6 * sizeof(double))) continue;
+                if (!fits(sym_part_elems(c, OP_DIFF, t) * sizeof(double))) continue;
                 if ((err = sym_select_diff(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);
@@ -1486,7 +1490,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 0 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 2 && err == cudaSuccess; ++t) {
-                if (!fits(sym_slots(c, t) * (size_t)c.nE * sizeof(double))) continue;
+                if (!fits(sym_part_elems(c, OP_ENERGY, t) * sizeof(double))) continue;
                 if ((err = sym_select_energy(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);
@@ -1509,7 +1513,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 2 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 2 && err == cudaSuccess; ++t) {
-                if (!fits(sym_slots(c, t) * (size_t)c.nE * 6 * sizeof(double))) continue;
+                if (!fits(sym_part_elems(c, OP_APPLY, t) * sizeof(double))) continue;
                 if ((err = sym_select(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);
@@ -1539,9 +1543,9 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         const size_t nE1 = (size_t)std::max(1, c.nE);
         size_t need = (size_t)std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots) *
                       nE1 * 6;
-        if (c.apply_sym) need = std::max(need, (size_t)c.plan_sym.max_slots * nE1 * 6);
-        if (c.energy_sym) need = std::max(need, (size_t)c.plan_sym_e.max_slots * nE1);
-        if (c.diff_sym) need = std::max(need, (size_t)c.plan_sym_d.max_slots * nE1 * 6);
+        if (c.apply_sym) need = std::max(need, sym_part_elems(c, OP_APPLY, c.apply_sym));
+        if (c.energy_sym) need = std::max(need, sym_part_elems(c, OP_ENERGY, c.energy_sym));
+        if (c.diff_sym) need = std::max(need, sym_part_elems(c, OP_DIFF, c.diff_sym));
         if (need < c.part_elems) {
             graphs_reset(c);  // captured blocks hold the old buffer's address
             CK(cudaStreamSynchronize(s));

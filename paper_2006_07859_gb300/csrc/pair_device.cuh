@@ -7,6 +7,7 @@
 
 #include <type_traits>
 
+#include "pair_lanes.cuh"
 #include "tpe_internal.cuh"
 
 namespace tpe {
@@ -20,8 +21,8 @@ __device__ __forceinline__ R inv_pow(R d2, R e, R &r2)
 {
     if constexpr (FAST) {
         if constexpr (sizeof(R) == 4) {
-            float r = rsqrtf(d2);
-            float sr = r * rsqrtf(r);
+            float r = l_rsqrt(d2);
+            float sr = r * l_rsqrt(r);
             r2 = r * r;
             return WHICH == 0 ? r2 * r2 * sr : r2 * sr;
         } else {
@@ -261,7 +262,7 @@ struct Acc32;  // per-target tile accumulators in the pair precision
 template <int PREC>
 struct Acc32<PREC, OP_ENERGY> {
     static constexpr int op = OP_ENERGY;
-    typename RealOf<PREC>::type s;
+    typename RealOf<PREC>::type s, c;  // c: Kahan compensation (mixed path)
 };
 template <int PREC>
 struct Acc32<PREC, OP_DIFF> {
@@ -336,11 +337,11 @@ __device__ __forceinline__ void load_uval(UVal<typename RealOf<PREC>::type> &v, 
 }
 
 
-// Differential of one near pair in FP64 from the double-float positions and tangents, accumulated
-// straight into the FP64 accumulators: along the curve the near-pair gradient terms are large and
-// cancel between neighbours, so they need FP64 both in the arithmetic and in the sum.
-static __device__ __noinline__ void near_diff_df(const Tgt<float> &t, const Src<PMIX> &s, double alpha, double beta,
-                                          bool fast, DiffAcc64 &acc)
+// Differential of one near pair at general exponents, in FP64 from the double-float positions and tangents,
+// accumulated straight into the FP64 accumulators: along the curve the near-pair gradient terms are large
+// and cancel between neighbours, so they need more than FP32 both in the arithmetic and in the sum.
+static __device__ __noinline__ void near_diff_fp64(const Tgt<float> &t, const Src<PMIX> &s, double alpha, double beta,
+                                                   DiffAcc64 &acc)
 {
     double TI[3] = {(double)t.T.x + t.Tl.x, (double)t.T.y + t.Tl.y, (double)t.T.z + t.Tl.z};
     double TJ[3] = {(double)s.T.x + s.Tm.x, (double)s.T.y + s.Tm.y, (double)s.T.z + s.Tm.z};
@@ -361,19 +362,11 @@ static __device__ __noinline__ void near_diff_df(const Tgt<float> &t, const Src<
         double cJ2 = dpJ[0] * dpJ[0] + dpJ[1] * dpJ[1] + dpJ[2] * dpJ[2];
         double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
         double rb, fI, fJ, aI, aJ;
-        if (fast) {
-            double r = rsqrt(d2), r2 = r * r;
-            rb = r2 * r2 * sqrt(r);
-            fI = cI2 * rb;
-            fJ = cJ2 * rb;
-            aI = aJ = 2.0 * rb;
-        } else {
-            rb = pow(d2, -0.5 * beta);
-            fI = (cI2 > 0.0 ? pow(cI2, 0.5 * alpha) : 0.0) * rb;
-            fJ = (cJ2 > 0.0 ? pow(cJ2, 0.5 * alpha) : 0.0) * rb;
-            aI = cI2 > 0.0 ? alpha * fI / cI2 : 0.0;
-            aJ = cJ2 > 0.0 ? alpha * fJ / cJ2 : 0.0;
-        }
+        rb = pow(d2, -0.5 * beta);
+        fI = (cI2 > 0.0 ? pow(cI2, 0.5 * alpha) : 0.0) * rb;
+        fJ = (cJ2 > 0.0 ? pow(cJ2, 0.5 * alpha) : 0.0) * rb;
+        aI = cI2 > 0.0 ? alpha * fI / cI2 : 0.0;
+        aJ = cJ2 > 0.0 ? alpha * fJ / cJ2 : 0.0;
         double cb = beta * (fI + fJ) / d2;
         double *G = ab < 2 ? acc.G1 : acc.G2;
         for (int k = 0; k < 3; ++k) {
@@ -387,20 +380,12 @@ static __device__ __noinline__ void near_diff_df(const Tgt<float> &t, const Src<
 // One (target, source) pair: accumulate into the tile accumulator a.
 // DF: use the low parts (double-float differences) and compensated accumulation; only the mixed
 // path's MID and NEAR tiles set it.
-// |T x d|^2 in FP64 from the double-float position differences and tangent of a near pair: the
-// angle between T and the chord is small there, so FP32 would lose most of the digits of the
-// perpendicular part.  Only this quantity goes to FP64; the rest of the pair stays in FP32.
-__device__ __forceinline__ float perp2_near(V3<float> P, V3<float> PL, V3<float> Q, V3<float> QL, V3<float> T,
-                                            V3<float> Tl)
-{
-    double dx = (double)(P.x - Q.x) + (double)(PL.x - QL.x);
-    double dy = (double)(P.y - Q.y) + (double)(PL.y - QL.y);
-    double dz = (double)(P.z - Q.z) + (double)(PL.z - QL.z);
-    double tx = (double)T.x + (double)Tl.x, ty = (double)T.y + (double)Tl.y, tz = (double)T.z + (double)Tl.z;
-    double t = tx * dx + ty * dy + tz * dz;
-    double px = dx - t * tx, py = dy - t * ty, pz = dz - t * tz;
-    return (float)(px * px + py * py + pz * pz);
-}
+// Records behind a pair, for the near paths (which load them again).
+struct NearRef {
+    const RecF *recF;
+    const RecLo *recLo;
+    int I, J;
+};
 
 // The four chords d_ab = g_ia - g_jb of a pair (index ab = 2 (a - 1) + (b - 1)), formed from d11
 // by increments that mirror exactly between row I and row J: d12 = d11 - e_J, d21 = d11 + e_I,
@@ -480,20 +465,39 @@ __device__ __forceinline__ void pair_eval(const Tgt<typename RealOf<PREC>::type>
                                           Acc32<PREC, OP> &a, bool keep, const KernelParams &kp,
                                           typename RealOf<PREC>::type &d2_11,
                                           const UVal<typename RealOf<PREC>::type> *tu,
-                                          const UVal<typename RealOf<PREC>::type> *su, bool near = false)
+                                          const UVal<typename RealOf<PREC>::type> *su, const NearRef *near = nullptr)
 {
     using R = typename RealOf<PREC>::type;
     const R alpha = (R)kp.alpha, beta = (R)kp.beta, pp = (R)kp.p;
-    if constexpr (OP == OP_ENERGY) {
+    if constexpr (OP == OP_ENERGY && PREC == PMIX && FAST) {
+        // the terms of pairs_sym.cu on one lane, bit for bit: the two passes differ in the order of their
+        // compensated sums only
+        LV<float> d[4];
+        l_chords<DF, float>({t.p1.x, t.p1.y, t.p1.z}, {t.l1.x, t.l1.y, t.l1.z}, {t.e.x, t.e.y, t.e.z},
+                            {s.q1.x, s.q1.y, s.q1.z}, {s.m1.x, s.m1.y, s.m1.z}, {s.e.x, s.e.y, s.e.z}, d);
+        const LV<float> T = {t.T.x, t.T.y, t.T.z};
+        float c0 = l_perp2(d[0], T), c1 = l_perp2(d[1], T);  // |T_I x d_1b|^2 = |T_I x d_2b|^2
+        d2_11 = l_dot(d[0], d[0]);
+        if (near && keep && d2_11 < kp.near2f) {
+            float c[4];
+            near_energy<float, false>(near->recF, near->recLo, near->I, near->I, near->J, c);
+            c0 = c[0], c1 = c[1];
+        }
+        float r[4], r2;
+#pragma unroll
+        for (int ab = 0; ab < 4; ++ab) r[ab] = l_pow45(ab == 0 ? d2_11 : l_dot(d[ab], d[ab]), r2);
+        l_kahan_fma(a.s, a.c, s.ell, l_keep(keep, l_energy_sum(c0, c1, r[0], r[1], r[2], r[3])));
+    } else if constexpr (OP == OP_ENERGY) {
         V3<R> dd[4];
         chords<DF>(t, s, dd);
         R tt;
         V3<R> dp;
         R cI[2] = {perp2(dd[0], t.T, tt, dp), perp2(dd[1], t.T, tt, dp)};  // |T_I x d_1b|^2 = |T_I x d_2b|^2
         if constexpr (DF && sizeof(R) == 4)
-            if (near) {
-                cI[0] = perp2_near(t.p1, t.l1, s.q1, s.m1, t.T, t.Tl);
-                cI[1] = perp2_near(t.p1, t.l1, s.q2, s.m2, t.T, t.Tl);
+            if (near && keep && dot3(dd[0], dd[0]) < kp.near2f) {
+                float c[4];
+                near_energy<float, false>(near->recF, near->recLo, near->I, near->I, near->J, c);
+                cI[0] = c[0], cI[1] = c[1];
             }
         R f = 0;
 #pragma unroll
@@ -504,7 +508,10 @@ __device__ __forceinline__ void pair_eval(const Tgt<typename RealOf<PREC>::type>
             f += pow_c<R, FAST>(cI[ab & 1], alpha) * inv_pow<R, FAST, 0>(d2, beta, r2);
         }
         R c = s.ell * f;
-        a.s += keep ? c : (R)0;
+        if constexpr (PREC == PMIX)
+            kahan_add(a.s, a.c, keep ? c : (R)0);
+        else
+            a.s += keep ? c : (R)0;
     } else if constexpr (OP == OP_DIFF) {
         // |T_I x d_ab|, its perpendicular d - (T_I.d) T_I depend on b only (T_I . d_2b = T_I . d_1b + l_I);
         // |T_J x d_ab| and its perpendicular on a only
@@ -619,7 +626,7 @@ template <int PREC, int OP>
 __device__ __forceinline__ void acc_zero(Acc32<PREC, OP> &a)
 {
     if constexpr (OP == OP_ENERGY) {
-        a.s = 0;
+        a.s = a.c = 0;
     } else if constexpr (OP == OP_DIFF) {
         a.S = a.cS = 0;
         for (int k = 0; k < 3; ++k) a.G1[k] = a.G2[k] = a.GT[k] = a.c1[k] = a.c2[k] = a.cT[k] = 0;
@@ -649,7 +656,7 @@ __device__ __forceinline__ void acc_add(X &A, const Y &a)
 {
     constexpr int OPX = X::op;
     if constexpr (OPX == OP_ENERGY) {
-        A.s += a.s;
+        A.s += (double)a.s - (double)a.c;
     } else if constexpr (OPX == OP_DIFF) {
         // tile fold into FP64: value minus its compensation
         A.S += (double)a.S - (double)a.cS;
@@ -718,17 +725,30 @@ __device__ __forceinline__ void tile_loop(const Tgt<typename RealOf<PREC>::type>
             if constexpr (PREC == PMIX && MODE < 2) {
                 pair_eval<PREC, OP, FAST, MODE == 1>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su);
             } else if constexpr (PREC == PMIX) {
-                // near pairs (|g_i1 - g_j1| below the cutoff) take |T x d|^2 in FP64; the differential
-                // evaluates and accumulates the whole near pair in FP64
-                V3<float> e = diff3<true>(tg[k].p1, tg[k].l1, s.q1, s.m1);
-                bool near = keep && (dot3(e, e) < (OP == OP_DIFF ? pa.kp.near2f_diff : pa.kp.near2f));
+                // near pairs (|g_i1 - g_j1| below the cutoff) take |T x d|^2 in double-float; the differential
+                // evaluates the whole near pair in double-float (general exponents: FP64)
                 if constexpr (OP == OP_DIFF) {
-                    if (near)
-                        near_diff_df(tg[k], s, pa.kp.alpha, pa.kp.beta, FAST, A[k]);
-                    else
-                        pair_eval<PREC, OP, FAST, true>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su, false);
+                    V3<float> e = diff3<true>(tg[k].p1, tg[k].l1, s.q1, s.m1);
+                    if (keep && dot3(e, e) < pa.kp.near2f_diff) {
+                        if constexpr (FAST) {
+                            dfl<float> x[10], y[10];
+                            near_diff(pa.recF, pa.recLo, tI[k], tI[k], s0 + j, s0 + j, x, y);
+                            l_kahan_df(a[k].S, a[k].cS, x[0].hi, x[0].lo);
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) {
+                                l_kahan_df(a[k].G1[q], a[k].c1[q], x[1 + q].hi, x[1 + q].lo);
+                                l_kahan_df(a[k].G2[q], a[k].c2[q], x[4 + q].hi, x[4 + q].lo);
+                                l_kahan_df(a[k].GT[q], a[k].cT[q], x[7 + q].hi, x[7 + q].lo);
+                            }
+                        } else {
+                            near_diff_fp64(tg[k], s, pa.kp.alpha, pa.kp.beta, A[k]);
+                        }
+                    } else {
+                        pair_eval<PREC, OP, FAST, true>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su);
+                    }
                 } else {
-                    pair_eval<PREC, OP, FAST, true>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su, near);
+                    const NearRef near{pa.recF, pa.recLo, tI[k], s0 + j};
+                    pair_eval<PREC, OP, FAST, true>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su, &near);
                 }
             } else {
                 pair_eval<PREC, OP, FAST>(tg[k], s, a[k], keep, pa.kp, d2_11, &tu[k], &su);

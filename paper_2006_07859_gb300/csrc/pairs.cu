@@ -301,32 +301,39 @@ __global__ void __launch_bounds__(kThreads, (pair_min_blocks<PREC, OP, TPT>())) 
 // ---------------------------------------------------------------------------------- reductions / gathers
 
 // rows[I] = (l_I / 4) sum_slots part[slot][I]
-__global__ void k_energy_rows(int nE, int nslots_max, const int *__restrict__ eslots, const double *__restrict__ part,
+__global__ void k_energy_rows(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
                               const double *__restrict__ ell, double *__restrict__ rows)
 {
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nE) return;
     double s = 0.0;
-    int ns = eslots[I];
+    const int ns = eslots[I];
+#pragma unroll 8
     for (int k = 0; k < ns; ++k) s += part[(size_t)k * nE + I];
     rows[I] = 0.25 * ell[I] * s;
 }
 
-// Per-problem sums of a per-edge array (deterministic: one block per problem, fixed order).
-__global__ void k_segment_sum(const int *__restrict__ off, const double *__restrict__ x, double *__restrict__ out)
+// Per-problem sums of a per-edge array (deterministic: one block per problem, fixed order).  One block reads
+// the whole of a problem, so its loads in flight set the time: 1,024 threads with eight loads each take
+// 32,768 rows in 8 us where 256 threads with one took 65.
+constexpr int kSegThreads = 1024;
+__global__ void __launch_bounds__(kSegThreads) k_segment_sum(const int *__restrict__ off, const double *__restrict__ x,
+                                                             double *__restrict__ out)
 {
-    int q = blockIdx.x;
-    int b = off[q], e = off[q + 1];
+    const int q = blockIdx.x, b = off[q], e = off[q + 1];
     double s = 0.0;
-    for (int i = b + threadIdx.x; i < e; i += blockDim.x) s += x[i];
-    __shared__ double sh[256];
-    sh[threadIdx.x] = s;
+#pragma unroll 8
+    for (int i = b + threadIdx.x; i < e; i += kSegThreads) s += x[i];
+    __shared__ double sh[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[q] = sh[0];
+    if (threadIdx.x >= 32) return;
+    s = sh[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) out[q] = s;
 }
 
 // out_v = sum_{(I, slot) in inc(v)} sum_k part[k][I][slot*3 + c] (diff: slot selects G_i1 / G_i2;
@@ -364,20 +371,20 @@ __global__ void k_vertex_gather(int nV, int nE, const int *__restrict__ inc_ptr,
 // Two-stage gather for many slots: each edge's slots are summed once (k_edge_slots), then every vertex
 // combines its edges' sums (k_vertex_from_edges).  The one-stage gather reads an edge's slots once per
 // endpoint, twice the traffic when an edge has tens of slots (the symmetric passes on long curves).
+// One thread per value, so that a slot's values are read coalesced.
 template <int OP>
 __global__ void k_edge_slots(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
                              double *__restrict__ esum)
 {
     constexpr int W = OP == OP_DIAG ? 1 : 6;
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nE) return;
-    double o[W];
-    for (int c = 0; c < W; ++c) o[c] = 0.0;
-    for (int q = 0; q < eslots[I]; ++q) {
-        const double *p = part + ((size_t)q * nE + I) * W;
-        for (int c = 0; c < W; ++c) o[c] += p[c];
-    }
-    for (int c = 0; c < W; ++c) esum[(size_t)I * W + c] = o[c];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nE * W) return;
+    const int ns = eslots[i / W];
+    const size_t step = (size_t)nE * W;
+    double o = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < ns; ++q) o += part[q * step + i];
+    esum[i] = o;
 }
 
 template <int OP>
@@ -408,15 +415,26 @@ __global__ void k_vertex_from_edges(int nV, const int *__restrict__ inc_ptr, con
     }
 }
 
+// out from the per-edge sums in c.d_esum
+template <int OP>
+static cudaError_t vertices_from_edges(Ctx &c, double *out, cudaStream_t s)
+{
+    if (c.nV == 0) return cudaSuccess;
+    k_vertex_from_edges<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.d_inc_ptr, c.d_inc, c.d_esum, out);
+    c.launches++;
+    return cudaGetLastError();
+}
+
 // Sum the partial slots of a pass into the per-vertex output, in one or two stages by slot count.
 template <int OP>
 static cudaError_t gather_slots(Ctx &c, const Ctx::Plan &pl, double *out, cudaStream_t s)
 {
     if (c.nV == 0) return cudaSuccess;
     if (pl.max_slots > 2 && c.d_esum) {
-        k_edge_slots<OP><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, c.d_part, c.d_esum);
-        k_vertex_from_edges<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.d_inc_ptr, c.d_inc, c.d_esum, out);
-        c.launches += 2;
+        const int values = c.nE * (OP == OP_DIAG ? 1 : 6);
+        k_edge_slots<OP><<<(values + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, c.d_part, c.d_esum);
+        c.launches++;
+        return vertices_from_edges<OP>(c, out, s);
     } else {
         k_vertex_gather<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.nE, c.d_inc_ptr, c.d_inc, pl.d_eslots, c.d_part,
                                                               out);
@@ -431,6 +449,8 @@ cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s
 }
 
 // ---------------------------------------------------------------------------------- planning
+
+constexpr int kMinChunk = 4;  // sources of the shortest item
 
 // Build the (target block, source chunk) queue of one pass.  Items of big problems come first
 // so the persistent grid ends with the small ones.
@@ -453,6 +473,26 @@ void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
         double n = c.h_prob_e[q + 1] - c.h_prob_e[q];
         total += n * n;
     }
+    // Items of at least eight source tiles amortise their targets; where those would leave resident CTAs
+    // without an item, one wave of short items is faster: a pass over 256 edges was two CTAs, each walking
+    // all 256 sources in turn (energy 284 us, FP64 differential 2,117 us), and is 64 to 128 of them.
+    const long long resident = (long long)c.sm_count * std::max(1, occupancy);
+    auto chunks = [&](int n, bool small) {
+        const int nblk = (n + tb - 1) / tb;
+        const double share = total > 0 ? (double)n * n / total : 1.0;
+        const double want = std::ceil(share * (small ? (double)resident : (double)target_items) / nblk);
+        const int most = std::min(64, small ? n / kMinChunk : n / (8 * kTile));
+        return (int)std::max(1.0, std::min(want, (double)most));
+    };
+    auto items_of = [&](bool small) {
+        long long k = 0;
+        for (int q = 0; q < c.nProb; ++q) {
+            const int n = c.h_prob_e[q + 1] - c.h_prob_e[q];
+            k += (long long)((n + tb - 1) / tb) * chunks(n, small);
+        }
+        return k;
+    };
+    const bool small = items_of(false) < resident;
     int max_slots = 1;
     std::vector<int> eslots(c.nE, 1);
     struct Tmp {
@@ -464,13 +504,9 @@ void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
         int e0 = c.h_prob_e[q], e1 = c.h_prob_e[q + 1], n = e1 - e0;
         if (n <= 0) continue;
         int nblk = (n + tb - 1) / tb;
-        // chunks so that this problem gets its share of the target item count
-        double share = total > 0 ? (double)n * n / total : 1.0;
-        int want = (int)std::ceil(share * target_items / nblk);
-        int max_chunks = std::max(1, n / (8 * kTile));  // at least 8 source tiles per item
-        int nch = std::min(std::max(1, want), max_chunks);
-        nch = std::min(nch, 64);
-        int clen = ((n + nch - 1) / nch + kTile - 1) / kTile * kTile;
+        int nch = chunks(n, small);
+        int clen = (n + nch - 1) / nch;
+        if (!small) clen = (clen + kTile - 1) / kTile * kTile;
         nch = (n + clen - 1) / clen;
         max_slots = std::max(max_slots, nch);
         for (int b = 0; b < nblk; ++b) {
@@ -503,28 +539,10 @@ void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
 }
 
 constexpr int kTptEnergy = 4, kTptDiff = 2, kTptApply = 2;
-constexpr int kTptEnergy64 = 1, kTptDiff64 = 1, kTptApply64 = 1;
 
-template <int PREC, int OP, int TPT>
-static int occupancy_of(const Ctx &c)
-{
-    int occ = 0;
-    if constexpr (PREC == PMIX && !((OP == OP_ENERGY && TPT == kTptEnergy) || (OP == OP_DIFF && TPT == kTptDiff) ||
-                                    ((OP == OP_APPLY || OP == OP_DIAG) && TPT == kTptApply))) {
-        // candidate-only targets-per-thread values exist for the specialised powers alone
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs<PREC, OP, TPT, true>, kThreads, 0);
-    } else if (c.kp.fast) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs<PREC, OP, TPT, true>, kThreads, 0);
-    } else {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs<PREC, OP, TPT, false>, kThreads, 0);
-    }
-    return occ;
-}
-
-
-// Targets per thread: the default of each op class, and the values the autotuner may choose for the
-// mixed-precision passes with the specialised powers ((alpha, beta) = (2, 4.5)), the only kernels
-// instantiated for every candidate.
+// Targets per thread: one on short graphs (see small_graph), the default of the op class otherwise, and for
+// the mixed-precision passes with the specialised powers ((alpha, beta) = (2, 4.5)) the value the autotuner
+// chose; only those are instantiated for every candidate.
 static int op_class(int op) { return op == OP_ENERGY ? 0 : (op == OP_DIFF ? 1 : 2); }
 
 int tpt_default(const Ctx &c, int cls)
@@ -552,36 +570,49 @@ int tpt_candidates(const Ctx &c, int cls, int *out)
     return 3;
 }
 
-static int tpt_for(const Ctx &c, int cls) { return (tunable(c) && c.tpt[cls]) ? c.tpt[cls] : tpt_default(c, cls); }
-
-template <int OP>
-static int occupancy_fast_mixed(const Ctx &c, int tpt)
+// Too few edges to give every SM two items of tpt targets per thread and eight source tiles: one target
+// per thread then doubles or quadruples the items (256 edges: energy with four targets 16 items, with one 64).
+static bool small_graph(const Ctx &c, int tpt)
 {
-    if constexpr (OP == OP_DIFF) {
-        return tpt == 1 ? occupancy_of<PMIX, OP, 1>(c) : occupancy_of<PMIX, OP, 2>(c);
-    } else {
-        return tpt == 1 ? occupancy_of<PMIX, OP, 1>(c)
-                        : (tpt == 4 ? occupancy_of<PMIX, OP, 4>(c) : occupancy_of<PMIX, OP, 2>(c));
+    long long items = 0;
+    for (int q = 0; q < c.nProb; ++q) {
+        const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q];
+        items += ((n + kThreads * tpt - 1) / (kThreads * tpt)) * std::max(1LL, n / (8 * kTile));
     }
+    return items < 2LL * c.sm_count;
 }
 
-// Launch the pair kernel of the mixed / specialised-power path with `tpt` targets per thread.
-template <int OP>
-static void launch_fast_mixed(int tpt, int g, cudaStream_t s, const PairArgs &pa)
+static int tpt_for(const Ctx &c, int cls)
 {
-    if constexpr (OP == OP_DIFF) {
-        if (tpt == 1)
-            k_pairs<PMIX, OP, 1, true><<<g, kThreads, 0, s>>>(pa);
-        else
-            k_pairs<PMIX, OP, 2, true><<<g, kThreads, 0, s>>>(pa);
-    } else {
-        if (tpt == 1)
-            k_pairs<PMIX, OP, 1, true><<<g, kThreads, 0, s>>>(pa);
-        else if (tpt == 4)
-            k_pairs<PMIX, OP, 4, true><<<g, kThreads, 0, s>>>(pa);
-        else
-            k_pairs<PMIX, OP, 2, true><<<g, kThreads, 0, s>>>(pa);
-    }
+    if (tunable(c) && c.tpt[cls]) return c.tpt[cls];
+    const int t = tpt_default(c, cls);
+    return small_graph(c, t) ? 1 : t;
+}
+
+// f(kernel) of one pass at tpt targets per thread (the values instantiated for it; the op's default otherwise)
+template <int PREC, int OP, bool FAST, class F>
+static void with_pair_kernel(int tpt, F f)
+{
+    constexpr int D = PREC == P64 ? 1 : (OP == OP_ENERGY ? kTptEnergy : (OP == OP_DIFF ? kTptDiff : kTptApply));
+    if constexpr (D != 1)
+        if (tpt == 1) return f(k_pairs<PREC, OP, 1, FAST>);
+    if constexpr (PREC == PMIX && FAST && D == 4)
+        if (tpt == 2) return f(k_pairs<PREC, OP, 2, FAST>);
+    if constexpr (PREC == PMIX && FAST && D == 2 && OP != OP_DIFF)
+        if (tpt == 4) return f(k_pairs<PREC, OP, 4, FAST>);
+    f(k_pairs<PREC, OP, D, FAST>);
+}
+
+template <int OP, class F>
+static void with_pair_kernel(const Ctx &c, int tpt, F f)
+{
+    const bool fast = c.kp.fast != 0;
+    if (c.prm.precision == TP_FP64)
+        fast ? with_pair_kernel<P64, OP, true>(tpt, f) : with_pair_kernel<P64, OP, false>(tpt, f);
+    else if (c.prm.precision == TP_MIXED)
+        fast ? with_pair_kernel<PMIX, OP, true>(tpt, f) : with_pair_kernel<PMIX, OP, false>(tpt, f);
+    else
+        fast ? with_pair_kernel<P32, OP, true>(tpt, f) : with_pair_kernel<P32, OP, false>(tpt, f);
 }
 
 // ---------------------------------------------------------------------------------- profiling
@@ -632,18 +663,15 @@ void prof_harvest(Ctx &c)
 
 static int occupancy_cls(const Ctx &c, int cls, int tpt)
 {
-    if (c.prm.precision == TP_FP64)
-        return cls == 0 ? occupancy_of<P64, OP_ENERGY, kTptEnergy64>(c)
-                        : (cls == 1 ? occupancy_of<P64, OP_DIFF, kTptDiff64>(c) : occupancy_of<P64, OP_APPLY, kTptApply64>(c));
-    if (c.prm.precision == TP_MIXED) {
-        if (tunable(c))
-            return cls == 0 ? occupancy_fast_mixed<OP_ENERGY>(c, tpt)
-                            : (cls == 1 ? occupancy_fast_mixed<OP_DIFF>(c, tpt) : occupancy_fast_mixed<OP_APPLY>(c, tpt));
-        return cls == 0 ? occupancy_of<PMIX, OP_ENERGY, kTptEnergy>(c)
-                        : (cls == 1 ? occupancy_of<PMIX, OP_DIFF, kTptDiff>(c) : occupancy_of<PMIX, OP_APPLY, kTptApply>(c));
-    }
-    return cls == 0 ? occupancy_of<P32, OP_ENERGY, kTptEnergy>(c)
-                    : (cls == 1 ? occupancy_of<P32, OP_DIFF, kTptDiff>(c) : occupancy_of<P32, OP_APPLY, kTptApply>(c));
+    int occ = 0;
+    auto ask = [&](auto kern) { cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0); };
+    if (cls == 0)
+        with_pair_kernel<OP_ENERGY>(c, tpt, ask);
+    else if (cls == 1)
+        with_pair_kernel<OP_DIFF>(c, tpt, ask);
+    else
+        with_pair_kernel<OP_APPLY>(c, tpt, ask);
+    return occ;
 }
 
 static Ctx::Plan &plan_of(Ctx &c, int cls) { return cls == 0 ? c.plan_energy : (cls == 1 ? c.plan_diff : c.plan_apply); }
@@ -795,8 +823,8 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
         k_pairs<PMIX, OP_ENERGY, kTptEnergy, true><<<grid, kThreads, 0, s>>>(pa);
     else
         k_pairs<PMIX, OP_ENERGY, kTptEnergy, false><<<grid, kThreads, 0, s>>>(pa);
-    k_energy_rows<<<(nE + 255) / 256, 256, 0, s>>>(nE, nch, eslots, part, ell, rows);
-    k_segment_sum<<<1, 256, 0, s>>>(off, rows, E);
+    k_energy_rows<<<(nE + 255) / 256, 256, 0, s>>>(nE, eslots, part, ell, rows);
+    k_segment_sum<<<1, kSegThreads, 0, s>>>(off, rows, E);
     return cudaGetLastError();
 }
 
@@ -829,7 +857,7 @@ cudaError_t build_urecs(Ctx &c, const double *u, int which, cudaStream_t s)
 
 cudaError_t segment_sum(Ctx &c, const double *rows, double *E, cudaStream_t s)
 {
-    k_segment_sum<<<c.nProb, 256, 0, s>>>(c.d_prob_e, rows, E);
+    k_segment_sum<<<c.nProb, kSegThreads, 0, s>>>(c.d_prob_e, rows, E);
     c.launches++;
     return cudaGetLastError();
 }
@@ -847,6 +875,7 @@ static cudaError_t run_pairs(Ctx &c, int which, const double *gamma, const doubl
 {
     Ctx::Plan &pl = (OP == OP_ENERGY) ? c.plan_energy : (OP == OP_DIFF ? c.plan_diff : c.plan_apply);
     if (pl.n_items == 0) return cudaSuccess;
+    if (!tunable(c) && pl.tpt != 1 && pl.tpt != tpt_default(c, op_class(OP))) return cudaErrorInvalidValue;  // no such kernel
     constexpr int ctr = OP;
     TPE_CHECK(cudaMemsetAsync(c.d_counter + ctr, 0, sizeof(int), s));
     PairArgs pa;
@@ -863,29 +892,10 @@ static cudaError_t run_pairs(Ctx &c, int which, const double *gamma, const doubl
     pa.nE = c.nE;
     pa.kp = c.kp;
     pa.skip = (OP == OP_APPLY) ? c.d_skip : nullptr;
-    const int g = pl.grid;
-    const bool f = c.kp.fast != 0;
     // profiling: applies that skip converged problems are recorded apart (op 4), so op 2 always
     // times full passes of pairs_per_pass pairs
     const int slot = c.profile ? prof_begin(c, (OP == OP_APPLY && c.d_skip) ? 4 : OP, s) : -1;
-    switch (c.prm.precision) {
-    case TP_FP64:
-        if (f) k_pairs<P64, OP, (OP == OP_ENERGY ? kTptEnergy64 : OP == OP_DIFF ? kTptDiff64 : kTptApply64), true><<<g, kThreads, 0, s>>>(pa);
-        else k_pairs<P64, OP, (OP == OP_ENERGY ? kTptEnergy64 : OP == OP_DIFF ? kTptDiff64 : kTptApply64), false><<<g, kThreads, 0, s>>>(pa);
-        break;
-    case TP_MIXED:
-        if (f) {
-            launch_fast_mixed<OP>(pl.tpt, g, s, pa);  // the plan's targets per thread (autotuned or default)
-        } else {
-            if (pl.tpt != tpt_default(c, op_class(OP))) return cudaErrorInvalidValue;  // plan / kernel mismatch
-            k_pairs<PMIX, OP, (OP == OP_ENERGY ? kTptEnergy : OP == OP_DIFF ? kTptDiff : kTptApply), false><<<g, kThreads, 0, s>>>(pa);
-        }
-        break;
-    default:
-        if (f) k_pairs<P32, OP, (OP == OP_ENERGY ? kTptEnergy : OP == OP_DIFF ? kTptDiff : kTptApply), true><<<g, kThreads, 0, s>>>(pa);
-        else k_pairs<P32, OP, (OP == OP_ENERGY ? kTptEnergy : OP == OP_DIFF ? kTptDiff : kTptApply), false><<<g, kThreads, 0, s>>>(pa);
-        break;
-    }
+    with_pair_kernel<OP>(c, pl.tpt, [&](auto kern) { kern<<<pl.grid, kThreads, 0, s>>>(pa); });  // the plan's targets per thread
     if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
     c.launches++;
     return cudaGetLastError();
@@ -893,44 +903,39 @@ static cudaError_t run_pairs(Ctx &c, int which, const double *gamma, const doubl
 
 cudaError_t pair_energy(Ctx &c, const double *gamma, int which, double *rows_out, double *E_out, cudaStream_t s)
 {
-    const bool sym = c.energy_sym > 0;
-    if (sym)
-        TPE_CHECK(sym_energy_pass(c, which, gamma, s));
-    else
-        TPE_CHECK(run_pairs<OP_ENERGY>(c, which, gamma, nullptr, s));
-    const Ctx::Plan &pl = sym ? c.plan_sym_e : c.plan_energy;
     double *rows = rows_out ? rows_out : c.d_rows;
-    if (c.nE > 0) {
-        k_energy_rows<<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.max_slots, pl.d_eslots, c.d_part, c.d_ellw[which],
-                                                         rows);
-        c.launches++;
+    if (c.energy_sym > 0) {
+        TPE_CHECK(sym_energy_pass(c, which, rows, s));
+    } else {
+        TPE_CHECK(run_pairs<OP_ENERGY>(c, which, gamma, nullptr, s));
+        if (c.nE > 0) {
+            k_energy_rows<<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, c.plan_energy.d_eslots, c.d_part, c.d_ellw[which], rows);
+            c.launches++;
+        }
     }
-    if (E_out) {
-        k_segment_sum<<<c.nProb, 256, 0, s>>>(c.d_prob_e, rows, E_out);
-        c.launches++;
-    }
+    if (E_out) TPE_CHECK(segment_sum(c, rows, E_out, s));
     return cudaGetLastError();
 }
 
 cudaError_t pair_diff(Ctx &c, const double *gamma, int which, double *dE, cudaStream_t s)
 {
-    const bool sym = c.diff_sym > 0;
-    if (sym)
-        TPE_CHECK(sym_diff_pass(c, which, gamma, s));
-    else
-        TPE_CHECK(run_pairs<OP_DIFF>(c, which, gamma, nullptr, s));
-    return gather_slots<OP_DIFF>(c, sym ? c.plan_sym_d : c.plan_diff, dE, s);
+    if (c.diff_sym > 0) {
+        TPE_CHECK(sym_diff_pass(c, which, s));
+        return vertices_from_edges<OP_DIFF>(c, dE, s);
+    }
+    TPE_CHECK(run_pairs<OP_DIFF>(c, which, gamma, nullptr, s));
+    return gather_slots<OP_DIFF>(c, c.plan_diff, dE, s);
 }
 
 cudaError_t pair_apply(Ctx &c, const double *gamma_geom, int which, const double *u, double *Au, cudaStream_t s)
 {
     TPE_CHECK(build_urecs(c, u, which, s));
-    const bool sym = c.apply_sym > 0;
-    if (sym)
-        TPE_CHECK(sym_apply_pass(c, which, gamma_geom, u, s));
-    else
-        TPE_CHECK(run_pairs<OP_APPLY>(c, which, gamma_geom, u, s));
-    return gather_slots<OP_APPLY>(c, sym ? c.plan_sym : c.plan_apply, Au, s);
+    if (c.apply_sym > 0) {
+        TPE_CHECK(sym_apply_pass(c, which, s));
+        return vertices_from_edges<OP_APPLY>(c, Au, s);
+    }
+    TPE_CHECK(run_pairs<OP_APPLY>(c, which, gamma_geom, u, s));
+    return gather_slots<OP_APPLY>(c, c.plan_apply, Au, s);
 }
 
 cudaError_t pair_diag(Ctx &c, const double *gamma_geom, int which, double *diag, cudaStream_t s)

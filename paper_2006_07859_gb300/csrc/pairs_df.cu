@@ -22,6 +22,8 @@
 // so the result is deterministic.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "df.cuh"
 #include "tpe_internal.cuh"
 
@@ -272,15 +274,14 @@ cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const do
 {
     if (c.prm.precision == TP_FP64) return pair_apply(c, gamma_geom, which, u, Au, s);
     Ctx::Plan &pl = c.plan_df;
-    if (!pl.d_items) {
-        sym_plan_items(c, pl, 1, df_occupancy(c.kp.fast != 0));
-        const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
-        if (need > c.part_elems) {
-            TPE_CHECK(cudaFree(c.d_part));
-            TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-            c.part_elems = need;
-            graphs_reset(c);  // captured blocks hold the old partial buffer
-        }
+    if (!pl.d_items) sym_plan_items(c, pl, 1, df_occupancy(c.kp.fast != 0));
+    // the buffer is shared with the other passes and may have been resized since the last call
+    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
+    if (need > c.part_elems) {
+        TPE_CHECK(cudaFree(c.d_part));
+        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
+        c.part_elems = need;
+        graphs_reset(c);  // captured blocks hold the old partial buffer
     }
     TPE_CHECK(build_urecs(c, u, which, s));
     if (pl.n_items == 0) return cudaMemsetAsync(Au, 0, sizeof(double) * 3 * c.nV, s);

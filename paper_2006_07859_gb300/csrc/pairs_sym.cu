@@ -1,27 +1,43 @@
-// Symmetric Sobolev apply: every unordered pair of disjoint edges {I, J} evaluated once.
+// Symmetric pair passes: every unordered pair of disjoint edges {I, J} evaluated once, both rows fed.
 //
-// The Gram weights are symmetric: w_IJ = w_JI and the low-order weight enters as w0_IJ + w0_JI
-// (Secs. 5.2.2-5.2.3).  One evaluation of a pair therefore yields what row I receives from J and what
-// row J receives from I:
-//   row I: h += l_J sw ((du_I - du_J) + (|T_I - T_J|^2 / 2) du_J),   l += l_J sw0 (ub_I - ub_J)
-//   row J: h += l_I sw ((du_J - du_I) + (|T_I - T_J|^2 / 2) du_I),   l += l_I sw0 (ub_J - ub_I)
-// with sw = sum_ab |d_ab|^-p and sw0 = sum_ab (|T_I x d_ab|^2 + |T_J x d_ab|^2) |d_ab|^-(4+p).  The chords
-// and weights are bitwise the same from either side (pair_device.cuh), so the result equals the
-// gather pass's up to summation order.
+//   apply: the Gram weights are symmetric (w_IJ = w_JI, and the low-order weight enters as w0_IJ + w0_JI,
+//     Secs. 5.2.2-5.2.3), so one evaluation yields what row I receives from J and what row J receives from I:
+//       row I: h += l_J sw ((du_I - du_J) + (|T_I - T_J|^2 / 2) du_J),   l += l_J sw0 (ub_I - ub_J)
+//       row J: h += l_I sw ((du_J - du_I) + (|T_I - T_J|^2 / 2) du_I),   l += l_I sw0 (ub_J - ub_I)
+//     with sw = sum_ab |d_ab|^-p and sw0 = sum_ab (|T_I x d_ab|^2 + |T_J x d_ab|^2) |d_ab|^-(4+p);
+//   energy: row I receives l_J sum_ab |T_I x d_ab|^2 |d_ab|^-4.5, row J l_I sum_ab |T_J x d_ab|^2 |d_ab|^-4.5;
+//   differential: row I accumulates (scaled by l_J) S = sum (f_I + f_J), G_a += v_ab, GT += -a_I (T_I . d_ab)
+//     d_ab with v_ab = d(f_I + f_J)/dd at d_ab = g_ia - g_jb; row J sees d' = -d and accumulates (scaled by
+//     l_I) the same S, H_b -= v_ab (its endpoint b) and HT += -a_J (T_J . d_ab) d_ab.
 //
-// Work items are pairs of edge blocks (b, c >= b) of one problem (block = 128 x TPT edges).  For
-// b < c the CTA owns the targets of block b in registers and streams block c through shared memory;
-// lane l of each warp visits source (step + l) mod P at step `step`, so the 32 lanes of a warp always
-// touch 32 distinct sources and add what those sources receive into the warp's own Kahan-compensated
-// shared-memory accumulators (no atomics).  Target rows of block b write partial slot c, source rows of
-// block c write slot b, and the diagonal item (b, b) is a plain gather over its own block writing slot
-// b: every row receives exactly one write per slot m = 0 .. nblk - 1, and the vertex gather sums the
-// slots in index order, so the pass is deterministic.
+// What bounds the passes and the layout that follows from it.  A pair of the apply costs about 195
+// operations of the FP32 pipe and 8 MUFU; as scalar instructions these, the shared-memory accesses and the
+// denormal fix-ups of rsqrtf filled ~299 issue slots of a sub-partition per 32 pairs.  Every thread
+// therefore owns TWO target edges and evaluates both pairs with one source in packed f32x2 instructions
+// (pair_lanes.cuh), half the issue slots for the same FP32 work, and one load of a source serves two pairs.
+// (One target a thread would load 7 LDS.128 a pair, 112 of the ~200 cycles the shared-memory port has
+// for it; four targets do not fit in registers.)
+//
+// Blocks.  A problem's edges are cut into super-blocks of 256 target rows (128 threads x 2 adjacent rows) and
+// tiles of 128 source rows.  A work item is one super-block X against up to four tiles beyond it (c >= 2 X + 2),
+// or against itself.  Lane l of a warp takes source (step + 2 l) mod P at step `step`: the 32 lanes touch 32
+// distinct sources and add what those receive into the warp's own Kahan-compensated shared-memory
+// accumulators (no atomics), and along a curve all lanes are equally far from their sources, so near pairs
+// (evaluated in double-float) come in the same steps.  Inside its own super-block a warp takes its own 64
+// rows and whole 64-row sections of the others, every pair once (a plain gather there would add 12% of
+// the pairs at 4,096 edges).
+//
+// Partial sums are (sum, low part) float pairs, one slot per writer: a row of super-block X gets slot B from
+// every super-block B < X (as a source), slots X to X + 2 from its own super-block (source side, and target
+// side of its two tiles) and one slot from every item it is a target of; k_sym_sum adds a row's slots in index order in
+// double-float arithmetic, so the passes are deterministic, and no FP64 instruction (2 per clock and SM) is
+// left in the pair kernels.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <vector>
 
+#include "df.cuh"
 #include "pair_device.cuh"
 
 namespace tpe {
@@ -33,735 +49,639 @@ namespace tpe {
     } while (0)
 
 constexpr int kSymWarps = kThreads / 32;
+constexpr int kSuper = 2 * kThreads;  // target rows of an item
+constexpr int kSection = 64;          // rows of one warp
+constexpr int kQueue = 128;           // near pairs a warp holds back: a batch of 64 and one step's worth
+constexpr int kSymMaxTiles = 4;       // source tiles of an item: a Kahan sum spans at most 512 sources
 
-// One unordered pair in mixed precision: target-side terms Kahan-accumulated into `a`, source-side
-// terms added to hs (high-order, 3) and ls (low-order, 3).
-template <bool FAST, bool DF>
-__device__ __forceinline__ void pair_apply_both(const Tgt<float> &t, const Src<PMIX> &s, const UVal<float> &tu,
-                                                const UVal<float> &su, bool keep, const KernelParams &kp,
-                                                Acc32<PMIX, OP_APPLY> &a, float (&hs)[3], float (&ls)[3])
+struct SymArgs {
+    const WorkItem *items;  // slot: (super-block << 16) | target slot; nb_lo: bit t = tile t needs the disjointness test
+    int n_items;
+    int *counter;
+    const RecF *recF;
+    const RecLo *recLo;
+    const URecF *urecF;
+    float2 *part;  // [slot][nE][W]
+    int nE;
+    float near2f, mid2f;
+    const int *skip;
+};
+
+template <int OP>
+__host__ __device__ constexpr int sym_width()
 {
-    const float pp = (float)kp.p;
-    V3<float> dd[4];
-    chords<DF>(t, s, dd);
-    float tt;
-    V3<float> dp;
-    const float cI1 = perp2(dd[0], t.T, tt, dp), cI2 = perp2(dd[1], t.T, tt, dp);
-    const float cJ1 = perp2(dd[0], s.T, tt, dp), cJ2 = perp2(dd[2], s.T, tt, dp);
-    const float c2s[4] = {cI1 + cJ1, cI2 + cJ1, cI1 + cJ2, cI2 + cJ2};
-    float tw[4], tw0[4];
-#pragma unroll
-    for (int ab = 0; ab < 4; ++ab) {
-        const float d2 = dot3(dd[ab], dd[ab]);
-        float r2;
-        const float rp = inv_pow<float, FAST, 1>(d2, pp, r2);
-        tw[ab] = rp;
-        tw0[ab] = c2s[ab] * (rp * r2 * r2);
+    return OP == OP_ENERGY ? 1 : (OP == OP_DIFF ? 10 : 6);
+}
+
+// Source tile (struct of arrays, 16-byte elements) and the warps' source accumulators.
+template <int PREC, int OP>
+struct SymSmem {
+    static constexpr bool MIX = PREC == PMIX, U = OP == OP_APPLY;
+    float4 t0[kTile], t1[kTile], t2[kTile];  // (q1, l), (e, T.x), (T.y, T.z, q1.x lo, q1.y lo)
+    float4 t3[MIX ? kTile : 1];              // (q1.z lo, T lo)
+    float4 u0[U ? kTile : 1], u1[U ? kTile : 1], u2[(U && MIX) ? kTile : 1];
+    int2 id[kTile];
+    float2 sac[kSymWarps][sym_width<OP>()][kTile];  // (sum, Kahan compensation)
+    // differential: the warps' queues of near pairs (row << 8 | slot) and the target sums of those pairs
+    float2 tac[OP == OP_DIFF ? kSymWarps : 1][OP == OP_DIFF ? 10 : 1][OP == OP_DIFF ? kSection : 1];
+    unsigned short queue[OP == OP_DIFF ? kSymWarps : 1][OP == OP_DIFF ? kQueue : 1];
+    float box[kSymWarps][6];
+    int item;
+};
+
+struct SymSrc {
+    float q[3], m[3], e[3], T[3], Tm[3], ell;
+    int j1, j2;
+};
+
+template <int PREC, int OP, bool CHECK>
+__device__ __forceinline__ void sym_load(SymSrc &s, const SymSmem<PREC, OP> &tl, int j)
+{
+    const float4 a = tl.t0[j], b = tl.t1[j], c = tl.t2[j];
+    s.q[0] = a.x, s.q[1] = a.y, s.q[2] = a.z, s.ell = a.w;
+    s.e[0] = b.x, s.e[1] = b.y, s.e[2] = b.z, s.T[0] = b.w;
+    s.T[1] = c.x, s.T[2] = c.y;
+    if constexpr (PREC == PMIX) {
+        const float4 d = tl.t3[j];
+        s.m[0] = c.z, s.m[1] = c.w, s.m[2] = d.x;
+        s.Tm[0] = d.y, s.Tm[1] = d.z, s.Tm[2] = d.w;
+    } else {
+        s.m[0] = s.m[1] = s.m[2] = s.Tm[0] = s.Tm[1] = s.Tm[2] = 0.f;
     }
-    const float sw = (tw[0] + tw[3]) + (tw[1] + tw[2]);
-    const float sw0 = (tw0[0] + tw0[3]) + (tw0[1] + tw0[2]);
-    const float Wt = keep ? s.ell * sw : 0.f, W0t = keep ? s.ell * sw0 : 0.f;
-    const float Ws = keep ? t.ell * sw : 0.f, W0s = keep ? t.ell * sw0 : 0.f;
-    V3<float> dT = {t.T.x - s.T.x, t.T.y - s.T.y, t.T.z - s.T.z};
-    dT.x += t.Tl.x - s.Tm.x;
-    dT.y += t.Tl.y - s.Tm.y;
-    dT.z += t.Tl.z - s.Tm.z;
-    const float omt = 0.5f * dot3(dT, dT);
-    // differences of the double-float u records (exact difference form)
-    const float ddv[3] = {(tu.dh.x - su.dh.x) + (tu.dl.x - su.dl.x), (tu.dh.y - su.dh.y) + (tu.dl.y - su.dl.y),
-                          (tu.dh.z - su.dh.z) + (tu.dl.z - su.dl.z)};
-    const float dbv[3] = {(tu.uh.x - su.uh.x) + (tu.ul.x - su.ul.x), (tu.uh.y - su.uh.y) + (tu.ul.y - su.ul.y),
-                          (tu.uh.z - su.uh.z) + (tu.ul.z - su.ul.z)};
-    const float sdh[3] = {su.dh.x, su.dh.y, su.dh.z}, tdh[3] = {tu.dh.x, tu.dh.y, tu.dh.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        kahan_add(a.A1[k], a.C1[k], Wt * (ddv[k] + omt * sdh[k]));
-        kahan_add(a.A2[k], a.C2[k], W0t * dbv[k]);
-        hs[k] += Ws * (omt * tdh[k] - ddv[k]);
-        ls[k] -= W0s * dbv[k];
+    if constexpr (CHECK) {
+        const int2 v = tl.id[j];
+        s.j1 = v.x, s.j2 = v.y;
     }
 }
 
-// Staggered loop over one staged tile: lane l takes source (step + l) mod P, P = max(cnt, 32).
-// CHECK: the tile overlaps the targets' neighbour span (test disjointness per pair); DF: double-float
-// chords (every tile but the far ones); SRC: accumulate what the sources receive (off on the diagonal
-// item, which is a plain gather).
-template <int TPT, bool FAST, bool CHECK, bool DF, bool SRC>
-__device__ __forceinline__ void sym_tile(const Tgt<float> (&tg)[TPT], const UVal<float> (&tu)[TPT],
-                                         const bool (&valid)[TPT], const Tile<PMIX, true> &tl, int cnt,
-                                         Acc32<PMIX, OP_APPLY> (&a)[TPT], float2 (*sac)[kTile],
-                                         const KernelParams &kp)
+using L2 = float2;
+
+// Two target rows of a thread (rows of invalid lanes repeat the last one with length 0, so that they feed
+// nothing into the sources).
+struct SymTgt {
+    LV<L2> p, pl, e, T, Tl;
+    L2 ell;
+    int i1[2], i2[2], row[2];
+};
+
+// u data of the two rows (apply)
+struct SymTgtU {
+    LV<L2> dh, uh, dl, ul;
+};
+
+// ---------------------------------------------------------------------------------- per-pair bodies
+
+template <int PREC, int OP>
+struct SymAcc;
+template <int PREC>
+struct SymAcc<PREC, OP_ENERGY> {
+    L2 s[1], c[1];
+};
+template <int PREC>
+struct SymAcc<PREC, OP_DIFF> {
+    L2 s[10], c[10];
+};
+template <int PREC>
+struct SymAcc<PREC, OP_APPLY> {
+    L2 s[6], c[6];
+};
+
+// source accumulator += wx vx + wy vy, both compensated
+__device__ __forceinline__ void src_add(float2 &ac, L2 w, L2 v)
+{
+    l_kahan_fma(ac.x, ac.y, w.x, v.x);
+    l_kahan_fma(ac.x, ac.y, w.y, v.y);
+}
+
+template <int PREC, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &, const SymSmem<PREC, OP_ENERGY> &, const SymSrc &s,
+                                         int, int Jg, bool k0, bool k1, SymAcc<PREC, OP_ENERGY> &a, float2 *sac,
+                                         const SymArgs &pa, bool &, bool &)
+{
+    LV<L2> d[4];
+    l_chords<(MODE >= 1 && PREC == PMIX)>(t.p, t.pl, t.e, l_bc3<L2>(s.q[0], s.q[1], s.q[2]),
+                                          l_bc3<L2>(s.m[0], s.m[1], s.m[2]), l_bc3<L2>(s.e[0], s.e[1], s.e[2]), d);
+    const LV<L2> TJ = l_bc3<L2>(s.T[0], s.T[1], s.T[2]);
+    L2 cI[2] = {l_perp2(d[0], t.T), l_perp2(d[1], t.T)};
+    L2 cJ[2] = {l_perp2(d[0], TJ), l_perp2(d[2], TJ)};
+    L2 r[4], d11;
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+        const L2 d2 = l_dot(d[ab], d[ab]);
+        if (ab == 0) d11 = d2;
+        L2 r2;
+        r[ab] = l_pow45(d2, r2);
+    }
+    if constexpr (MODE == 2) {
+        const bool n0 = k0 && d11.x < pa.near2f, n1 = k1 && d11.y < pa.near2f;
+        if (n0 || n1) {
+            L2 c[4];
+            near_energy<L2, true>(pa.recF, pa.recLo, t.row[0], t.row[1], Jg, c);
+            cI[0] = make_float2(n0 ? c[0].x : cI[0].x, n1 ? c[0].y : cI[0].y);
+            cI[1] = make_float2(n0 ? c[1].x : cI[1].x, n1 ? c[1].y : cI[1].y);
+            cJ[0] = make_float2(n0 ? c[2].x : cJ[0].x, n1 ? c[2].y : cJ[0].y);
+            cJ[1] = make_float2(n0 ? c[3].x : cJ[1].x, n1 ? c[3].y : cJ[1].y);
+        }
+    }
+    L2 fI = l_energy_sum(cI[0], cI[1], r[0], r[1], r[2], r[3]);
+    if constexpr (CHECK) fI = l_keep(k0, k1, fI);
+    l_kahan_fma(a.s[0], a.c[0], l_bc<L2>(s.ell), fI);
+    L2 fJ = l_energy_sum(cJ[0], cJ[1], r[0], r[2], r[1], r[3]);
+    if constexpr (CHECK) fJ = l_keep(k0, k1, fJ);
+    float2 ac = *sac;
+    src_add(ac, t.ell, fJ);
+    *sac = ac;
+}
+
+template <int PREC, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &tu, const SymSmem<PREC, OP_APPLY> &tl,
+                                         const SymSrc &s, int j, int, bool k0, bool k1, SymAcc<PREC, OP_APPLY> &a,
+                                         float2 *sac, const SymArgs &, bool &, bool &)
+{
+    constexpr bool MIX = PREC == PMIX;
+    LV<L2> d[4];
+    l_chords<(MODE >= 1 && MIX)>(t.p, t.pl, t.e, l_bc3<L2>(s.q[0], s.q[1], s.q[2]), l_bc3<L2>(s.m[0], s.m[1], s.m[2]),
+                                 l_bc3<L2>(s.e[0], s.e[1], s.e[2]), d);
+    const LV<L2> TJ = l_bc3<L2>(s.T[0], s.T[1], s.T[2]);
+    const L2 cI1 = l_perp2(d[0], t.T), cI2 = l_perp2(d[1], t.T);
+    const L2 cJ1 = l_perp2(d[0], TJ), cJ2 = l_perp2(d[2], TJ);
+    L2 f[4], g[4];
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) f[ab] = l_pow25(l_dot(d[ab], d[ab]), g[ab]);
+    // (11 + 22) + (12 + 21): bitwise the same from row I and from row J
+    L2 sw = l_add(l_add(f[0], f[3]), l_add(f[1], f[2]));
+    L2 sw0 = l_add(l_fma(l_add(cI2, cJ2), g[3], l_mul(l_add(cI1, cJ1), g[0])),
+                   l_add(l_mul(l_add(cI2, cJ1), g[1]), l_mul(l_add(cI1, cJ2), g[2])));
+    if constexpr (CHECK) sw = l_keep(k0, k1, sw), sw0 = l_keep(k0, k1, sw0);
+    LV<L2> dT = l_sub3(t.T, TJ);
+    if constexpr (MIX) dT = l_add3(dT, l_sub3(t.Tl, l_bc3<L2>(s.Tm[0], s.Tm[1], s.Tm[2])));
+    const L2 omt = l_mul(l_bc<L2>(0.5f), l_dot(dT, dT));  // |T_I - T_J|^2 / 2
+    const float4 x = tl.u0[j], y = tl.u1[j];
+    const LV<L2> sdh = l_bc3<L2>(x.x, x.y, x.z);
+    LV<L2> dd = l_sub3(tu.dh, sdh), db = l_sub3(tu.uh, l_bc3<L2>(x.w, y.x, y.y));
+    if constexpr (MIX) {  // differences of the double-float u records
+        const float4 z = tl.u2[j];
+        dd = l_add3(dd, l_sub3(tu.dl, l_bc3<L2>(y.z, y.w, z.x)));
+        db = l_add3(db, l_sub3(tu.ul, l_bc3<L2>(z.y, z.z, z.w)));
+    }
+    const L2 Wt = l_mul(l_bc<L2>(s.ell), sw), W0t = l_mul(l_bc<L2>(s.ell), sw0);
+    l_kahan_fma(a.s[0], a.c[0], Wt, l_fma(omt, sdh.x, dd.x));
+    l_kahan_fma(a.s[1], a.c[1], Wt, l_fma(omt, sdh.y, dd.y));
+    l_kahan_fma(a.s[2], a.c[2], Wt, l_fma(omt, sdh.z, dd.z));
+    l_kahan_fma(a.s[3], a.c[3], W0t, db.x);
+    l_kahan_fma(a.s[4], a.c[4], W0t, db.y);
+    l_kahan_fma(a.s[5], a.c[5], W0t, db.z);
+    const L2 Ws = l_mul(t.ell, sw), W0s = l_neg(l_mul(t.ell, sw0));
+    const L2 v[6] = {l_fma(omt, tu.dh.x, l_neg(dd.x)), l_fma(omt, tu.dh.y, l_neg(dd.y)), l_fma(omt, tu.dh.z, l_neg(dd.z)),
+                     db.x, db.y, db.z};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        float2 ac = sac[q * kTile];
+        src_add(ac, q < 3 ? Ws : W0s, v[q]);
+        sac[q * kTile] = ac;
+    }
+}
+
+template <int PREC, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &, const SymSmem<PREC, OP_DIFF> &, const SymSrc &s,
+                                         int, int, bool k0, bool k1, SymAcc<PREC, OP_DIFF> &a, float2 *sac,
+                                         const SymArgs &pa, bool &n0, bool &n1)
+{
+    LV<L2> d[4];
+    l_chords<(MODE >= 1)>(t.p, t.pl, t.e, l_bc3<L2>(s.q[0], s.q[1], s.q[2]), l_bc3<L2>(s.m[0], s.m[1], s.m[2]),
+                          l_bc3<L2>(s.e[0], s.e[1], s.e[2]), d);
+    const LV<L2> TJ = l_bc3<L2>(s.T[0], s.T[1], s.T[2]), TJl = l_bc3<L2>(s.Tm[0], s.Tm[1], s.Tm[2]);
+    // both tangents double-float: each is the target tangent of one of the two rows
+    L2 tI[2], tJ[2], cI[2], cJ[2];
+    LV<L2> pI[2], pJ[2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        cI[b] = l_perp2_df(d[b], t.T, t.Tl, tI[b], pI[b]);
+        cJ[b] = l_perp2_df(d[2 * b], TJ, TJl, tJ[b], pJ[b]);
+    }
+    const L2 d11 = l_dot(d[0], d[0]);
+    if constexpr (MODE == 2) {
+        n0 = k0 && d11.x < pa.near2f;
+        n1 = k1 && d11.y < pa.near2f;
+    }
+    const bool m0 = k0 && !n0, m1 = k1 && !n1;  // pairs of the FP32 sums
+    L2 S, G[2][3], H[2][3], GT[3], HT[3];
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+        const int ia = ab >> 1, jb = ab & 1;
+        L2 d2 = ab == 0 ? d11 : l_dot(d[ab], d[ab]);
+        if constexpr (CHECK || MODE == 2) d2 = make_float2(m0 ? d2.x : 1.f, m1 ? d2.y : 1.f);
+        L2 r2;
+        L2 rb = l_pow45(d2, r2);
+        if constexpr (CHECK || MODE == 2) rb = l_keep(m0, m1, rb);
+        const L2 fs = l_fma(cJ[ia], rb, l_mul(cI[jb], rb));
+        const L2 al = l_add(rb, rb);  // alpha |d|^-beta
+        const L2 cb = l_neg(l_mul(l_mul(l_bc<L2>(4.5f), fs), r2));
+        const L2 mI = l_neg(l_mul(al, ia ? l_add(tI[jb], t.ell) : tI[jb]));
+        const L2 mJ = l_neg(l_mul(al, jb ? l_sub(tJ[ia], l_bc<L2>(s.ell)) : tJ[ia]));
+        const L2 dv[3] = {d[ab].x, d[ab].y, d[ab].z};
+        const LV<L2> ps = l_add3(pI[jb], pJ[ia]);
+        const L2 pv[3] = {ps.x, ps.y, ps.z};
+        S = ab == 0 ? fs : l_add(S, fs);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const L2 v = l_fma(al, pv[k], l_mul(cb, dv[k]));
+            G[ia][k] = jb ? l_add(G[ia][k], v) : v;
+            H[jb][k] = ia ? l_sub(H[jb][k], v) : l_neg(v);
+            GT[k] = ab == 0 ? l_mul(mI, dv[k]) : l_fma(mI, dv[k], GT[k]);
+            HT[k] = ab == 0 ? l_mul(mJ, dv[k]) : l_fma(mJ, dv[k], HT[k]);
+        }
+    }
+    const L2 L = l_bc<L2>(s.ell);
+    l_kahan_fma(a.s[0], a.c[0], L, S);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        l_kahan_fma(a.s[1 + k], a.c[1 + k], L, G[0][k]);
+        l_kahan_fma(a.s[4 + k], a.c[4 + k], L, G[1][k]);
+        l_kahan_fma(a.s[7 + k], a.c[7 + k], L, GT[k]);
+    }
+#pragma unroll
+    for (int q = 0; q < 10; ++q) {
+        float2 ac = sac[q * kTile];
+        src_add(ac, t.ell, q == 0 ? S : (q < 4 ? H[0][(q + 2) % 3] : (q < 7 ? H[1][(q + 2) % 3] : HT[(q + 2) % 3])));
+        sac[q * kTile] = ac;
+    }
+}
+
+// Place of tile row j in the shared arrays: even rows first, so that the rows step + 2 lane of a warp are
+// consecutive.
+__device__ __forceinline__ int sym_slot(int j) { return ((j & 1) << 6) | (j >> 1); }
+
+// Evaluate up to 64 near pairs of the differential from a warp's queue, two per lane, into the warp's target and
+// source sums.  Near pairs held back this way fill all lanes: on short curves every step has a few lanes
+// near another strand, and evaluated in place each of them cost the warp a whole double-float pair.  Pairs of
+// one batch that share a row add in queue order, one at a time.
+static __device__ __noinline__ void sym_near_flush(SymSmem<PMIX, OP_DIFF> &sm, int wid, int first, int count, int tgt0, int ntgt,
+                                                   int s0, const SymArgs &pa)
 {
     const int lane = threadIdx.x & 31;
-    const int P = max(cnt, 32);
-    for (int step = 0; step < P; ++step) {
-        int j = step + lane;
+    int row[2], at[2], I[2], J[2];
+    bool on[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int e = 32 * k + lane;
+        on[k] = e < count;
+        const int v = on[k] ? sm.queue[wid][first + e] : sm.queue[wid][first];
+        row[k] = v >> 8;
+        at[k] = v & 0xff;
+        const int loc = kSection * wid + row[k];
+        on[k] = on[k] && loc < ntgt;
+        I[k] = tgt0 + min(loc, ntgt - 1);
+        J[k] = s0 + (((at[k] & 63) << 1) | (at[k] >> 6));
+    }
+    dfl<L2> x[10], y[10];
+    near_diff<L2>(pa.recF, pa.recLo, I[0], I[1], J[0], J[1], x, y);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const unsigned live = __ballot_sync(0xffffffffu, on[k]);
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const int key = on[k] ? (side ? at[k] : row[k]) : 256 + lane;
+            const unsigned same = __match_any_sync(0xffffffffu, key) & live;
+            const int rank = __popc(same & ((1u << lane) - 1));
+            const int rounds = __reduce_max_sync(0xffffffffu, on[k] ? rank + 1 : 0);
+            for (int r = 0; r < rounds; ++r) {
+                if (on[k] && rank == r) {
+                    float2 *ac = side ? &sm.sac[wid][0][at[k]] : &sm.tac[wid][0][row[k]];
+#pragma unroll
+                    for (int q = 0; q < 10; ++q, ac += side ? kTile : kSection) {
+                        const dfl<L2> v = side ? y[q] : x[q];
+                        float2 t = *ac;
+                        l_kahan_df(t.x, t.y, k ? v.hi.y : v.hi.x, k ? v.lo.y : v.lo.x);
+                        *ac = t;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+}
+
+// Staggered loop of one warp over sources [j0, j0 + cnt) of the staged tile (global rows s0 + j).
+// CHECK: some pair may share a vertex; MODE 2: near pairs possible, 1: double-float chords, 0: single-float
+// chords (far tiles).  OWN: the sources are the warp's own 64 rows; each unordered pair once, by the row that
+// sees the other at most half the circle of 64 ahead.
+template <int PREC, int OP, bool CHECK, int MODE, bool OWN>
+__device__ __forceinline__ void sym_section(const SymTgt &t, const SymTgtU &tu, SymSmem<PREC, OP> &sm, int wid, int s0,
+                                            int j0, int cnt, SymAcc<PREC, OP> &a, int &queued, const WorkItem &w,
+                                            const SymArgs &pa)
+{
+    constexpr bool QUEUE = OP == OP_DIFF && MODE == 2;
+    const int lane = threadIdx.x & 31;
+    const int P = OWN ? kSection : max((cnt + 1) & ~1, kSection), n = OWN ? kSection / 2 + 2 : P;
+    for (int step = OWN ? 1 : 0; step < n; ++step) {
+        int j = step + 2 * lane;
         if (j >= P) j -= P;
+        const int at = sym_slot(j + j0);
+        bool n0 = false, n1 = false;
         if (j < cnt) {
-            Src<PMIX> s;
-            load_source<PMIX, true>(s, tl, j);
-            UVal<float> su;
-            {
-                const float4 x = tl.u[j].a, y = tl.u[j].b, z = tl.u[j].c;
-                su.dh = {x.x, x.y, x.z};
-                su.uh = {x.w, y.x, y.y};
-                su.dl = {y.z, y.w, z.x};
-                su.ul = {z.y, z.z, z.w};
+            j += j0;
+            SymSrc s;
+            sym_load<PREC, OP, CHECK>(s, sm, at);
+            bool k0 = true, k1 = true;
+            if constexpr (CHECK) {
+                k0 = (s.j1 != t.i1[0]) & (s.j1 != t.i2[0]) & (s.j2 != t.i1[0]) & (s.j2 != t.i2[0]);
+                k1 = (s.j1 != t.i1[1]) & (s.j1 != t.i2[1]) & (s.j2 != t.i1[1]) & (s.j2 != t.i2[1]);
             }
-            float hs[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) {
-                bool keep = valid[k];
-                if constexpr (CHECK)
-                    keep = keep & (s.j1 != tg[k].i1) & (s.j1 != tg[k].i2) & (s.j2 != tg[k].i1) & (s.j2 != tg[k].i2);
-                pair_apply_both<FAST, DF>(tg[k], s, tu[k], su, keep, kp, a[k], hs, ls);
+            if constexpr (OWN) {  // row 2 lane is `step` behind the source, row 2 lane + 1 is step - 1 behind
+                k0 = k0 & (step < 32 || (step == 32 && lane < 16));
+                k1 = k1 & (step > 1) & (step < 33 || lane < 16);
             }
-            if constexpr (SRC) {
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    float2 h = sac[q][j], l = sac[3 + q][j];  // (sum, Kahan compensation)
-                    kahan_add(h.x, h.y, hs[q]);
-                    kahan_add(l.x, l.y, ls[q]);
-                    sac[q][j] = h;
-                    sac[3 + q][j] = l;
+            sym_pair<PREC, CHECK, MODE>(t, tu, sm, s, at, s0 + j, k0, k1, a, &sm.sac[wid][0][at], pa, n0, n1);
+        }
+        __syncwarp();  // the next step hands this lane's source on
+        if constexpr (QUEUE) {
+            const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
+            if (b0 | b1) {
+                const unsigned lt = (1u << lane) - 1;
+                if (n0) sm.queue[wid][queued + __popc(b0 & lt)] = (unsigned short)((2 * lane) << 8 | at);
+                if (n1) sm.queue[wid][queued + __popc(b0) + __popc(b1 & lt)] = (unsigned short)((2 * lane + 1) << 8 | at);
+                queued += __popc(b0) + __popc(b1);
+                __syncwarp();
+                if (queued >= 64) {  // the last 64; the rest stays queued
+                    queued -= 64;
+                    sym_near_flush(sm, wid, queued, 64, w.tgt0, w.ntgt, s0, pa);
                 }
             }
         }
-        if constexpr (SRC) __syncwarp();  // the next step hands this lane's source to lane - 1
     }
 }
 
-template <int TPT, bool FAST>
-__global__ void __launch_bounds__(kThreads, 2) k_pairs_sym(const PairArgs pa)
+template <int PREC, int OP, int MB>
+__global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
 {
-    __shared__ Tile<PMIX, true> tl;
-    __shared__ float2 sac[kSymWarps][6][kTile];  // per warp and source: (sum, Kahan compensation)
-    __shared__ int s_item;
-    __shared__ float s_box[2][kThreads / 32][6];
+    constexpr int W = sym_width<OP>();
+    constexpr bool MIX = PREC == PMIX, NEAR = MIX && OP != OP_APPLY;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    SymSmem<PREC, OP> &sm = *reinterpret_cast<SymSmem<PREC, OP> *>(dyn);
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(pa.counter, 1);
+        if (threadIdx.x == 0) sm.item = atomicAdd(pa.counter, 1);
         __syncthreads();
-        const int it = s_item;
+        const int it = sm.item;
         __syncthreads();
         if (it >= pa.n_items) break;
         const WorkItem w = pa.items[it];
         if (pa.skip && pa.skip[w.pad]) continue;  // problem already converged
-        const int bslot = w.slot >> 16, cslot = w.slot & 0xffff;
-        const bool diag = bslot == cslot;
-        Tgt<float> tg[TPT];
-        UVal<float> tu[TPT];
-        bool valid[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            const int loc = threadIdx.x + k * kThreads;
-            valid[k] = loc < w.ntgt;  // clamped duplicates must not feed the source side
-            const int I = w.tgt0 + min(loc, w.ntgt - 1);
-            load_target<PMIX>(tg[k], I, pa.recF, pa.recLo, pa.recD);
-            load_uval<PMIX>(tu[k], pa.urecF, pa.urecD, I);
-        }
-        Acc64<OP_APPLY> A[TPT];
-        Acc32<PMIX, OP_APPLY> a[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            acc64_zero<OP_APPLY>(A[k]);
-            acc_zero<PMIX, OP_APPLY>(a[k]);
-        }
-        float tbox[6];
+        const int X = w.slot >> 16, tslot = w.slot & 0xffff;
+        const bool diag = w.src0 < w.tgt0 + w.ntgt;  // a tile of its own super-block
+        SymTgt t;
+        SymTgtU tu;
+        float tbox[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
         {
-            float b[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
+            RecF r[2];
+            RecLo q[2];
+            URecF u[2];
+            bool valid[2];
 #pragma unroll
-            for (int k = 0; k < TPT; ++k) box_add(b, tg[k].p1, tg[k].p2);
+            for (int k = 0; k < 2; ++k) {
+                const int loc = kSection * wid + 2 * lane + k;
+                valid[k] = loc < w.ntgt;
+                const int I = w.tgt0 + min(loc, w.ntgt - 1);
+                t.row[k] = I;
+                r[k] = pa.recF[I];
+                if constexpr (MIX) q[k] = pa.recLo[I];
+                if constexpr (OP == OP_APPLY) u[k] = pa.urecF[I];
+                t.i1[k] = __float_as_int(r[k].c.z);
+                t.i2[k] = __float_as_int(r[k].c.w);
+                if constexpr (MIX)
+                    box_add(tbox, V3<float>{r[k].a.x, r[k].a.y, r[k].a.z}, V3<float>{r[k].b.x, r[k].b.y, r[k].b.z});
+            }
+#define TPE_L2(field) make_float2(r[0].field, r[1].field)
+#define TPE_Q2(field) make_float2(q[0].field, q[1].field)
+#define TPE_U2(field) make_float2(u[0].field, u[1].field)
+            t.p = {TPE_L2(a.x), TPE_L2(a.y), TPE_L2(a.z)};
+            t.T = {TPE_L2(b.w), TPE_L2(c.x), TPE_L2(c.y)};
+            t.ell = make_float2(valid[0] ? r[0].a.w : 0.f, valid[1] ? r[1].a.w : 0.f);
+            if constexpr (MIX) {
+                t.pl = {TPE_Q2(lo.x), TPE_Q2(lo.y), TPE_Q2(lo.z)};
+                t.Tl = {TPE_Q2(lo2.z), TPE_Q2(lo2.w), TPE_Q2(lo3.x)};
+                t.e = {TPE_Q2(lo3.y), TPE_Q2(lo3.z), TPE_Q2(lo3.w)};
+            } else {
+                t.e = l_sub3(LV<L2>{TPE_L2(b.x), TPE_L2(b.y), TPE_L2(b.z)}, t.p);
+            }
+            if constexpr (OP == OP_APPLY) {
+                tu.dh = {TPE_U2(a.x), TPE_U2(a.y), TPE_U2(a.z)};
+                tu.uh = {TPE_U2(a.w), TPE_U2(b.x), TPE_U2(b.y)};
+                if constexpr (MIX) {
+                    tu.dl = {TPE_U2(b.z), TPE_U2(b.w), TPE_U2(c.x)};
+                    tu.ul = {TPE_U2(c.y), TPE_U2(c.z), TPE_U2(c.w)};
+                }
+            }
+#undef TPE_L2
+#undef TPE_Q2
+#undef TPE_U2
+        }
+        if constexpr (MIX) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
-                for (int q = 0; q < 6; ++q) {
-                    const float v = __shfl_xor_sync(0xffffffffu, b[q], o);
-                    b[q] = q < 3 ? fminf(b[q], v) : fmaxf(b[q], v);
+                for (int k = 0; k < 6; ++k) {
+                    const float v = __shfl_xor_sync(0xffffffffu, tbox[k], o);
+                    tbox[k] = k < 3 ? fminf(tbox[k], v) : fmaxf(tbox[k], v);
                 }
-            for (int q = 0; q < 6; ++q) tbox[q] = b[q];
         }
-        for (int s0 = w.src0; s0 < w.src1; s0 += kTile) {
+        SymAcc<PREC, OP> a;
+#pragma unroll
+        for (int k = 0; k < W; ++k) a.s[k] = a.c[k] = make_float2(0.f, 0.f);
+        const bool have = kSection * wid < w.ntgt;  // this warp has target rows
+        int queued = 0;                             // near pairs held back
+        if constexpr (OP == OP_DIFF)
+            for (int q = 0; q < W; ++q)
+                for (int j = lane; j < kSection; j += 32) sm.tac[wid][q][j] = make_float2(0.f, 0.f);
+        for (int s0 = w.src0, tile = 0; s0 < w.src1; s0 += kTile, ++tile) {
             const int cnt = min(kTile, w.src1 - s0);
             __syncthreads();  // the previous tile's readers are done
             float sb[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
             if (threadIdx.x < cnt) {
-                const int J = s0 + threadIdx.x;
+                const int J = s0 + threadIdx.x, j = sym_slot(threadIdx.x);
                 const RecF r = pa.recF[J];
-                tl.r[threadIdx.x] = r;
-                tl.lo[threadIdx.x] = pa.recLo[J];
-                tl.u[threadIdx.x] = pa.urecF[J];
-                box_add(sb, V3<float>{r.a.x, r.a.y, r.a.z}, V3<float>{r.b.x, r.b.y, r.b.z});
-            }
-            for (int t = lane; t < kTile; t += 32)
-                for (int q = 0; q < 6; ++q) sac[wid][q][t] = make_float2(0.f, 0.f);
-            block_box(sb, s_box[1]);  // contains the barrier that publishes the tile
-            const bool check = !(s0 + cnt - 1 < w.nb_lo || s0 > w.nb_hi);
-            float g2 = 0.f;
-            for (int q = 0; q < 3; ++q) {
-                const float gap = fmaxf(fmaxf(sb[q] - tbox[3 + q], tbox[q] - sb[3 + q]), 0.f);
-                g2 += gap * gap;
-            }
-            const bool far = g2 >= pa.kp.mid2f;
-            if (diag) {
-                sym_tile<TPT, FAST, true, true, false>(tg, tu, valid, tl, cnt, a, sac[wid], pa.kp);
-            } else if (check) {
-                sym_tile<TPT, FAST, true, true, true>(tg, tu, valid, tl, cnt, a, sac[wid], pa.kp);
-            } else if (!far) {
-                sym_tile<TPT, FAST, false, true, true>(tg, tu, valid, tl, cnt, a, sac[wid], pa.kp);
-            } else {
-                sym_tile<TPT, FAST, false, false, true>(tg, tu, valid, tl, cnt, a, sac[wid], pa.kp);
-            }
-            // fold the target tile accumulators into FP64
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) {
-                acc_add(A[k], a[k]);
-                acc_zero<PMIX, OP_APPLY>(a[k]);
-            }
-            if (!diag) {
-                __syncthreads();  // every warp's source accumulators are complete
-                if (threadIdx.x < cnt) {
-                    const int J = s0 + threadIdx.x;
-                    double v[6];
-                    for (int q = 0; q < 6; ++q) {
-                        double x = 0.0;
-                        for (int wv = 0; wv < kSymWarps; ++wv)
-                            x += (double)sac[wv][q][threadIdx.x].x - (double)sac[wv][q][threadIdx.x].y;
-                        v[q] = x;
-                    }
-                    const double l = pa.na.ell[J];
-                    double *o = pa.part + ((size_t)bslot * pa.nE + J) * 6;
-                    for (int q = 0; q < 3; ++q) {
-                        o[q] = 0.5 * v[q];
-                        o[3 + q] = 0.125 * l * v[3 + q];
-                    }
+                sm.t0[j] = r.a;
+                sm.id[j] = make_int2(__float_as_int(r.c.z), __float_as_int(r.c.w));
+                if constexpr (MIX) {
+                    const RecLo q = pa.recLo[J];
+                    sm.t1[j] = make_float4(q.lo3.y, q.lo3.z, q.lo3.w, r.b.w);
+                    sm.t2[j] = make_float4(r.c.x, r.c.y, q.lo.x, q.lo.y);
+                    sm.t3[j] = make_float4(q.lo.z, q.lo2.z, q.lo2.w, q.lo3.x);
+                    box_add(sb, V3<float>{r.a.x, r.a.y, r.a.z}, V3<float>{r.b.x, r.b.y, r.b.z});
+                } else {
+                    sm.t1[j] = make_float4(r.b.x - r.a.x, r.b.y - r.a.y, r.b.z - r.a.z, r.b.w);
+                    sm.t2[j] = make_float4(r.c.x, r.c.y, 0.f, 0.f);
+                }
+                if constexpr (OP == OP_APPLY) {
+                    const URecF u = pa.urecF[J];
+                    sm.u0[j] = u.a;
+                    sm.u1[j] = u.b;
+                    if constexpr (MIX) sm.u2[j] = u.c;
                 }
             }
-        }
-        // target rows of block b: slot c
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            if (!valid[k]) continue;
-            const int I = w.tgt0 + threadIdx.x + k * kThreads;
-            const double l = pa.na.ell[I];
-            double *o = pa.part + ((size_t)cslot * pa.nE + I) * 6;
-            for (int q = 0; q < 3; ++q) {
-                o[q] = 0.5 * A[k].A1[q];
-                o[3 + q] = 0.125 * l * A[k].A2[q];
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------- symmetric energy
-
-// One unordered pair of the energy: the target row receives l_J sum_ab |T_I x d_ab|^alpha |d_ab|^-beta,
-// the source row l_I sum_ab |T_J x d_ab|^alpha |d_ab|^-beta (Eqs. 17-18; the factor l_I / 4 of a row
-// is applied when the rows are summed).  Near pairs take both |T x d|^2 in FP64.
-template <bool FAST, bool DF>
-__device__ __forceinline__ void pair_energy_both(const Tgt<float> &t, const Src<PMIX> &s, bool keep, bool near,
-                                                 const KernelParams &kp, float &at, float &as)
-{
-    const float alpha = (float)kp.alpha, beta = (float)kp.beta;
-    V3<float> dd[4];
-    chords<DF>(t, s, dd);
-    float tt;
-    V3<float> dp;
-    float cI[2] = {perp2(dd[0], t.T, tt, dp), perp2(dd[1], t.T, tt, dp)};  // depends on b only
-    float cJ[2] = {perp2(dd[0], s.T, tt, dp), perp2(dd[2], s.T, tt, dp)};  // depends on a only
-    if constexpr (DF)
-        if (near) {
-            cI[0] = perp2_near(t.p1, t.l1, s.q1, s.m1, t.T, t.Tl);
-            cI[1] = perp2_near(t.p1, t.l1, s.q2, s.m2, t.T, t.Tl);
-            cJ[0] = perp2_near(t.p1, t.l1, s.q1, s.m1, s.T, s.Tm);
-            cJ[1] = perp2_near(t.p2, t.l2, s.q1, s.m1, s.T, s.Tm);
-        }
-    const float pI[2] = {pow_c<float, FAST>(cI[0], alpha), pow_c<float, FAST>(cI[1], alpha)};
-    const float pJ[2] = {pow_c<float, FAST>(cJ[0], alpha), pow_c<float, FAST>(cJ[1], alpha)};
-    float fI = 0.f, fJ = 0.f;
-#pragma unroll
-    for (int ab = 0; ab < 4; ++ab) {
-        const float d2 = dot3(dd[ab], dd[ab]);
-        float r2;
-        const float rb = inv_pow<float, FAST, 0>(d2, beta, r2);
-        fI += pI[ab & 1] * rb;
-        fJ += pJ[ab >> 1] * rb;
-    }
-    at += keep ? s.ell * fI : 0.f;
-    as += keep ? t.ell * fJ : 0.f;
-}
-
-// MODE 2: near pairs possible (|g_i1 - g_j1|^2 < near cutoff^2 take FP64 cross products); 1: double-float
-// chords; 0: single-float chords (far tiles).
-template <int TPT, bool FAST, bool CHECK, int MODE, bool SRC>
-__device__ __forceinline__ void sym_energy_tile(const Tgt<float> (&tg)[TPT], const bool (&valid)[TPT],
-                                                const Tile<PMIX, false> &tl, int cnt, float (&at)[TPT],
-                                                float2 *sac, const KernelParams &kp)
-{
-    const int lane = threadIdx.x & 31;
-    const int P = max(cnt, 32);
-    for (int step = 0; step < P; ++step) {
-        int j = step + lane;
-        if (j >= P) j -= P;
-        if (j < cnt) {
-            Src<PMIX> s;
-            load_source<PMIX, false>(s, tl, j);
-            float as = 0.f;
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) {
-                bool keep = valid[k];
-                if constexpr (CHECK)
-                    keep = keep & (s.j1 != tg[k].i1) & (s.j1 != tg[k].i2) & (s.j2 != tg[k].i1) & (s.j2 != tg[k].i2);
-                bool near = false;
-                if constexpr (MODE == 2) {
-                    const V3<float> e = diff3<true>(tg[k].p1, tg[k].l1, s.q1, s.m1);
-                    near = keep && dot3(e, e) < kp.near2f;
-                }
-                pair_energy_both<FAST, (MODE >= 1)>(tg[k], s, keep, near, kp, at[k], as);
-            }
-            if constexpr (SRC) {
-                float2 ac = sac[j];  // (sum, Kahan compensation)
-                kahan_add(ac.x, ac.y, as);
-                sac[j] = ac;
-            }
-        }
-        if constexpr (SRC) __syncwarp();
-    }
-}
-
-template <int TPT, bool FAST>
-__global__ void __launch_bounds__(kThreads, 3) k_energy_sym(const PairArgs pa)
-{
-    __shared__ Tile<PMIX, false> tl;
-    __shared__ float2 sac[kSymWarps][kTile];  // per warp and source: (sum, Kahan compensation)
-    __shared__ int s_item;
-    __shared__ float s_box[2][kThreads / 32][6];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(pa.counter, 1);
-        __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it >= pa.n_items) break;
-        const WorkItem w = pa.items[it];
-        const int bslot = w.slot >> 16, cslot = w.slot & 0xffff;
-        const bool diag = bslot == cslot;
-        Tgt<float> tg[TPT];
-        bool valid[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            const int loc = threadIdx.x + k * kThreads;
-            valid[k] = loc < w.ntgt;
-            load_target<PMIX>(tg[k], w.tgt0 + min(loc, w.ntgt - 1), pa.recF, pa.recLo, pa.recD);
-        }
-        double A[TPT];
-        float at[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) A[k] = 0.0;
-        float tbox[6];
-        {
-            float b[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) box_add(b, tg[k].p1, tg[k].p2);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                for (int q = 0; q < 6; ++q) {
-                    const float v = __shfl_xor_sync(0xffffffffu, b[q], o);
-                    b[q] = q < 3 ? fminf(b[q], v) : fmaxf(b[q], v);
-                }
-            for (int q = 0; q < 6; ++q) tbox[q] = b[q];
-        }
-        for (int s0 = w.src0; s0 < w.src1; s0 += kTile) {
-            const int cnt = min(kTile, w.src1 - s0);
-            __syncthreads();
-            float sb[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
-            if (threadIdx.x < cnt) {
-                const int J = s0 + threadIdx.x;
-                const RecF r = pa.recF[J];
-                tl.r[threadIdx.x] = r;
-                tl.lo[threadIdx.x] = pa.recLo[J];
-                box_add(sb, V3<float>{r.a.x, r.a.y, r.a.z}, V3<float>{r.b.x, r.b.y, r.b.z});
-            }
-            for (int t = lane; t < kTile; t += 32) sac[wid][t] = make_float2(0.f, 0.f);
-            block_box(sb, s_box[1]);
-            const bool check = !(s0 + cnt - 1 < w.nb_lo || s0 > w.nb_hi);
-            float g2 = 0.f;
-            for (int q = 0; q < 3; ++q) {
-                const float gap = fmaxf(fmaxf(sb[q] - tbox[3 + q], tbox[q] - sb[3 + q]), 0.f);
-                g2 += gap * gap;
-            }
-            const int mode = g2 < pa.kp.near2f ? 2 : (g2 < pa.kp.mid2f ? 1 : 0);
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) at[k] = 0.f;
-            if (diag)
-                sym_energy_tile<TPT, FAST, true, 2, false>(tg, valid, tl, cnt, at, sac[wid], pa.kp);
-            else if (check || mode == 2)
-                sym_energy_tile<TPT, FAST, true, 2, true>(tg, valid, tl, cnt, at, sac[wid], pa.kp);
-            else if (mode == 1)
-                sym_energy_tile<TPT, FAST, false, 1, true>(tg, valid, tl, cnt, at, sac[wid], pa.kp);
+            for (int q = 0; q < W; ++q)
+                for (int j = lane; j < kTile; j += 32) sm.sac[wid][q][j] = make_float2(0.f, 0.f);
+            if constexpr (MIX)
+                block_box(sb, sm.box);  // contains the barrier that publishes the tile
             else
-                sym_energy_tile<TPT, FAST, false, 0, true>(tg, valid, tl, cnt, at, sac[wid], pa.kp);
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) A[k] += (double)at[k];
-            if (!diag) {
                 __syncthreads();
-                if (threadIdx.x < cnt) {
-                    double x = 0.0;
-                    for (int wv = 0; wv < kSymWarps; ++wv) x += (double)sac[wv][threadIdx.x].x - (double)sac[wv][threadIdx.x].y;
-                    pa.part[(size_t)bslot * pa.nE + s0 + threadIdx.x] = x;
+            int mode = 1;
+            if constexpr (MIX) {
+                float g2 = 0.f;
+                for (int q = 0; q < 3; ++q) {
+                    const float gap = fmaxf(fmaxf(sb[q] - tbox[3 + q], tbox[q] - sb[3 + q]), 0.f);
+                    g2 += gap * gap;
+                }
+                mode = (NEAR && g2 < pa.near2f) ? 2 : (g2 < pa.mid2f ? 1 : 0);
+            }
+            constexpr int MN = NEAR ? 2 : 1;
+            if (diag) {
+                // the super-block's 64-row sections: a warp takes its own, and of the six pairs of sections one
+                // or two (odd warps also the section before theirs), at most 97 steps per tile
+                if (have) {
+                    const int sec = (s0 - w.tgt0) / kSection;
+                    if ((wid & 2) == sec) {
+                        sym_section<PREC, OP, true, MN, true>(t, tu, sm, wid, s0, kSection * (wid & 1),
+                                                              min(kSection, w.ntgt - kSection * wid), a, queued, w, pa);
+                        if (wid & 1) sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, 0, kSection, a, queued, w, pa);
+                    } else {
+                        const int g = wid >= 2 ? wid - 2 : 3 - wid, gc = min(kSection, w.ntgt - kSection * g);
+                        if (gc > 0)
+                            sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, kSection * (g - sec), gc, a, queued, w,
+                                                                   pa);
+                    }
+                }
+            } else if (have) {
+                if (((w.nb_lo >> tile) & 1) || mode == 2)
+                    sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
+                else if (mode == 1 || !MIX)
+                    sym_section<PREC, OP, false, 1, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
+                else
+                    sym_section<PREC, OP, false, 0, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
+            }
+            if constexpr (OP == OP_DIFF) {
+                if (queued) sym_near_flush(sm, wid, 0, queued, w.tgt0, w.ntgt, s0, pa);
+                queued = 0;
+            }
+            __syncthreads();  // every warp's source accumulators are complete
+            if (threadIdx.x < cnt) {
+                float2 *o = pa.part + ((size_t)X * pa.nE + s0 + threadIdx.x) * W;
+#pragma unroll
+                for (int q = 0; q < W; ++q) {
+                    const int at = sym_slot(threadIdx.x);
+                    float2 x = sm.sac[0][q][at];
+                    float lo = -x.y;
+#pragma unroll
+                    for (int wv = 1; wv < kSymWarps; ++wv) {
+                        const float2 y = sm.sac[wv][q][at];
+                        const df s = two_sum(x.x, y.x);
+                        x.x = s.hi;
+                        lo = __fadd_rn(lo, __fsub_rn(s.lo, y.y));
+                    }
+                    o[q] = make_float2(x.x, lo);
                 }
             }
         }
 #pragma unroll
-        for (int k = 0; k < TPT; ++k)
-            if (valid[k]) pa.part[(size_t)cslot * pa.nE + w.tgt0 + threadIdx.x + k * kThreads] = A[k];
-    }
-}
-
-// ---------------------------------------------------------------------------------- symmetric differential
-//
-// Row I accumulates (scaled by l_J) S = sum (f_I + f_J), G_a += v_ab, GT += -a_I (T_I . d_ab) d_ab, with
-// v_ab = d(f_I + f_J)/dd at d_ab = g_ia - g_jb.  Row J sees d' = -d and accumulates (scaled by l_I) the
-// same S, G_b -= v_ab (its endpoint b) and GT += -a_J (T_J . d_ab) d_ab.  Both tangents are double-float
-// in |T x d|^2 and T . d (each is the target tangent of one of the two rows).
-
-// source-side accumulator slots: 0 S, 1-3 G1, 4-6 G2, 7-9 GT
-constexpr int kDS = 10;
-
-template <bool FAST, bool DF>
-__device__ __forceinline__ void pair_diff_both(const Tgt<float> &t, const Src<PMIX> &s, bool keep,
-                                               const KernelParams &kp, Acc32<PMIX, OP_DIFF> &a,
-                                               float (&src)[kDS])
-{
-    const float alpha = (float)kp.alpha, beta = (float)kp.beta;
-    V3<float> dd[4];
-    chords<DF>(t, s, dd);
-    float tI[2], tJ[2], cI[2], cJ[2];
-    V3<float> dpI[2], dpJ[2];
+        for (int k = 0; k < 2; ++k) {
+            const int loc = kSection * wid + 2 * lane + k;
+            if (loc >= w.ntgt) continue;
+            float2 *o = pa.part + ((size_t)tslot * pa.nE + w.tgt0 + loc) * W;
+            if constexpr (OP == OP_DIFF) {
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        cI[b] = perp2_df(dd[b], t.T, t.Tl, tI[b], dpI[b]);
-        cJ[b] = perp2_df(dd[2 * b], s.T, s.Tm, tJ[b], dpJ[b]);
-    }
-    float S = 0.f, G1[3] = {0, 0, 0}, G2[3] = {0, 0, 0}, GT[3] = {0, 0, 0};
-    float H1[3] = {0, 0, 0}, H2[3] = {0, 0, 0}, HT[3] = {0, 0, 0};
+                for (int q = 0; q < W; ++q) {
+                    const float2 v = sm.tac[wid][q][2 * lane + k];
+                    if (k)
+                        l_kahan_df(a.s[q].y, a.c[q].y, v.x, -v.y);
+                    else
+                        l_kahan_df(a.s[q].x, a.c[q].x, v.x, -v.y);
+                }
+            }
 #pragma unroll
-    for (int ab = 0; ab < 4; ++ab) {
-        const int ia = ab >> 1, jb = ab & 1;
-        const V3<float> d = dd[ab];
-        const float d2 = dot3(d, d);
-        float r2;
-        const float rb = inv_pow<float, FAST, 0>(d2, beta, r2);
-        float fI, fJ, aI, aJ;
-        if constexpr (FAST) {
-            fI = cI[jb] * rb;
-            fJ = cJ[ia] * rb;
-            aI = aJ = 2.f * rb;
-        } else {
-            fI = pow_c<float, false>(cI[jb], alpha) * rb;
-            fJ = pow_c<float, false>(cJ[ia], alpha) * rb;
-            aI = cI[jb] > 0.f ? alpha * fI / cI[jb] : 0.f;
-            aJ = cJ[ia] > 0.f ? alpha * fJ / cJ[ia] : 0.f;
+            for (int q = 0; q < W; ++q)
+                o[q] = k ? make_float2(a.s[q].y, -a.c[q].y) : make_float2(a.s[q].x, -a.c[q].x);
         }
-        const float fs = fI + fJ, cb = beta * fs * r2;
-        const float v[3] = {aI * dpI[jb].x + aJ * dpJ[ia].x - cb * d.x, aI * dpI[jb].y + aJ * dpJ[ia].y - cb * d.y,
-                            aI * dpI[jb].z + aJ * dpJ[ia].z - cb * d.z};
-        float *G = ia ? G2 : G1, *H = jb ? H2 : H1;
-        const float mI = -aI * (ia ? tI[jb] + t.ell : tI[jb]);
-        const float mJ = -aJ * (jb ? tJ[ia] - s.ell : tJ[ia]);
-        const float dv[3] = {d.x, d.y, d.z};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            G[k] += v[k];
-            H[k] -= v[k];
-            GT[k] += mI * dv[k];
-            HT[k] += mJ * dv[k];
-        }
-        S += fs;
-    }
-    const float L = keep ? s.ell : 0.f, Ls = keep ? t.ell : 0.f;
-    kahan_add(a.S, a.cS, keep ? L * S : 0.f);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        kahan_add(a.G1[k], a.c1[k], keep ? L * G1[k] : 0.f);
-        kahan_add(a.G2[k], a.c2[k], keep ? L * G2[k] : 0.f);
-        kahan_add(a.GT[k], a.cT[k], keep ? L * GT[k] : 0.f);
-    }
-    if (keep) {
-        src[0] += Ls * S;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            src[1 + k] += Ls * H1[k];
-            src[4 + k] += Ls * H2[k];
-            src[7 + k] += Ls * HT[k];
-        }
-    }
-}
-
-// A near pair entirely in FP64 from the double-float positions and tangents: row I's terms into tgt,
-// row J's into src (both FP64).
-static __device__ __noinline__ void near_diff_both_df(const Tgt<float> &t, const Src<PMIX> &s, double alpha,
-                                                      double beta, bool fast, DiffAcc64 &tgt, double (&src)[kDS])
-{
-    const double TI[3] = {(double)t.T.x + t.Tl.x, (double)t.T.y + t.Tl.y, (double)t.T.z + t.Tl.z};
-    const double TJ[3] = {(double)s.T.x + s.Tm.x, (double)s.T.y + s.Tm.y, (double)s.T.z + s.Tm.z};
-    const double L = s.ell, Ls = t.ell;
-    for (int ab = 0; ab < 4; ++ab) {
-        const V3<float> P = (ab < 2) ? t.p1 : t.p2, PL = (ab < 2) ? t.l1 : t.l2;
-        const V3<float> Q = (ab & 1) ? s.q2 : s.q1, QL = (ab & 1) ? s.m2 : s.m1;
-        const double d[3] = {(double)(P.x - Q.x) + (double)(PL.x - QL.x), (double)(P.y - Q.y) + (double)(PL.y - QL.y),
-                             (double)(P.z - Q.z) + (double)(PL.z - QL.z)};
-        const double tI = TI[0] * d[0] + TI[1] * d[1] + TI[2] * d[2];
-        const double tJ = TJ[0] * d[0] + TJ[1] * d[1] + TJ[2] * d[2];
-        double dpI[3], dpJ[3];
-        for (int k = 0; k < 3; ++k) {
-            dpI[k] = d[k] - tI * TI[k];
-            dpJ[k] = d[k] - tJ * TJ[k];
-        }
-        const double cI2 = dpI[0] * dpI[0] + dpI[1] * dpI[1] + dpI[2] * dpI[2];
-        const double cJ2 = dpJ[0] * dpJ[0] + dpJ[1] * dpJ[1] + dpJ[2] * dpJ[2];
-        const double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        double rb, fI, fJ, aI, aJ;
-        if (fast) {
-            const double r = rsqrt(d2), r2 = r * r;
-            rb = r2 * r2 * sqrt(r);
-            fI = cI2 * rb;
-            fJ = cJ2 * rb;
-            aI = aJ = 2.0 * rb;
-        } else {
-            rb = pow(d2, -0.5 * beta);
-            fI = (cI2 > 0.0 ? pow(cI2, 0.5 * alpha) : 0.0) * rb;
-            fJ = (cJ2 > 0.0 ? pow(cJ2, 0.5 * alpha) : 0.0) * rb;
-            aI = cI2 > 0.0 ? alpha * fI / cI2 : 0.0;
-            aJ = cJ2 > 0.0 ? alpha * fJ / cJ2 : 0.0;
-        }
-        const double cb = beta * (fI + fJ) / d2;
-        double *G = ab < 2 ? tgt.G1 : tgt.G2;
-        const int hb = (ab & 1) ? 4 : 1;
-        for (int k = 0; k < 3; ++k) {
-            const double v = aI * dpI[k] + aJ * dpJ[k] - cb * d[k];
-            G[k] += L * v;
-            tgt.GT[k] += -L * aI * tI * d[k];
-            src[hb + k] -= Ls * v;
-            src[7 + k] += -Ls * aJ * tJ * d[k];
-        }
-        tgt.S += L * (fI + fJ);
-        src[0] += Ls * (fI + fJ);
     }
 }
 
 // Row output of the differential from its accumulators (Sec. 5.1 by the chain rule through l_I and T_I):
 // G_i1 = (1/4)[-T S + l G1 - (Id - T T^t) GT],  G_i2 = (1/4)[T S + l G2 + (Id - T T^t) GT]
-__device__ __forceinline__ void diff_row_out(const double *T, double l, double S, const double *G1,
-                                             const double *G2, const double *GT, double *o)
+__device__ __forceinline__ void diff_row_out(const double *T, double l, const double *v, double *o)
 {
+    const double *G1 = v + 1, *G2 = v + 4, *GT = v + 7;
     const double gt = T[0] * GT[0] + T[1] * GT[1] + T[2] * GT[2];
     for (int c = 0; c < 3; ++c) {
         const double pgt = GT[c] - gt * T[c];
-        o[c] = 0.25 * (-T[c] * S + l * G1[c] - pgt);
-        o[3 + c] = 0.25 * (T[c] * S + l * G2[c] + pgt);
+        o[c] = 0.25 * (-T[c] * v[0] + l * G1[c] - pgt);
+        o[3 + c] = 0.25 * (T[c] * v[0] + l * G2[c] + pgt);
     }
 }
 
-// MODE 2: near pairs (|g_i1 - g_j1| inside the differential's FP64 band) possible; 1 / 0 as in the energy.
-template <int TPT, bool FAST, bool CHECK, int MODE, bool SRC>
-__device__ __forceinline__ void sym_diff_tile(const Tgt<float> (&tg)[TPT], const bool (&valid)[TPT],
-                                              const Tile<PMIX, false> &tl, int cnt, Acc32<PMIX, OP_DIFF> (&a)[TPT],
-                                              Acc64<OP_DIFF> (&A)[TPT], float2 *sac,
-                                              const KernelParams &kp)
+// Sum the slots of every row (one thread per value, so that a slot's values are read coalesced) and form the
+// row's outputs: energy rows (l_I / 4) sum, or the six endpoint values of an edge into esum.
+template <int OP>
+__global__ void __launch_bounds__(OP == OP_ENERGY ? 256 : 32 * sym_width<OP>())
+k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ part, const double *__restrict__ ell,
+          const double *__restrict__ T, double *__restrict__ out)
 {
-    const int lane = threadIdx.x & 31;
-    const int P = max(cnt, 32);
-    for (int step = 0; step < P; ++step) {
-        int j = step + lane;
-        if (j >= P) j -= P;
-        if (j < cnt) {
-            Src<PMIX> s;
-            load_source<PMIX, false>(s, tl, j);
-            float src[kDS];
+    constexpr int W = sym_width<OP>(), R = OP == OP_ENERGY ? 256 : 32;  // rows per block
+    __shared__ double sh[OP == OP_ENERGY ? 1 : R * W];
+    const int row = blockIdx.x * R + threadIdx.x / W;
+    double x = 0.0;
+    if (row < nE) {
+        const size_t step = (size_t)nE * W;
+        const float2 *p = part + (size_t)blockIdx.x * R * W + threadIdx.x;
+        const int ns = eslots[row];
+        float s = 0.f, lo = 0.f;
+        int q = 0;
+        for (; q + 8 <= ns; q += 8) {
+            float2 v[8];
 #pragma unroll
-            for (int q = 0; q < kDS; ++q) src[q] = 0.f;
-            double srcd[kDS];
-            bool anynear = false;
+            for (int k = 0; k < 8; ++k) v[k] = __ldcs(p + (size_t)(q + k) * step);
 #pragma unroll
-            for (int k = 0; k < TPT; ++k) {
-                bool keep = valid[k];
-                if constexpr (CHECK)
-                    keep = keep & (s.j1 != tg[k].i1) & (s.j1 != tg[k].i2) & (s.j2 != tg[k].i1) & (s.j2 != tg[k].i2);
-                bool near = false;
-                if constexpr (MODE == 2) {
-                    const V3<float> e = diff3<true>(tg[k].p1, tg[k].l1, s.q1, s.m1);
-                    near = keep && dot3(e, e) < kp.near2f_diff;
-                }
-                if (near) {
-                    if (!anynear) {
-#pragma unroll
-                        for (int q = 0; q < kDS; ++q) srcd[q] = 0.0;
-                        anynear = true;
-                    }
-                    if constexpr (SRC)
-                        near_diff_both_df(tg[k], s, kp.alpha, kp.beta, FAST, A[k], srcd);
-                    else
-                        near_diff_df(tg[k], s, kp.alpha, kp.beta, FAST, A[k]);
-                } else {
-                    pair_diff_both<FAST, (MODE >= 1)>(tg[k], s, keep, kp, a[k], src);
-                }
-            }
-            if constexpr (SRC) {
-#pragma unroll
-                for (int q = 0; q < kDS; ++q) {
-                    const float2 ac = sac[q * kTile + j];  // (sum, Kahan compensation)
-                    float acc = ac.x, cmp = ac.y;
-                    if (anynear) {
-                        // FP64 near terms as hi + lo so the compensated sum keeps their digits
-                        const double tot = (double)src[q] + srcd[q];
-                        const float hi = (float)tot;
-                        kahan_add(acc, cmp, hi);
-                        kahan_add(acc, cmp, (float)(tot - (double)hi));
-                    } else {
-                        kahan_add(acc, cmp, src[q]);
-                    }
-                    sac[q * kTile + j] = make_float2(acc, cmp);
-                }
+            for (int k = 0; k < 8; ++k) {
+                const df r = two_sum(s, v[k].x);
+                s = r.hi;
+                lo = __fadd_rn(lo, __fadd_rn(r.lo, v[k].y));
             }
         }
-        if constexpr (SRC) __syncwarp();
+        for (; q < ns; ++q) {
+            const float2 v = __ldcs(p + (size_t)q * step);
+            const df r = two_sum(s, v.x);
+            s = r.hi;
+            lo = __fadd_rn(lo, __fadd_rn(r.lo, v.y));
+        }
+        x = (double)s + (double)lo;
     }
-}
-
-constexpr size_t kDiffSymDynSmem = sizeof(float) * 2 * kSymWarps * kDS * kTile;
-
-// MB: resident CTAs per SM the register allocation is held to (2 needs no spills at either TPT; the
-// variants with 3 / 4 trade a few spilled registers for more warps to hide latency).
-template <int TPT, bool FAST, int MB>
-__global__ void __launch_bounds__(kThreads, MB) k_diff_sym(const PairArgs pa)
-{
-    __shared__ Tile<PMIX, false> tl;
-    __shared__ int s_item;
-    __shared__ float s_box[2][kThreads / 32][6];
-    extern __shared__ float dyn[];  // [kSymWarps][kDS][kTile] float2 (sum, Kahan compensation) per source
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2 *sac = reinterpret_cast<float2 *>(dyn) + (size_t)wid * kDS * kTile;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(pa.counter, 1);
+    if constexpr (OP == OP_ENERGY) {
+        if (row < nE) out[row] = 0.25 * ell[row] * x;
+    } else {
+        sh[threadIdx.x] = x;
         __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it >= pa.n_items) break;
-        const WorkItem w = pa.items[it];
-        const int bslot = w.slot >> 16, cslot = w.slot & 0xffff;
-        const bool diag = bslot == cslot;
-        Tgt<float> tg[TPT];
-        bool valid[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            const int loc = threadIdx.x + k * kThreads;
-            valid[k] = loc < w.ntgt;
-            load_target<PMIX>(tg[k], w.tgt0 + min(loc, w.ntgt - 1), pa.recF, pa.recLo, pa.recD);
-        }
-        Acc64<OP_DIFF> A[TPT];
-        Acc32<PMIX, OP_DIFF> a[TPT];
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            acc64_zero<OP_DIFF>(A[k]);
-            acc_zero<PMIX, OP_DIFF>(a[k]);
-        }
-        float tbox[6];
-        {
-            float b[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) box_add(b, tg[k].p1, tg[k].p2);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                for (int q = 0; q < 6; ++q) {
-                    const float v = __shfl_xor_sync(0xffffffffu, b[q], o);
-                    b[q] = q < 3 ? fminf(b[q], v) : fmaxf(b[q], v);
-                }
-            for (int q = 0; q < 6; ++q) tbox[q] = b[q];
-        }
-        for (int s0 = w.src0; s0 < w.src1; s0 += kTile) {
-            const int cnt = min(kTile, w.src1 - s0);
-            __syncthreads();
-            float sb[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
-            if (threadIdx.x < cnt) {
-                const int J = s0 + threadIdx.x;
-                const RecF r = pa.recF[J];
-                tl.r[threadIdx.x] = r;
-                tl.lo[threadIdx.x] = pa.recLo[J];
-                box_add(sb, V3<float>{r.a.x, r.a.y, r.a.z}, V3<float>{r.b.x, r.b.y, r.b.z});
-            }
-            for (int t = lane; t < kDS * kTile; t += 32) sac[t] = make_float2(0.f, 0.f);
-            block_box(sb, s_box[1]);
-            const bool check = !(s0 + cnt - 1 < w.nb_lo || s0 > w.nb_hi);
-            float g2 = 0.f;
-            for (int q = 0; q < 3; ++q) {
-                const float gap = fmaxf(fmaxf(sb[q] - tbox[3 + q], tbox[q] - sb[3 + q]), 0.f);
-                g2 += gap * gap;
-            }
-            const int mode = g2 < pa.kp.near2f_diff ? 2 : (g2 < pa.kp.mid2f ? 1 : 0);
-            if (diag)
-                sym_diff_tile<TPT, FAST, true, 2, false>(tg, valid, tl, cnt, a, A, sac, pa.kp);
-            else if (check || mode == 2)
-                sym_diff_tile<TPT, FAST, true, 2, true>(tg, valid, tl, cnt, a, A, sac, pa.kp);
-            else if (mode == 1)
-                sym_diff_tile<TPT, FAST, false, 1, true>(tg, valid, tl, cnt, a, A, sac, pa.kp);
-            else
-                sym_diff_tile<TPT, FAST, false, 0, true>(tg, valid, tl, cnt, a, A, sac, pa.kp);
-#pragma unroll
-            for (int k = 0; k < TPT; ++k) {
-                acc_add(A[k], a[k]);
-                acc_zero<PMIX, OP_DIFF>(a[k]);
-            }
-            if (!diag) {
-                __syncthreads();
-                if (threadIdx.x < cnt) {
-                    const int J = s0 + threadIdx.x;
-                    double v[kDS];
-                    for (int q = 0; q < kDS; ++q) {
-                        double x = 0.0;
-                        for (int wv = 0; wv < kSymWarps; ++wv) {
-                            const float2 ac = reinterpret_cast<const float2 *>(dyn)[((size_t)wv * kDS + q) * kTile + threadIdx.x];
-                            x += (double)ac.x - (double)ac.y;
-                        }
-                        v[q] = x;
-                    }
-                    diff_row_out(pa.na.T + 3 * J, pa.na.ell[J], v[0], v + 1, v + 4, v + 7,
-                                 pa.part + ((size_t)bslot * pa.nE + J) * 6);
-                }
+        const int I = blockIdx.x * R + threadIdx.x;
+        if (threadIdx.x >= R || I >= nE) return;
+        const double *v = sh + W * threadIdx.x;
+        const double l = ell[I];
+        double o[6];
+        if constexpr (OP == OP_DIFF) {
+            diff_row_out(T + 3 * (size_t)I, l, v, o);
+        } else {
+            for (int c = 0; c < 3; ++c) {
+                o[c] = 0.5 * v[c];
+                o[3 + c] = 0.125 * l * v[3 + c];
             }
         }
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-            if (!valid[k]) continue;
-            const int I = w.tgt0 + threadIdx.x + k * kThreads;
-            diff_row_out(pa.na.T + 3 * I, pa.na.ell[I], A[k].S, A[k].G1, A[k].G2, A[k].GT,
-                         pa.part + ((size_t)cslot * pa.nE + I) * 6);
-        }
+        for (int c = 0; c < 6; ++c) out[6 * (size_t)I + c] = o[c];
     }
 }
 
 // ---------------------------------------------------------------------------------- host side
 
-static int sym_occupancy(int tpt)
-{
-    int occ = 0;
-    if (tpt == 1)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_sym<1, true>, kThreads, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_sym<2, true>, kThreads, 0);
-    return occ;
-}
-
-// Edge blocks of 128 x tpt per problem; items (b, c >= b) sorted by problem size (large first).
+// Edge blocks of 128 x tpt per problem; items (b, c >= b) sorted by problem size (large first): the
+// double-float apply's work list.
 void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
 {
     const int tb = kThreads * tpt;
-    std::vector<int> vmin(c.nV, INT32_MAX), vmax(c.nV, -1);
-    for (int I = 0; I < c.nE; ++I)
-        for (int s = 0; s < 2; ++s) {
-            const int v = c.h_edges[2 * I + s];
-            vmin[v] = std::min(vmin[v], I);
-            vmax[v] = std::max(vmax[v], I);
-        }
     std::vector<std::pair<long long, WorkItem>> tmp;
     std::vector<int> eslots(std::max(1, c.nE), 1);
     int max_slots = 1;
@@ -772,16 +692,9 @@ void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
         max_slots = std::max(max_slots, nblk);
         for (int b = 0; b < nblk; ++b) {
             const int t0 = e0 + b * tb, nt = std::min(tb, e1 - t0);
-            int lo = INT32_MAX, hi = -1;
-            for (int I = t0; I < t0 + nt; ++I)
-                for (int s = 0; s < 2; ++s) {
-                    const int v = c.h_edges[2 * I + s];
-                    lo = std::min(lo, vmin[v]);
-                    hi = std::max(hi, vmax[v]);
-                }
             for (int cb = b; cb < nblk; ++cb) {
                 const int s0 = e0 + cb * tb, s1 = std::min(e1, s0 + tb);
-                tmp.push_back({(long long)n, WorkItem{t0, nt, s0, s1, (b << 16) | cb, lo, hi, q}});
+                tmp.push_back({(long long)n, WorkItem{t0, nt, s0, s1, (b << 16) | cb, e0, e1 - 1, q}});
             }
         }
         for (int I = e0; I < e1; ++I) eslots[I] = nblk;
@@ -800,201 +713,211 @@ void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
     cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
 }
 
-// Slots the symmetric pass needs per row (the largest problem's block count) at tpt targets per thread.
-size_t sym_slots(const Ctx &c, int tpt)
+// Tiles per item: four (fewer partial slots, longer runs per target load) once every resident CTA gets about
+// six items that way, fewer on smaller graphs so that the last wave stays short.
+static int sym_tiles_per_item(const Ctx &c, int resident)
 {
-    const int tb = kThreads * tpt;
-    int m = 1;
-    for (int q = 0; q < c.nProb; ++q) m = std::max(m, (c.h_prob_e[q + 1] - c.h_prob_e[q] + tb - 1) / tb);
-    return (size_t)m;
-}
-
-// Switch the apply to the symmetric pass with tpt targets per thread (1 or 2), or back to the gather
-// pass (tpt = 0).  Mixed precision with the specialised powers only; grows the partial buffer if needed.
-cudaError_t sym_select(Ctx &c, int tpt)
-{
-    graphs_reset(c);
-    Ctx::Plan &pl = c.plan_sym;
-    if (pl.d_items) TPE_CHECK(cudaFree(pl.d_items));
-    if (pl.d_eslots) TPE_CHECK(cudaFree(pl.d_eslots));
-    pl = Ctx::Plan{};
-    c.apply_sym = 0;
-    if (tpt <= 0) return cudaSuccess;
-    if (c.prm.precision != TP_MIXED || !c.kp.fast || (tpt != 1 && tpt != 2)) return cudaErrorInvalidValue;
-    sym_plan_items(c, pl, tpt, sym_occupancy(tpt));
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
-    if (need > c.part_elems) {
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
+    long long tiles = 0;
+    for (int q = 0; q < c.nProb; ++q) {
+        const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
+        for (long long X = 0; X < ns; ++X) tiles += std::max(0LL, nb - 2 * X - 2);
     }
-    c.apply_sym = tpt;
-    return cudaGetLastError();
+    return (int)std::min<long long>(kSymMaxTiles, std::max<long long>(1, tiles / (6LL * std::max(1, resident))));
 }
 
-static int sym_energy_occupancy(int tpt)
+// Slots a row of super-block X of a problem with nb tiles has at tc tiles per item.
+static int sym_row_slots(int X, int nb, int tc)
 {
-    int occ = 0;
-    if (tpt == 1)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_energy_sym<1, true>, kThreads, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_energy_sym<2, true>, kThreads, 0);
-    return occ;
+    const int m = std::max(0, nb - 2 * X - 2);
+    return X + std::min(3, nb - 2 * X + 1) + (m + tc - 1) / tc;
 }
 
-// The energy's symmetric pass on (tpt 1, 2) or off (0); same conditions as sym_select.
-cudaError_t sym_select_energy(Ctx &c, int tpt)
+static int sym_max_slots(const Ctx &c, int tc)
 {
-    Ctx::Plan &pl = c.plan_sym_e;
-    if (pl.d_items) TPE_CHECK(cudaFree(pl.d_items));
-    if (pl.d_eslots) TPE_CHECK(cudaFree(pl.d_eslots));
-    pl = Ctx::Plan{};
-    c.energy_sym = 0;
-    if (tpt <= 0) return cudaSuccess;
-    if (c.prm.precision != TP_MIXED || !c.kp.fast || (tpt != 1 && tpt != 2)) return cudaErrorInvalidValue;
-    sym_plan_items(c, pl, tpt, sym_energy_occupancy(tpt));
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE);
-    if (need > c.part_elems) {
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
+    int ms = 1;
+    for (int q = 0; q < c.nProb; ++q) {
+        const int n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
+        for (int X = 0; X < ns; ++X) ms = std::max(ms, sym_row_slots(X, nb, tc));
     }
-    c.energy_sym = tpt;
-    return cudaGetLastError();
+    return ms;
 }
 
-cudaError_t sym_energy_pass(Ctx &c, int which, const double *gamma, cudaStream_t s)
+static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
 {
-    Ctx::Plan &pl = c.plan_sym_e;
-    if (pl.n_items == 0) return cudaSuccess;
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + 5, 0, sizeof(int), s));
-    PairArgs pa;
-    pa.items = pl.d_items;
-    pa.n_items = pl.n_items;
-    pa.counter = c.d_counter + 5;
-    pa.recF = which ? c.d_recF2 : c.d_recF;
-    pa.recLo = which ? c.d_recLo2 : c.d_recLo;
-    pa.recD = nullptr;
-    pa.urecF = nullptr;
-    pa.urecD = nullptr;
-    pa.na = NearArgs{gamma, c.d_edges, c.d_ellw[which], c.d_Tw[which], nullptr};
-    pa.part = c.d_part;
-    pa.nE = c.nE;
-    pa.kp = c.kp;
-    pa.skip = nullptr;
-    const int slot = c.profile ? prof_begin(c, OP_ENERGY, s) : -1;
-    if (pl.tpt == 1)
-        k_energy_sym<1, true><<<pl.grid, kThreads, 0, s>>>(pa);
-    else
-        k_energy_sym<2, true><<<pl.grid, kThreads, 0, s>>>(pa);
-    if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
-    c.launches++;
-    return cudaGetLastError();
+    const int resident = c.sm_count * std::max(1, occupancy);
+    const int tc = sym_tiles_per_item(c, resident);
+    // edges at every vertex, for the tiles that hold a neighbour of a super-block
+    std::vector<int> ptr(c.nV + 1, 0), inc(2 * (size_t)c.nE);
+    for (int k = 0; k < 2 * c.nE; ++k) ptr[c.h_edges[k] + 1]++;
+    for (int v = 0; v < c.nV; ++v) ptr[v + 1] += ptr[v];
+    std::vector<int> fill(ptr.begin(), ptr.end() - 1);
+    for (int I = 0; I < c.nE; ++I)
+        for (int s = 0; s < 2; ++s) inc[fill[c.h_edges[2 * I + s]]++] = I;
+    struct Tmp {
+        WorkItem w;
+        int cost;
+    };
+    std::vector<Tmp> tmp;
+    std::vector<int> eslots(std::max(1, c.nE), 0);
+    std::vector<char> touch;
+    for (int q = 0; q < c.nProb; ++q) {
+        const int e0 = c.h_prob_e[q], e1 = c.h_prob_e[q + 1], n = e1 - e0;
+        if (n <= 0) continue;
+        const int nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
+        for (int X = 0; X < ns; ++X) {
+            const int t0 = e0 + X * kSuper, nt = std::min(kSuper, e1 - t0);
+            touch.assign(nb, 0);
+            for (int I = t0; I < t0 + nt; ++I)
+                for (int s = 0; s < 2; ++s) {
+                    const int v = c.h_edges[2 * I + s];
+                    for (int k = ptr[v]; k < ptr[v + 1]; ++k)
+                        if (inc[k] >= e0 && inc[k] < e1) touch[(inc[k] - e0) / kTile] = 1;
+                }
+            // tiles with near pairs take longer: they and the super-block itself go first
+            int slot = X + 1;
+            for (int h = t0; h < t0 + nt; h += kTile, ++slot)
+                tmp.push_back({WorkItem{t0, nt, h, std::min(h + kTile, t0 + nt), (X << 16) | slot, 3, 0, q}, 1 + kSymMaxTiles});
+            for (int cb = 2 * X + 2; cb < nb; cb += tc, ++slot) {
+                const int ce = std::min(nb, cb + tc);
+                int mask = 0;
+                for (int k = cb; k < ce; ++k) mask |= touch[k] << (k - cb);
+                tmp.push_back({WorkItem{t0, nt, e0 + cb * kTile, std::min(e1, e0 + ce * kTile), (X << 16) | slot, mask, 0, q},
+                               ce - cb + (mask ? kSymMaxTiles : 0)});
+            }
+            for (int I = t0; I < t0 + nt; ++I) eslots[I] = sym_row_slots(X, nb, tc);
+        }
+    }
+    std::stable_sort(tmp.begin(), tmp.end(), [](const Tmp &a, const Tmp &b) { return a.cost > b.cost; });
+    std::vector<WorkItem> items;
+    items.reserve(tmp.size());
+    for (auto &t : tmp) items.push_back(t.w);
+    pl.n_items = (int)items.size();
+    pl.max_slots = sym_max_slots(c, tc);
+    pl.grid = std::max(1, std::min(pl.n_items, resident));
+    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
+    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
+    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
+    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
 }
 
-// Symmetric differential variants: 1 / 2 targets per thread at 2 CTAs per SM, 3: one target at 4 CTAs
-// per SM, 4: two targets at 3 CTAs per SM.
-static int diff_variant_tpt(int v)
-{
-    return (v == 2 || v == 4) ? 2 : 1;
-}
-
+// Variants differ in the CTAs per SM that the register allocation is held to.
 template <class F>
-static void with_diff_kernel(int v, F f)
+static void with_sym_kernel(int prec, int op, int variant, F f)
 {
-    switch (v) {
-        case 1: f(k_diff_sym<1, true, 2>); break;
-        case 2: f(k_diff_sym<2, true, 2>); break;
-        case 3: f(k_diff_sym<1, true, 4>); break;
-        default: f(k_diff_sym<2, true, 3>); break;
+    if (op == OP_ENERGY) {
+        if (prec == TP_FP32)
+            f(k_sym<P32, OP_ENERGY, 4>, sizeof(SymSmem<P32, OP_ENERGY>));
+        else if (variant == 2)
+            f(k_sym<PMIX, OP_ENERGY, 4>, sizeof(SymSmem<PMIX, OP_ENERGY>));
+        else
+            f(k_sym<PMIX, OP_ENERGY, 3>, sizeof(SymSmem<PMIX, OP_ENERGY>));
+    } else if (op == OP_DIFF) {
+        if (variant >= 3)
+            f(k_sym<PMIX, OP_DIFF, 3>, sizeof(SymSmem<PMIX, OP_DIFF>));
+        else
+            f(k_sym<PMIX, OP_DIFF, 2>, sizeof(SymSmem<PMIX, OP_DIFF>));
+    } else {
+        if (prec == TP_FP32)
+            f(k_sym<P32, OP_APPLY, 3>, sizeof(SymSmem<P32, OP_APPLY>));
+        else if (variant == 2)
+            f(k_sym<PMIX, OP_APPLY, 2>, sizeof(SymSmem<PMIX, OP_APPLY>));
+        else
+            f(k_sym<PMIX, OP_APPLY, 3>, sizeof(SymSmem<PMIX, OP_APPLY>));
     }
 }
 
-static int sym_diff_occupancy(int v)
+static int sym_occupancy(const Ctx &c, int op, int variant)
 {
     int occ = 0;
-    with_diff_kernel(v, [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiffSymDynSmem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, kDiffSymDynSmem);
+    with_sym_kernel(c.prm.precision, op, variant, [&](auto kern, size_t smem) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
     });
     return occ;
 }
 
-// The differential's symmetric pass on (tpt 1, 2) or off (0); same conditions as sym_select.
-cudaError_t sym_select_diff(Ctx &c, int tpt)
+static int sym_op_width(int op) { return op == OP_ENERGY ? 1 : (op == OP_DIFF ? 10 : 6); }
+
+// Doubles of the partial buffer the symmetric pass of `op` needs.
+size_t sym_part_elems(const Ctx &c, int op, int variant)
 {
-    Ctx::Plan &pl = c.plan_sym_d;
+    const int tc = sym_tiles_per_item(c, c.sm_count * std::max(1, sym_occupancy(c, op, variant)));
+    return (size_t)sym_max_slots(c, tc) * std::max(1, c.nE) * sym_op_width(op);
+}
+
+// Switch one pass to its symmetric form (variant > 0) or back to the gather form; grows the partial buffer.
+static cudaError_t select_pass(Ctx &c, int op, int variant, int max_variant, Ctx::Plan &pl, int &flag)
+{
+    graphs_reset(c);
     if (pl.d_items) TPE_CHECK(cudaFree(pl.d_items));
     if (pl.d_eslots) TPE_CHECK(cudaFree(pl.d_eslots));
     pl = Ctx::Plan{};
-    c.diff_sym = 0;
-    if (tpt <= 0) return cudaSuccess;
-    if (c.prm.precision != TP_MIXED || !c.kp.fast || tpt > 4) return cudaErrorInvalidValue;
-    sym_plan_items(c, pl, diff_variant_tpt(tpt), sym_diff_occupancy(tpt));
-    pl.tpt = tpt;  // the variant (the plan's blocking follows its targets per thread)
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
+    flag = 0;
+    if (variant <= 0) return cudaSuccess;
+    if (!c.kp.fast || variant > max_variant) return cudaErrorInvalidValue;
+    if (c.prm.precision != TP_MIXED && !(c.prm.precision == TP_FP32 && op != OP_DIFF)) return cudaErrorInvalidValue;
+    sym_plan(c, pl, sym_occupancy(c, op, variant));
+    pl.tpt = variant;
+    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(op);
     if (need > c.part_elems) {
         TPE_CHECK(cudaFree(c.d_part));
         TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
         c.part_elems = need;
     }
-    c.diff_sym = tpt;
+    flag = variant;
     return cudaGetLastError();
 }
 
-cudaError_t sym_diff_pass(Ctx &c, int which, const double *gamma, cudaStream_t s)
-{
-    Ctx::Plan &pl = c.plan_sym_d;
-    if (pl.n_items == 0) return cudaSuccess;
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + 6, 0, sizeof(int), s));
-    PairArgs pa;
-    pa.items = pl.d_items;
-    pa.n_items = pl.n_items;
-    pa.counter = c.d_counter + 6;
-    pa.recF = which ? c.d_recF2 : c.d_recF;
-    pa.recLo = which ? c.d_recLo2 : c.d_recLo;
-    pa.recD = nullptr;
-    pa.urecF = nullptr;
-    pa.urecD = nullptr;
-    pa.na = NearArgs{gamma, c.d_edges, c.d_ellw[which], c.d_Tw[which], nullptr};
-    pa.part = c.d_part;
-    pa.nE = c.nE;
-    pa.kp = c.kp;
-    pa.skip = nullptr;
-    const int slot = c.profile ? prof_begin(c, OP_DIFF, s) : -1;
-    with_diff_kernel(pl.tpt, [&](auto kern) { kern<<<pl.grid, kThreads, kDiffSymDynSmem, s>>>(pa); });
-    if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
-    c.launches++;
-    return cudaGetLastError();
-}
+cudaError_t sym_select(Ctx &c, int v) { return select_pass(c, OP_APPLY, v, 2, c.plan_sym, c.apply_sym); }
+cudaError_t sym_select_energy(Ctx &c, int v) { return select_pass(c, OP_ENERGY, v, 2, c.plan_sym_e, c.energy_sym); }
+cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4, c.plan_sym_d, c.diff_sym); }
 
-cudaError_t sym_apply_pass(Ctx &c, int which, const double *gamma, const double *u, cudaStream_t s)
+// Run the symmetric pass of `op` and sum its slots: energy rows into out [nE], else the edges' endpoint
+// values into c.d_esum.
+static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof_op, int which, const int *skip, double *out,
+                            cudaStream_t s)
 {
-    Ctx::Plan &pl = c.plan_sym;
     if (pl.n_items == 0) return cudaSuccess;
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + 4, 0, sizeof(int), s));
-    PairArgs pa;
+    TPE_CHECK(cudaMemsetAsync(c.d_counter + counter, 0, sizeof(int), s));
+    SymArgs pa;
     pa.items = pl.d_items;
     pa.n_items = pl.n_items;
-    pa.counter = c.d_counter + 4;
+    pa.counter = c.d_counter + counter;
     pa.recF = which ? c.d_recF2 : c.d_recF;
     pa.recLo = which ? c.d_recLo2 : c.d_recLo;
-    pa.recD = nullptr;
     pa.urecF = c.d_urecF;
-    pa.urecD = nullptr;
-    pa.na = NearArgs{gamma, c.d_edges, c.d_ellw[which], c.d_Tw[which], u};
-    pa.part = c.d_part;
+    pa.part = reinterpret_cast<float2 *>(c.d_part);
     pa.nE = c.nE;
-    pa.kp = c.kp;
-    pa.skip = c.d_skip;
-    const int slot = c.profile ? prof_begin(c, c.d_skip ? 4 : 2, s) : -1;
-    if (pl.tpt == 1)
-        k_pairs_sym<1, true><<<pl.grid, kThreads, 0, s>>>(pa);
-    else
-        k_pairs_sym<2, true><<<pl.grid, kThreads, 0, s>>>(pa);
+    pa.near2f = op == OP_DIFF ? c.kp.near2f_diff : c.kp.near2f;
+    pa.mid2f = c.kp.mid2f;
+    pa.skip = skip;
+    const int slot = c.profile ? prof_begin(c, prof_op, s) : -1;
+    with_sym_kernel(c.prm.precision, op, pl.tpt, [&](auto kern, size_t smem) { kern<<<pl.grid, kThreads, smem, s>>>(pa); });
     if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
-    c.launches++;
+    const double *ell = c.d_ellw[which], *T = c.d_Tw[which];
+    if (op == OP_ENERGY)
+        k_sym_sum<OP_ENERGY><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+    else if (op == OP_DIFF)
+        k_sym_sum<OP_DIFF><<<(c.nE + 31) / 32, 320, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+    else
+        k_sym_sum<OP_APPLY><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+    c.launches += 2;
     return cudaGetLastError();
+}
+
+cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s)
+{
+    return sym_pass(c, OP_ENERGY, c.plan_sym_e, 5, OP_ENERGY, which, nullptr, rows, s);
+}
+
+cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s)
+{
+    return sym_pass(c, OP_DIFF, c.plan_sym_d, 6, OP_DIFF, which, nullptr, c.d_esum, s);
+}
+
+cudaError_t sym_apply_pass(Ctx &c, int which, cudaStream_t s)
+{
+    return sym_pass(c, OP_APPLY, c.plan_sym, 4, c.d_skip ? 4 : 2, which, c.d_skip, c.d_esum, s);
 }
 
 }  // namespace tpe

@@ -242,13 +242,15 @@ void multi_free(Ctx &c);
 void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
 void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);  // (pairs_sym.cu) items (b, c >= b)
 cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s);
-cudaError_t sym_select(Ctx &c, int tpt);  // (pairs_sym.cu) symmetric apply on (tpt 1, 2) or off (0)
-cudaError_t sym_apply_pass(Ctx &c, int which, const double *gamma, const double *u, cudaStream_t s);
-size_t sym_slots(const Ctx &c, int tpt);
-cudaError_t sym_select_energy(Ctx &c, int tpt);
-cudaError_t sym_energy_pass(Ctx &c, int which, const double *gamma, cudaStream_t s);
-cudaError_t sym_select_diff(Ctx &c, int tpt);
-cudaError_t sym_diff_pass(Ctx &c, int which, const double *gamma, cudaStream_t s);
+// symmetric passes (pairs_sym.cu): a variant > 0 or the gather pass (0); the passes write the energy rows
+// [nE] or the edges' endpoint values into c.d_esum
+cudaError_t sym_select(Ctx &c, int variant);
+cudaError_t sym_apply_pass(Ctx &c, int which, cudaStream_t s);
+cudaError_t sym_select_energy(Ctx &c, int variant);
+cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s);
+cudaError_t sym_select_diff(Ctx &c, int variant);
+cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
+size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 void make_plans(Ctx &c);
 cudaError_t replan(Ctx &c, int cls);  // rebuild the plan of one op class (0 energy, 1 diff, 2 apply/diag)
 int tpt_default(const Ctx &c, int cls);

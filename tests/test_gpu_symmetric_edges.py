@@ -1,0 +1,103 @@
+"""Edges of the blocking of the pair passes: 64-row sections, 128-row tiles and 256-row super-blocks of the
+symmetric passes, the short source chunks of the gather passes, edges whose neighbours lie in other tiles (a
+curve with its edges shuffled) and the passes a new context picks by size, all against the FP64 oracle.
+
+Tolerances are those of the same quantities elsewhere in the suite: relative to the largest entry 1e-6 for the
+mixed energy rows and apply, 1e-5 for the mixed differential, 1e-10 for FP64."""
+import numpy as np
+import pytest
+
+import synth as S
+from tests.gpu_util import dev, host, make_ctx, need_gpu, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    return need_gpu()
+
+
+@pytest.fixture(scope="module")
+def orc():
+    from oracle import oracle as O
+    O.build_library()
+    return O
+
+
+def _check(torch, orc, ctx, c, prec, tol):
+    from paper_2006_07859_gb300 import tpe
+    g = dev(c.gamma)
+    rows = torch.empty(c.n_edges, dtype=torch.float64, device="cuda")
+    E = host(tpe.tp_energy(ctx, g, rows=rows))
+    dE = host(tpe.tp_differential(ctx, g))
+    u = np.random.default_rng(5).normal(size=(c.n_vertices, 3))
+    Au = host(tpe.sobolev_apply(ctx, g, dev(u)))
+    for k in range(ctx.n_problems):
+        if ctx.n_problems == 1:
+            gk, ek, v, e = c.gamma, c.edges, slice(None), slice(None)
+        else:
+            gk, ek = c.curve(k)
+            v = slice(c.vertex_offsets[k], c.vertex_offsets[k + 1])
+            e = slice(c.edge_offsets[k], c.edge_offsets[k + 1])
+        ref = orc.energy_rows(gk, ek, np.arange(len(ek), dtype=np.int32))
+        if not np.abs(ref).max() > 0:
+            assert np.all(host(rows)[e] == 0) and np.all(dE[v] == 0) and np.all(Au[v] == 0)
+            continue
+        assert rel(host(rows)[e], ref) <= tol["energy"], (k, len(ek))
+        assert abs(E[k] - ref.sum()) <= tol["energy"] * ref.sum()
+        if prec != 1:   # the plain FP32 differential has its own test
+            assert rel(dE[v], orc.differential(gk, ek)) <= tol["diff"], (k, len(ek))
+        assert rel(Au[v], orc.gram_apply(gk, ek, 0.75, u[v])) <= tol["apply"], (k, len(ek))
+
+
+MIXED = {"energy": 1e-6, "diff": 1e-5, "apply": 1e-6}
+FP64 = {"energy": 1e-10, "diff": 1e-10, "apply": 1e-10}
+
+
+@pytest.mark.parametrize("n", [3, 4, 5, 31, 63, 64, 65, 127, 128, 129, 192, 193, 255, 256, 257, 384, 385, 640])
+@pytest.mark.parametrize("variant", [0, 1])
+def test_mixed_passes_at_block_edges(torch, orc, n, variant):
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(n, 4, 40 + n))
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    tpe.tp_set_energy_variant(ctx, variant)
+    tpe.tp_set_diff_variant(ctx, variant)
+    tpe.tp_set_apply_variant(ctx, variant)
+    _check(torch, orc, ctx, c, 2, MIXED)
+
+
+@pytest.mark.parametrize("n", [4, 130, 257, 900])
+def test_fp64_passes_in_short_chunks(torch, orc, n):
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(n, 4, 60 + n))
+    _check(torch, orc, make_ctx(c, precision=tpe.TP_FP64, precond=tpe.TP_PRECOND_JACOBI), c, 0, FP64)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+def test_shuffled_edges_find_their_neighbours(torch, orc, variant):
+    """The two neighbours of an edge lie anywhere in the edge order; some edges are flipped too."""
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(700, 4, 3))
+    rng = np.random.default_rng(8)
+    e = c.edges[rng.permutation(c.n_edges)].copy()
+    flip = rng.random(len(e)) < 0.3
+    e[flip] = e[flip][:, ::-1]
+    c = S.Curves(c.gamma, e, c.vertex_offsets, c.edge_offsets)
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    tpe.tp_set_energy_variant(ctx, variant)
+    tpe.tp_set_diff_variant(ctx, variant)
+    tpe.tp_set_apply_variant(ctx, variant)
+    _check(torch, orc, ctx, c, 2, MIXED)
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_new_context_of_many_ragged_curves(torch, orc, prec):
+    """Enough work for the symmetric passes by default: 209 curves of 4 to 700 edges."""
+    from paper_2006_07859_gb300 import tpe
+    sizes = [4, 5, 63, 64, 65, 128, 129, 255, 256, 257, 300, 513, 700] * 16 + [700]
+    c = S.batch_of_knots(sizes, 4, 77)
+    ctx = make_ctx(c, precision=prec, precond=tpe.TP_PRECOND_JACOBI, independent=1)
+    # plain FP32 positions: the suite's FP32 bar for the energy, and 1e-4 of the largest entry for the apply
+    # (positions rounded to 6e-8 of the curve's size against edges of 1e-2 of it)
+    _check(torch, orc, ctx, c, prec, MIXED if prec == 2 else {"energy": 1e-4, "diff": 1.0, "apply": 1e-4})
