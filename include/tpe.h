@@ -516,7 +516,9 @@ TPE_API tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, do
 /* Select the apply pass: symmetric_tpt = 0 the gather pass (every ordered pair), 1 or 2 the symmetric pass
  * (every unordered pair evaluated once, two targets per thread in packed arithmetic; both rows receive their
  * terms; TP_MIXED with (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED), its registers held to three
- * (1) or two (2) resident CTAs per SM.  Both are deterministic and differ only in summation order.  May grow the partial-sum buffer. */
+ * (1) or two (2) resident CTAs per SM.  A new context has the symmetric pass where its work list fills the GPU
+ * and its partial sums take at most 1 GiB, the gather pass elsewhere.  Both are deterministic and differ
+ * only in summation order.  May grow the partial-sum buffer. */
 TPE_API tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt);
 
 /* The same choice for the energy pass (0: gather, 1 or 2: symmetric at three or four resident CTAs per SM; the

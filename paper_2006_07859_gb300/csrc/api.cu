@@ -434,6 +434,7 @@ tp_status tp_create(tp_ctx **out, int nV, int nE, const int32_t *edges_host, int
     int ms = std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots);
     c.part_elems = (size_t)ms * std::max(1, nE) * 6;
     CK(dalloc(&c.d_part, c.part_elems));
+    CK(sym_defaults(c));
     CK(dalloc(&c.d_rows, nE));
     CK(dalloc(&c.d_esum, 6 * (size_t)nE));
     CK(dalloc(&c.d_x0L0, 4 * (size_t)c.nProb));

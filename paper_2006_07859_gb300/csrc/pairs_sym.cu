@@ -872,6 +872,29 @@ cudaError_t sym_select(Ctx &c, int v) { return select_pass(c, OP_APPLY, v, 2, c.
 cudaError_t sym_select_energy(Ctx &c, int v) { return select_pass(c, OP_ENERGY, v, 2, c.plan_sym_e, c.energy_sym); }
 cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4, c.plan_sym_d, c.diff_sym); }
 
+// The passes a new context runs in symmetric form: those whose work list, one tile per item, gives every
+// resident CTA an item, while the partial sums stay below 1 GiB.  With fewer items the gather pass's short
+// chunks spread the work better (mixed precision, one knot, gather / symmetric: 1,000 edges energy 42 / 96 us,
+// differential 117 / 515 us; 4,096 edges 101 / 107 and 573 / 683; 8,192 edges 280 / 181 and 1,137 / 944;
+// 8 x 4,096 edges 488 / 322, differential 2,835 / 1,211, apply 956 / 553).
+cudaError_t sym_defaults(Ctx &c)
+{
+    if (!c.kp.fast || c.prm.precision == TP_FP64) return cudaSuccess;
+    long long items = 0;
+    for (int q = 0; q < c.nProb; ++q) {
+        const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
+        for (long long X = 0; X < ns; ++X) items += nb - 2 * X;
+    }
+    auto pays = [&](int op) {
+        return items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1)) &&
+               sym_part_elems(c, op, 1) * sizeof(double) <= (size_t)1 << 30;
+    };
+    if (pays(OP_ENERGY)) TPE_CHECK(sym_select_energy(c, 1));
+    if (c.prm.precision == TP_MIXED && pays(OP_DIFF)) TPE_CHECK(sym_select_diff(c, 1));
+    if (pays(OP_APPLY)) TPE_CHECK(sym_select(c, 1));
+    return cudaSuccess;
+}
+
 // Run the symmetric pass of `op` and sum its slots: energy rows into out [nE], else the edges' endpoint
 // values into c.d_esum.
 static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof_op, int which, const int *skip, double *out,

@@ -250,6 +250,7 @@ cudaError_t sym_select_energy(Ctx &c, int variant);
 cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s);
 cudaError_t sym_select_diff(Ctx &c, int variant);
 cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
+cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 void make_plans(Ctx &c);
 cudaError_t replan(Ctx &c, int cls);  // rebuild the plan of one op class (0 energy, 1 diff, 2 apply/diag)
