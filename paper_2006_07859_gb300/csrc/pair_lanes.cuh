@@ -170,8 +170,8 @@ __device__ __forceinline__ L l_energy_sum(L c0, L c1, L r11, L r12, L r21, L r22
 // terms (which cancel between a vertex's two edges) need more than FP32.  They are evaluated in
 // double-float arithmetic on the FP32 pipe (about 2^-44): an FP64 instruction of a warp holds its
 // sub-partition's FP64 pipe for 64 cycles, and one near pair of the differential takes ~500 of them
-// (33,000 cycles) against ~1,800 FP32 instructions here.  The pairs are not renormalised after an operation
-// (lo stays within a few ulp of hi, its own rounding at 2^-47).  The functions load the records themselves
+// (33,000 cycles) against ~1,800 FP32 instructions here.  The pairs are renormalised only where a difference
+// cancels (elsewhere lo stays within a few ulp of hi, its own rounding at 2^-47).  The functions load the records themselves
 // and are not inlined, and the differential's is unrolled over one endpoint only: unrolled over both, 48 KB of
 // straight-line code ran at the instruction cache's rate (23,000 cycles a call).
 
@@ -188,6 +188,14 @@ __device__ __forceinline__ dfl<L> l_two_sum(L a, L b)
 }
 template <class L>
 __device__ __forceinline__ dfl<L> l_dfneg(dfl<L> x) { return {l_neg(x.hi), l_neg(x.lo)}; }
+// hi and lo of x with |lo| <= ulp(hi) / 2: needed after a difference that cancels, where lo would be left as large
+// as hi (products drop lo lo)
+template <class L>
+__device__ __forceinline__ dfl<L> l_dfnorm(dfl<L> x)
+{
+    const L s = l_add(x.hi, x.lo);
+    return {s, l_sub(x.lo, l_sub(s, x.hi))};
+}
 // error 2^-47 (|x| + |y|)
 template <class L>
 __device__ __forceinline__ dfl<L> l_dfadd(dfl<L> x, dfl<L> y)
@@ -236,7 +244,8 @@ template <class L>
 __device__ __forceinline__ dfv<L> l_dfperp(const dfv<L> &d, dfl<L> t, const dfv<L> &T)
 {
     const dfl<L> n = l_dfneg(t);
-    return {l_dfadd(d.x, l_dfmul(n, T.x)), l_dfadd(d.y, l_dfmul(n, T.y)), l_dfadd(d.z, l_dfmul(n, T.z))};
+    return {l_dfnorm(l_dfadd(d.x, l_dfmul(n, T.x))), l_dfnorm(l_dfadd(d.y, l_dfmul(n, T.y))),
+            l_dfnorm(l_dfadd(d.z, l_dfmul(n, T.z)))};
 }
 
 // The edges of a lane as the near paths see them: endpoints (hi, lo), tangent (hi, lo), length.

@@ -448,6 +448,8 @@ cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s
     return gather_slots<OP_APPLY>(c, pl, Au, s);
 }
 
+cudaError_t vertices_apply(Ctx &c, double *Au, cudaStream_t s) { return vertices_from_edges<OP_APPLY>(c, Au, s); }
+
 // ---------------------------------------------------------------------------------- planning
 
 constexpr int kMinChunk = 4;  // sources of the shortest item

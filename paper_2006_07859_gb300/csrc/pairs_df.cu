@@ -1,28 +1,22 @@
-// Sobolev apply in double-float arithmetic: the accurate operator that certifies the residuals of the
-// mixed-precision solves.
+// Sobolev apply in double-float arithmetic at general exponents: the accurate operator that certifies the
+// residuals of the mixed-precision solves ((alpha, beta) = (2, 4.5) runs the packed pass of pairs_sym.cu).
 //
-// The product is the same as the gather pass of pairs.cu (Secs. 5.2.2-5.2.3): for every ordered pair
-// (I, J) of disjoint edges
+// For every pair of disjoint edges (Secs. 5.2.2-5.2.3)
 //   h_I += 2 w_IJ [(du_I - du_J) + (|T_I - T_J|^2 / 2) du_J],     l_I += (w0_IJ + w0_JI)(ub_I - ub_J),
 // w_IJ = (1/4) l_I l_J sum_ab |d_ab|^-p, w0_IJ + w0_JI = (1/4) l_I l_J sum_ab (|T_I x d_ab|^2 + |T_J x d_ab|^2)
-// |d_ab|^-(4+p), d_ab = g_ia - g_jb; (A u) at i1, i2 = -/+ h_I / l_I + l_I / 2.  Here every quantity is a
-// double-float (hi + lo, ~48 bits) built from the FP64 positions, tangents, lengths and u: the chords,
-// |d|^2, the powers (rsqrt and sqrt of the FP32 pipe, each refined by one exact-residual correction),
-// |T x d|^2 = |d|^2 - (T . d)^2, the weights and the products with the u differences.  Each term is
-// then correct to ~1e-13 relative, about 2^24 times better than the FP32 pair arithmetic of the mixed
-// pass, so a residual b - A x formed with this pass is exact to far below the 1e-6 the solves certify.
-// Row sums are double-float per tile and FP64 across tiles.  General exponents take the power in FP64.
+// |d_ab|^-(4+p), d_ab = g_ia - g_jb; (A u) at i1, i2 = -/+ h_I / l_I + l_I / 2.  Every quantity is a
+// double-float (hi + lo, ~48 bits) built from the FP64 positions, tangents, lengths and u, with
+// |T x d|^2 = |d|^2 - (T . d)^2; the powers are FP64 and bound the pass.
 //
-// The pass is symmetric (as pairs_sym.cu): the Gram weights satisfy w_IJ = w_JI and enter the low-order
-// form as w0_IJ + w0_JI, so one evaluation of an unordered pair {I, J} yields what row I receives from J
-// and what row J receives from I.  Items are edge-block pairs (b, c >= b); lane l of a warp takes source
-// (step + l) mod P at each step, and the source rows' terms go to per-warp double-float accumulators in
-// shared memory (no atomics); target rows of block b write partial slot c, source rows of block c slot
-// b, the diagonal item (b, b) is a plain gather writing slot b.  Every row receives one write per slot,
-// so the result is deterministic.
+// The weights are symmetric, so one evaluation of an unordered pair yields both rows' terms.  Items are
+// edge-block pairs (b, c >= b); lane l of a warp takes source (step + l) mod P at each step, and the source
+// rows' terms go to per-warp double-float accumulators in shared memory (no atomics); target rows of block b
+// write partial slot c, source rows of block c slot b, the diagonal item (b, b) is a plain gather writing slot
+// b.  Every row receives one write per slot, so the result is deterministic.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "df.cuh"
 #include "tpe_internal.cuh"
@@ -84,38 +78,16 @@ __device__ __forceinline__ df df3_dot(const DfV3 &a, const DfV3 &b)
 
 __device__ __forceinline__ df df3_norm2(const DfV3 &a) { return df_add(df_add(df_sqr(a.x), df_sqr(a.y)), df_sqr(a.z)); }
 
-// F = |d|^-p and G = |d|^-(4+p) from d2 = |d|^2 (p = 2.5 in the fast path).
-// r0 = rsqrt(d2.hi) has some ulp of error; rho = 1 - d2 r0^2 is formed exactly enough through fma
-// (r0^2 = a + b exactly), and r = r0 (1 + eps), eps = rho / 2 + 3 rho^2 / 8.  sqrt(r0) = q0 + (r0 - q0^2)
-// / (2 q0) likewise.  Then |d|^-2.5 = r0^2 sqrt(r0) (1 + eps)^2.5 and |d|^-2 = r0^2 (1 + eps)^2.
-template <bool FAST>
+// F = |d|^-p and G = |d|^-(4+p) from d2 = |d|^2, the power in FP64
 __device__ __forceinline__ void df_powers(df d2, double p, df &F, df &G)
 {
-    if constexpr (FAST) {
-        const float r0 = rsqrtf(d2.hi);
-        const float a = __fmul_rn(r0, r0);
-        const float b = __fmaf_rn(r0, r0, -a);
-        float rho = __fmaf_rn(-d2.hi, a, 1.f);
-        rho = __fmaf_rn(-d2.hi, b, rho);
-        rho = __fmaf_rn(-d2.lo, a, rho);
-        const float eps = rho * (0.5f + 0.375f * rho);
-        const float q0 = sqrtf(r0);
-        const float dq = __fmaf_rn(-q0, q0, r0) * (0.5f / q0);
-        const df R2 = fast_two_sum(a, b);
-        const df Q = fast_two_sum(q0, dq);
-        F = df_scale1p(df_mul(R2, Q), eps * (2.5f + 1.875f * eps));
-        const df Rsq = df_scale1p(R2, eps * (2.f + eps));  // |d|^-2
-        G = df_mul(F, df_sqr(Rsq));
-    } else {
-        const double d2d = df_to_double(d2);
-        const double f = pow(d2d, -0.5 * p);
-        F = df_from_double(f);
-        G = df_from_double(f / (d2d * d2d));
-    }
+    const double d2d = df_to_double(d2);
+    const double f = pow(d2d, -0.5 * p);
+    F = df_from_double(f);
+    G = df_from_double(f / (d2d * d2d));
 }
 
 // One unordered pair {I, J}: row I's terms into (A1, A2), row J's into (H, L) (all double-float).
-template <bool FAST>
 __device__ __forceinline__ void df_pair_both(const DfEdge &t, const DfEdge &s, double p, df (&A1)[3], df (&A2)[3],
                                              df (&H)[3], df (&L)[3])
 {
@@ -128,7 +100,7 @@ __device__ __forceinline__ void df_pair_both(const DfEdge &t, const DfEdge &s, d
 #pragma unroll
     for (int ab = 0; ab < 4; ++ab) {
         d2[ab] = df_add_pos(df_add_pos(df_sqr(d[ab].x), df_sqr(d[ab].y)), df_sqr(d[ab].z));
-        df_powers<FAST>(d2[ab], p, F[ab], G[ab]);
+        df_powers(d2[ab], p, F[ab], G[ab]);
     }
     // |T_I x d_ab|^2 depends on b only, |T_J x d_ab|^2 on a only (g_i2 = g_i1 + l_I T_I)
     const df tI1 = df3_dot(t.T, d[0]), tI2 = df3_dot(t.T, d[1]);
@@ -155,8 +127,7 @@ __device__ __forceinline__ void df_pair_both(const DfEdge &t, const DfEdge &s, d
     }
 }
 
-template <bool FAST>
-__global__ void __launch_bounds__(kThreads, 2) k_apply_df_sym(const DfArgs a)
+__global__ void __launch_bounds__(kThreads, 2) k_apply_df_general(const DfArgs a)
 {
     constexpr int kW = kThreads / 32;
     __shared__ RecF sr[kTile];
@@ -207,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_apply_df_sym(const DfArgs a)
                     if (keep) {
                         df H[3] = {df_make(0.f), df_make(0.f), df_make(0.f)};
                         df L[3] = {df_make(0.f), df_make(0.f), df_make(0.f)};
-                        df_pair_both<FAST>(t, s, a.p, A1, A2, H, L);
+                        df_pair_both(t, s, a.p, A1, A2, H, L);
                         if (!diag) {
 #pragma unroll
                             for (int q = 0; q < 3; ++q) {
@@ -257,33 +228,74 @@ __global__ void __launch_bounds__(kThreads, 2) k_apply_df_sym(const DfArgs a)
     }
 }
 
-static int df_occupancy(bool fast)
+// Edge blocks of 128 per problem; items (b, c >= b) sorted by problem size (large first).
+static void plan_items(Ctx &c, Ctx::Plan &pl, int occupancy)
+{
+    const int tb = kThreads;
+    std::vector<std::pair<long long, WorkItem>> tmp;
+    std::vector<int> eslots(std::max(1, c.nE), 1);
+    int max_slots = 1;
+    for (int q = 0; q < c.nProb; ++q) {
+        const int e0 = c.h_prob_e[q], e1 = c.h_prob_e[q + 1], n = e1 - e0;
+        if (n <= 0) continue;
+        const int nblk = (n + tb - 1) / tb;
+        max_slots = std::max(max_slots, nblk);
+        for (int b = 0; b < nblk; ++b) {
+            const int t0 = e0 + b * tb, nt = std::min(tb, e1 - t0);
+            for (int cb = b; cb < nblk; ++cb) {
+                const int s0 = e0 + cb * tb, s1 = std::min(e1, s0 + tb);
+                tmp.push_back({(long long)n, WorkItem{t0, nt, s0, s1, (b << 16) | cb, e0, e1 - 1, q}});
+            }
+        }
+        for (int I = e0; I < e1; ++I) eslots[I] = nblk;
+    }
+    std::stable_sort(tmp.begin(), tmp.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+    std::vector<WorkItem> items;
+    items.reserve(tmp.size());
+    for (auto &t : tmp) items.push_back(t.second);
+    pl.n_items = (int)items.size();
+    pl.max_slots = max_slots;
+    pl.tpt = 1;
+    pl.grid = std::max(1, std::min(pl.n_items, c.sm_count * std::max(1, occupancy)));
+    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
+    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
+    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
+    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
+}
+
+static int df_occupancy()
 {
     int occ = 0;
-    if (fast)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_df_sym<true>, kThreads, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_df_sym<false>, kThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_df_general, kThreads, 0);
     return occ;
 }
 
-// Au = A-bar u in double-float arithmetic on the geometry slot `which` (records built for that curve).
-// Contexts in FP64 run their own FP64 pass instead.  Uses its own work list of edge-block pairs (128-edge
-// blocks) and the context's partial-sum buffer (one slot per block of the largest problem).
+// Au = A-bar u in double-float arithmetic on the geometry slot `which` (records built for that curve): the
+// packed pass of pairs_sym.cu with the specialised powers, the pass above otherwise.  Contexts in FP64 run
+// their own FP64 pass instead.  Work list and partial sums are built and grown at the first call.
 cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const double *u, double *Au, cudaStream_t s)
 {
     if (c.prm.precision == TP_FP64) return pair_apply(c, gamma_geom, which, u, Au, s);
     Ctx::Plan &pl = c.plan_df;
-    if (!pl.d_items) sym_plan_items(c, pl, 1, df_occupancy(c.kp.fast != 0));
+    if (pl.d_items && (pl.tpt == 1) == (c.kp.fast != 0)) {  // the exponents changed since the last call
+        TPE_CHECK(cudaFree(pl.d_items));
+        TPE_CHECK(cudaFree(pl.d_eslots));
+        pl = Ctx::Plan{};
+    }
+    TPE_CHECK(build_urecs(c, u, which, s));
+    if (c.kp.fast) {
+        TPE_CHECK(sym_apply_accurate_pass(c, which, s));
+        return vertices_apply(c, Au, s);
+    }
+    if (!pl.d_items) plan_items(c, pl, df_occupancy());
     // the buffer is shared with the other passes and may have been resized since the last call
     const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
     if (need > c.part_elems) {
+        graphs_reset(c);  // captured blocks hold the old partial buffer
         TPE_CHECK(cudaFree(c.d_part));
         TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
         c.part_elems = need;
-        graphs_reset(c);  // captured blocks hold the old partial buffer
     }
-    TPE_CHECK(build_urecs(c, u, which, s));
     if (pl.n_items == 0) return cudaMemsetAsync(Au, 0, sizeof(double) * 3 * c.nV, s);
     TPE_CHECK(cudaMemsetAsync(c.d_counter + 7, 0, sizeof(int), s));
     DfArgs a;
@@ -300,10 +312,7 @@ cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const do
     a.p = c.kp.p;
     a.skip = c.d_skip;
     const int slot = c.profile ? prof_begin(c, 5, s) : -1;
-    if (c.kp.fast)
-        k_apply_df_sym<true><<<pl.grid, kThreads, 0, s>>>(a);
-    else
-        k_apply_df_sym<false><<<pl.grid, kThreads, 0, s>>>(a);
+    k_apply_df_general<<<pl.grid, kThreads, 0, s>>>(a);
     if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
     c.launches++;
     TPE_CHECK(cudaGetLastError());

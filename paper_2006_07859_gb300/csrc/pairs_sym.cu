@@ -61,6 +61,7 @@ struct SymArgs {
     const RecF *recF;
     const RecLo *recLo;
     const URecF *urecF;
+    const float *ell_lo;  // PDF
     float2 *part;  // [slot][nE][W]
     int nE;
     float near2f, mid2f;
@@ -76,9 +77,10 @@ __host__ __device__ constexpr int sym_width()
 // Source tile (struct of arrays, 16-byte elements) and the warps' source accumulators.
 template <int PREC, int OP>
 struct SymSmem {
-    static constexpr bool MIX = PREC == PMIX, U = OP == OP_APPLY;
+    static constexpr bool MIX = PREC != P32, U = OP == OP_APPLY;
     float4 t0[kTile], t1[kTile], t2[kTile];  // (q1, l), (e, T.x), (T.y, T.z, q1.x lo, q1.y lo)
     float4 t3[MIX ? kTile : 1];              // (q1.z lo, T lo)
+    float4 t4[PREC == PDF ? kTile : 1];      // (e lo, l lo)
     float4 u0[U ? kTile : 1], u1[U ? kTile : 1], u2[(U && MIX) ? kTile : 1];
     int2 id[kTile];
     float2 sac[kSymWarps][sym_width<OP>()][kTile];  // (sum, Kahan compensation)
@@ -90,7 +92,8 @@ struct SymSmem {
 };
 
 struct SymSrc {
-    float q[3], m[3], e[3], T[3], Tm[3], ell;
+    float q[3], m[3], e[3], T[3], Tm[3], ell;  // PDF: em the low part of e
+    float em[3], ell_lo;
     int j1, j2;
 };
 
@@ -101,7 +104,11 @@ __device__ __forceinline__ void sym_load(SymSrc &s, const SymSmem<PREC, OP> &tl,
     s.q[0] = a.x, s.q[1] = a.y, s.q[2] = a.z, s.ell = a.w;
     s.e[0] = b.x, s.e[1] = b.y, s.e[2] = b.z, s.T[0] = b.w;
     s.T[1] = c.x, s.T[2] = c.y;
-    if constexpr (PREC == PMIX) {
+    if constexpr (PREC == PDF) {
+        const float4 d = tl.t4[j];
+        s.em[0] = d.x, s.em[1] = d.y, s.em[2] = d.z, s.ell_lo = d.w;
+    }
+    if constexpr (PREC != P32) {
         const float4 d = tl.t3[j];
         s.m[0] = c.z, s.m[1] = c.w, s.m[2] = d.x;
         s.Tm[0] = d.y, s.Tm[1] = d.z, s.Tm[2] = d.w;
@@ -119,8 +126,9 @@ using L2 = float2;
 // Two target rows of a thread (rows of invalid lanes repeat the last one with length 0, so that they feed
 // nothing into the sources).
 struct SymTgt {
-    LV<L2> p, pl, e, T, Tl;
-    L2 ell;
+    LV<L2> p, pl, e, T, Tl;  // PDF: el the low part of e
+    LV<L2> el;
+    L2 ell, ell_lo;
     int i1[2], i2[2], row[2];
 };
 
@@ -193,11 +201,117 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &, const
     *sac = ac;
 }
 
+// F = |d|^-2.5 and G = |d|^-6.5 in double-float from |d|^2: r0 = rsqrt(d2.hi), its residual rho = 1 - d2 r0^2 formed
+// through fma, |d|^-1 = r0 (1 + eps) with eps = rho / 2 + 3 rho^2 / 8, and sqrt(r0) = q0 + (r0 - q0^2) / (2 q0).
+__device__ __forceinline__ void sym_df_powers(dfl<L2> d2, dfl<L2> &F, dfl<L2> &G)
+{
+    const L2 r0 = l_rsqrt(d2.hi);
+    const L2 a = l_mul(r0, r0), b = l_fma(r0, r0, l_neg(a));
+    L2 rho = l_fma(l_neg(d2.hi), a, l_bc<L2>(1.f));
+    rho = l_fma(l_neg(d2.hi), b, rho);
+    rho = l_fma(l_neg(d2.lo), a, rho);
+    const L2 eps = l_mul(rho, l_fma(l_bc<L2>(0.375f), rho, l_bc<L2>(0.5f)));
+    const L2 iq = l_mul(l_bc<L2>(0.5f), l_rsqrt(r0));
+    L2 q0 = l_mul(r0, l_add(iq, iq));
+    q0 = l_fma(l_fma(l_neg(q0), q0, r0), iq, q0);  // to half an ulp: dq leaves out (r0 - q0^2)^2 / (8 q0^3)
+    const L2 dq = l_mul(l_fma(l_neg(q0), q0, r0), iq);
+    const dfl<L2> R = {a, b};
+    F = l_dfscale(l_dfmul(R, dfl<L2>{q0, dq}), l_mul(eps, l_fma(l_bc<L2>(1.875f), eps, l_bc<L2>(2.5f))));
+    const dfl<L2> R2 = l_dfscale(R, l_mul(eps, l_add(l_bc<L2>(2.f), eps)));  // |d|^-2
+    G = l_dfmul(F, l_dfsqr(R2));
+}
+
+// a - b with both parts' differences exact: rounding al - bl leaves 2^-49 |a|, which for neighbouring edges (|a - b|
+// ~ 1e-3 |a|) is a thousand times the rounding of everything else (5.6e-13 against 1.5e-13 in A u at 500 edges).
+template <class L>
+__device__ __forceinline__ dfl<L> l_dfdiff(L ah, L al, L bh, L bl)
+{
+    const dfl<L> s = l_two_sum(ah, l_neg(bh)), t = l_two_sum(al, l_neg(bl));
+    const dfl<L> r = l_dfnorm(dfl<L>{s.hi, l_add(s.lo, t.hi)});
+    return l_dfnorm(dfl<L>{r.hi, l_add(r.lo, t.lo)});
+}
+
+// source sum += both lanes' double-float terms
+__device__ __forceinline__ void src_add_df(float2 &ac, dfl<L2> v)
+{
+    l_kahan_df(ac.x, ac.y, v.hi.x, v.lo.x);
+    l_kahan_df(ac.x, ac.y, v.hi.y, v.lo.y);
+}
+
+// The accurate apply: every quantity of the pair a double-float, about 1,000 operations against the mixed
+// apply's 195; FP32 operand reads bound it (8 x 4,096 edges 2.78 ms; one target per thread in scalar double-float
+// arithmetic took 4.75).  Its error against FP64 stays that of fully renormalised arithmetic (1.5e-13 at 500
+// edges, 8.8e-13 at 4,096, random u) as long as the differences are exact and t is renormalised before t^2.
+// Sums are (sum, minus low part) like the compensated ones.
+template <bool CHECK>
+__device__ __forceinline__ void sym_pair_df(const SymTgt &t, const SymTgtU &tu, const SymSmem<PDF, OP_APPLY> &tl,
+                                            const SymSrc &s, int j, bool k0, bool k1, SymAcc<PDF, OP_APPLY> &a,
+                                            float2 *sac)
+{
+    const dfv<L2> TI = {{t.T.x, t.Tl.x}, {t.T.y, t.Tl.y}, {t.T.z, t.Tl.z}};
+    const dfv<L2> TJ = {{l_bc<L2>(s.T[0]), l_bc<L2>(s.Tm[0])}, {l_bc<L2>(s.T[1]), l_bc<L2>(s.Tm[1])},
+                        {l_bc<L2>(s.T[2]), l_bc<L2>(s.Tm[2])}};
+    const dfv<L2> eI = {{t.e.x, t.el.x}, {t.e.y, t.el.y}, {t.e.z, t.el.z}};
+    const dfv<L2> eJ = {{l_bc<L2>(-s.e[0]), l_bc<L2>(-s.em[0])}, {l_bc<L2>(-s.e[1]), l_bc<L2>(-s.em[1])},
+                        {l_bc<L2>(-s.e[2]), l_bc<L2>(-s.em[2])}};
+    const auto add3 = [](const dfv<L2> &x, const dfv<L2> &y) {
+        return dfv<L2>{l_dfnorm(l_dfadd(x.x, y.x)), l_dfnorm(l_dfadd(x.y, y.y)), l_dfnorm(l_dfadd(x.z, y.z))};
+    };
+    dfv<L2> dd4[4];
+    dd4[0] = {l_dfdiff(t.p.x, t.pl.x, l_bc<L2>(s.q[0]), l_bc<L2>(s.m[0])),
+              l_dfdiff(t.p.y, t.pl.y, l_bc<L2>(s.q[1]), l_bc<L2>(s.m[1])),
+              l_dfdiff(t.p.z, t.pl.z, l_bc<L2>(s.q[2]), l_bc<L2>(s.m[2]))};
+    dd4[1] = add3(dd4[0], eJ);
+    dd4[2] = add3(dd4[0], eI);
+    dd4[3] = add3(dd4[1], eI);
+    dfl<L2> d2[4], F[4], G[4], cI[2], cJ[2];
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+        const dfv<L2> &d = dd4[ab];
+        d2[ab] = l_dfnorm2(d);
+        sym_df_powers(d2[ab], F[ab], G[ab]);
+        // |T_I x d_ab|^2 depends on b only, |T_J x d_ab|^2 on a only (g_i2 = g_i1 + l_I T_I)
+        if (ab < 2) cI[ab] = l_dfnorm(l_dfadd(d2[ab], l_dfneg(l_dfsqr(l_dfnorm(l_dfdot(TI, d))))));
+        if (!(ab & 1)) cJ[ab >> 1] = l_dfnorm(l_dfadd(d2[ab], l_dfneg(l_dfsqr(l_dfnorm(l_dfdot(TJ, d))))));
+    }
+    dfl<L2> sw = l_dfadd(l_dfadd(F[0], F[3]), l_dfadd(F[1], F[2]));
+    dfl<L2> sw0 = l_dfadd(l_dfadd(l_dfmul(l_dfadd(cI[0], cJ[0]), G[0]), l_dfmul(l_dfadd(cI[1], cJ[1]), G[3])),
+                          l_dfadd(l_dfmul(l_dfadd(cI[1], cJ[0]), G[1]), l_dfmul(l_dfadd(cI[0], cJ[1]), G[2])));
+    if constexpr (CHECK) {
+        sw = {l_keep(k0, k1, sw.hi), l_keep(k0, k1, sw.lo)};
+        sw0 = {l_keep(k0, k1, sw0.hi), l_keep(k0, k1, sw0.lo)};
+    }
+    const dfl<L2> ls = {l_bc<L2>(s.ell), l_bc<L2>(s.ell_lo)}, lt = {t.ell, t.ell_lo};
+    const dfl<L2> Wt = l_dfmul(ls, sw), W0t = l_dfmul(ls, sw0), Ws = l_dfmul(lt, sw), W0s = l_dfneg(l_dfmul(lt, sw0));
+    const dfv<L2> dT = {l_dfdiff(TI.x.hi, TI.x.lo, TJ.x.hi, TJ.x.lo), l_dfdiff(TI.y.hi, TI.y.lo, TJ.y.hi, TJ.y.lo),
+                        l_dfdiff(TI.z.hi, TI.z.lo, TJ.z.hi, TJ.z.lo)};
+    const dfl<L2> n2 = l_dfnorm2(dT), omt = {l_mul(l_bc<L2>(0.5f), n2.hi), l_mul(l_bc<L2>(0.5f), n2.lo)};
+    const float4 x = tl.u0[j], y = tl.u1[j], z = tl.u2[j];
+    const L2 sd[3] = {l_bc<L2>(x.x), l_bc<L2>(x.y), l_bc<L2>(x.z)}, sdl[3] = {l_bc<L2>(y.z), l_bc<L2>(y.w), l_bc<L2>(z.x)};
+    const L2 sb[3] = {l_bc<L2>(x.w), l_bc<L2>(y.x), l_bc<L2>(y.y)}, sbl[3] = {l_bc<L2>(z.y), l_bc<L2>(z.z), l_bc<L2>(z.w)};
+    const L2 td[3] = {tu.dh.x, tu.dh.y, tu.dh.z}, tdl[3] = {tu.dl.x, tu.dl.y, tu.dl.z};
+    const L2 tb[3] = {tu.uh.x, tu.uh.y, tu.uh.z}, tbl[3] = {tu.ul.x, tu.ul.y, tu.ul.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const dfl<L2> dd = l_dfdiff(td[k], tdl[k], sd[k], sdl[k]), db = l_dfdiff(tb[k], tbl[k], sb[k], sbl[k]);
+        // row I: (du_I - du_J) + omt du_J;  row J: (du_J - du_I) + omt du_I
+        const dfl<L2> h = l_dfmul(Wt, l_dfadd(dd, l_dfmul(omt, dfl<L2>{sd[k], sdl[k]}))), m = l_dfmul(W0t, db);
+        l_kahan_df(a.s[k], a.c[k], h.hi, h.lo);
+        l_kahan_df(a.s[3 + k], a.c[3 + k], m.hi, m.lo);
+        float2 ac = sac[k * kTile], bc = sac[(3 + k) * kTile];
+        src_add_df(ac, l_dfmul(Ws, l_dfadd(l_dfmul(omt, dfl<L2>{td[k], tdl[k]}), l_dfneg(dd))));
+        src_add_df(bc, l_dfmul(W0s, db));
+        sac[k * kTile] = ac;
+        sac[(3 + k) * kTile] = bc;
+    }
+}
+
 template <int PREC, bool CHECK, int MODE>
 __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &tu, const SymSmem<PREC, OP_APPLY> &tl,
                                          const SymSrc &s, int j, int, bool k0, bool k1, SymAcc<PREC, OP_APPLY> &a,
                                          float2 *sac, const SymArgs &, bool &, bool &)
 {
+    if constexpr (PREC == PDF) return sym_pair_df<CHECK>(t, tu, tl, s, j, k0, k1, a, sac);
     constexpr bool MIX = PREC == PMIX;
     LV<L2> d[4];
     l_chords<(MODE >= 1 && MIX)>(t.p, t.pl, t.e, l_bc3<L2>(s.q[0], s.q[1], s.q[2]), l_bc3<L2>(s.m[0], s.m[1], s.m[2]),
@@ -416,7 +530,7 @@ template <int PREC, int OP, int MB>
 __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
 {
     constexpr int W = sym_width<OP>();
-    constexpr bool MIX = PREC == PMIX, NEAR = MIX && OP != OP_APPLY;
+    constexpr bool MIX = PREC != P32, DF = PREC == PDF, NEAR = PREC == PMIX && OP != OP_APPLY;
     extern __shared__ __align__(16) unsigned char dyn[];
     SymSmem<PREC, OP> &sm = *reinterpret_cast<SymSmem<PREC, OP> *>(dyn);
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -461,7 +575,16 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
             if constexpr (MIX) {
                 t.pl = {TPE_Q2(lo.x), TPE_Q2(lo.y), TPE_Q2(lo.z)};
                 t.Tl = {TPE_Q2(lo2.z), TPE_Q2(lo2.w), TPE_Q2(lo3.x)};
-                t.e = {TPE_Q2(lo3.y), TPE_Q2(lo3.z), TPE_Q2(lo3.w)};
+                if constexpr (DF) {
+                    const dfl<L2> ex = l_dfdiff(TPE_L2(b.x), TPE_Q2(lo.w), t.p.x, t.pl.x),
+                                  ey = l_dfdiff(TPE_L2(b.y), TPE_Q2(lo2.x), t.p.y, t.pl.y),
+                                  ez = l_dfdiff(TPE_L2(b.z), TPE_Q2(lo2.y), t.p.z, t.pl.z);
+                    t.e = {ex.hi, ey.hi, ez.hi};
+                    t.el = {ex.lo, ey.lo, ez.lo};
+                    t.ell_lo = make_float2(valid[0] ? pa.ell_lo[t.row[0]] : 0.f, valid[1] ? pa.ell_lo[t.row[1]] : 0.f);
+                } else {
+                    t.e = {TPE_Q2(lo3.y), TPE_Q2(lo3.z), TPE_Q2(lo3.w)};
+                }
             } else {
                 t.e = l_sub3(LV<L2>{TPE_L2(b.x), TPE_L2(b.y), TPE_L2(b.z)}, t.p);
             }
@@ -504,7 +627,14 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
                 sm.id[j] = make_int2(__float_as_int(r.c.z), __float_as_int(r.c.w));
                 if constexpr (MIX) {
                     const RecLo q = pa.recLo[J];
-                    sm.t1[j] = make_float4(q.lo3.y, q.lo3.z, q.lo3.w, r.b.w);
+                    if constexpr (DF) {
+                        const dfl<float> ex = l_dfdiff(r.b.x, q.lo.w, r.a.x, q.lo.x), ey = l_dfdiff(r.b.y, q.lo2.x, r.a.y, q.lo.y),
+                                         ez = l_dfdiff(r.b.z, q.lo2.y, r.a.z, q.lo.z);
+                        sm.t1[j] = make_float4(ex.hi, ey.hi, ez.hi, r.b.w);
+                        sm.t4[j] = make_float4(ex.lo, ey.lo, ez.lo, pa.ell_lo[J]);
+                    } else {
+                        sm.t1[j] = make_float4(q.lo3.y, q.lo3.z, q.lo3.w, r.b.w);
+                    }
                     sm.t2[j] = make_float4(r.c.x, r.c.y, q.lo.x, q.lo.y);
                     sm.t3[j] = make_float4(q.lo.z, q.lo2.z, q.lo2.w, q.lo3.x);
                     box_add(sb, V3<float>{r.a.x, r.a.y, r.a.z}, V3<float>{r.b.x, r.b.y, r.b.z});
@@ -532,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
                     const float gap = fmaxf(fmaxf(sb[q] - tbox[3 + q], tbox[q] - sb[3 + q]), 0.f);
                     g2 += gap * gap;
                 }
-                mode = (NEAR && g2 < pa.near2f) ? 2 : (g2 < pa.mid2f ? 1 : 0);
+                mode = (NEAR && g2 < pa.near2f) ? 2 : (DF || g2 < pa.mid2f ? 1 : 0);
             }
             constexpr int MN = NEAR ? 2 : 1;
             if (diag) {
@@ -556,7 +686,7 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
                     sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
                 else if (mode == 1 || !MIX)
                     sym_section<PREC, OP, false, 1, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
-                else
+                else if constexpr (PREC == PMIX)
                     sym_section<PREC, OP, false, 0, false>(t, tu, sm, wid, s0, 0, cnt, a, queued, w, pa);
             }
             if constexpr (OP == OP_DIFF) {
@@ -619,7 +749,8 @@ __device__ __forceinline__ void diff_row_out(const double *T, double l, const do
 
 // Sum the slots of every row (one thread per value, so that a slot's values are read coalesced) and form the
 // row's outputs: energy rows (l_I / 4) sum, or the six endpoint values of an edge into esum.
-template <int OP>
+// D64: in FP64 (the accurate apply), else in double-float.
+template <int OP, bool D64 = false>
 __global__ void __launch_bounds__(OP == OP_ENERGY ? 256 : 32 * sym_width<OP>())
 k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ part, const double *__restrict__ ell,
           const double *__restrict__ T, double *__restrict__ out)
@@ -640,6 +771,10 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
             for (int k = 0; k < 8; ++k) v[k] = __ldcs(p + (size_t)(q + k) * step);
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
+                if constexpr (D64) {
+                    x += (double)v[k].x + (double)v[k].y;
+                    continue;
+                }
                 const df r = two_sum(s, v[k].x);
                 s = r.hi;
                 lo = __fadd_rn(lo, __fadd_rn(r.lo, v[k].y));
@@ -647,11 +782,15 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
         }
         for (; q < ns; ++q) {
             const float2 v = __ldcs(p + (size_t)q * step);
+            if constexpr (D64) {
+                x += (double)v.x + (double)v.y;
+                continue;
+            }
             const df r = two_sum(s, v.x);
             s = r.hi;
             lo = __fadd_rn(lo, __fadd_rn(r.lo, v.y));
         }
-        x = (double)s + (double)lo;
+        if constexpr (!D64) x = (double)s + (double)lo;
     }
     if constexpr (OP == OP_ENERGY) {
         if (row < nE) out[row] = 0.25 * ell[row] * x;
@@ -676,42 +815,6 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
 }
 
 // ---------------------------------------------------------------------------------- host side
-
-// Edge blocks of 128 x tpt per problem; items (b, c >= b) sorted by problem size (large first): the
-// double-float apply's work list.
-void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
-{
-    const int tb = kThreads * tpt;
-    std::vector<std::pair<long long, WorkItem>> tmp;
-    std::vector<int> eslots(std::max(1, c.nE), 1);
-    int max_slots = 1;
-    for (int q = 0; q < c.nProb; ++q) {
-        const int e0 = c.h_prob_e[q], e1 = c.h_prob_e[q + 1], n = e1 - e0;
-        if (n <= 0) continue;
-        const int nblk = (n + tb - 1) / tb;
-        max_slots = std::max(max_slots, nblk);
-        for (int b = 0; b < nblk; ++b) {
-            const int t0 = e0 + b * tb, nt = std::min(tb, e1 - t0);
-            for (int cb = b; cb < nblk; ++cb) {
-                const int s0 = e0 + cb * tb, s1 = std::min(e1, s0 + tb);
-                tmp.push_back({(long long)n, WorkItem{t0, nt, s0, s1, (b << 16) | cb, e0, e1 - 1, q}});
-            }
-        }
-        for (int I = e0; I < e1; ++I) eslots[I] = nblk;
-    }
-    std::stable_sort(tmp.begin(), tmp.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
-    std::vector<WorkItem> items;
-    items.reserve(tmp.size());
-    for (auto &t : tmp) items.push_back(t.second);
-    pl.n_items = (int)items.size();
-    pl.max_slots = max_slots;
-    pl.tpt = tpt;
-    pl.grid = std::max(1, std::min(pl.n_items, c.sm_count * std::max(1, occupancy)));
-    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
-    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
-    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
-    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
-}
 
 // Tiles per item: four (fewer partial slots, longer runs per target load) once every resident CTA gets about
 // six items that way, fewer on smaller graphs so that the last wave stays short.
@@ -800,6 +903,8 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
     cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
 }
 
+constexpr int kSymAccurate = 100;  // the apply in double-float
+
 // Variants differ in the CTAs per SM that the register allocation is held to.
 template <class F>
 static void with_sym_kernel(int prec, int op, int variant, F f)
@@ -817,7 +922,9 @@ static void with_sym_kernel(int prec, int op, int variant, F f)
         else
             f(k_sym<PMIX, OP_DIFF, 2>, sizeof(SymSmem<PMIX, OP_DIFF>));
     } else {
-        if (prec == TP_FP32)
+        if (variant == kSymAccurate)
+            f(k_sym<PDF, OP_APPLY, 2>, sizeof(SymSmem<PDF, OP_APPLY>));
+        else if (prec == TP_FP32)
             f(k_sym<P32, OP_APPLY, 3>, sizeof(SymSmem<P32, OP_APPLY>));
         else if (variant == 2)
             f(k_sym<PMIX, OP_APPLY, 2>, sizeof(SymSmem<PMIX, OP_APPLY>));
@@ -900,7 +1007,7 @@ cudaError_t sym_defaults(Ctx &c)
 static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof_op, int which, const int *skip, double *out,
                             cudaStream_t s)
 {
-    if (pl.n_items == 0) return cudaSuccess;
+    if (pl.n_items == 0) return cudaSuccess;  // no edges: nothing reads the sums
     TPE_CHECK(cudaMemsetAsync(c.d_counter + counter, 0, sizeof(int), s));
     SymArgs pa;
     pa.items = pl.d_items;
@@ -909,6 +1016,7 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
     pa.recF = which ? c.d_recF2 : c.d_recF;
     pa.recLo = which ? c.d_recLo2 : c.d_recLo;
     pa.urecF = c.d_urecF;
+    pa.ell_lo = c.d_ell_lo[which];
     pa.part = reinterpret_cast<float2 *>(c.d_part);
     pa.nE = c.nE;
     pa.near2f = op == OP_DIFF ? c.kp.near2f_diff : c.kp.near2f;
@@ -922,6 +1030,8 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
         k_sym_sum<OP_ENERGY><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     else if (op == OP_DIFF)
         k_sym_sum<OP_DIFF><<<(c.nE + 31) / 32, 320, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+    else if (pl.tpt == kSymAccurate)
+        k_sym_sum<OP_APPLY, true><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     else
         k_sym_sum<OP_APPLY><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     c.launches += 2;
@@ -941,6 +1051,25 @@ cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s)
 cudaError_t sym_apply_pass(Ctx &c, int which, cudaStream_t s)
 {
     return sym_pass(c, OP_APPLY, c.plan_sym, 4, c.d_skip ? 4 : 2, which, c.d_skip, c.d_esum, s);
+}
+
+// The accurate apply (edges' endpoint values into c.d_esum); its plan is built at the first call.
+cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s)
+{
+    Ctx::Plan &pl = c.plan_df;
+    if (!pl.d_items) {
+        sym_plan(c, pl, sym_occupancy(c, OP_APPLY, kSymAccurate));
+        pl.tpt = kSymAccurate;
+    }
+    // the buffer is shared with the other passes and may have been resized since the last call
+    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(OP_APPLY);
+    if (need > c.part_elems) {
+        graphs_reset(c);  // captured blocks hold the old partial buffer
+        TPE_CHECK(cudaFree(c.d_part));
+        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
+        c.part_elems = need;
+    }
+    return sym_pass(c, OP_APPLY, pl, 7, 5, which, c.d_skip, c.d_esum, s);
 }
 
 }  // namespace tpe

@@ -22,7 +22,7 @@ struct PinState;
 struct BhState;
 
 // Precision of the pair arithmetic.
-enum Prec { P64 = 0, P32 = 1, PMIX = 2 };
+enum Prec { P64 = 0, P32 = 1, PMIX = 2, PDF = 3 };  // PDF: double-float throughout (the accurate apply)
 
 // Which quantity a pair pass accumulates.
 enum PairOp { OP_ENERGY = 0, OP_DIFF = 1, OP_APPLY = 2, OP_DIAG = 3 };
@@ -133,7 +133,7 @@ struct Ctx {
     int energy_sym = 0;      // > 0: the energy runs the symmetric pass with this many targets per thread
     Plan plan_sym_d;         // symmetric differential (pairs_sym.cu)
     int diff_sym = 0;        // > 0: the differential runs the symmetric pass
-    Plan plan_df;            // double-float apply (pairs_df.cu), built at its first use
+    Plan plan_df;            // double-float apply, built at its first use (tpt 1: general exponents)
     Plan plan_multi;         // multi-field apply (pairs_multi.cu), built at its first use
     URecF *d_urecMF = nullptr;  // multi-field apply: per-edge records of kMultiG fields (FP32 contexts)
     URecD *d_urecMD = nullptr;  // the same in FP64 contexts
@@ -240,8 +240,8 @@ cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const 
                              cudaStream_t s);
 void multi_free(Ctx &c);
 void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
-void sym_plan_items(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);  // (pairs_sym.cu) items (b, c >= b)
 cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s);
+cudaError_t vertices_apply(Ctx &c, double *Au, cudaStream_t s);  // from the per-edge sums in c.d_esum
 // symmetric passes (pairs_sym.cu): a variant > 0 or the gather pass (0); the passes write the energy rows
 // [nE] or the edges' endpoint values into c.d_esum
 cudaError_t sym_select(Ctx &c, int variant);
@@ -250,6 +250,7 @@ cudaError_t sym_select_energy(Ctx &c, int variant);
 cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s);
 cudaError_t sym_select_diff(Ctx &c, int variant);
 cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
+cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s);  // specialised powers; grows c.d_part
 cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 void make_plans(Ctx &c);
