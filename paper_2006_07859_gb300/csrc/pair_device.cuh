@@ -26,10 +26,21 @@ __device__ __forceinline__ R inv_pow(R d2, R e, R &r2)
             r2 = r * r;
             return WHICH == 0 ? r2 * r2 * sr : r2 * sr;
         } else {
-            double r = rsqrt(d2);
-            double sr = sqrt(r);
-            r2 = r * r;
-            return WHICH == 0 ? r2 * r2 * sr : r2 * sr;
+            // y = |d|^-1/2 = d2^-1/4: two hardware approximations (2^-22), then one step of the series of
+            // (1 - e)^-1/4 with e = 1 - d2 y^4 (|e| < 2e-6, the cubic term is below 2^-53).  Ten FP64
+            // instructions where rsqrt() and sqrt() take about twenty: the FP64 passes are bound by their
+            // number (2 per clock and SM).
+            double r0, q0;
+            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d2));
+            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(q0) : "d"(r0));
+            double y = r0 * q0;
+            const double y2 = y * y;
+            const double e = fma(-d2, y2 * y2, 1.0);
+            y = fma(y, e * fma(0.15625, e, 0.25), y);
+            if (!(d2 > 0.0)) y = 1.0 / d2;  // coincident points: infinite, as the plain formula has it
+            const double yy = y * y;
+            r2 = yy * yy;
+            return WHICH == 0 ? r2 * r2 * y : r2 * y;
         }
     } else {
         if constexpr (sizeof(R) == 4) {
@@ -239,6 +250,13 @@ struct ApplyAcc64 {
 };
 
 // ---------------------------------------------------------------------------------- the pair kernel
+
+// A block that finds the queue empty (it >= n_items; thread 0 of every block draws one such number): the last of
+// them resets the counter for the next launch, which saves a memset before every pass.
+__device__ __forceinline__ void queue_done(int it, int n_items, int *counter)
+{
+    if (threadIdx.x == 0 && it == n_items + (int)gridDim.x - 1) *counter = 0;
+}
 
 struct PairArgs {
     const WorkItem *items;

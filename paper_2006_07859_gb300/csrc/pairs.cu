@@ -41,6 +41,21 @@ namespace tpe {
 
 // ---------------------------------------------------------------------------------- K0: edge records
 
+// isfinite without an FP64 comparison
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// a / b from ib = 1 / b with one residual correction: within an ulp of the quotient, three FP64 instructions after
+// the shared reciprocal.  An infinite or zero quotient has no residual and stays as it is.
+__device__ __forceinline__ double div_by(double a, double b, double ib)
+{
+    const double q = a * ib, r = fma(-q, b, a);
+    return finite64(r) ? fma(r, ib, q) : q;
+}
+
+// The per-edge kernels run in blocks of 64: FP64 instructions bound them (2 per clock and SM), so what counts is
+// that a short graph spreads over many SMs (256 edges in one block of 256 took 10 us).
+constexpr int kRecThreads = 64;
+
 __global__ void k_records(int nE, const double *__restrict__ g, const int *__restrict__ E, RecF *__restrict__ recF,
                           RecLo *__restrict__ recLo, RecD *__restrict__ recD, double *__restrict__ ell,
                           double *__restrict__ T, double *__restrict__ x, int *__restrict__ err,
@@ -56,7 +71,8 @@ __global__ void k_records(int nE, const double *__restrict__ g, const int *__res
         e[k] = p2[k] - p1[k];
     }
     double l = sqrt(e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
-    bool fin = isfinite(l) && isfinite(p1[0] + p1[1] + p1[2]) && isfinite(p2[0] + p2[1] + p2[2]);
+    bool fin = finite64(l);
+    for (int k = 0; k < 3; ++k) fin = fin && finite64(p1[k]) && finite64(p2[k]);
     if (!fin) {
         atomicCAS(err, 0, (int)TP_ERR_NONFINITE);
         l = 1.0;
@@ -64,7 +80,8 @@ __global__ void k_records(int nE, const double *__restrict__ g, const int *__res
         atomicCAS(err, 0, (int)TP_ERR_DEGENERATE_EDGE);
         l = 1.0;
     }
-    double t[3] = {e[0] / l, e[1] / l, e[2] / l};
+    const double li = 1.0 / l;
+    double t[3] = {div_by(e[0], l, li), div_by(e[1], l, li), div_by(e[2], l, li)};
     ell[I] = l;
     if (ell_lo) ell_lo[I] = (float)(l - (double)(float)l);
     for (int k = 0; k < 3; ++k) {
@@ -114,10 +131,11 @@ __global__ void k_urecs(int nE, const double *__restrict__ u, const int *__restr
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nE) return;
     int i1 = E[2 * I], i2 = E[2 * I + 1];
-    double l = ell[I], du[3], ub[3];
+    const double l = ell[I], li = 1.0 / l;
+    double du[3], ub[3];
     for (int k = 0; k < 3; ++k) {
         double a = u[3 * i1 + k], b = u[3 * i2 + k];
-        du[k] = (b - a) / l;
+        du[k] = div_by(b - a, l, li);
         ub[k] = 0.5 * (a + b);
     }
     if (uf) {
@@ -172,7 +190,10 @@ __global__ void __launch_bounds__(kThreads, (pair_min_blocks<PREC, OP, TPT>())) 
         __syncthreads();
         const int it = s_item;
         __syncthreads();
-        if (it >= pa.n_items) break;
+        if (it >= pa.n_items) {
+            queue_done(it, pa.n_items, pa.counter);
+            break;
+        }
         const WorkItem w = pa.items[it];
         if (pa.skip && pa.skip[w.pad]) continue;  // problem already converged: its output is not used
         Tgt<R> tg[TPT];
@@ -300,17 +321,30 @@ __global__ void __launch_bounds__(kThreads, (pair_min_blocks<PREC, OP, TPT>())) 
 
 // ---------------------------------------------------------------------------------- reductions / gathers
 
-// rows[I] = (l_I / 4) sum_slots part[slot][I]
-__global__ void k_energy_rows(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
-                              const double *__restrict__ ell, double *__restrict__ rows)
+// Sum of the ns slots of value i (slot stride `step`) by the eight warps of a 256-thread block, 32 values a
+// block: warp w adds slots w, w + 8, ... and the partial sums are added in warp order.  Valid in warp 0.  One
+// thread per value waits for 64 slots in turn (12 us at 256 edges).
+__device__ __forceinline__ double slot_sum(const double *part, size_t step, size_t i, int ns, double (*sh)[32])
 {
-    int I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nE) return;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    const int ns = eslots[I];
-#pragma unroll 8
-    for (int k = 0; k < ns; ++k) s += part[(size_t)k * nE + I];
-    rows[I] = 0.25 * ell[I] * s;
+#pragma unroll 4
+    for (int k = w; k < ns; k += 8) s += part[k * step + i];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0)
+        for (int k = 1; k < 8; ++k) s += sh[k][lane];
+    return s;
+}
+
+// rows[I] = (l_I / 4) sum_slots part[slot][I]; 32 rows per block
+__global__ void __launch_bounds__(256) k_energy_rows(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
+                                                     const double *__restrict__ ell, double *__restrict__ rows)
+{
+    __shared__ double sh[8][32];
+    const int I = blockIdx.x * 32 + (threadIdx.x & 31);
+    const double s = slot_sum(part, nE, min(I, nE - 1), I < nE ? eslots[I] : 0, sh);
+    if (threadIdx.x < 32 && I < nE) rows[I] = 0.25 * ell[I] * s;
 }
 
 // Per-problem sums of a per-edge array (deterministic: one block per problem, fixed order).  One block reads
@@ -371,20 +405,15 @@ __global__ void k_vertex_gather(int nV, int nE, const int *__restrict__ inc_ptr,
 // Two-stage gather for many slots: each edge's slots are summed once (k_edge_slots), then every vertex
 // combines its edges' sums (k_vertex_from_edges).  The one-stage gather reads an edge's slots once per
 // endpoint, twice the traffic when an edge has tens of slots (the symmetric passes on long curves).
-// One thread per value, so that a slot's values are read coalesced.
 template <int OP>
-__global__ void k_edge_slots(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
-                             double *__restrict__ esum)
+__global__ void __launch_bounds__(256) k_edge_slots(int nE, const int *__restrict__ eslots, const double *__restrict__ part,
+                                                    double *__restrict__ esum)
 {
     constexpr int W = OP == OP_DIAG ? 1 : 6;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nE * W) return;
-    const int ns = eslots[i / W];
-    const size_t step = (size_t)nE * W;
-    double o = 0.0;
-#pragma unroll 8
-    for (int q = 0; q < ns; ++q) o += part[q * step + i];
-    esum[i] = o;
+    __shared__ double sh[8][32];
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31), n = nE * W;
+    const double s = slot_sum(part, n, min(i, n - 1), i < n ? eslots[i / W] : 0, sh);
+    if (threadIdx.x < 32 && i < n) esum[i] = s;
 }
 
 template <int OP>
@@ -415,12 +444,12 @@ __global__ void k_vertex_from_edges(int nV, const int *__restrict__ inc_ptr, con
     }
 }
 
-// out from the per-edge sums in c.d_esum
+// out from per-edge sums
 template <int OP>
-static cudaError_t vertices_from_edges(Ctx &c, double *out, cudaStream_t s)
+static cudaError_t vertices_from_edges(Ctx &c, const double *esum, double *out, cudaStream_t s)
 {
     if (c.nV == 0) return cudaSuccess;
-    k_vertex_from_edges<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.d_inc_ptr, c.d_inc, c.d_esum, out);
+    k_vertex_from_edges<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.d_inc_ptr, c.d_inc, esum, out);
     c.launches++;
     return cudaGetLastError();
 }
@@ -432,9 +461,9 @@ static cudaError_t gather_slots(Ctx &c, const Ctx::Plan &pl, double *out, cudaSt
     if (c.nV == 0) return cudaSuccess;
     if (pl.max_slots > 2 && c.d_esum) {
         const int values = c.nE * (OP == OP_DIAG ? 1 : 6);
-        k_edge_slots<OP><<<(values + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, c.d_part, c.d_esum);
+        k_edge_slots<OP><<<(values + 31) / 32, 256, 0, s>>>(c.nE, pl.d_eslots, c.d_part, c.d_esum);
         c.launches++;
-        return vertices_from_edges<OP>(c, out, s);
+        return vertices_from_edges<OP>(c, c.d_esum, out, s);
     } else {
         k_vertex_gather<OP><<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.nE, c.d_inc_ptr, c.d_inc, pl.d_eslots, c.d_part,
                                                               out);
@@ -448,7 +477,10 @@ cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s
     return gather_slots<OP_APPLY>(c, pl, Au, s);
 }
 
-cudaError_t vertices_apply(Ctx &c, double *Au, cudaStream_t s) { return vertices_from_edges<OP_APPLY>(c, Au, s); }
+cudaError_t vertices_apply(Ctx &c, const double *esum, double *Au, cudaStream_t s)
+{
+    return vertices_from_edges<OP_APPLY>(c, esum, Au, s);
+}
 
 // ---------------------------------------------------------------------------------- planning
 
@@ -765,7 +797,7 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
     *status = 0;
     if (nE == 0) return cudaMemsetAsync(E, 0, sizeof(double), s);
     TPE_CHECK(cudaMemsetAsync(err, 0, sizeof(int), s));
-    k_records<<<(nE + 255) / 256, 256, 0, s>>>(nE, gamma, edges, recF, recLo, nullptr, ell, T, x, err, nullptr);
+    k_records<<<(nE + kRecThreads - 1) / kRecThreads, kRecThreads, 0, s>>>(nE, gamma, edges, recF, recLo, nullptr, ell, T, x, err, nullptr);
     k_static_stats<<<1, 256, 0, s>>>(nV, nE, gamma, ell, scal);
     TPE_CHECK(cudaGetLastError());
     // the cutoffs are kernel arguments: read the two statistics and the error word (synchronises)
@@ -825,7 +857,7 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
         k_pairs<PMIX, OP_ENERGY, kTptEnergy, true><<<grid, kThreads, 0, s>>>(pa);
     else
         k_pairs<PMIX, OP_ENERGY, kTptEnergy, false><<<grid, kThreads, 0, s>>>(pa);
-    k_energy_rows<<<(nE + 255) / 256, 256, 0, s>>>(nE, eslots, part, ell, rows);
+    k_energy_rows<<<(nE + 31) / 32, 256, 0, s>>>(nE, eslots, part, ell, rows);
     k_segment_sum<<<1, kSegThreads, 0, s>>>(off, rows, E);
     return cudaGetLastError();
 }
@@ -834,14 +866,14 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
 
 cudaError_t build_records(Ctx &c, const double *gamma, int which, cudaStream_t s)
 {
-    int nb = (c.nE + 255) / 256;
+    int nb = (c.nE + kRecThreads - 1) / kRecThreads;
     const bool p64 = c.prm.precision == TP_FP64;
     RecF *rf = p64 ? nullptr : (which ? c.d_recF2 : c.d_recF);
     // the low parts serve the mixed pair passes and, in FP32 contexts too, the double-float apply
     RecLo *rl = p64 ? nullptr : (which ? c.d_recLo2 : c.d_recLo);
     RecD *rd = p64 ? (which ? c.d_recD2 : c.d_recD) : nullptr;
     if (c.nE == 0) return cudaSuccess;
-    k_records<<<nb, 256, 0, s>>>(c.nE, gamma, c.d_edges, rf, rl, rd, c.d_ellw[which], c.d_Tw[which], c.d_xw[which], c.d_err,
+    k_records<<<nb, kRecThreads, 0, s>>>(c.nE, gamma, c.d_edges, rf, rl, rd, c.d_ellw[which], c.d_Tw[which], c.d_xw[which], c.d_err,
                                  p64 ? nullptr : c.d_ell_lo[which]);
     c.launches++;
     return cudaGetLastError();
@@ -850,9 +882,9 @@ cudaError_t build_records(Ctx &c, const double *gamma, int which, cudaStream_t s
 cudaError_t build_urecs(Ctx &c, const double *u, int which, cudaStream_t s)
 {
     if (c.nE == 0) return cudaSuccess;
-    int nb = (c.nE + 255) / 256;
+    int nb = (c.nE + kRecThreads - 1) / kRecThreads;
     const bool p64 = c.prm.precision == TP_FP64;
-    k_urecs<<<nb, 256, 0, s>>>(c.nE, u, c.d_edges, c.d_ellw[which], p64 ? nullptr : c.d_urecF, p64 ? c.d_urecD : nullptr);
+    k_urecs<<<nb, kRecThreads, 0, s>>>(c.nE, u, c.d_edges, c.d_ellw[which], p64 ? nullptr : c.d_urecF, p64 ? c.d_urecD : nullptr);
     c.launches++;
     return cudaGetLastError();
 }
@@ -867,7 +899,7 @@ cudaError_t segment_sum(Ctx &c, const double *rows, double *E, cudaStream_t s)
 cudaError_t build_urecs_into(Ctx &c, const double *u, int which, URecF *uf, URecD *ud, cudaStream_t s)
 {
     if (c.nE == 0) return cudaSuccess;
-    k_urecs<<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, u, c.d_edges, c.d_ellw[which], uf, ud);
+    k_urecs<<<(c.nE + kRecThreads - 1) / kRecThreads, kRecThreads, 0, s>>>(c.nE, u, c.d_edges, c.d_ellw[which], uf, ud);
     c.launches++;
     return cudaGetLastError();
 }
@@ -879,7 +911,6 @@ static cudaError_t run_pairs(Ctx &c, int which, const double *gamma, const doubl
     if (pl.n_items == 0) return cudaSuccess;
     if (!tunable(c) && pl.tpt != 1 && pl.tpt != tpt_default(c, op_class(OP))) return cudaErrorInvalidValue;  // no such kernel
     constexpr int ctr = OP;
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + ctr, 0, sizeof(int), s));
     PairArgs pa;
     pa.items = pl.d_items;
     pa.n_items = pl.n_items;
@@ -911,7 +942,7 @@ cudaError_t pair_energy(Ctx &c, const double *gamma, int which, double *rows_out
     } else {
         TPE_CHECK(run_pairs<OP_ENERGY>(c, which, gamma, nullptr, s));
         if (c.nE > 0) {
-            k_energy_rows<<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, c.plan_energy.d_eslots, c.d_part, c.d_ellw[which], rows);
+            k_energy_rows<<<(c.nE + 31) / 32, 256, 0, s>>>(c.nE, c.plan_energy.d_eslots, c.d_part, c.d_ellw[which], rows);
             c.launches++;
         }
     }
@@ -923,7 +954,7 @@ cudaError_t pair_diff(Ctx &c, const double *gamma, int which, double *dE, cudaSt
 {
     if (c.diff_sym > 0) {
         TPE_CHECK(sym_diff_pass(c, which, s));
-        return vertices_from_edges<OP_DIFF>(c, dE, s);
+        return vertices_from_edges<OP_DIFF>(c, c.d_esum, dE, s);
     }
     TPE_CHECK(run_pairs<OP_DIFF>(c, which, gamma, nullptr, s));
     return gather_slots<OP_DIFF>(c, c.plan_diff, dE, s);
@@ -934,7 +965,7 @@ cudaError_t pair_apply(Ctx &c, const double *gamma_geom, int which, const double
     TPE_CHECK(build_urecs(c, u, which, s));
     if (c.apply_sym > 0) {
         TPE_CHECK(sym_apply_pass(c, which, s));
-        return vertices_from_edges<OP_APPLY>(c, Au, s);
+        return vertices_from_edges<OP_APPLY>(c, c.d_esum, Au, s);
     }
     TPE_CHECK(run_pairs<OP_APPLY>(c, which, gamma_geom, u, s));
     return gather_slots<OP_APPLY>(c, c.plan_apply, Au, s);

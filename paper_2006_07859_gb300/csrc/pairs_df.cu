@@ -285,7 +285,7 @@ cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const do
     TPE_CHECK(build_urecs(c, u, which, s));
     if (c.kp.fast) {
         TPE_CHECK(sym_apply_accurate_pass(c, which, s));
-        return vertices_apply(c, Au, s);
+        return vertices_apply(c, c.d_esum, Au, s);
     }
     if (!pl.d_items) plan_items(c, pl, df_occupancy());
     // the buffer is shared with the other passes and may have been resized since the last call
@@ -297,11 +297,11 @@ cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const do
         c.part_elems = need;
     }
     if (pl.n_items == 0) return cudaMemsetAsync(Au, 0, sizeof(double) * 3 * c.nV, s);
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + 7, 0, sizeof(int), s));
+    TPE_CHECK(cudaMemsetAsync(c.d_counter + 9, 0, sizeof(int), s));
     DfArgs a;
     a.items = pl.d_items;
     a.n_items = pl.n_items;
-    a.counter = c.d_counter + 7;
+    a.counter = c.d_counter + 9;
     a.recF = which ? c.d_recF2 : c.d_recF;
     a.recLo = which ? c.d_recLo2 : c.d_recLo;
     a.ell_lo = c.d_ell_lo[which];

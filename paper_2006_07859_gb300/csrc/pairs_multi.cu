@@ -215,11 +215,25 @@ static cudaError_t multi_init(Ctx &c)
     const size_t ne = (size_t)std::max(1, c.nE);
     if (c.prm.precision == TP_FP64)
         TPE_CHECK(cudaMalloc(&c.d_urecMD, sizeof(URecD) * kMultiG * ne));
-    else
+    else if (!c.d_urecMF)
         TPE_CHECK(cudaMalloc(&c.d_urecMF, sizeof(URecF) * kMultiG * ne));
     TPE_CHECK(cudaMalloc(&c.d_partM, sizeof(double) * (size_t)c.plan_multi.max_slots * ne * 6 * kMultiG));
     c.multi_ready = 1;
     return cudaGetLastError();
+}
+
+static cudaError_t apply_multi_sym(Ctx &c, int which, const double *U, double *AU, int m, cudaStream_t s)
+{
+    const size_t ne = (size_t)c.nE, nv3 = 3 * (size_t)c.nV;
+    if (!c.d_urecMF) TPE_CHECK(cudaMalloc(&c.d_urecMF, sizeof(URecF) * kMultiG * ne));
+    if (!c.d_esum2) TPE_CHECK(cudaMalloc(&c.d_esum2, sizeof(double) * 12 * ne));
+    int f = 0;
+    for (; f + 2 <= m; f += 2) {
+        for (int g = 0; g < 2; ++g) TPE_CHECK(build_urecs_into(c, U + (f + g) * nv3, which, c.d_urecMF + g * ne, nullptr, s));
+        TPE_CHECK(sym_apply2_pass(c, which, s));
+        for (int g = 0; g < 2; ++g) TPE_CHECK(vertices_apply(c, c.d_esum2 + 6 * g * ne, AU + (f + g) * nv3, s));
+    }
+    return f < m ? pair_apply(c, nullptr, which, U + f * nv3, AU + f * nv3, s) : cudaSuccess;
 }
 
 cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const double *U, double *AU, int m,
@@ -230,6 +244,10 @@ cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const 
         if (m > 0 && c.nV > 0) TPE_CHECK(cudaMemsetAsync(AU, 0, sizeof(double) * 3 * c.nV * (size_t)m, s));
         return cudaSuccess;
     }
+    // Contexts that run the symmetric apply take the fields two by two through its two-field form (four would
+    // not fit in registers): 16,384 edges, four fields 2 x 1,480 us against 3,736 us for the four-field gather pass
+    // below, which evaluates every ordered pair.
+    if (c.apply_sym > 0 && c.prm.precision == TP_MIXED) return apply_multi_sym(c, which, U, AU, m, s);
     TPE_CHECK(multi_init(c));
     const Ctx::Plan &pl = c.plan_multi;
     const bool p64 = c.prm.precision == TP_FP64;
@@ -287,6 +305,11 @@ void multi_free(Ctx &c)
     cudaFree(c.d_urecMF);
     cudaFree(c.d_urecMD);
     cudaFree(c.d_partM);
+    cudaFree(c.plan_sym2.d_items);
+    cudaFree(c.plan_sym2.d_eslots);
+    cudaFree(c.d_esum2);
+    c.plan_sym2 = Ctx::Plan{};
+    c.d_esum2 = nullptr;
     c.plan_multi = Ctx::Plan{};
     c.d_urecMF = nullptr;
     c.d_urecMD = nullptr;

@@ -71,17 +71,24 @@ struct SymArgs {
 template <int OP>
 __host__ __device__ constexpr int sym_width()
 {
-    return OP == OP_ENERGY ? 1 : (OP == OP_DIFF ? 10 : 6);
+    return OP == OP_ENERGY ? 1 : (OP == OP_DIFF ? 10 : (OP == OP_APPLY2 ? 12 : 6));
+}
+// vector fields of the pass
+template <int OP>
+__host__ __device__ constexpr int sym_fields()
+{
+    return OP == OP_APPLY ? 1 : (OP == OP_APPLY2 ? 2 : 0);
 }
 
 // Source tile (struct of arrays, 16-byte elements) and the warps' source accumulators.
 template <int PREC, int OP>
 struct SymSmem {
-    static constexpr bool MIX = PREC != P32, U = OP == OP_APPLY;
+    static constexpr bool MIX = PREC != P32;
+    static constexpr int F = sym_fields<OP>() ? sym_fields<OP>() : 1, U = sym_fields<OP>() ? kTile : 1;
     float4 t0[kTile], t1[kTile], t2[kTile];  // (q1, l), (e, T.x), (T.y, T.z, q1.x lo, q1.y lo)
     float4 t3[MIX ? kTile : 1];              // (q1.z lo, T lo)
     float4 t4[PREC == PDF ? kTile : 1];      // (e lo, l lo)
-    float4 u0[U ? kTile : 1], u1[U ? kTile : 1], u2[(U && MIX) ? kTile : 1];
+    float4 u0[F][U], u1[F][U], u2[F][MIX ? U : 1];  // u records
     int2 id[kTile];
     float2 sac[kSymWarps][sym_width<OP>()][kTile];  // (sum, Kahan compensation)
     // differential: the warps' queues of near pairs (row << 8 | slot) and the target sums of those pairs
@@ -153,6 +160,10 @@ template <int PREC>
 struct SymAcc<PREC, OP_APPLY> {
     L2 s[6], c[6];
 };
+template <int PREC>
+struct SymAcc<PREC, OP_APPLY2> {
+    L2 s[12], c[12];
+};
 
 // source accumulator += wx vx + wy vy, both compensated
 __device__ __forceinline__ void src_add(float2 &ac, L2 w, L2 v)
@@ -162,7 +173,7 @@ __device__ __forceinline__ void src_add(float2 &ac, L2 w, L2 v)
 }
 
 template <int PREC, bool CHECK, int MODE>
-__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &, const SymSmem<PREC, OP_ENERGY> &, const SymSrc &s,
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const SymSmem<PREC, OP_ENERGY> &, const SymSrc &s,
                                          int, int Jg, bool k0, bool k1, SymAcc<PREC, OP_ENERGY> &a, float2 *sac,
                                          const SymArgs &pa, bool &, bool &)
 {
@@ -286,7 +297,7 @@ __device__ __forceinline__ void sym_pair_df(const SymTgt &t, const SymTgtU &tu, 
     const dfv<L2> dT = {l_dfdiff(TI.x.hi, TI.x.lo, TJ.x.hi, TJ.x.lo), l_dfdiff(TI.y.hi, TI.y.lo, TJ.y.hi, TJ.y.lo),
                         l_dfdiff(TI.z.hi, TI.z.lo, TJ.z.hi, TJ.z.lo)};
     const dfl<L2> n2 = l_dfnorm2(dT), omt = {l_mul(l_bc<L2>(0.5f), n2.hi), l_mul(l_bc<L2>(0.5f), n2.lo)};
-    const float4 x = tl.u0[j], y = tl.u1[j], z = tl.u2[j];
+    const float4 x = tl.u0[0][j], y = tl.u1[0][j], z = tl.u2[0][j];
     const L2 sd[3] = {l_bc<L2>(x.x), l_bc<L2>(x.y), l_bc<L2>(x.z)}, sdl[3] = {l_bc<L2>(y.z), l_bc<L2>(y.w), l_bc<L2>(z.x)};
     const L2 sb[3] = {l_bc<L2>(x.w), l_bc<L2>(y.x), l_bc<L2>(y.y)}, sbl[3] = {l_bc<L2>(z.y), l_bc<L2>(z.z), l_bc<L2>(z.w)};
     const L2 td[3] = {tu.dh.x, tu.dh.y, tu.dh.z}, tdl[3] = {tu.dl.x, tu.dl.y, tu.dl.z};
@@ -306,12 +317,10 @@ __device__ __forceinline__ void sym_pair_df(const SymTgt &t, const SymTgtU &tu, 
     }
 }
 
-template <int PREC, bool CHECK, int MODE>
-__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &tu, const SymSmem<PREC, OP_APPLY> &tl,
-                                         const SymSrc &s, int j, int, bool k0, bool k1, SymAcc<PREC, OP_APPLY> &a,
-                                         float2 *sac, const SymArgs &, bool &, bool &)
+template <int PREC, int OP, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair_apply(const SymTgt &t, const SymTgtU *tus, const SymSmem<PREC, OP> &tl, const SymSrc &s,
+                                               int j, bool k0, bool k1, SymAcc<PREC, OP> &a, float2 *sac)
 {
-    if constexpr (PREC == PDF) return sym_pair_df<CHECK>(t, tu, tl, s, j, k0, k1, a, sac);
     constexpr bool MIX = PREC == PMIX;
     LV<L2> d[4];
     l_chords<(MODE >= 1 && MIX)>(t.p, t.pl, t.e, l_bc3<L2>(s.q[0], s.q[1], s.q[2]), l_bc3<L2>(s.m[0], s.m[1], s.m[2]),
@@ -330,34 +339,57 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &tu, con
     LV<L2> dT = l_sub3(t.T, TJ);
     if constexpr (MIX) dT = l_add3(dT, l_sub3(t.Tl, l_bc3<L2>(s.Tm[0], s.Tm[1], s.Tm[2])));
     const L2 omt = l_mul(l_bc<L2>(0.5f), l_dot(dT, dT));  // |T_I - T_J|^2 / 2
-    const float4 x = tl.u0[j], y = tl.u1[j];
-    const LV<L2> sdh = l_bc3<L2>(x.x, x.y, x.z);
-    LV<L2> dd = l_sub3(tu.dh, sdh), db = l_sub3(tu.uh, l_bc3<L2>(x.w, y.x, y.y));
-    if constexpr (MIX) {  // differences of the double-float u records
-        const float4 z = tl.u2[j];
-        dd = l_add3(dd, l_sub3(tu.dl, l_bc3<L2>(y.z, y.w, z.x)));
-        db = l_add3(db, l_sub3(tu.ul, l_bc3<L2>(z.y, z.z, z.w)));
-    }
     const L2 Wt = l_mul(l_bc<L2>(s.ell), sw), W0t = l_mul(l_bc<L2>(s.ell), sw0);
-    l_kahan_fma(a.s[0], a.c[0], Wt, l_fma(omt, sdh.x, dd.x));
-    l_kahan_fma(a.s[1], a.c[1], Wt, l_fma(omt, sdh.y, dd.y));
-    l_kahan_fma(a.s[2], a.c[2], Wt, l_fma(omt, sdh.z, dd.z));
-    l_kahan_fma(a.s[3], a.c[3], W0t, db.x);
-    l_kahan_fma(a.s[4], a.c[4], W0t, db.y);
-    l_kahan_fma(a.s[5], a.c[5], W0t, db.z);
     const L2 Ws = l_mul(t.ell, sw), W0s = l_neg(l_mul(t.ell, sw0));
-    const L2 v[6] = {l_fma(omt, tu.dh.x, l_neg(dd.x)), l_fma(omt, tu.dh.y, l_neg(dd.y)), l_fma(omt, tu.dh.z, l_neg(dd.z)),
-                     db.x, db.y, db.z};
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        float2 ac = sac[q * kTile];
-        src_add(ac, q < 3 ? Ws : W0s, v[q]);
-        sac[q * kTile] = ac;
+    for (int f = 0; f < sym_fields<OP>(); ++f) {
+        const SymTgtU &tu = tus[f];
+        const float4 x = tl.u0[f][j], y = tl.u1[f][j];
+        const LV<L2> sdh = l_bc3<L2>(x.x, x.y, x.z);
+        LV<L2> dd = l_sub3(tu.dh, sdh), db = l_sub3(tu.uh, l_bc3<L2>(x.w, y.x, y.y));
+        if constexpr (MIX) {  // differences of the double-float u records
+            const float4 z = tl.u2[f][j];
+            dd = l_add3(dd, l_sub3(tu.dl, l_bc3<L2>(y.z, y.w, z.x)));
+            db = l_add3(db, l_sub3(tu.ul, l_bc3<L2>(z.y, z.z, z.w)));
+        }
+        L2 *as = a.s + 6 * f, *ac = a.c + 6 * f;
+        l_kahan_fma(as[0], ac[0], Wt, l_fma(omt, sdh.x, dd.x));
+        l_kahan_fma(as[1], ac[1], Wt, l_fma(omt, sdh.y, dd.y));
+        l_kahan_fma(as[2], ac[2], Wt, l_fma(omt, sdh.z, dd.z));
+        l_kahan_fma(as[3], ac[3], W0t, db.x);
+        l_kahan_fma(as[4], ac[4], W0t, db.y);
+        l_kahan_fma(as[5], ac[5], W0t, db.z);
+        const L2 v[6] = {l_fma(omt, tu.dh.x, l_neg(dd.x)), l_fma(omt, tu.dh.y, l_neg(dd.y)),
+                         l_fma(omt, tu.dh.z, l_neg(dd.z)), db.x, db.y, db.z};
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            float2 *p = sac + (6 * f + q) * kTile, x2 = *p;
+            src_add(x2, q < 3 ? Ws : W0s, v[q]);
+            *p = x2;
+        }
     }
 }
 
 template <int PREC, bool CHECK, int MODE>
-__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU &, const SymSmem<PREC, OP_DIFF> &, const SymSrc &s,
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *tu, const SymSmem<PREC, OP_APPLY> &tl, const SymSrc &s,
+                                         int j, int, bool k0, bool k1, SymAcc<PREC, OP_APPLY> &a, float2 *sac, const SymArgs &,
+                                         bool &, bool &)
+{
+    if constexpr (PREC == PDF)
+        sym_pair_df<CHECK>(t, tu[0], tl, s, j, k0, k1, a, sac);
+    else
+        sym_pair_apply<PREC, OP_APPLY, CHECK, MODE>(t, tu, tl, s, j, k0, k1, a, sac);
+}
+template <int PREC, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *tu, const SymSmem<PREC, OP_APPLY2> &tl, const SymSrc &s,
+                                         int j, int, bool k0, bool k1, SymAcc<PREC, OP_APPLY2> &a, float2 *sac, const SymArgs &,
+                                         bool &, bool &)
+{
+    sym_pair_apply<PREC, OP_APPLY2, CHECK, MODE>(t, tu, tl, s, j, k0, k1, a, sac);
+}
+
+template <int PREC, bool CHECK, int MODE>
+__device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const SymSmem<PREC, OP_DIFF> &, const SymSrc &s,
                                          int, int, bool k0, bool k1, SymAcc<PREC, OP_DIFF> &a, float2 *sac,
                                          const SymArgs &pa, bool &n0, bool &n1)
 {
@@ -481,7 +513,7 @@ static __device__ __noinline__ void sym_near_flush(SymSmem<PMIX, OP_DIFF> &sm, i
 // chords (far tiles).  OWN: the sources are the warp's own 64 rows; each unordered pair once, by the row that
 // sees the other at most half the circle of 64 ahead.
 template <int PREC, int OP, bool CHECK, int MODE, bool OWN>
-__device__ __forceinline__ void sym_section(const SymTgt &t, const SymTgtU &tu, SymSmem<PREC, OP> &sm, int wid, int s0,
+__device__ __forceinline__ void sym_section(const SymTgt &t, const SymTgtU *tu, SymSmem<PREC, OP> &sm, int wid, int s0,
                                             int j0, int cnt, SymAcc<PREC, OP> &a, int &queued, const WorkItem &w,
                                             const SymArgs &pa)
 {
@@ -530,7 +562,8 @@ template <int PREC, int OP, int MB>
 __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
 {
     constexpr int W = sym_width<OP>();
-    constexpr bool MIX = PREC != P32, DF = PREC == PDF, NEAR = PREC == PMIX && OP != OP_APPLY;
+    constexpr bool MIX = PREC != P32, DF = PREC == PDF, NEAR = PREC == PMIX && (OP == OP_ENERGY || OP == OP_DIFF);
+    constexpr int F = sym_fields<OP>();
     extern __shared__ __align__(16) unsigned char dyn[];
     SymSmem<PREC, OP> &sm = *reinterpret_cast<SymSmem<PREC, OP> *>(dyn);
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -539,18 +572,20 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
         __syncthreads();
         const int it = sm.item;
         __syncthreads();
-        if (it >= pa.n_items) break;
+        if (it >= pa.n_items) {
+            queue_done(it, pa.n_items, pa.counter);
+            break;
+        }
         const WorkItem w = pa.items[it];
         if (pa.skip && pa.skip[w.pad]) continue;  // problem already converged
         const int X = w.slot >> 16, tslot = w.slot & 0xffff;
         const bool diag = w.src0 < w.tgt0 + w.ntgt;  // a tile of its own super-block
         SymTgt t;
-        SymTgtU tu;
+        SymTgtU tu[F ? F : 1];
         float tbox[6] = {1e30f, 1e30f, 1e30f, -1e30f, -1e30f, -1e30f};
         {
             RecF r[2];
             RecLo q[2];
-            URecF u[2];
             bool valid[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -560,7 +595,6 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
                 t.row[k] = I;
                 r[k] = pa.recF[I];
                 if constexpr (MIX) q[k] = pa.recLo[I];
-                if constexpr (OP == OP_APPLY) u[k] = pa.urecF[I];
                 t.i1[k] = __float_as_int(r[k].c.z);
                 t.i2[k] = __float_as_int(r[k].c.w);
                 if constexpr (MIX)
@@ -588,12 +622,14 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
             } else {
                 t.e = l_sub3(LV<L2>{TPE_L2(b.x), TPE_L2(b.y), TPE_L2(b.z)}, t.p);
             }
-            if constexpr (OP == OP_APPLY) {
-                tu.dh = {TPE_U2(a.x), TPE_U2(a.y), TPE_U2(a.z)};
-                tu.uh = {TPE_U2(a.w), TPE_U2(b.x), TPE_U2(b.y)};
+#pragma unroll
+            for (int f = 0; f < F; ++f) {
+                const URecF u[2] = {pa.urecF[(size_t)f * pa.nE + t.row[0]], pa.urecF[(size_t)f * pa.nE + t.row[1]]};
+                tu[f].dh = {TPE_U2(a.x), TPE_U2(a.y), TPE_U2(a.z)};
+                tu[f].uh = {TPE_U2(a.w), TPE_U2(b.x), TPE_U2(b.y)};
                 if constexpr (MIX) {
-                    tu.dl = {TPE_U2(b.z), TPE_U2(b.w), TPE_U2(c.x)};
-                    tu.ul = {TPE_U2(c.y), TPE_U2(c.z), TPE_U2(c.w)};
+                    tu[f].dl = {TPE_U2(b.z), TPE_U2(b.w), TPE_U2(c.x)};
+                    tu[f].ul = {TPE_U2(c.y), TPE_U2(c.z), TPE_U2(c.w)};
                 }
             }
 #undef TPE_L2
@@ -642,11 +678,12 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
                     sm.t1[j] = make_float4(r.b.x - r.a.x, r.b.y - r.a.y, r.b.z - r.a.z, r.b.w);
                     sm.t2[j] = make_float4(r.c.x, r.c.y, 0.f, 0.f);
                 }
-                if constexpr (OP == OP_APPLY) {
-                    const URecF u = pa.urecF[J];
-                    sm.u0[j] = u.a;
-                    sm.u1[j] = u.b;
-                    if constexpr (MIX) sm.u2[j] = u.c;
+#pragma unroll
+                for (int f = 0; f < F; ++f) {
+                    const URecF u = pa.urecF[(size_t)f * pa.nE + J];
+                    sm.u0[f][j] = u.a;
+                    sm.u1[f][j] = u.b;
+                    if constexpr (MIX) sm.u2[f][j] = u.c;
                 }
             }
             for (int q = 0; q < W; ++q)
@@ -801,16 +838,18 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
         if (threadIdx.x >= R || I >= nE) return;
         const double *v = sh + W * threadIdx.x;
         const double l = ell[I];
-        double o[6];
-        if constexpr (OP == OP_DIFF) {
-            diff_row_out(T + 3 * (size_t)I, l, v, o);
-        } else {
-            for (int c = 0; c < 3; ++c) {
-                o[c] = 0.5 * v[c];
-                o[3 + c] = 0.125 * l * v[3 + c];
+        for (int f = 0; f < (OP == OP_APPLY2 ? 2 : 1); ++f, v += 6, out += 6 * (size_t)nE) {
+            double o[6];
+            if constexpr (OP == OP_DIFF) {
+                diff_row_out(T + 3 * (size_t)I, l, v, o);
+            } else {
+                for (int c = 0; c < 3; ++c) {
+                    o[c] = 0.5 * v[c];
+                    o[3 + c] = 0.125 * l * v[3 + c];
+                }
             }
+            for (int c = 0; c < 6; ++c) out[6 * (size_t)I + c] = o[c];
         }
-        for (int c = 0; c < 6; ++c) out[6 * (size_t)I + c] = o[c];
     }
 }
 
@@ -921,6 +960,8 @@ static void with_sym_kernel(int prec, int op, int variant, F f)
             f(k_sym<PMIX, OP_DIFF, 3>, sizeof(SymSmem<PMIX, OP_DIFF>));
         else
             f(k_sym<PMIX, OP_DIFF, 2>, sizeof(SymSmem<PMIX, OP_DIFF>));
+    } else if (op == OP_APPLY2) {
+        f(k_sym<PMIX, OP_APPLY2, 2>, sizeof(SymSmem<PMIX, OP_APPLY2>));
     } else {
         if (variant == kSymAccurate)
             f(k_sym<PDF, OP_APPLY, 2>, sizeof(SymSmem<PDF, OP_APPLY>));
@@ -943,7 +984,7 @@ static int sym_occupancy(const Ctx &c, int op, int variant)
     return occ;
 }
 
-static int sym_op_width(int op) { return op == OP_ENERGY ? 1 : (op == OP_DIFF ? 10 : 6); }
+static int sym_op_width(int op) { return op == OP_ENERGY ? 1 : (op == OP_DIFF ? 10 : (op == OP_APPLY2 ? 12 : 6)); }
 
 // Doubles of the partial buffer the symmetric pass of `op` needs.
 size_t sym_part_elems(const Ctx &c, int op, int variant)
@@ -1008,14 +1049,13 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
                             cudaStream_t s)
 {
     if (pl.n_items == 0) return cudaSuccess;  // no edges: nothing reads the sums
-    TPE_CHECK(cudaMemsetAsync(c.d_counter + counter, 0, sizeof(int), s));
     SymArgs pa;
     pa.items = pl.d_items;
     pa.n_items = pl.n_items;
     pa.counter = c.d_counter + counter;
     pa.recF = which ? c.d_recF2 : c.d_recF;
     pa.recLo = which ? c.d_recLo2 : c.d_recLo;
-    pa.urecF = c.d_urecF;
+    pa.urecF = op == OP_APPLY2 ? c.d_urecMF : c.d_urecF;
     pa.ell_lo = c.d_ell_lo[which];
     pa.part = reinterpret_cast<float2 *>(c.d_part);
     pa.nE = c.nE;
@@ -1030,6 +1070,8 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
         k_sym_sum<OP_ENERGY><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     else if (op == OP_DIFF)
         k_sym_sum<OP_DIFF><<<(c.nE + 31) / 32, 320, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+    else if (op == OP_APPLY2)
+        k_sym_sum<OP_APPLY2><<<(c.nE + 31) / 32, 384, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     else if (pl.tpt == kSymAccurate)
         k_sym_sum<OP_APPLY, true><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
     else
@@ -1053,23 +1095,35 @@ cudaError_t sym_apply_pass(Ctx &c, int which, cudaStream_t s)
     return sym_pass(c, OP_APPLY, c.plan_sym, 4, c.d_skip ? 4 : 2, which, c.d_skip, c.d_esum, s);
 }
 
-// The accurate apply (edges' endpoint values into c.d_esum); its plan is built at the first call.
-cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s)
+// Passes whose plan is built at the first call.
+static cudaError_t lazy_pass(Ctx &c, int op, Ctx::Plan &pl, int variant, int counter, int prof_op, int which, const int *skip,
+                             double *out, cudaStream_t s)
 {
-    Ctx::Plan &pl = c.plan_df;
     if (!pl.d_items) {
-        sym_plan(c, pl, sym_occupancy(c, OP_APPLY, kSymAccurate));
-        pl.tpt = kSymAccurate;
+        sym_plan(c, pl, sym_occupancy(c, op, variant));
+        pl.tpt = variant;
     }
     // the buffer is shared with the other passes and may have been resized since the last call
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(OP_APPLY);
+    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(op);
     if (need > c.part_elems) {
         graphs_reset(c);  // captured blocks hold the old partial buffer
         TPE_CHECK(cudaFree(c.d_part));
         TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
         c.part_elems = need;
     }
-    return sym_pass(c, OP_APPLY, pl, 7, 5, which, c.d_skip, c.d_esum, s);
+    return sym_pass(c, op, pl, counter, prof_op, which, skip, out, s);
+}
+
+// The accurate apply: edges' endpoint values into c.d_esum.
+cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s)
+{
+    return lazy_pass(c, OP_APPLY, c.plan_df, kSymAccurate, 7, 5, which, c.d_skip, c.d_esum, s);
+}
+
+// Two vector fields, the weights once per pair.
+cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s)
+{
+    return lazy_pass(c, OP_APPLY2, c.plan_sym2, 1, 10, 7, which, nullptr, c.d_esum2, s);
 }
 
 }  // namespace tpe

@@ -25,7 +25,7 @@ struct BhState;
 enum Prec { P64 = 0, P32 = 1, PMIX = 2, PDF = 3 };  // PDF: double-float throughout (the accurate apply)
 
 // Which quantity a pair pass accumulates.
-enum PairOp { OP_ENERGY = 0, OP_DIFF = 1, OP_APPLY = 2, OP_DIAG = 3 };
+enum PairOp { OP_ENERGY = 0, OP_DIFF = 1, OP_APPLY = 2, OP_DIAG = 3, OP_APPLY2 = 4 };  // OP_APPLY2: two vector fields
 
 constexpr int kThreads = 128;  // threads per CTA of the pair passes
 constexpr int kTile = 128;     // source edges staged in shared memory per tile
@@ -139,6 +139,8 @@ struct Ctx {
     URecD *d_urecMD = nullptr;  // the same in FP64 contexts
     double *d_partM = nullptr;  // multi-field apply: partial sums [slot][nE][6 kMultiG]
     int multi_ready = 0;
+    Plan plan_sym2;             // symmetric multi-field apply (two fields per pass), built at its first use
+    double *d_esum2 = nullptr;  // its per-edge sums [2][nE][6]
     int *d_counter = nullptr;  // persistent-queue counters [16]
     // edge records
     RecF *d_recF = nullptr, *d_recF2 = nullptr;
@@ -241,7 +243,7 @@ cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const 
 void multi_free(Ctx &c);
 void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
 cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s);
-cudaError_t vertices_apply(Ctx &c, double *Au, cudaStream_t s);  // from the per-edge sums in c.d_esum
+cudaError_t vertices_apply(Ctx &c, const double *esum, double *Au, cudaStream_t s);  // from per-edge sums
 // symmetric passes (pairs_sym.cu): a variant > 0 or the gather pass (0); the passes write the energy rows
 // [nE] or the edges' endpoint values into c.d_esum
 cudaError_t sym_select(Ctx &c, int variant);
@@ -251,6 +253,7 @@ cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s);
 cudaError_t sym_select_diff(Ctx &c, int variant);
 cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
 cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s);  // specialised powers; grows c.d_part
+cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: c.d_urecMF into c.d_esum2; grows c.d_part
 cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 void make_plans(Ctx &c);

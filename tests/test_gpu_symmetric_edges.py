@@ -101,3 +101,31 @@ def test_new_context_of_many_ragged_curves(torch, orc, prec):
     # plain FP32 positions: the suite's FP32 bar for the energy, and 1e-4 of the largest entry for the apply
     # (positions rounded to 6e-8 of the curve's size against edges of 1e-2 of it)
     _check(torch, orc, ctx, c, prec, MIXED if prec == 2 else {"energy": 1e-4, "diff": 1.0, "apply": 1e-4})
+
+
+@pytest.mark.parametrize("m", [1, 2, 3, 5])
+def test_multi_field_apply_on_the_symmetric_pass(torch, orc, m):
+    """Fields two by two and an odd last one, per field against the oracle and against the single apply (1e-6 of
+    the largest entry each, the mixed apply's bar)."""
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(449, 4, 12))
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    tpe.tp_set_apply_variant(ctx, 1)
+    U = np.random.default_rng(m).normal(size=(m, c.n_vertices, 3))
+    AU = host(tpe.sobolev_apply_multi(ctx, dev(c.gamma), dev(U)))
+    for f in range(m):
+        assert rel(AU[f], orc.gram_apply(c.gamma, c.edges, 0.75, U[f])) <= 1e-6
+        assert rel(AU[f], host(tpe.sobolev_apply(ctx, dev(c.gamma), dev(U[f])))) <= 1e-6
+
+
+def test_accurate_apply_after_a_change_of_exponents(torch, orc):
+    """The accurate apply's work list follows the exponents of the context (tolerance of its own tests)."""
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(300, 4, 21))
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    u = np.random.default_rng(2).normal(size=(c.n_vertices, 3))
+    for alpha, beta in ((2.0, 4.5), (3.0, 6.0), (2.0, 4.5)):
+        ctx.set_params(alpha=alpha, beta=beta)
+        ref = orc.gram_apply(c.gamma, c.edges, orc.sigma_of(alpha, beta), u)
+        assert rel(host(tpe.sobolev_apply_accurate(ctx, dev(c.gamma), dev(u))), ref) <= 1e-11
+        assert rel(host(tpe.sobolev_apply(ctx, dev(c.gamma), dev(u))), ref) <= 1e-5
