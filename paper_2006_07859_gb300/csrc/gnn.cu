@@ -48,7 +48,10 @@ constexpr int oW1 = 0, ob1 = oW1 + kH * kF, oW2s = ob1 + kH, oW2n = oW2s + kH * 
               kNParams = ob4 + kO;
 constexpr int kWgBlocks = 256;  // blocks of the weight-gradient kernels (fixed: deterministic sums)
 constexpr int kWgSub = 32;      // edges staged per sub-tile
-constexpr int kWgMax = kH * kH + kH;
+constexpr int kWgSmallBlocks = 1024, kWgSmall = 1024;  // the same of the two small layers (195 and 576 entries)
+constexpr int kWgMax = 2 * kH * kH + kH;  // entries of a block's partial: self and neighbour weights, biases
+
+static_assert((size_t)kWgSmallBlocks * kWgSmall <= (size_t)kWgBlocks * kWgMax && kH * kF + kH <= kWgSmall, "partials");
 
 struct GnnState {
     float *master = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;  // [P]
@@ -159,9 +162,20 @@ __global__ void __launch_bounds__(128) k_gnn_l1(int nE, const float *__restrict_
 // its data gradient [dh | dm] = dz [Ws | Wn] (K = 64, N = 128).  The weights are BF16 already; each FP32
 // activation is split into three BF16 terms (x = x1 + x2 + x3 to ~2^-24), so the products carry the
 // FP32 activations' digits and the layers compute what the CUDA-core form computes, up to the order of
-// the FP32 sums.  A block of 64 threads (two warps of 16 rows) takes 32 edges; the operand tiles sit in
-// shared memory with padded rows.
-constexpr int kTcRows = 32;
+// the FP32 sums.  A block of 128 threads (four warps of 16 rows) takes 64 edges; the operand tiles sit in
+// shared memory with padded rows.  What bounds the layers is staging, not the products (1.6 GFLOP at 32,768
+// edges): with weights staged one BF16 value per instruction for every 32 edges they took 68 and 51 us, with
+// 16-byte loads, 64 edges a block and 32-bit fragment loads 17 and 15 (cold caches).
+constexpr int kTcRows = 64, kTcThreads = 2 * kTcRows;
+
+__device__ __forceinline__ float4 relu4(float4 v)
+{
+    return make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+}
+__device__ __forceinline__ float4 avg4(float4 a, float4 b)
+{
+    return make_float4(0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z), 0.5f * (a.w + b.w));
+}
 
 __device__ __forceinline__ uint32_t bf_pack(__nv_bfloat16 lo, __nv_bfloat16 hi)
 {
@@ -197,10 +211,10 @@ __device__ __forceinline__ void tc_rows16(const float *X, int r0, const __nv_bfl
 #pragma unroll
     for (int kk = 0; kk < K; kk += 16) {
         const int c0 = kk + 2 * q;
-        const float x[8] = {X[(r0 + g) * LDX + c0],         X[(r0 + g) * LDX + c0 + 1],
-                            X[(r0 + g + 8) * LDX + c0],     X[(r0 + g + 8) * LDX + c0 + 1],
-                            X[(r0 + g) * LDX + c0 + 8],     X[(r0 + g) * LDX + c0 + 9],
-                            X[(r0 + g + 8) * LDX + c0 + 8], X[(r0 + g + 8) * LDX + c0 + 9]};
+        const float *xr = X + (r0 + g) * LDX + c0, *xs = xr + 8 * LDX;
+        const float2 x01 = *reinterpret_cast<const float2 *>(xr), x23 = *reinterpret_cast<const float2 *>(xs),
+                     x45 = *reinterpret_cast<const float2 *>(xr + 8), x67 = *reinterpret_cast<const float2 *>(xs + 8);
+        const float x[8] = {x01.x, x01.y, x23.x, x23.y, x45.x, x45.y, x67.x, x67.y};
         __nv_bfloat16 t[8][3];
 #pragma unroll
         for (int e = 0; e < 8; ++e) bf_split3(x[e], t[e]);
@@ -212,7 +226,7 @@ __device__ __forceinline__ void tc_rows16(const float *X, int r0, const __nv_bfl
 #pragma unroll
         for (int nt = 0; nt < N / 8; ++nt) {
             const __nv_bfloat16 *bc = Bt + (nt * 8 + g) * LDB + c0;
-            const uint32_t b0 = bf_pack(bc[0], bc[1]), b1 = bf_pack(bc[8], bc[9]);
+            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(bc), b1 = *reinterpret_cast<const uint32_t *>(bc + 8);
             // smallest terms first
             mma_bf16_16816(acc[nt], a[2], b0, b1);
             mma_bf16_16816(acc[nt], a[1], b0, b1);
@@ -221,32 +235,38 @@ __device__ __forceinline__ void tc_rows16(const float *X, int r0, const __nv_bfl
     }
 }
 
+constexpr int kLmpLdx = 2 * kH + 4, kLmpLdb = 2 * kH + 8, kBmatLdx = kH + 4, kBmatLdb = kH + 8;
+constexpr size_t kLmpSmem = sizeof(float) * kTcRows * kLmpLdx + sizeof(__nv_bfloat16) * kH * kLmpLdb;
+
 // zout = Ws relu(zin) + Wn avg(relu(zin[I-1]), relu(zin[I+1])) + b on the tensor cores
-__global__ void __launch_bounds__(64) k_gnn_lmp_tc(int nE, const int *__restrict__ eprev, const int *__restrict__ enext,
-                                                   const float *__restrict__ zin, const __nv_bfloat16 *__restrict__ w,
-                                                   int oWs, int oWn, int ob, float *__restrict__ zout)
+__global__ void __launch_bounds__(kTcThreads) k_gnn_lmp_tc(int nE, const int *__restrict__ eprev,
+                                                           const int *__restrict__ enext, const float *__restrict__ zin,
+                                                           const __nv_bfloat16 *__restrict__ w, int oWs, int oWn, int ob,
+                                                           float *__restrict__ zout)
 {
-    constexpr int K = 2 * kH, LDX = K + 4, LDB = K + 8;
-    __shared__ __align__(16) float X[kTcRows * LDX];
-    __shared__ __align__(16) __nv_bfloat16 Bt[kH * LDB];
+    constexpr int K = 2 * kH, LDX = kLmpLdx, LDB = kLmpLdb;
+    extern __shared__ __align__(16) unsigned char gnn_smem[];
+    float *X = reinterpret_cast<float *>(gnn_smem);
+    __nv_bfloat16 *Bt = reinterpret_cast<__nv_bfloat16 *>(X + kTcRows * LDX);
     __shared__ float bias[kH];
-    for (int t = threadIdx.x; t < kH * K; t += blockDim.x) {
-        const int n = t / K, k = t % K;
-        Bt[n * LDB + k] = k < kH ? w[oWs + n * kH + k] : w[oWn + n * kH + (k - kH)];
+    // weight rows of 64 in 16-byte pieces (the parameter blocks start at multiples of 16 bytes)
+    for (int t = threadIdx.x; t < kH * K / 8; t += kTcThreads) {
+        const int n = t / (K / 8), k = 8 * (t % (K / 8));
+        const __nv_bfloat16 *src = w + (k < kH ? oWs + n * kH + k : oWn + n * kH + (k - kH));
+        *reinterpret_cast<uint4 *>(Bt + n * LDB + k) = *reinterpret_cast<const uint4 *>(src);
     }
-    for (int t = threadIdx.x; t < kH; t += blockDim.x) bias[t] = bf(w, ob + t);
+    for (int t = threadIdx.x; t < kH; t += kTcThreads) bias[t] = bf(w, ob + t);
     const int I0 = blockIdx.x * kTcRows;
-    for (int t = threadIdx.x; t < kTcRows * K; t += blockDim.x) {
-        const int r = t / K, k = t % K, I = I0 + r;
-        float v = 0.f;
+    const float4 *z4 = reinterpret_cast<const float4 *>(zin);
+    for (int t = threadIdx.x; t < kTcRows * kH / 4; t += kTcThreads) {
+        const int r = t / (kH / 4), k = t % (kH / 4), I = I0 + r;
+        float4 h = make_float4(0.f, 0.f, 0.f, 0.f), m = h;
         if (I < nE) {
-            if (k < kH)
-                v = fmaxf(zin[(size_t)I * kH + k], 0.f);
-            else
-                v = 0.5f * (fmaxf(zin[(size_t)eprev[I] * kH + k - kH], 0.f) +
-                            fmaxf(zin[(size_t)enext[I] * kH + k - kH], 0.f));
+            h = relu4(z4[(size_t)I * (kH / 4) + k]);
+            m = avg4(relu4(z4[(size_t)eprev[I] * (kH / 4) + k]), relu4(z4[(size_t)enext[I] * (kH / 4) + k]));
         }
-        X[r * LDX + k] = v;
+        *reinterpret_cast<float4 *>(X + r * LDX + 4 * k) = h;
+        *reinterpret_cast<float4 *>(X + r * LDX + kH + 4 * k) = m;
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
@@ -267,21 +287,27 @@ __global__ void __launch_bounds__(64) k_gnn_lmp_tc(int nE, const int *__restrict
 }
 
 // dh = dz Ws, dm = dz Wn on the tensor cores (dh[k] = sum_o dz[o] Ws[o][k])
-__global__ void __launch_bounds__(64) k_gnn_bmat_tc(int nE, const float *__restrict__ dz,
-                                                    const __nv_bfloat16 *__restrict__ w, int oWs, int oWn,
-                                                    float *__restrict__ dh, float *__restrict__ dm)
+__global__ void __launch_bounds__(kTcThreads) k_gnn_bmat_tc(int nE, const float *__restrict__ dz,
+                                                            const __nv_bfloat16 *__restrict__ w, int oWs, int oWn,
+                                                            float *__restrict__ dh, float *__restrict__ dm)
 {
-    constexpr int K = kH, N = 2 * kH, LDX = K + 4, LDB = K + 8;
+    constexpr int K = kH, N = 2 * kH, LDX = kBmatLdx, LDB = kBmatLdb;
     __shared__ __align__(16) float X[kTcRows * LDX];
     __shared__ __align__(16) __nv_bfloat16 Bt[N * LDB];
-    for (int t = threadIdx.x; t < N * K; t += blockDim.x) {
-        const int n = t / K, o = t % K;  // Bt[n][o] = Ws[o][n] (n < 64), Wn[o][n - 64]
-        Bt[n * LDB + o] = n < kH ? w[oWs + o * kH + n] : w[oWn + o * kH + (n - kH)];
+    for (int t = threadIdx.x; t < N * K / 8; t += kTcThreads) {  // Bt[n][o] = Ws[o][n] (n < 64), Wn[o][n - 64]
+        const int o = t % K, n = 8 * (t / K);
+        const uint4 v = *reinterpret_cast<const uint4 *>(w + (n < kH ? oWs + o * kH + n : oWn + o * kH + (n - kH)));
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            Bt[(n + e) * LDB + o] = __ushort_as_bfloat16((unsigned short)(u[e >> 1] >> (16 * (e & 1))));
     }
     const int I0 = blockIdx.x * kTcRows;
-    for (int t = threadIdx.x; t < kTcRows * K; t += blockDim.x) {
-        const int r = t / K, k = t % K, I = I0 + r;
-        X[r * LDX + k] = I < nE ? dz[(size_t)I * kH + k] : 0.f;
+    const float4 *d4 = reinterpret_cast<const float4 *>(dz);
+    for (int t = threadIdx.x; t < kTcRows * kH / 4; t += kTcThreads) {
+        const int r = t / (kH / 4), k = t % (kH / 4), I = I0 + r;
+        *reinterpret_cast<float4 *>(X + r * LDX + 4 * k) =
+            I < nE ? d4[(size_t)I * (kH / 4) + k] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
@@ -342,106 +368,178 @@ __global__ void k_gnn_vlog(int nV, const int *__restrict__ inc_ptr, const int *_
 
 // ---------------------------------------------------------------------------------- backward
 
-// dz3 = (dout W4) * [z3 > 0]
-__global__ void k_gnn_bout(int nE, const float *__restrict__ dout, const float *__restrict__ z3,
-                           const __nv_bfloat16 *__restrict__ w, float *__restrict__ dz3)
+// The weight-gradient kernels leave one partial per block over a contiguous range of edges, entries in a fixed
+// order, and k_gnn_wreduce adds the blocks' partials in a fixed order: deterministic sums.
+
+__device__ __forceinline__ int block_edges(int nE, int &e1)
 {
-    __shared__ float W[kO * kH];
-    for (int t = threadIdx.x; t < kO * kH; t += blockDim.x) W[t] = bf(w, oW4 + t);
-    __syncthreads();
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nE) return;
-    const float da = dout[kO * I], db = dout[kO * I + 1], dc = dout[kO * I + 2];
-    for (int k = 0; k < kH; ++k) {
-        const float z = z3[(size_t)I * kH + k];
-        dz3[(size_t)I * kH + k] = z > 0.f ? fmaf(da, W[k], fmaf(db, W[kH + k], dc * W[2 * kH + k])) : 0.f;
+    const int per = (nE + gridDim.x - 1) / gridDim.x, e0 = blockIdx.x * per;
+    e1 = min(nE, e0 + per);
+    return e0;
+}
+
+// Sum of v over the four thread groups of a 256-thread block (group g: threads 64 g ..), valid in group 0.
+template <int N>
+__device__ __forceinline__ void sum_groups(float (&v)[N], float (*sh)[kH])
+{
+    const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        __syncthreads();
+        sh[g][t] = v[k];
+        __syncthreads();
+        if (g == 0) v[k] = ((sh[0][t] + sh[1][t]) + sh[2][t]) + sh[3][t];
     }
 }
 
-// Block partials of grad_W[o][k] = sum_I dz[I][o] x_I[k] and grad_b[o] = sum_I dz[I][o] over one
-// contiguous edge range per block.  x_I = relu(xin[I]) (mode 0), avg(relu(xin[I-1]), relu(xin[I+1]))
-// (mode 1) or xin[I] itself (mode 2: the features).
-template <int O, int K>
-__global__ void __launch_bounds__(256) k_gnn_wgrad(int nE, const float *__restrict__ dz, const float *__restrict__ xin,
-                                                   const int *__restrict__ eprev, const int *__restrict__ enext,
-                                                   int mode, float *__restrict__ wpart)
+// Read-out: dz3 = (dout W4) * [z3 > 0], and the block's partial of grad_W4[c][k] = sum_I dout[I][c] relu(z3[I][k]) (3 x
+// 64) and grad_b4[c] = sum_I dout[I][c].  Thread (group, k): one pass over z3, coalesced.
+__global__ void __launch_bounds__(256) k_gnn_bout(int nE, const float *__restrict__ dout, const float *__restrict__ z3,
+                                                  const __nv_bfloat16 *__restrict__ w, float *__restrict__ dz3,
+                                                  float *__restrict__ wpart)
 {
-    constexpr int NE = O * K + O;          // entries: weights then biases
-    constexpr int PER = (NE + 255) / 256;  // entries per thread
-    __shared__ float sd[kWgSub][O], sx[kWgSub][K];
-    const int per_blk = (nE + gridDim.x - 1) / gridDim.x;
-    const int e0 = blockIdx.x * per_blk, e1 = min(nE, e0 + per_blk);
-    float acc[PER];
-#pragma unroll
-    for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-    for (int base = e0; base < e1; base += kWgSub) {
-        for (int t = threadIdx.x; t < kWgSub * O; t += blockDim.x) {
-            const int e = t / O, o = t % O, I = base + e;
-            sd[e][o] = I < e1 ? dz[(size_t)I * O + o] : 0.f;
-        }
-        for (int t = threadIdx.x; t < kWgSub * K; t += blockDim.x) {
-            const int e = t / K, k = t % K, I = base + e;
-            float xv = 0.f;
-            if (I < e1) {
-                if (mode == 0)
-                    xv = fmaxf(xin[(size_t)I * K + k], 0.f);
-                else if (mode == 1)
-                    xv = 0.5f * (fmaxf(xin[(size_t)eprev[I] * K + k], 0.f) + fmaxf(xin[(size_t)enext[I] * K + k], 0.f));
-                else
-                    xv = xin[(size_t)I * K + k];
-            }
-            sx[e][k] = xv;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int ent = threadIdx.x + 256 * q;
-            if (ent < O * K) {
-                const int o = ent / K, k = ent % K;
-                float s = acc[q];
+    __shared__ float sh[4][kH];
+    const int g = threadIdx.x >> 6, k = threadIdx.x & 63;
+    const float w0 = bf(w, oW4 + k), w1 = bf(w, oW4 + kH + k), w2 = bf(w, oW4 + 2 * kH + k);
+    int e1;
+    const int e0 = block_edges(nE, e1);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
-                for (int e = 0; e < kWgSub; ++e) s = fmaf(sd[e][o], sx[e][k], s);
-                acc[q] = s;
-            } else if (ent < NE) {
-                const int o = ent - O * K;
-                float s = acc[q];
-                for (int e = 0; e < kWgSub; ++e) s += sd[e][o];
-                acc[q] = s;
+    for (int I = e0 + g; I < e1; I += 4) {
+        const float z = z3[(size_t)I * kH + k], da = dout[kO * I], db = dout[kO * I + 1], dc = dout[kO * I + 2];
+        dz3[(size_t)I * kH + k] = z > 0.f ? fmaf(da, w0, fmaf(db, w1, dc * w2)) : 0.f;
+        const float h = fmaxf(z, 0.f);
+        acc[0] = fmaf(da, h, acc[0]);
+        acc[1] = fmaf(db, h, acc[1]);
+        acc[2] = fmaf(dc, h, acc[2]);
+        acc[3] += k == 0 ? da : (k == 1 ? db : dc);
+    }
+    sum_groups(acc, sh);
+    if (g == 0) {
+        float *o = wpart + (size_t)blockIdx.x * kWgSmall;
+        for (int c = 0; c < kO; ++c) o[c * kH + k] = acc[c];
+        if (k < kO) o[kO * kH + k] = acc[3];
+    }
+}
+
+// A message-passing layer's weights: the block's partial of sum_I dz[I][o] [h_I | m_I][k] (64 x 128, h = relu(zin), m
+// the average of the neighbours' h) and of sum_I dz[I][o].  Each thread owns a 4 x 8 tile of the entries, so an
+// edge costs it three 16-byte shared loads for 32 products (one product per two loads took 2 x 53 us a layer).
+__global__ void __launch_bounds__(256) k_gnn_wgrad(int nE, const float *__restrict__ dz, const float *__restrict__ zin,
+                                                   const int *__restrict__ eprev, const int *__restrict__ enext,
+                                                   float *__restrict__ wpart)
+{
+    __shared__ __align__(16) float sd[kWgSub][kH], sx[kWgSub][2 * kH];
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;  // outputs 4 ty .., inputs 4 tx .. and 64 + 4 tx ..
+    int e1;
+    const int e0 = block_edges(nE, e1);
+    float acc[4][8], bias[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    const float4 *d4 = reinterpret_cast<const float4 *>(dz), *z4 = reinterpret_cast<const float4 *>(zin);
+    for (int base = e0; base < e1; base += kWgSub) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < kWgSub * kH / 4; t += 256) {
+            const int r = t / (kH / 4), k = t % (kH / 4), I = base + r;
+            float4 d = make_float4(0.f, 0.f, 0.f, 0.f), h = d, m = d;
+            if (I < e1) {
+                d = d4[(size_t)I * (kH / 4) + k];
+                h = relu4(z4[(size_t)I * (kH / 4) + k]);
+                m = avg4(relu4(z4[(size_t)eprev[I] * (kH / 4) + k]), relu4(z4[(size_t)enext[I] * (kH / 4) + k]));
             }
+            reinterpret_cast<float4 *>(sd[r])[k] = d;
+            reinterpret_cast<float4 *>(sx[r])[k] = h;
+            reinterpret_cast<float4 *>(sx[r])[kH / 4 + k] = m;
         }
         __syncthreads();
-    }
+#pragma unroll 4
+        for (int e = 0; e < kWgSub; ++e) {
+            const float4 d = reinterpret_cast<const float4 *>(sd[e])[ty];
+            const float4 h = reinterpret_cast<const float4 *>(sx[e])[tx], m = reinterpret_cast<const float4 *>(sx[e])[16 + tx];
+            const float dv[4] = {d.x, d.y, d.z, d.w}, xv[8] = {h.x, h.y, h.z, h.w, m.x, m.y, m.z, m.w};
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int ent = threadIdx.x + 256 * q;
-        if (ent < NE) wpart[(size_t)blockIdx.x * kWgMax + ent] = acc[q];
+            for (int i = 0; i < 4; ++i) {
+                bias[i] += dv[i];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(dv[i], xv[j], acc[i][j]);
+            }
+        }
+    }
+    float *o = wpart + (size_t)blockIdx.x * kWgMax;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int out = 4 * ty + i;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            o[out * kH + 4 * tx + j] = acc[i][j];
+            o[kH * kH + out * kH + 4 * tx + j] = acc[i][4 + j];
+        }
+        if (tx == 0) o[2 * kH * kH + out] = bias[i];
     }
 }
 
-// grad[oW + e] (and the biases at ob) = sum of the block partials, in block order
-__global__ void k_gnn_wreduce(int nW, int nB, int nblk, const float *__restrict__ wpart, int oW, int ob,
-                              float *__restrict__ grad)
+// grad[o0 + e] for the first n0 entries, grad[o1 + e - n0] for the next n1 and grad[o2 + e - n0 - n1] for the last n2:
+// the blocks' partials added by eight warps (warp w: blocks w, w + 8, ...), then the warps in order.
+__global__ void __launch_bounds__(256) k_gnn_wreduce(int n0, int o0, int n1, int o1, int n2, int o2, int nblk, int stride,
+                                                     const float *__restrict__ wpart, float *__restrict__ grad)
 {
-    const int ent = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ent >= nW + nB) return;
+    __shared__ float sh[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ent = blockIdx.x * 32 + lane, n = n0 + n1 + n2;
     float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += wpart[(size_t)b * kWgMax + ent];
-    if (ent < nW)
-        grad[oW + ent] = s;
-    else
-        grad[ob + ent - nW] = s;
+    if (ent < n)
+#pragma unroll 8
+        for (int b = w; b < nblk; b += 8) s += wpart[(size_t)b * stride + ent];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w || ent >= n) return;
+    for (int k = 1; k < 8; ++k) s += sh[k][lane];
+    grad[ent < n0 ? o0 + ent : (ent < n0 + n1 ? o1 + ent - n0 : o2 + ent - n0 - n1)] = s;
 }
 
-// dzin = (dh + (dm[I+1] + dm[I-1]) / 2) * [zin > 0], written over dh (m[J] averages h[J-1], h[J+1])
+// dzin = (dh + (dm[I+1] + dm[I-1]) / 2) * [zin > 0], written over dh (m[J] averages h[J-1], h[J+1]); one thread per
+// four values, coalesced
 __global__ void k_gnn_bcombine(int nE, const int *__restrict__ eprev, const int *__restrict__ enext,
-                               const float *__restrict__ dm, const float *__restrict__ zin, float *__restrict__ dh)
+                               const float4 *__restrict__ dm, const float4 *__restrict__ zin, float4 *__restrict__ dh)
 {
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, I = t / (kH / 4), k = t % (kH / 4);
     if (I >= nE) return;
-    const int P = eprev[I], N = enext[I];
-    for (int k = 0; k < kH; ++k) {
-        const float g = dh[(size_t)I * kH + k] + 0.5f * (dm[(size_t)N * kH + k] + dm[(size_t)P * kH + k]);
-        dh[(size_t)I * kH + k] = zin[(size_t)I * kH + k] > 0.f ? g : 0.f;
+    const float4 z = zin[t], d = dh[t], n = dm[(size_t)enext[I] * (kH / 4) + k], p = dm[(size_t)eprev[I] * (kH / 4) + k];
+    dh[t] = make_float4(z.x > 0.f ? d.x + 0.5f * (n.x + p.x) : 0.f, z.y > 0.f ? d.y + 0.5f * (n.y + p.y) : 0.f,
+                        z.z > 0.f ? d.z + 0.5f * (n.z + p.z) : 0.f, z.w > 0.f ? d.w + 0.5f * (n.w + p.w) : 0.f);
+}
+
+// The first layer: dz1 = (dh + (dm[I+1] + dm[I-1]) / 2) * [z1 > 0] and the block's partial of grad_W1[o][k] = sum_I
+// dz1[I][o] f[I][k] (64 x 8) and grad_b1[o] = sum_I dz1[I][o].  Thread (group, o).
+__global__ void __launch_bounds__(256) k_gnn_wgrad1(int nE, const int *__restrict__ eprev, const int *__restrict__ enext,
+                                                    const float *__restrict__ dh, const float *__restrict__ dm,
+                                                    const float *__restrict__ z1, const float *__restrict__ feat,
+                                                    float *__restrict__ wpart)
+{
+    __shared__ float sh[4][kH];
+    const int g = threadIdx.x >> 6, o = threadIdx.x & 63;
+    int e1;
+    const int e0 = block_edges(nE, e1);
+    float acc[kF + 1];
+#pragma unroll
+    for (int k = 0; k <= kF; ++k) acc[k] = 0.f;
+#pragma unroll 4
+    for (int I = e0 + g; I < e1; I += 4) {
+        const float z = z1[(size_t)I * kH + o];
+        float d = dh[(size_t)I * kH + o] + 0.5f * (dm[(size_t)enext[I] * kH + o] + dm[(size_t)eprev[I] * kH + o]);
+        d = z > 0.f ? d : 0.f;
+        const float4 a = reinterpret_cast<const float4 *>(feat)[2 * (size_t)I], b = reinterpret_cast<const float4 *>(feat)[2 * (size_t)I + 1];
+        const float x[kF] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int k = 0; k < kF; ++k) acc[k] = fmaf(d, x[k], acc[k]);
+        acc[kF] += d;
+    }
+    sum_groups(acc, sh);
+    if (g == 0) {
+        float *p = wpart + (size_t)blockIdx.x * kWgSmall;
+        for (int k = 0; k < kF; ++k) p[o * kF + k] = acc[k];
+        p[kH * kF + o] = acc[kF];
     }
 }
 
@@ -634,6 +732,7 @@ int gnn_num_params() { return kNParams; }
 cudaError_t gnn_alloc(Ctx &c)
 {
     if (c.gnn) return cudaSuccess;
+    TPE_CHECK(cudaFuncSetAttribute(k_gnn_lmp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLmpSmem));
     c.gnn = new GnnState();
     GnnState &G = *c.gnn;
     const size_t nE = std::max(1, c.nE), nV = std::max(1, c.nV);
@@ -746,51 +845,47 @@ cudaError_t gnn_forward(Ctx &c, cudaStream_t s)
     const int nb = (c.nE + 127) / 128;
     k_gnn_l1<<<nb, 128, 0, s>>>(c.nE, G.feat, G.wb, G.z1);
     const int ntc = (c.nE + kTcRows - 1) / kTcRows;
-    k_gnn_lmp_tc<<<ntc, 64, 0, s>>>(c.nE, G.eprev, G.enext, G.z1, G.wb, oW2s, oW2n, ob2, G.z2);
-    k_gnn_lmp_tc<<<ntc, 64, 0, s>>>(c.nE, G.eprev, G.enext, G.z2, G.wb, oW3s, oW3n, ob3, G.z3);
+    k_gnn_lmp_tc<<<ntc, kTcThreads, kLmpSmem, s>>>(c.nE, G.eprev, G.enext, G.z1, G.wb, oW2s, oW2n, ob2, G.z2);
+    k_gnn_lmp_tc<<<ntc, kTcThreads, kLmpSmem, s>>>(c.nE, G.eprev, G.enext, G.z2, G.wb, oW3s, oW3n, ob3, G.z3);
     k_gnn_out<<<nb, 128, 0, s>>>(c.nE, G.z3, G.wb, G.out, G.ew);
     k_gnn_vlog<<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, c.d_inc_ptr, c.d_inc, G.out, G.vlog);
     c.launches += 5;
     return cudaGetLastError();
 }
 
-template <int O, int K>
-static cudaError_t wgrad(Ctx &c, const float *dz, const float *x, int mode, int oW, int ob, float *grad,
-                         cudaStream_t s)
+static void wreduce(GnnState &G, int nblk, int stride, int n0, int o0, int n1, int o1, int n2, int o2, float *grad, cudaStream_t s)
 {
-    GnnState &G = *c.gnn;
-    const int nblk = std::max(1, std::min(kWgBlocks, (c.nE + kWgSub - 1) / kWgSub));
-    k_gnn_wgrad<O, K><<<nblk, 256, 0, s>>>(c.nE, dz, x, G.eprev, G.enext, mode, G.wpart);
-    const int nb = ob >= 0 ? O : 0, n = O * K + nb;
-    k_gnn_wreduce<<<(n + 255) / 256, 256, 0, s>>>(O * K, nb, nblk, G.wpart, oW, ob, grad);
-    c.launches += 2;
-    return cudaGetLastError();
+    k_gnn_wreduce<<<(n0 + n1 + n2 + 31) / 32, 256, 0, s>>>(n0, o0, n1, o1, n2, o2, nblk, stride, G.wpart, grad);
 }
 
 // Parameter gradient (FP32, [P]) of a scalar whose derivative with respect to the outputs of the
-// last forward pass is dout [nE][2].
+// last forward pass is dout [nE][3].
 cudaError_t gnn_backward(Ctx &c, const float *dout, float *grad, cudaStream_t s)
 {
     GnnState &G = *c.gnn;
-    const int nb = (c.nE + 127) / 128;
-    // read-out: W4, b4, then dz3 into bA
-    TPE_CHECK((wgrad<kO, kH>(c, dout, G.z3, 0, oW4, ob4, grad, s)));
-    k_gnn_bout<<<nb, 128, 0, s>>>(c.nE, dout, G.z3, G.wb, G.bA);
-    c.launches++;
-    // layer 3: x = h2 (self) and avg h2 (neighbours)
-    TPE_CHECK((wgrad<kH, kH>(c, G.bA, G.z2, 0, oW3s, ob3, grad, s)));
-    TPE_CHECK((wgrad<kH, kH>(c, G.bA, G.z2, 1, oW3n, -1, grad, s)));
-    k_gnn_bmat_tc<<<(c.nE + kTcRows - 1) / kTcRows, 64, 0, s>>>(c.nE, G.bA, G.wb, oW3s, oW3n, G.bB, G.bC);
-    k_gnn_bcombine<<<nb, 128, 0, s>>>(c.nE, G.eprev, G.enext, G.bC, G.z2, G.bB);  // dz2 in bB
-    c.launches += 2;
-    // layer 2
-    TPE_CHECK((wgrad<kH, kH>(c, G.bB, G.z1, 0, oW2s, ob2, grad, s)));
-    TPE_CHECK((wgrad<kH, kH>(c, G.bB, G.z1, 1, oW2n, -1, grad, s)));
-    k_gnn_bmat_tc<<<(c.nE + kTcRows - 1) / kTcRows, 64, 0, s>>>(c.nE, G.bB, G.wb, oW2s, oW2n, G.bA, G.bC);
-    k_gnn_bcombine<<<nb, 128, 0, s>>>(c.nE, G.eprev, G.enext, G.bC, G.z1, G.bA);  // dz1 in bA
-    c.launches += 2;
-    // layer 1: x = the features
-    TPE_CHECK((wgrad<kH, kF>(c, G.bA, G.feat, 2, oW1, ob1, grad, s)));
+    const int nblk = std::max(1, std::min(kWgBlocks, (c.nE + kWgSub - 1) / kWgSub));
+    const int nsmall = std::max(1, std::min(kWgSmallBlocks, (c.nE + kWgSub - 1) / kWgSub));
+    const int ntc = (c.nE + kTcRows - 1) / kTcRows, n4 = c.nE * (kH / 4);
+    auto combine = [&](const float *zin, float *dh) {
+        k_gnn_bcombine<<<(n4 + 255) / 256, 256, 0, s>>>(c.nE, G.eprev, G.enext, reinterpret_cast<const float4 *>(G.bC),
+                                                        reinterpret_cast<const float4 *>(zin), reinterpret_cast<float4 *>(dh));
+    };
+    // read-out: W4, b4, and dz3 into bA
+    k_gnn_bout<<<nsmall, 256, 0, s>>>(c.nE, dout, G.z3, G.wb, G.bA, G.wpart);
+    wreduce(G, nsmall, kWgSmall, kO * kH, oW4, kO, ob4, 0, 0, grad, s);
+    // layer 3 on z2: its weights, then dz2 in bB
+    k_gnn_wgrad<<<nblk, 256, 0, s>>>(c.nE, G.bA, G.z2, G.eprev, G.enext, G.wpart);
+    wreduce(G, nblk, kWgMax, kH * kH, oW3s, kH * kH, oW3n, kH, ob3, grad, s);
+    k_gnn_bmat_tc<<<ntc, kTcThreads, 0, s>>>(c.nE, G.bA, G.wb, oW3s, oW3n, G.bB, G.bC);
+    combine(G.z2, G.bB);
+    // layer 2 on z1: its weights, then dh1 in bA and dm1 in bC
+    k_gnn_wgrad<<<nblk, 256, 0, s>>>(c.nE, G.bB, G.z1, G.eprev, G.enext, G.wpart);
+    wreduce(G, nblk, kWgMax, kH * kH, oW2s, kH * kH, oW2n, kH, ob2, grad, s);
+    k_gnn_bmat_tc<<<ntc, kTcThreads, 0, s>>>(c.nE, G.bB, G.wb, oW2s, oW2n, G.bA, G.bC);
+    // layer 1 on the features
+    k_gnn_wgrad1<<<nsmall, 256, 0, s>>>(c.nE, G.eprev, G.enext, G.bA, G.bC, G.z1, G.feat, G.wpart);
+    wreduce(G, nsmall, kWgSmall, kH * kF, oW1, kH, ob1, 0, 0, grad, s);
+    c.launches += 11;
     return cudaGetLastError();
 }
 
