@@ -128,31 +128,34 @@ __global__ void k_coarse_factor(const CoarseCurve *__restrict__ cc, double *__re
     }
 }
 
-// w[j][q] = Z_j^T r: one block per (curve, j)
-__global__ void k_coarse_restrict(const CoarseCurve *__restrict__ cc, const double *__restrict__ r,
-                                  double *__restrict__ w)
+// w[j][q] = Z_j^T r: one block per (curve, j), of one warp for hats of up to kRestrictWarp vertices and of four
+// above that.  Latency bounds it (a few dependent loads): the warp's shuffles take the place of seven barriers.
+constexpr int kRestrictWarp = 256;
+__global__ void __launch_bounds__(128) k_coarse_restrict(const CoarseCurve *__restrict__ cc,
+                                                         const double *__restrict__ r, double *__restrict__ w)
 {
     const CoarseCurve C = cc[blockIdx.x];
     const int j = blockIdx.y;
     if (j >= C.m - 1) return;
     int lo, len;
     hat_support(j, C.n, C.m, lo, len);
-    __shared__ double sh[3][128];
+    __shared__ double sh[4][3];
     double s[3] = {0, 0, 0};
     for (int k = threadIdx.x; k < len; k += blockDim.x) {
         int i = ((lo + k) % C.n + C.n) % C.n;
         double z = hat(i, j, C.n, C.m);
         for (int q = 0; q < 3; ++q) s[q] += z * r[3 * (C.v0 + i) + q];
     }
-    for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] = s[q];
+    for (int o = 16; o > 0; o >>= 1)
+        for (int q = 0; q < 3; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int q = 0; q < 3; ++q) sh[threadIdx.x >> 5][q] = s[q];
     __syncthreads();
-    for (int wv = 64; wv > 0; wv >>= 1) {
-        if (threadIdx.x < wv)
-            for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + wv];
-        __syncthreads();
+    if (threadIdx.x < 3) {
+        double x = sh[0][threadIdx.x];
+        for (int k = 1; k < (int)blockDim.x / 32; ++k) x += sh[k][threadIdx.x];
+        w[C.woff + 3 * j + threadIdx.x] = x;
     }
-    if (threadIdx.x == 0)
-        for (int q = 0; q < 3; ++q) w[C.woff + 3 * j + q] = sh[q][0];
 }
 
 // y = (Z^T A Z)^-1 w per curve: one warp per row (8 rows per block, blockIdx.y the curve).  The lanes
@@ -187,9 +190,9 @@ __global__ void __launch_bounds__(32 * kSolveRows) k_coarse_solve(const CoarseCu
         for (int q = 0; q < 3; ++q) y[C.woff + 3 * r + q] = s[q];
 }
 
-// z[v] += sum_j Z_j(i) y_j (each vertex lies in at most two hats)
+// z[v] += sum_j Z_j(i) (w_j - w2_j) (each vertex lies in at most two hats; w2 may be NULL)
 __global__ void k_coarse_prolong(int nV, const CoarseCurve *__restrict__ cc, const int *__restrict__ vcurve,
-                                 const double *__restrict__ w, double *__restrict__ z)
+                                 const double *__restrict__ w, const double *__restrict__ w2, double *__restrict__ z)
 {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nV) return;
@@ -202,7 +205,7 @@ __global__ void k_coarse_prolong(int nV, const CoarseCurve *__restrict__ cc, con
         int j = (j0 + dj) % C.m;
         if (j >= C.m - 1) continue;
         double h = hat(i, j, C.n, C.m);
-        for (int q = 0; q < 3; ++q) acc[q] += h * w[C.woff + 3 * j + q];
+        for (int q = 0; q < 3; ++q) acc[q] += h * (w[C.woff + 3 * j + q] - (w2 ? w2[C.woff + 3 * j + q] : 0.0));
     }
     for (int q = 0; q < 3; ++q) z[3 * v + q] += acc[q];
 }
@@ -222,23 +225,27 @@ __global__ void k_az_store(int nV, int b, const CoarseCurve *__restrict__ cc, co
 }
 
 // out[v] = r[v] - sum_j AZ[j][v] w[j] (three components; each vertex reads its curve's column entries,
-// consecutive vertices read consecutive addresses of a column).  The coefficients w of a chunk of
-// columns are staged in shared memory, and the column loop is unrolled so that every thread keeps
-// several independent loads in flight (the pass streams n (m - 1) doubles from memory).
-constexpr int kAzChunk = 512;
-__global__ void __launch_bounds__(256) k_az_prolong_sub(int nV, const CoarseCurve *__restrict__ cc,
-                                                        const int *__restrict__ vcurve, const double *__restrict__ AZ,
-                                                        const double *__restrict__ w, const double *__restrict__ r,
-                                                        double *__restrict__ out, int max_mm)
+// consecutive vertices read consecutive addresses of a column).  A block serves 32 vertices and its warps split
+// the columns: FP64 FMAs bound the pass (64 cycles a warp instruction), and a warp with every column of its 32
+// vertices would leave the 608 schedulers one or two warps each; with a quarter of the columns per warp the work
+// spreads evenly and four times the loads are in flight.  8 curves of 4,096, 128 hats: 26 us (the
+// FMAs alone take 21), with a thread per vertex 40.
+constexpr int kAzChunk = 512, kAzWarps = 4;
+__global__ void __launch_bounds__(32 * kAzWarps) k_az_prolong_sub(int nV, const CoarseCurve *__restrict__ cc,
+                                                                  const int *__restrict__ vcurve, const double *__restrict__ AZ,
+                                                                  const double *__restrict__ w, const double *__restrict__ r,
+                                                                  double *__restrict__ out, int max_mm)
 {
     __shared__ double sw[3 * kAzChunk];
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double part[kAzWarps][3][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int v = blockIdx.x * 32 + lane;
     const int vc = min(v, nV - 1);
     const CoarseCurve C = cc[vcurve[vc]];
     const int i = vc - C.v0, mm = C.m - 1;
     const double *az = AZ + C.zoff + i;
-    // the block's vertices may span curves: each stages its own curve's coefficients chunk by chunk
-    const CoarseCurve C0 = cc[vcurve[min((int)(blockIdx.x * blockDim.x), nV - 1)]];
+    // the block's vertices may span curves: the coefficients of the first one's are staged chunk by chunk
+    const CoarseCurve C0 = cc[vcurve[blockIdx.x * 32]];
     const bool uniform = C0.woff == C.woff;
     const double *wc = w + C.woff;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -247,17 +254,18 @@ __global__ void __launch_bounds__(256) k_az_prolong_sub(int nV, const CoarseCurv
         __syncthreads();
         for (int t = threadIdx.x; t < 3 * cnt; t += blockDim.x) sw[t] = w[C0.woff + 3 * (long long)j0 + t];
         __syncthreads();
-        const int hi = min(mm, j0 + kAzChunk);
+        const int len = min(mm - j0, kAzChunk), per = (len + kAzWarps - 1) / kAzWarps;  // len <= 0: no columns left
+        const int lo = j0 + warp * per, hi = j0 + min(len, (warp + 1) * per);
         if (uniform) {
-#pragma unroll 8
-            for (int j = j0; j < hi; ++j) {
+#pragma unroll 16
+            for (int j = lo; j < hi; ++j) {
                 const double a = az[(long long)j * C.n];
                 s0 += a * sw[3 * (j - j0)];
                 s1 += a * sw[3 * (j - j0) + 1];
                 s2 += a * sw[3 * (j - j0) + 2];
             }
         } else {
-            for (int j = j0; j < hi; ++j) {
+            for (int j = lo; j < hi; ++j) {
                 const double a = az[(long long)j * C.n];
                 s0 += a * wc[3 * j];
                 s1 += a * wc[3 * j + 1];
@@ -265,10 +273,15 @@ __global__ void __launch_bounds__(256) k_az_prolong_sub(int nV, const CoarseCurv
             }
         }
     }
-    if (v >= nV) return;
-    out[3 * v] = r[3 * v] - s0;
-    out[3 * v + 1] = r[3 * v + 1] - s1;
-    out[3 * v + 2] = r[3 * v + 2] - s2;
+    part[warp][0][lane] = s0;
+    part[warp][1][lane] = s1;
+    part[warp][2][lane] = s2;
+    __syncthreads();
+    if (v >= nV || warp >= 3) return;
+    double acc = part[0][warp][lane];  // warp q finishes component q
+#pragma unroll
+    for (int k = 1; k < kAzWarps; ++k) acc += part[k][warp][lane];
+    out[3 * v + warp] = r[3 * v + warp] - acc;
 }
 
 // w[j][q] = sum_i AZ[j][i] y[v0 + i][q]: one block per (curve, kAzCols consecutive columns), so that each
@@ -285,6 +298,7 @@ __global__ void __launch_bounds__(256) k_az_restrict(const CoarseCurve *__restri
     double s[kAzCols][3];
 #pragma unroll
     for (int c = 0; c < kAzCols; ++c) s[c][0] = s[c][1] = s[c][2] = 0.0;
+#pragma unroll 2
     for (int i = threadIdx.x; i < C.n; i += blockDim.x) {
         const double *yy = y + 3 * (size_t)(C.v0 + i);
         const double y0 = yy[0], y1 = yy[1], y2 = yy[2];
@@ -297,28 +311,29 @@ __global__ void __launch_bounds__(256) k_az_restrict(const CoarseCurve *__restri
                 s[c][2] += a * y2;
             }
     }
-    __shared__ double sh[8][kAzCols * 3];
+    // warp sums by halving (a lane keeps half of its values at every step): 31 FP64 additions where 24 values by
+    // plain shuffles take 120, which was a third of the kernel (FP64: 64 cycles a warp instruction)
+    __shared__ double sh[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[32];
 #pragma unroll
-    for (int c = 0; c < kAzCols; ++c)
+    for (int t = 0; t < 32; ++t) v[t] = t < 3 * kAzCols ? s[t / 3][t % 3] : 0.0;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            double x = s[c][q];
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) sh[warp][3 * c + q] = x;
+    for (int half = 16; half > 0; half >>= 1) {
+        const bool up = lane & half;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
         }
+    }
+    sh[warp][lane] = v[0];  // lane t holds value t
     __syncthreads();
     if (threadIdx.x < 3 * nc) {
         double x = 0.0;
         for (int k = 0; k < 8; ++k) x += sh[k][threadIdx.x];
         w[C.woff + 3 * (long long)j0 + threadIdx.x] = x;
     }
-}
-
-__global__ void k_coarse_sub(long long n, const double *__restrict__ a, double *__restrict__ b)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = a[i] - b[i];
 }
 
 // The balancing form's extra storage (the A Z columns and two coarse vectors), allocated when that
@@ -384,6 +399,7 @@ cudaError_t coarse_init(Ctx &c)
         woff += 3LL * (C.m - 1);
         zoff += (long long)(C.m - 1) * C.n;
         S.max_m = std::max(S.max_m, C.m);
+        if (2 * (C.n / C.m) > kRestrictWarp) S.restrict_threads = 128;
         S.curves.push_back(C);
         for (int v = C.v0; v < C.v0 + C.n; ++v) vc[v] = k;
     }
@@ -465,10 +481,10 @@ cudaError_t coarse_apply(Ctx &c, const double *r, double *z, cudaStream_t s)
 {
     if (!c.coarse || !c.coarse->ready) return cudaSuccess;
     CoarseState &S = *c.coarse;
-    k_coarse_restrict<<<dim3(c.nCurves, S.max_m), 128, 0, s>>>(S.d_curves, r, S.d_w);
+    k_coarse_restrict<<<dim3(c.nCurves, S.max_m), S.restrict_threads, 0, s>>>(S.d_curves, r, S.d_w);
     k_coarse_solve<<<dim3((S.max_m - 1 + kSolveRows - 1) / kSolveRows, c.nCurves), 32 * kSolveRows,
                      sizeof(double) * 3 * (S.max_m - 1), s>>>(S.d_curves, S.d_L, S.d_w, S.d_w2);
-    k_coarse_prolong<<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w2, z);
+    k_coarse_prolong<<<(c.nV + 255) / 256, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w2, nullptr, z);
     c.launches += 3;
     return cudaGetLastError();
 }
@@ -484,9 +500,9 @@ cudaError_t coarse_balanced_apply(Ctx &c, const double *r, double *z, cudaStream
     const size_t smem = sizeof(double) * 3 * (S.max_m - 1);
     const int nb = (c.nV + 255) / 256;
     // c1 = E^-1 Z^T r,  r2 = r - (A Z) c1
-    k_coarse_restrict<<<dim3(c.nCurves, S.max_m), 128, 0, s>>>(S.d_curves, r, S.d_w);
+    k_coarse_restrict<<<dim3(c.nCurves, S.max_m), S.restrict_threads, 0, s>>>(S.d_curves, r, S.d_w);
     k_coarse_solve<<<gsolve, 32 * kSolveRows, smem, s>>>(S.d_curves, S.d_L, S.d_w, S.d_w2);
-    k_az_prolong_sub<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_AZ, S.d_w2, r, S.d_r2, S.max_m - 1);
+    k_az_prolong_sub<<<(c.nV + 31) / 32, 32 * kAzWarps, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_AZ, S.d_w2, r, S.d_r2, S.max_m - 1);
     c.launches += 3;
     // y = S r2 (into z)
     if (learned) {
@@ -498,10 +514,8 @@ cudaError_t coarse_balanced_apply(Ctx &c, const double *r, double *z, cudaStream
     // c2 = E^-1 (A Z)^T y;  z = y + Z (c1 - c2)
     k_az_restrict<<<dim3(c.nCurves, (S.max_m - 1 + kAzCols - 1) / kAzCols), 256, 0, s>>>(S.d_curves, S.d_AZ, z, S.d_w3);
     k_coarse_solve<<<gsolve, 32 * kSolveRows, smem, s>>>(S.d_curves, S.d_L, S.d_w3, S.d_w4);
-    const long long nw = (long long)S.curves.back().woff + 3LL * (S.curves.back().m - 1);
-    k_coarse_sub<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(nw, S.d_w2, S.d_w4);
-    k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w4, z);
-    c.launches += 4;
+    k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w2, S.d_w4, z);
+    c.launches += 3;
     return cudaGetLastError();
 }
 
@@ -525,20 +539,20 @@ cudaError_t coarse_balanced_part(Ctx &c, int which, const double *v, double *out
     if (which == 2)
         k_az_restrict<<<dim3(c.nCurves, (S.max_m - 1 + kAzCols - 1) / kAzCols), 256, 0, s>>>(S.d_curves, S.d_AZ, v, S.d_w3);
     else
-        k_coarse_restrict<<<dim3(c.nCurves, S.max_m), 128, 0, s>>>(S.d_curves, v, S.d_w3);
+        k_coarse_restrict<<<dim3(c.nCurves, S.max_m), S.restrict_threads, 0, s>>>(S.d_curves, v, S.d_w3);
     k_coarse_solve<<<gsolve, 32 * kSolveRows, smem, s>>>(S.d_curves, S.d_L, S.d_w3, S.d_w4);
     c.launches += 2;
     if (which == 0) {
         TPE_CHECK(cudaMemsetAsync(out, 0, sizeof(double) * 3 * c.nV, s));
-        k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w4, out);
+        k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w4, nullptr, out);
         c.launches++;
     } else if (which == 1) {
-        k_az_prolong_sub<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_AZ, S.d_w4, v, out, S.max_m - 1);
+        k_az_prolong_sub<<<(c.nV + 31) / 32, 32 * kAzWarps, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_AZ, S.d_w4, v, out, S.max_m - 1);
         c.launches++;
     } else {
         if (out != v) TPE_CHECK(cudaMemcpyAsync(out, v, sizeof(double) * 3 * c.nV, cudaMemcpyDeviceToDevice, s));
         k_coarse_neg<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(nw, S.d_w4);
-        k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w4, out);
+        k_coarse_prolong<<<nb, 256, 0, s>>>(c.nV, S.d_curves, S.d_vcurve, S.d_w4, nullptr, out);
         c.launches += 2;
     }
     return cudaGetLastError();

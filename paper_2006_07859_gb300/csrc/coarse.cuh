@@ -38,6 +38,7 @@ struct tpe::CoarseState {
                              // balancing form, assembled by the A Z pass
     double *d_r2 = nullptr;  // balancing form: r - A Q r, [nV][3]
     int max_m = 0;
+    int restrict_threads = 32;   // block of the restriction, by the longest hat
     int ready = 0;
     int balanced = 0;        // the AZ columns are kept (every problem is one curve)
     // A Z pass (every curve's coarse space has at least kMinPassCoarse hats)

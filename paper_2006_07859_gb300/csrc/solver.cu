@@ -40,34 +40,78 @@ struct RedArgs {
     double *sums;          // [nprob][K]
 };
 
+// Warp sums of K values by halving: at each step a lane keeps one half of its values and adds the other lane's,
+// so 32 lanes x K values take about P + log2(32 / P) FP64 additions (P: K rounded up to a power of two) instead
+// of 5 K.  FP64 instructions bound these kernels (64 cycles a warp): 7 values by plain shuffles cost 2,240
+// cycles.  Afterwards v[0] of a lane holds the sum of value index(lane); lanes that differ in the low bits agree.
+template <int P, int MASK>
+__device__ __forceinline__ void warp_halve(double *v, int lane)
+{
+    if constexpr (MASK > 0) {
+        if constexpr (P > 1) {
+            const bool up = lane & MASK;
+#pragma unroll
+            for (int i = 0; i < P / 2; ++i) {
+                const double send = up ? v[i] : v[i + P / 2], keep = up ? v[i + P / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, MASK);
+            }
+            warp_halve<P / 2, MASK / 2>(v, lane);
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], MASK);
+            warp_halve<1, MASK / 2>(v, lane);
+        }
+    }
+}
+template <int K>
+__host__ __device__ constexpr int pow2_at_least()
+{
+    int p = 1;
+    while (p < K) p *= 2;
+    return p;
+}
+
 // Block-reduce K values, publish the block partial, and in the last block sum the partials of
 // every problem into sums[q][k].  Returns true in the last block (all threads).
 template <int K>
 __device__ bool reduce_phase(double (&s)[K], const RedArgs &ra)
 {
-    __shared__ double sh[K][kRedThreads];
+    constexpr int P = pow2_at_least<K>(), W = kRedThreads / 32;
+    static_assert(P <= 16, "one value per lane group");
+    __shared__ double sh[W][P];
     __shared__ bool last;
-    for (int k = 0; k < K; ++k) sh[k][threadIdx.x] = s[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) v[k] = k < K ? s[k] : 0.0;
+    warp_halve<P, 16>(v, lane);
+    if ((lane & (32 / P - 1)) == 0) sh[warp][lane / (32 / P)] = v[0];  // lane bits from the top select the half kept
     __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int k = 0; k < K; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < K; ++k) ra.partial[(size_t)blockIdx.x * K + k] = sh[k][0];
+    if (threadIdx.x < K) {
+        double acc = sh[0][threadIdx.x];
+        for (int w = 1; w < W; ++w) acc += sh[w][threadIdx.x];
+        ra.partial[(size_t)blockIdx.x * K + threadIdx.x] = acc;
         __threadfence();
-        last = (atomicAdd(ra.counter, 1u) == gridDim.x - 1);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = (atomicAdd(ra.counter, 1u) == gridDim.x - 1);
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    for (int q = threadIdx.x; q < ra.nprob; q += blockDim.x) {
-        for (int k = 0; k < K; ++k) {
-            double acc = 0.0;
-            for (int ch = ra.prob_c0[q]; ch < ra.prob_c0[q + 1]; ++ch) acc += __ldcg(&ra.partial[(size_t)ch * K + k]);
-            ra.sums[(size_t)q * K + k] = acc;
+    // G lanes per (problem, value), as many as the block has; each adds every G-th chunk, then the group adds up
+    const int total = ra.nprob * K;
+    int G = 32;
+    while (G > 1 && (long long)G * total > kRedThreads) G /= 2;
+    const int sub = threadIdx.x & (G - 1);
+    for (int base = 0; base < total; base += kRedThreads / G) {
+        const int i = base + threadIdx.x / G, q = i / K, k = i % K;
+        double acc = 0.0;
+        if (i < total) {
+            const int c1 = ra.prob_c0[q + 1];
+#pragma unroll 4
+            for (int ch = ra.prob_c0[q] + sub; ch < c1; ch += G) acc += __ldcg(&ra.partial[(size_t)ch * K + k]);
         }
+        for (int o = G / 2; o > 0; o /= 2) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (i < total && sub == 0) ra.sums[(size_t)q * K + k] = acc;
     }
     if (threadIdx.x == 0) *ra.counter = 0u;
     __threadfence();
@@ -132,10 +176,16 @@ cudaError_t solver_setup(Ctx &c)
 {
     c.sol = new SolverState();
     SolverState &s = S(c);
-    // chunks of 2048 elements (8 per thread): measured faster on the benchmark step than chunks sized to
-    // two per SM (more blocks, each with one element per thread, made the CG kernels slower)
-    make_red_plan(c.h_prob_v, 2048, &s.v_lo, &s.v_c0, &s.v_n);
-    make_red_plan(c.h_prob_e, 2048, &s.e_lo, &s.e_c0, &s.e_n);
+    // chunks of one to eight elements per thread: two blocks per SM where the graph is large enough.  FP64
+    // instructions bound the CG kernels, so idle SMs cost most (8 x 4,096 vertices, 16 blocks of 2,048: 22 us a
+    // reduction kernel, 128 blocks of 256: 11 us); the last block's share stays small because its threads split
+    // the chunks of a problem.
+    auto cap = [&](const std::vector<int32_t> &off) {
+        const int per = (int)((off.back() - off[0]) / (2LL * std::max(1, c.sm_count)) + 1);
+        return std::min(2048, std::max(kRedThreads, (per + kRedThreads - 1) / kRedThreads * kRedThreads));
+    };
+    make_red_plan(c.h_prob_v, cap(c.h_prob_v), &s.v_lo, &s.v_c0, &s.v_n);
+    make_red_plan(c.h_prob_e, cap(c.h_prob_e), &s.e_lo, &s.e_c0, &s.e_n);
     int mx = std::max(std::max(s.v_n, s.e_n), 1);
     TPE_CHECK(cudaMalloc(&s.partial, sizeof(double) * (size_t)mx * 16));
     TPE_CHECK(cudaMalloc(&s.counters, sizeof(unsigned) * 8));

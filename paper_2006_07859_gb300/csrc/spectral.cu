@@ -109,9 +109,12 @@ __device__ void fft_batch(double2 *a, int G, int M, int logM, const double2 *__r
             int i = g * M + grp * (half << 1) + pos, j = i + half;
             double2 w = tw[pos * step];
             if (inv) w.y = -w.y;
-            double2 u = a[i], v = cmul(a[j], w);
-            a[i] = make_double2(u.x + v.x, u.y + v.y);
-            a[j] = make_double2(u.x - v.x, u.y - v.y);
+            // s = u + w b by four FMAs and u - w b = 2 u - s by two: six FP64 instructions, where the product and
+            // the two sums take eight (the FP64 unit bounds every transform: 64 cycles per warp instruction)
+            const double2 u = a[i], b = a[j];
+            const double2 sum = make_double2(fma(-w.y, b.y, fma(w.x, b.x, u.x)), fma(w.y, b.x, fma(w.x, b.y, u.y)));
+            a[i] = sum;
+            a[j] = make_double2(fma(2.0, u.x, -sum.x), fma(2.0, u.y, -sum.y));
         }
         __syncthreads();
     }
@@ -209,11 +212,29 @@ __device__ __forceinline__ double2 twiddle_full(const double2 *__restrict__ tw, 
     return w;
 }
 
+__device__ __forceinline__ double flip_if(double x, unsigned m)
+{
+    return __hiloint2double(__double2hiint(x) ^ (int)m, __double2loint(x));  // m: 0 or the sign bit
+}
+
+// One radix-2 step across lanes: the lane with `bit` clear gets own + other, the other one other - own.
+__device__ __forceinline__ double2 lane_butterfly(double2 a, int bit, int lane)
+{
+    const unsigned m = lane & bit ? 0x80000000u : 0u;
+    return make_double2(__shfl_xor_sync(0xffffffffu, a.x, bit) + flip_if(a.x, m),
+                        __shfl_xor_sync(0xffffffffu, a.y, bit) + flip_if(a.y, m));
+}
+
 // z = D^-1/2 F^-1 diag(ilam) F D^-1/2 r for one (curve, component) per cluster.  Index m = m1 + 8 m2,
-// k = k2 + N2 k1.  Rank m1 transforms its column over m2 and twists by W_n^{m1 k2}; rank q then owns
-// rows k2 in [q N2/8, (q+1) N2/8): an 8-point DFT over m1 gathered from the cluster, the division by the
-// symbol, the 8-point inverse DFT over k1 and the twist W_n^{-m1 k2}; finally rank m1 gathers row m1 of
-// every k2 and transforms back over k2.
+// k = k2 + N2 k1.  Rank m1 transforms its column over m2 and twists by W_n^{m1 k2}; rank q then owns a share
+// of the rows k2: an 8-point DFT over m1 gathered from the cluster, the division by the symbol, the 8-point
+// inverse DFT over k1 and the twist W_n^{-m1 k2}; finally rank m1 gathers row m1 of every k2 and transforms back.
+//
+// FP64 instructions bound it (64 cycles a warp).  The columns are real and the symbol is even, so the spectrum of
+// a column is Hermitian: N2 real values take an N2/2-point complex transform, and only k2 = 0..N2/2 pass the middle
+// step, one lane per (k2, m1) with the 8-point DFTs across lanes (all four schedulers work, where a thread per
+// k2 with 64 twiddled products kept one busy).  Twice the even part of the symbol is used, which is all that reaches
+// the real part of the result.  8 curves of 4,096: 27.7 us, before 46.7.
 __global__ void __cluster_dims__(kClusterFFT, 1, 1) __launch_bounds__(kClusterThreads)
     k_spec_cluster(const SpecCurve *__restrict__ curves, const int *__restrict__ idx, const double *__restrict__ r,
                    double *__restrict__ z, const double *__restrict__ dinv, const double2 *__restrict__ tw,
@@ -225,57 +246,70 @@ __global__ void __cluster_dims__(kClusterFFT, 1, 1) __launch_bounds__(kClusterTh
     const int cidx = idx[tr / 3], comp = tr % 3;
     if (skip && skip[indep ? cidx : 0]) return;  // converged problem: the whole cluster leaves
     const SpecCurve C = curves[cidx];
-    const int n = C.n, N2 = n / kClusterFFT, logN2 = C.logM - 3, per = N2 / kClusterFFT;
-    const int sN = kMaxFFT / n, s8 = kMaxFFT / kClusterFFT;
-    __shared__ double2 Y[kClusterMaxN2];
-    __shared__ double2 V[kClusterMaxN2];
-    for (int m2 = threadIdx.x; m2 < N2; m2 += blockDim.x) {
-        const int v = C.v0 + rank + kClusterFFT * m2;
-        Y[m2] = make_double2(r[3 * v + comp] * dinv[v], 0.0);
+    const int n = C.n, N2 = n / kClusterFFT, H = N2 / 2, logH = C.logM - 4;
+    const int per = (H + 1 + kClusterFFT - 1) / kClusterFFT;
+    const int sN = kMaxFFT / n, s2 = kMaxFFT / N2;
+    __shared__ double2 Y[kClusterMaxN2 / 2 + 1];
+    __shared__ double2 V[kClusterMaxN2 / 2 + kClusterFFT];
+    for (int t = threadIdx.x; t < H; t += blockDim.x) {
+        const int v = C.v0 + rank + 2 * kClusterFFT * t, v2 = v + kClusterFFT;
+        Y[t] = make_double2(r[3 * v + comp] * dinv[v], r[3 * v2 + comp] * dinv[v2]);
     }
     __syncthreads();
-    fft_batch(Y, 1, N2, logN2, tw, false);
-    for (int k2 = threadIdx.x; k2 < N2; k2 += blockDim.x)
-        Y[k2] = cmul(Y[k2], twiddle_full(tw, ((rank * k2) % n) * sN, false));
+    fft_batch(Y, 1, H, logH, tw, false);
+    // twice the column's spectrum: X_k = E + w O, X_{H-k} = conj(E - w O), w = exp(-2 pi i k / N2)
+    for (int k = threadIdx.x; k <= H / 2; k += blockDim.x) {
+        const double2 a = Y[k], b = Y[(H - k) & (H - 1)];
+        const double2 E = make_double2(a.x + b.x, a.y - b.y), O = make_double2(a.y + b.y, b.x - a.x);
+        const double2 wO = cmul(O, twiddle_full(tw, k * s2, false));
+        Y[k] = make_double2(E.x + wO.x, E.y + wO.y);
+        Y[H - k] = make_double2(E.x - wO.x, wO.y - E.y);
+    }
     cl.sync();
-    for (int t = threadIdx.x; t < per; t += blockDim.x) {
-        const int k2 = rank * per + t;
-        double2 a[kClusterFFT], X[kClusterFFT];
-#pragma unroll
-        for (int m1 = 0; m1 < kClusterFFT; ++m1) a[m1] = cl.map_shared_rank(Y, m1)[k2];
-#pragma unroll
-        for (int k1 = 0; k1 < kClusterFFT; ++k1) {
-            double2 sacc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int m1 = 0; m1 < kClusterFFT; ++m1) {
-                const double2 p = cmul(a[m1], twiddle_full(tw, ((m1 * k1) % kClusterFFT) * s8, false));
-                sacc.x += p.x;
-                sacc.y += p.y;
-            }
-            const double f = ilam[C.v0 + k2 + N2 * k1];
-            X[k1] = make_double2(sacc.x * f, sacc.y * f);
-        }
-#pragma unroll
-        for (int m1 = 0; m1 < kClusterFFT; ++m1) {
-            double2 sacc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int k1 = 0; k1 < kClusterFFT; ++k1) {
-                const double2 p = cmul(X[k1], twiddle_full(tw, ((m1 * k1) % kClusterFFT) * s8, true));
-                sacc.x += p.x;
-                sacc.y += p.y;
-            }
-            V[t * kClusterFFT + m1] = cmul(sacc, twiddle_full(tw, ((m1 * k2) % n) * sN, true));
-        }
+    const int lane = threadIdx.x & 31, m1 = lane & 7, k1 = (int)(__brev((unsigned)m1) >> 29), pos = m1 & 3;
+    const double h = 0.70710678118654752440;
+    // W_8^pos for the lanes with bit 4 set, 1 for the others
+    const double2 w8 = !(m1 & 4) ? make_double2(1.0, 0.0)
+                                 : make_double2(pos == 0 ? 1.0 : pos == 1 ? h : pos == 2 ? 0.0 : -h,
+                                                pos == 0 ? 0.0 : pos == 2 ? -1.0 : -h);
+    for (int base = 0; base < per * kClusterFFT; base += blockDim.x) {  // uniform: the shuffles need whole warps
+        const int t = (base + threadIdx.x) / kClusterFFT, k2 = min(rank * per + t, H);
+        const double2 tws = twiddle_full(tw, m1 * k2 * sN, false);
+        double2 a = cmul(cl.map_shared_rank(Y, m1)[k2], tws);
+        // forward, decimation in frequency: the lane of input m1 ends with output k1
+        a = cmul(lane_butterfly(a, 4, lane), w8);
+        a = lane_butterfly(a, 2, lane);
+        if (pos == 3) a = make_double2(a.y, -a.x);
+        a = lane_butterfly(a, 1, lane);
+        const int k = k2 + N2 * k1;
+        const double f = ilam[C.v0 + k] + ilam[C.v0 + (k ? n - k : 0)];
+        a = make_double2(a.x * f, a.y * f);
+        // inverse, decimation in time: back to m1
+        a = lane_butterfly(a, 1, lane);
+        if (pos == 3) a = make_double2(-a.y, a.x);
+        a = cmul(lane_butterfly(a, 2, lane), cconj(w8));
+        a = lane_butterfly(a, 4, lane);
+        if (t < per) V[t * kClusterFFT + m1] = cmul(a, cconj(tws));
     }
     cl.sync();  // every rank's V is complete; nobody reads Y any more
-    for (int k2 = threadIdx.x; k2 < N2; k2 += blockDim.x)
+    for (int k2 = threadIdx.x; k2 <= H; k2 += blockDim.x)
         Y[k2] = cl.map_shared_rank(V, k2 / per)[(k2 % per) * kClusterFFT + rank];
     __syncthreads();
-    fft_batch(Y, 1, N2, logN2, tw, true);
-    const double sc = 1.0 / n;
-    for (int m2 = threadIdx.x; m2 < N2; m2 += blockDim.x) {
-        const int v = C.v0 + rank + kClusterFFT * m2;
-        z[3 * v + comp] = Y[m2].x * sc * dinv[v];
+    // Hermitian spectrum of a real column to the N2/2-point transform of its even and odd entries
+    for (int k = threadIdx.x; k <= H / 2; k += blockDim.x) {
+        const double2 a = Y[k], b = Y[H - k];
+        const double2 E = make_double2(a.x + b.x, a.y - b.y);
+        const double2 O = cmul(make_double2(a.x - b.x, a.y + b.y), twiddle_full(tw, k * s2, true));
+        Y[k] = make_double2(E.x - O.y, E.y + O.x);
+        if (k) Y[H - k] = make_double2(E.x + O.y, O.x - E.y);
+    }
+    __syncthreads();
+    fft_batch(Y, 1, H, logH, tw, true);
+    const double sc = 0.25 / n;  // the halves of the spectrum and of the symbol's even part
+    for (int t = threadIdx.x; t < H; t += blockDim.x) {
+        const int v = C.v0 + rank + 2 * kClusterFFT * t, v2 = v + kClusterFFT;
+        z[3 * v + comp] = Y[t].x * sc * dinv[v];
+        z[3 * v2 + comp] = Y[t].y * sc * dinv[v2];
     }
     cl.sync();  // the other ranks may still read this rank's V
 }
