@@ -432,7 +432,7 @@ tp_status tp_create(tp_ctx **out, int nV, int nE, const int32_t *edges_host, int
     make_plans(c);
     CK(cudaGetLastError());
     int ms = std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots);
-    c.part_elems = (size_t)ms * std::max(1, nE) * 6;
+    c.part_elems = std::max((size_t)ms * std::max(1, nE) * 6, sym_default_elems(c));
     CK(dalloc(&c.d_part, c.part_elems));
     CK(sym_defaults(c));
     CK(dalloc(&c.d_rows, nE));

@@ -750,7 +750,7 @@ __device__ __forceinline__ void tile_loop(const Tgt<typename RealOf<PREC>::type>
                     if (keep && dot3(e, e) < pa.kp.near2f_diff) {
                         if constexpr (FAST) {
                             dfl<float> x[10], y[10];
-                            near_diff(pa.recF, pa.recLo, tI[k], tI[k], s0 + j, s0 + j, x, y);
+                            near_diff(pa.recF, pa.recLo, tI[k], s0 + j, x, y);
                             l_kahan_df(a[k].S, a[k].cS, x[0].hi, x[0].lo);
 #pragma unroll
                             for (int q = 0; q < 3; ++q) {

@@ -170,10 +170,14 @@ __device__ __forceinline__ L l_energy_sum(L c0, L c1, L r11, L r12, L r21, L r22
 // terms (which cancel between a vertex's two edges) need more than FP32.  They are evaluated in
 // double-float arithmetic on the FP32 pipe (about 2^-44): an FP64 instruction of a warp holds its
 // sub-partition's FP64 pipe for 64 cycles, and one near pair of the differential takes ~500 of them
-// (33,000 cycles) against ~1,800 FP32 instructions here.  The pairs are renormalised only where a difference
+// (33,000 cycles) against ~2,000 FP32 instructions here.  The pairs are renormalised only where a difference
 // cancels (elsewhere lo stays within a few ulp of hi, its own rounding at 2^-47).  The functions load the records themselves
-// and are not inlined, and the differential's is unrolled over one endpoint only: unrolled over both, 48 KB of
-// straight-line code ran at the instruction cache's rate (23,000 cycles a call).
+// and are not inlined.  The instruction cache bounds the differential's: unrolled over both endpoints, 48 KB of
+// straight-line code took 23,000 cycles a call, and unrolled over one (22 KB) it still left the warps waiting for
+// instructions 30% of the time.  It is rolled over both endpoints (13 KB) and takes one pair a lane: packed
+// pairs do the same work of the FP32 pipe in half the instructions, but two rounds of the short code hit in
+// the cache (differential of 96 x 500 edges: packed, one endpoint unrolled 1,052 us, packed, rolled 1,060, single,
+// one unrolled 975, single, rolled 827).
 
 template <class L>
 struct dfl {
@@ -287,6 +291,17 @@ __device__ __forceinline__ dfv<L> near_chord(const NearEdge<L> &I, int a, const 
             l_two_sum(l_sub(I.p[a][2], J.p[b][2]), l_sub(I.l[a][2], J.l[b][2]))};
 }
 
+// the same with the endpoints chosen in a rolled loop
+template <class L>
+__device__ __forceinline__ dfv<L> near_chord_k(const NearEdge<L> &I, const NearEdge<L> &J, int a, int b)
+{
+#define TPE_C(q)                                                                \
+    l_two_sum(l_sub(a ? I.p[1][q] : I.p[0][q], b ? J.p[1][q] : J.p[0][q]), \
+              l_sub(a ? I.l[1][q] : I.l[0][q], b ? J.l[1][q] : J.l[0][q]))
+    return {TPE_C(0), TPE_C(1), TPE_C(2)};
+#undef TPE_C
+}
+
 // |T x d|^2 of a near pair, rounded to FP32
 template <class L>
 __device__ __forceinline__ L near_perp2(const dfv<L> &d, const dfv<L> &T)
@@ -331,57 +346,77 @@ __device__ __forceinline__ dfl<L> near_pow45(dfl<L> d2, dfl<L> &R2)
     return l_dfscale(F, l_mul(eps, l_fma(l_bc<L>(7.875f), eps, l_bc<L>(4.5f))));
 }
 
-// The differential's terms of one near pair (on the second lane I1, J1), scaled by the other row's length: row
-// I's (S, G1, G2, GT) into x and row J's (S, H1, H2, HT) into y, see pairs_sym.cu.
-template <class L>
-static __device__ __noinline__ void near_diff(const RecF *recF, const RecLo *recLo, int I0, int I1, int J0, int J1,
-                                              dfl<L> (&x)[10], dfl<L> (&y)[10])
+// The differential's terms of one near pair, scaled by the other row's length: row I's (S, G1, G2, GT) into x and
+// row J's (S, H1, H2, HT) into y, see pairs_sym.cu.
+static __device__ __noinline__ void near_diff(const RecF *recF, const RecLo *recLo, int I0, int J0, dfl<float> (&x)[10],
+                                              dfl<float> (&y)[10])
 {
+    using L = float;
     NearEdge<L> I, J;
-    near_load(I, recF, recLo, I0, I1);
-    near_load(J, recF, recLo, J0, J1);
-    const dfl<L> zero = {l_bc<L>(0.f), l_bc<L>(0.f)};
+    near_load(I, recF, recLo, I0, I0);
+    near_load(J, recF, recLo, J0, J0);
+    const dfl<L> zero = {0.f, 0.f};
     const dfv<L> TI = near_tangent(I), TJ = near_tangent(J);
     // |T_I x d_ab| and its perpendicular depend on b only, |T_J x d_ab| and its on a only
-    dfv<L> pI[2], pJ[2];
-    dfl<L> cI[2], cJ[2];
-#pragma unroll
+    dfv<L> pI[2] = {}, pJ[2] = {};
+    dfl<L> cI[2] = {}, cJ[2] = {};
+#pragma unroll 1
     for (int k = 0; k < 2; ++k) {
-        const dfv<L> dI = near_chord(I, 0, J, k), dJ = near_chord(I, k, J, 0);
-        pI[k] = l_dfperp(dI, l_dfdot(TI, dI), TI);
-        pJ[k] = l_dfperp(dJ, l_dfdot(TJ, dJ), TJ);
-        cI[k] = l_dfnorm2(pI[k]);
-        cJ[k] = l_dfnorm2(pJ[k]);
+        const dfv<L> dI = near_chord_k(I, J, 0, k), dJ = near_chord_k(I, J, k, 0);
+        pI[0] = pI[1];
+        pJ[0] = pJ[1];
+        cI[0] = cI[1];
+        cJ[0] = cJ[1];
+        pI[1] = l_dfperp(dI, l_dfdot(TI, dI), TI);
+        pJ[1] = l_dfperp(dJ, l_dfdot(TJ, dJ), TJ);
+        cI[1] = l_dfnorm2(pI[1]);
+        cJ[1] = l_dfnorm2(pJ[1]);
     }
     dfl<L> S = zero, H[2][3], GT[3] = {zero, zero, zero}, HT[3] = {zero, zero, zero};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) H[0][k] = H[1][k] = zero;
+    for (int k = 0; k < 3; ++k) H[0][k] = H[1][k] = x[4 + k] = zero;
 #pragma unroll 1
     for (int a = 0; a < 2; ++a) {
         dfl<L> G[3] = {zero, zero, zero};
-#pragma unroll
+#pragma unroll 1
         for (int b = 0; b < 2; ++b) {
-            const dfv<L> d = near_chord(I, 0, J, b);
+            const dfv<L> d = near_chord(I, 0, J, 0);
             dfl<L> r2;
             const dfl<L> rb = near_pow45(l_dfnorm2(d), r2);
-            const dfl<L> fs = l_dfmul(l_dfadd(cI[b], cJ[0]), rb);
+            const dfl<L> fs = l_dfmul(l_dfadd(cI[0], cJ[0]), rb);
             const dfl<L> al = {l_add(rb.hi, rb.hi), l_add(rb.lo, rb.lo)};  // alpha |d|^-beta
-            const dfl<L> cb = l_dfneg(l_dfmul(l_dfmulf(fs, l_bc<L>(4.5f)), r2));
+            const dfl<L> cb = l_dfneg(l_dfmul(l_dfmulf(fs, 4.5f), r2));
             const dfl<L> mI = l_dfneg(l_dfmul(al, l_dfdot(TI, d))), mJ = l_dfneg(l_dfmul(al, l_dfdot(TJ, d)));
-            const dfl<L> dk[3] = {d.x, d.y, d.z}, pi[3] = {pI[b].x, pI[b].y, pI[b].z}, pj[3] = {pJ[0].x, pJ[0].y, pJ[0].z};
+            const dfl<L> dk[3] = {d.x, d.y, d.z}, pi[3] = {pI[0].x, pI[0].y, pI[0].z}, pj[3] = {pJ[0].x, pJ[0].y, pJ[0].z};
             S = l_dfadd(S, fs);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const dfl<L> v = l_dfadd(l_dfmul(al, l_dfadd(pi[k], pj[k])), l_dfmul(cb, dk[k]));
                 G[k] = l_dfadd(G[k], v);
-                H[b][k] = l_dfadd(H[b][k], l_dfneg(v));
+                const dfl<L> h = l_dfadd(H[0][k], l_dfneg(v));
                 GT[k] = l_dfadd(GT[k], l_dfmul(mI, dk[k]));
                 HT[k] = l_dfadd(HT[k], l_dfmul(mJ, dk[k]));
+                // the other endpoint of J next
+                H[0][k] = H[1][k];
+                H[1][k] = h;
+                const L q = J.p[0][k], ql = J.l[0][k];
+                J.p[0][k] = J.p[1][k];
+                J.p[1][k] = q;
+                J.l[0][k] = J.l[1][k];
+                J.l[1][k] = ql;
             }
+            const dfv<L> pt = pI[0];
+            const dfl<L> ct = cI[0];
+            pI[0] = pI[1];
+            pI[1] = pt;
+            cI[0] = cI[1];
+            cI[1] = ct;
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            x[1 + 3 * a + k] = l_dfmulf(G[k], J.ell);
+            const dfl<L> xo = l_dfmulf(G[k], J.ell);
+            x[1 + k] = x[4 + k];
+            x[4 + k] = xo;
             // the second endpoint of I for the next round
             I.p[0][k] = I.p[1][k];
             I.l[0][k] = I.l[1][k];

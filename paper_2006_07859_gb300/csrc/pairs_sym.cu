@@ -19,7 +19,7 @@
 // for it; four targets do not fit in registers.)
 //
 // Blocks.  A problem's edges are cut into super-blocks of 256 target rows (128 threads x 2 adjacent rows) and
-// tiles of 128 source rows.  A work item is one super-block X against up to four tiles beyond it (c >= 2 X + 2),
+// tiles of 128 source rows.  A work item is one super-block X against half a tile to four tiles beyond it,
 // or against itself.  Lane l of a warp takes source (step + 2 l) mod P at step `step`: the 32 lanes touch 32
 // distinct sources and add what those receive into the warp's own Kahan-compensated shared-memory
 // accumulators (no atomics), and along a curve all lanes are equally far from their sources, so near pairs
@@ -458,47 +458,37 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const
 // consecutive.
 __device__ __forceinline__ int sym_slot(int j) { return ((j & 1) << 6) | (j >> 1); }
 
-// Evaluate up to 64 near pairs of the differential from a warp's queue, two per lane, into the warp's target and
+// Evaluate `count` near pairs of the differential from a warp's queue, 32 at a time, into the warp's target and
 // source sums.  Near pairs held back this way fill all lanes: on short curves every step has a few lanes
 // near another strand, and evaluated in place each of them cost the warp a whole double-float pair.  Pairs of
-// one batch that share a row add in queue order, one at a time.
+// one round that share a row add in queue order, one at a time.
 static __device__ __noinline__ void sym_near_flush(SymSmem<PMIX, OP_DIFF> &sm, int wid, int first, int count, int tgt0, int ntgt,
                                                    int s0, const SymArgs &pa)
 {
     const int lane = threadIdx.x & 31;
-    int row[2], at[2], I[2], J[2];
-    bool on[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int e = 32 * k + lane;
-        on[k] = e < count;
-        const int v = on[k] ? sm.queue[wid][first + e] : sm.queue[wid][first];
-        row[k] = v >> 8;
-        at[k] = v & 0xff;
-        const int loc = kSection * wid + row[k];
-        on[k] = on[k] && loc < ntgt;
-        I[k] = tgt0 + min(loc, ntgt - 1);
-        J[k] = s0 + (((at[k] & 63) << 1) | (at[k] >> 6));
-    }
-    dfl<L2> x[10], y[10];
-    near_diff<L2>(pa.recF, pa.recLo, I[0], I[1], J[0], J[1], x, y);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const unsigned live = __ballot_sync(0xffffffffu, on[k]);
+#pragma unroll 1
+    for (int base = 0; base < count; base += 32) {
+        bool on = base + lane < count;
+        const int v = sm.queue[wid][first + (on ? base + lane : 0)];
+        const int row = v >> 8, at = v & 0xff, loc = kSection * wid + row;
+        on = on && loc < ntgt;
+        dfl<float> x[10], y[10];
+        near_diff(pa.recF, pa.recLo, tgt0 + min(loc, ntgt - 1), s0 + (((at & 63) << 1) | (at >> 6)), x, y);
+        const unsigned live = __ballot_sync(0xffffffffu, on);
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
-            const int key = on[k] ? (side ? at[k] : row[k]) : 256 + lane;
+            const int key = on ? (side ? at : row) : 256 + lane;
             const unsigned same = __match_any_sync(0xffffffffu, key) & live;
             const int rank = __popc(same & ((1u << lane) - 1));
-            const int rounds = __reduce_max_sync(0xffffffffu, on[k] ? rank + 1 : 0);
+            const int rounds = __reduce_max_sync(0xffffffffu, on ? rank + 1 : 0);
             for (int r = 0; r < rounds; ++r) {
-                if (on[k] && rank == r) {
-                    float2 *ac = side ? &sm.sac[wid][0][at[k]] : &sm.tac[wid][0][row[k]];
+                if (on && rank == r) {
+                    float2 *ac = side ? &sm.sac[wid][0][at] : &sm.tac[wid][0][row];
 #pragma unroll
                     for (int q = 0; q < 10; ++q, ac += side ? kTile : kSection) {
-                        const dfl<L2> v = side ? y[q] : x[q];
+                        const dfl<float> v = side ? y[q] : x[q];
                         float2 t = *ac;
-                        l_kahan_df(t.x, t.y, k ? v.hi.y : v.hi.x, k ? v.lo.y : v.lo.x);
+                        l_kahan_df(t.x, t.y, v.hi, v.lo);
                         *ac = t;
                     }
                 }
@@ -511,16 +501,16 @@ static __device__ __noinline__ void sym_near_flush(SymSmem<PMIX, OP_DIFF> &sm, i
 // Staggered loop of one warp over sources [j0, j0 + cnt) of the staged tile (global rows s0 + j).
 // CHECK: some pair may share a vertex; MODE 2: near pairs possible, 1: double-float chords, 0: single-float
 // chords (far tiles).  OWN: the sources are the warp's own 64 rows; each unordered pair once, by the row that
-// sees the other at most half the circle of 64 ahead.
+// sees the other at most half the circle of 64 ahead.  Otherwise steps [first, last) of the circle (last < 0: all).
 template <int PREC, int OP, bool CHECK, int MODE, bool OWN>
 __device__ __forceinline__ void sym_section(const SymTgt &t, const SymTgtU *tu, SymSmem<PREC, OP> &sm, int wid, int s0,
                                             int j0, int cnt, SymAcc<PREC, OP> &a, int &queued, const WorkItem &w,
-                                            const SymArgs &pa)
+                                            const SymArgs &pa, int first = 0, int last = -1)
 {
     constexpr bool QUEUE = OP == OP_DIFF && MODE == 2;
     const int lane = threadIdx.x & 31;
-    const int P = OWN ? kSection : max((cnt + 1) & ~1, kSection), n = OWN ? kSection / 2 + 2 : P;
-    for (int step = OWN ? 1 : 0; step < n; ++step) {
+    const int P = OWN ? kSection : max((cnt + 1) & ~1, kSection), n = OWN ? kSection / 2 + 2 : (last < 0 ? P : last);
+    for (int step = OWN ? 1 : first; step < n; ++step) {
         int j = step + 2 * lane;
         if (j >= P) j -= P;
         const int at = sym_slot(j + j0);
@@ -703,14 +693,19 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
             }
             constexpr int MN = NEAR ? 2 : 1;
             if (diag) {
-                // the super-block's 64-row sections: a warp takes its own, and of the six pairs of sections one
-                // or two (odd warps also the section before theirs), at most 97 steps per tile
+                // the super-block's 64-row sections: in the tile of its own a warp takes those rows and half of the
+                // pairs with the tile's other section, in the other tile one whole section: 65 or 64 steps.  The pair
+                // of sections (even, odd) is cut where the even row 2 l sees sources 2 l to 2 l + 31 of the circle;
+                // the rest is steps 2 to 33 of the odd section against the even one.
                 if (have) {
                     const int sec = (s0 - w.tgt0) / kSection;
                     if ((wid & 2) == sec) {
                         sym_section<PREC, OP, true, MN, true>(t, tu, sm, wid, s0, kSection * (wid & 1),
                                                               min(kSection, w.ntgt - kSection * wid), a, queued, w, pa);
-                        if (wid & 1) sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, 0, kSection, a, queued, w, pa);
+                        const int o = (wid & 1) ^ 1, oc = min(kSection, w.ntgt - kSection * (wid ^ 1));
+                        if (oc > 0)
+                            sym_section<PREC, OP, true, MN, false>(t, tu, sm, wid, s0, kSection * o, oc, a, queued, w, pa,
+                                                                   o ? 0 : 2, o ? kSection / 2 : kSection / 2 + 2);
                     } else {
                         const int g = wid >= 2 ? wid - 2 : 3 - wid, gc = min(kSection, w.ntgt - kSection * g);
                         if (gc > 0)
@@ -855,31 +850,36 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
 
 // ---------------------------------------------------------------------------------- host side
 
-// Tiles per item: four (fewer partial slots, longer runs per target load) once every resident CTA gets about
-// six items that way, fewer on smaller graphs so that the last wave stays short.
-static int sym_tiles_per_item(const Ctx &c, int resident)
+// Source rows per item beyond the own super-block: four tiles (fewer partial slots, longer runs per target load) once
+// every resident CTA gets about six items that way, fewer on smaller graphs so that the last wave stays short, and
+// half a tile where even whole tiles would be fewer: an item among near pairs takes many times the others' time
+// (mixed, half / whole tiles: one knot of 4,096 edges differential 393 / 556 us, apply 103 / 107; 4 x 4,096 610 / 728 and
+// 282 / 319; 8 x 1,500 425 / 507 and 105 / 142; 96 x 500, where the super-blocks themselves hold the near pairs, 826 / 792
+// and 151 / 175).
+static int sym_item_span(const Ctx &c, int resident)
 {
     long long tiles = 0;
     for (int q = 0; q < c.nProb; ++q) {
         const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
         for (long long X = 0; X < ns; ++X) tiles += std::max(0LL, nb - 2 * X - 2);
     }
-    return (int)std::min<long long>(kSymMaxTiles, std::max<long long>(1, tiles / (6LL * std::max(1, resident))));
+    const long long per = tiles / (6LL * std::max(1, resident));
+    return per ? kTile * (int)std::min<long long>(kSymMaxTiles, per) : kTile / 2;
 }
 
-// Slots a row of super-block X of a problem with nb tiles has at tc tiles per item.
-static int sym_row_slots(int X, int nb, int tc)
+// Slots a row of super-block X of a problem with n rows has at `span` source rows per item.
+static int sym_row_slots(int X, int n, int span)
 {
-    const int m = std::max(0, nb - 2 * X - 2);
-    return X + std::min(3, nb - 2 * X + 1) + (m + tc - 1) / tc;
+    const int nb = (n + kTile - 1) / kTile, m = std::max(0, n - (X + 1) * kSuper);
+    return X + std::min(3, nb - 2 * X + 1) + (m + span - 1) / span;
 }
 
-static int sym_max_slots(const Ctx &c, int tc)
+static int sym_max_slots(const Ctx &c, int span)
 {
     int ms = 1;
     for (int q = 0; q < c.nProb; ++q) {
-        const int n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
-        for (int X = 0; X < ns; ++X) ms = std::max(ms, sym_row_slots(X, nb, tc));
+        const int n = c.h_prob_e[q + 1] - c.h_prob_e[q], ns = (n + kSuper - 1) / kSuper;
+        for (int X = 0; X < ns; ++X) ms = std::max(ms, sym_row_slots(X, n, span));
     }
     return ms;
 }
@@ -887,7 +887,7 @@ static int sym_max_slots(const Ctx &c, int tc)
 static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
 {
     const int resident = c.sm_count * std::max(1, occupancy);
-    const int tc = sym_tiles_per_item(c, resident);
+    const int span = sym_item_span(c, resident);
     // edges at every vertex, for the tiles that hold a neighbour of a super-block
     std::vector<int> ptr(c.nV + 1, 0), inc(2 * (size_t)c.nE);
     for (int k = 0; k < 2 * c.nE; ++k) ptr[c.h_edges[k] + 1]++;
@@ -919,14 +919,14 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
             int slot = X + 1;
             for (int h = t0; h < t0 + nt; h += kTile, ++slot)
                 tmp.push_back({WorkItem{t0, nt, h, std::min(h + kTile, t0 + nt), (X << 16) | slot, 3, 0, q}, 1 + kSymMaxTiles});
-            for (int cb = 2 * X + 2; cb < nb; cb += tc, ++slot) {
-                const int ce = std::min(nb, cb + tc);
+            for (int s0 = (X + 1) * kSuper; s0 < n; s0 += span, ++slot) {  // whole tiles, or half a tile
+                const int s1 = std::min(n, s0 + span);
                 int mask = 0;
-                for (int k = cb; k < ce; ++k) mask |= touch[k] << (k - cb);
-                tmp.push_back({WorkItem{t0, nt, e0 + cb * kTile, std::min(e1, e0 + ce * kTile), (X << 16) | slot, mask, 0, q},
-                               ce - cb + (mask ? kSymMaxTiles : 0)});
+                for (int k = s0; k < s1; k += kTile) mask |= touch[k / kTile] << ((k - s0) / kTile);
+                tmp.push_back({WorkItem{t0, nt, e0 + s0, e0 + s1, (X << 16) | slot, mask, 0, q},
+                               (s1 - s0 + kTile - 1) / kTile + (mask ? kSymMaxTiles : 0)});
             }
-            for (int I = t0; I < t0 + nt; ++I) eslots[I] = sym_row_slots(X, nb, tc);
+            for (int I = t0; I < t0 + nt; ++I) eslots[I] = sym_row_slots(X, n, span);
         }
     }
     std::stable_sort(tmp.begin(), tmp.end(), [](const Tmp &a, const Tmp &b) { return a.cost > b.cost; });
@@ -934,7 +934,7 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
     items.reserve(tmp.size());
     for (auto &t : tmp) items.push_back(t.w);
     pl.n_items = (int)items.size();
-    pl.max_slots = sym_max_slots(c, tc);
+    pl.max_slots = sym_max_slots(c, span);
     pl.grid = std::max(1, std::min(pl.n_items, resident));
     cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
     cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
@@ -989,8 +989,8 @@ static int sym_op_width(int op) { return op == OP_ENERGY ? 1 : (op == OP_DIFF ? 
 // Doubles of the partial buffer the symmetric pass of `op` needs.
 size_t sym_part_elems(const Ctx &c, int op, int variant)
 {
-    const int tc = sym_tiles_per_item(c, c.sm_count * std::max(1, sym_occupancy(c, op, variant)));
-    return (size_t)sym_max_slots(c, tc) * std::max(1, c.nE) * sym_op_width(op);
+    const int span = sym_item_span(c, c.sm_count * std::max(1, sym_occupancy(c, op, variant)));
+    return (size_t)sym_max_slots(c, span) * std::max(1, c.nE) * sym_op_width(op);
 }
 
 // Switch one pass to its symmetric form (variant > 0) or back to the gather form; grows the partial buffer.
@@ -1020,26 +1020,48 @@ cudaError_t sym_select(Ctx &c, int v) { return select_pass(c, OP_APPLY, v, 2, c.
 cudaError_t sym_select_energy(Ctx &c, int v) { return select_pass(c, OP_ENERGY, v, 2, c.plan_sym_e, c.energy_sym); }
 cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4, c.plan_sym_d, c.diff_sym); }
 
-// The passes a new context runs in symmetric form: those whose work list, one tile per item, gives every
-// resident CTA an item, while the partial sums stay below 1 GiB.  With fewer items the gather pass's short
-// chunks spread the work better (mixed precision, one knot, gather / symmetric: 1,000 edges energy 42 / 96 us,
-// differential 117 / 515 us; 4,096 edges 101 / 107 and 573 / 683; 8,192 edges 280 / 181 and 1,137 / 944;
-// 8 x 4,096 edges 488 / 322, differential 2,835 / 1,211, apply 956 / 553).
-cudaError_t sym_defaults(Ctx &c)
+// Whether a new context runs the pass of `op` in symmetric form: where a work list of whole tiles gives every
+// resident CTA an item, or (mixed precision) where the unordered pairs per SM reach 22,000, for the energy
+// 50,000; the partial sums stay below 1 GiB.  On smaller graphs the gather pass's short chunks spread the work better
+// and the symmetric pass waits for its longest item.  Gather / symmetric in us:
+//   edges      pairs/SM   differential    apply      energy
+//   2,000        13,000     268 / 320     50 / 55    47 / 64
+//   2,500        20,500     368 / 456     74 / 72    58 / 80
+//   3,000        29,600     448 / 414     96 / 72    67 / 81
+//   3,500        40,300     659 / 479    116 / 90    84 / 80
+//   4,096        55,200     589 / 402    123 / 104   96 / 90
+//   20 x 500     16,400     439 / 353     67 / 73    57 / 73
+//   12 x 1,000   39,400     550 / 398    114 / 91    89 / 100
+//   120 x 256    25,800     816 / 524     88 / 76    85 / 93
+static bool sym_pays(const Ctx &c, int op)
 {
-    if (!c.kp.fast || c.prm.precision == TP_FP64) return cudaSuccess;
+    if (!c.kp.fast || c.prm.precision == TP_FP64 || (op == OP_DIFF && c.prm.precision != TP_MIXED)) return false;
     long long items = 0;
+    double pairs = 0.0;
     for (int q = 0; q < c.nProb; ++q) {
         const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q], nb = (n + kTile - 1) / kTile, ns = (n + kSuper - 1) / kSuper;
         for (long long X = 0; X < ns; ++X) items += nb - 2 * X;
+        pairs += 0.5 * (double)n * (double)n;
     }
-    auto pays = [&](int op) {
-        return items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1)) &&
-               sym_part_elems(c, op, 1) * sizeof(double) <= (size_t)1 << 30;
-    };
-    if (pays(OP_ENERGY)) TPE_CHECK(sym_select_energy(c, 1));
-    if (c.prm.precision == TP_MIXED && pays(OP_DIFF)) TPE_CHECK(sym_select_diff(c, 1));
-    if (pays(OP_APPLY)) TPE_CHECK(sym_select(c, 1));
+    const bool fills = items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1)) ||
+                       (c.prm.precision == TP_MIXED && pairs >= (op == OP_ENERGY ? 50e3 : 22e3) * c.sm_count);
+    return fills && sym_part_elems(c, op, 1) * sizeof(double) <= (size_t)1 << 30;
+}
+
+// Doubles of the partial buffer a new context needs for them.
+size_t sym_default_elems(const Ctx &c)
+{
+    size_t need = 0;
+    for (int op : {OP_ENERGY, OP_DIFF, OP_APPLY})
+        if (sym_pays(c, op)) need = std::max(need, sym_part_elems(c, op, 1));
+    return need;
+}
+
+cudaError_t sym_defaults(Ctx &c)
+{
+    if (sym_pays(c, OP_ENERGY)) TPE_CHECK(sym_select_energy(c, 1));
+    if (sym_pays(c, OP_DIFF)) TPE_CHECK(sym_select_diff(c, 1));
+    if (sym_pays(c, OP_APPLY)) TPE_CHECK(sym_select(c, 1));
     return cudaSuccess;
 }
 

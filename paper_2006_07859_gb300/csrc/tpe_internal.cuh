@@ -254,6 +254,7 @@ cudaError_t sym_select_diff(Ctx &c, int variant);
 cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
 cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s);  // specialised powers; grows c.d_part
 cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: c.d_urecMF into c.d_esum2; grows c.d_part
+size_t sym_default_elems(const Ctx &c);
 cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 void make_plans(Ctx &c);

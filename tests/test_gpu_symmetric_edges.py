@@ -129,3 +129,26 @@ def test_accurate_apply_after_a_change_of_exponents(torch, orc):
         ref = orc.gram_apply(c.gamma, c.edges, orc.sigma_of(alpha, beta), u)
         assert rel(host(tpe.sobolev_apply_accurate(ctx, dev(c.gamma), dev(u))), ref) <= 1e-11
         assert rel(host(tpe.sobolev_apply(ctx, dev(c.gamma), dev(u))), ref) <= 1e-5
+
+
+# Both forms add the same FP32 pair terms (about 1e-6 of the largest entry each); a lost or doubled pair of the smallest
+# curves moves a row by 1e-2.
+@pytest.mark.parametrize("n,k", [(2600, 1), (300, 16), (65, 300), (3950, 1)])
+def test_new_context_between_the_passes(torch, n, k):
+    """Either side of the work from which a new context runs each pass in symmetric form, with half tiles per item
+    (152 SMs: 2,587 and 3,899 edges of one curve), against the gather form."""
+    from paper_2006_07859_gb300 import tpe
+    c = S.batch_of_knots([n] * k, 5, 31)
+    g, u = dev(c.gamma), dev(np.random.default_rng(5).normal(size=(c.n_vertices, 3)))
+    out = []
+    for gather in (False, True):
+        ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI, independent=1)
+        if gather:
+            tpe.tp_set_energy_variant(ctx, 0)
+            tpe.tp_set_diff_variant(ctx, 0)
+            tpe.tp_set_apply_variant(ctx, 0)
+        rows = torch.empty(c.n_edges, dtype=torch.float64, device="cuda")
+        tpe.tp_energy(ctx, g, rows=rows)
+        out.append([host(rows), host(tpe.tp_differential(ctx, g)), host(tpe.sobolev_apply(ctx, g, u))])
+    for new, old in zip(*out):
+        assert rel(new, old) <= 1e-5
