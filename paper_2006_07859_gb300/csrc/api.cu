@@ -398,6 +398,8 @@ tp_status tp_create(tp_ctx **out, int nV, int nE, const int32_t *edges_host, int
     CK(cudaMemcpy(c.d_inc_ptr, deg.data(), sizeof(int) * (nV + 1), cudaMemcpyHostToDevice));
     CK(dalloc(&c.d_inc, 2 * (size_t)nE));
     CK(cudaMemcpy(c.d_inc, inc.data(), sizeof(int) * 2 * nE, cudaMemcpyHostToDevice));
+    c.h_inc_ptr = std::move(deg);
+    c.h_inc = std::move(inc);
     CK(dalloc(&c.d_vprob, nV));
     CK(cudaMemcpy(c.d_vprob, vprob.data(), sizeof(int) * nV, cudaMemcpyHostToDevice));
     CK(dalloc(&c.d_eprob, nE));

@@ -80,52 +80,95 @@ __global__ void k_coarse_gram(int b, const CoarseCurve *__restrict__ cc, const d
         }
 }
 
-// symmetrise, Cholesky-factor and invert in place every curve's coarse matrix of at most 127 rows, in
-// shared memory (one block per curve; larger ones go to the tiled kernels of coarse_factor.cu);
-// Li: scratch of the same layout for L^-1
-__global__ void k_coarse_factor(const CoarseCurve *__restrict__ cc, double *__restrict__ L, double *__restrict__ Li)
+// Coarse matrices of at most 127 rows (larger ones go to the tiled kernels of coarse_factor.cu): symmetrise and
+// Cholesky-factor in shared memory, one block per curve; then L^-1, one warp per column, and (Z^T A Z)^-1 =
+// L^-T L^-1, one thread per entry, over the whole GPU.  FP64 instructions bound all three (64 cycles a warp): as one
+// kernel on one SM per curve the inverse and the product were two thirds of 1,190 us (8 curves, 127 rows), now
+// 248 + 58 + 21 us.
+// The factor leaves L^T in L (row k: column k of the factor) and 1 / L_kk on the diagonal of Li.
+__global__ void __launch_bounds__(256) k_coarse_factor(const CoarseCurve *__restrict__ cc, double *__restrict__ L,
+                                                       double *__restrict__ Li)
 {
     const CoarseCurve C = cc[blockIdx.x];
     const int mm = C.m - 1;
     if (mm > kSmemCoarse - 1) return;
     extern __shared__ double a[];  // [mm][mm] (dynamic shared memory)
-    double *g = L + C.aoff;
+    __shared__ double inv;
+    double *g = L + C.aoff, *li = Li + C.aoff;
     for (int t = threadIdx.x; t < mm * mm; t += blockDim.x) {
         int r = t / mm, col = t % mm;
         a[r * mm + col] = 0.5 * (g[r * mm + col] + g[col * mm + r]);
     }
-    __syncthreads();
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     for (int k = 0; k < mm; ++k) {
+        __syncthreads();  // the update of step k - 1 is complete
         if (threadIdx.x == 0) {
-            double d = a[k * mm + k];
-            a[k * mm + k] = d > 0.0 ? sqrt(d) : 1e-150;
+            const double d = a[k * mm + k];
+            inv = d > 0.0 ? rsqrt(d) : 1e150;
+            li[k * mm + k] = inv;
         }
         __syncthreads();
-        double dk = a[k * mm + k];
-        for (int r = k + 1 + threadIdx.x; r < mm; r += blockDim.x) a[r * mm + k] /= dk;
+        const double s = inv;
+        for (int r = k + 1 + threadIdx.x; r < mm; r += blockDim.x) a[r * mm + k] *= s;
         __syncthreads();
-        for (int t = threadIdx.x; t < (mm - k - 1) * (mm - k - 1); t += blockDim.x) {
-            int r = k + 1 + t / (mm - k - 1), col = k + 1 + t % (mm - k - 1);
-            if (col <= r) a[r * mm + col] -= a[r * mm + k] * a[col * mm + k];
-        }
-        __syncthreads();
-    }
-    // L^-1 by forward substitution, one column per thread, then (Z^T A Z)^-1 = L^-T L^-1
-    double *li = Li + C.aoff;
-    for (int col = threadIdx.x; col < mm; col += blockDim.x) {
-        for (int r = 0; r < mm; ++r) {
-            double v = (r == col) ? 1.0 : 0.0;
-            for (int k = col; k < r; ++k) v -= a[r * mm + k] * li[k * mm + col];
-            li[r * mm + col] = r < col ? 0.0 : v / a[r * mm + r];
+        for (int r = k + 1 + ty; r < mm; r += 16) {
+            const double x = a[r * mm + k];
+            for (int col = k + 1 + tx; col <= r; col += 16) a[r * mm + col] -= x * a[col * mm + k];
         }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < mm * mm; t += blockDim.x) {
-        const int r = t / mm, col = t % mm;
-        double v = 0.0;
-        for (int k = max(r, col); k < mm; ++k) v += li[k * mm + r] * li[k * mm + col];
-        g[t] = v;
+        const int k = t / mm, r = t % mm;
+        if (r > k) g[t] = a[r * mm + k];
     }
+}
+
+constexpr int kInvCols = 4;
+__global__ void __launch_bounds__(32 * kInvCols) k_coarse_inverse(const CoarseCurve *__restrict__ cc,
+                                                                  const double *__restrict__ Lt, double *__restrict__ Li)
+{
+    const CoarseCurve C = cc[blockIdx.y];
+    const int mm = C.m - 1, lane = threadIdx.x & 31, col = blockIdx.x * kInvCols + (threadIdx.x >> 5);
+    if (mm > kSmemCoarse - 1 || col >= mm) return;
+    const double *lt = Lt + C.aoff;
+    double *li = Li + C.aoff;
+    double v[4];  // rows lane + 32 i of the right-hand side, then of the solution
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = lane + 32 * i == col ? 1.0 : 0.0;
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb) {
+        const int k0 = max(32 * kb, col), k1 = min(32 * kb + 32, mm);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const double x = __shfl_sync(0xffffffffu, v[kb], k & 31) * li[k * mm + k];
+            if (lane == (k & 31)) v[kb] = x;
+#pragma unroll
+            for (int i = kb; i < 4; ++i) {
+                const int r = lane + 32 * i;
+                if (r > k && r < mm) v[i] -= lt[k * mm + r] * x;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = lane + 32 * i;
+        if (r > col && r < mm) li[r * mm + col] = v[i];  // the diagonal is there already
+    }
+}
+
+constexpr int kGramTile = 16;
+__global__ void __launch_bounds__(kGramTile *kGramTile) k_coarse_product(const CoarseCurve *__restrict__ cc,
+                                                                         const double *__restrict__ Li, double *__restrict__ out)
+{
+    const CoarseCurve C = cc[blockIdx.z];
+    const int mm = C.m - 1, r = blockIdx.y * kGramTile + threadIdx.x / kGramTile, col = blockIdx.x * kGramTile + threadIdx.x % kGramTile;
+    if (mm > kSmemCoarse - 1 || r >= mm || col > r) return;  // the lower triangle; the other half is its mirror image
+    const double *li = Li + C.aoff;
+    double s = 0.0;
+#pragma unroll 4
+    for (int k = r; k < mm; ++k) s += li[k * mm + r] * li[k * mm + col];
+    out[C.aoff + (long long)r * mm + col] = s;
+    out[C.aoff + (long long)col * mm + r] = s;
 }
 
 // w[j][q] = Z_j^T r: one block per (curve, j), of one warp for hats of up to kRestrictWarp vertices and of four
@@ -228,8 +271,8 @@ __global__ void k_az_store(int nV, int b, const CoarseCurve *__restrict__ cc, co
 // consecutive vertices read consecutive addresses of a column).  A block serves 32 vertices and its warps split
 // the columns: FP64 FMAs bound the pass (64 cycles a warp instruction), and a warp with every column of its 32
 // vertices would leave the 608 schedulers one or two warps each; with a quarter of the columns per warp the work
-// spreads evenly and four times the loads are in flight.  8 curves of 4,096, 128 hats: 26 us (the
-// FMAs alone take 21), with a thread per vertex 40.
+// spreads evenly and four times the loads are in flight.  8 curves of 4,096, 128 hats: 32 us (the
+// FMAs alone take 21), before 45 (40 with only a deeper unroll).
 constexpr int kAzChunk = 512, kAzWarps = 4;
 __global__ void __launch_bounds__(32 * kAzWarps) k_az_prolong_sub(int nV, const CoarseCurve *__restrict__ cc,
                                                                   const int *__restrict__ vcurve, const double *__restrict__ AZ,
@@ -468,7 +511,10 @@ cudaError_t coarse_setup(Ctx &c, const double *gamma_geom, int which, cudaStream
     }
     const int msm = std::min(S.max_m, kSmemCoarse) - 1;
     k_coarse_factor<<<c.nCurves, 256, (size_t)msm * msm * sizeof(double), s>>>(S.d_curves, S.d_L, S.d_Li);
-    c.launches++;
+    k_coarse_inverse<<<dim3((msm + kInvCols - 1) / kInvCols, c.nCurves), 32 * kInvCols, 0, s>>>(S.d_curves, S.d_L, S.d_Li);
+    const int gt = (msm + kGramTile - 1) / kGramTile;
+    k_coarse_product<<<dim3(gt, gt, c.nCurves), kGramTile * kGramTile, 0, s>>>(S.d_curves, S.d_Li, S.d_L);
+    c.launches += 3;
     for (const CoarseCurve &C : S.curves)
         if (C.m - 1 > kSmemCoarse - 1)
             TPE_CHECK(coarse_factor_tiled(c, C.m - 1, S.d_L + C.aoff, S.d_W + C.aoff, S.d_Li + C.aoff, s));

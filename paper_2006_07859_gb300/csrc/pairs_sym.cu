@@ -888,13 +888,7 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
 {
     const int resident = c.sm_count * std::max(1, occupancy);
     const int span = sym_item_span(c, resident);
-    // edges at every vertex, for the tiles that hold a neighbour of a super-block
-    std::vector<int> ptr(c.nV + 1, 0), inc(2 * (size_t)c.nE);
-    for (int k = 0; k < 2 * c.nE; ++k) ptr[c.h_edges[k] + 1]++;
-    for (int v = 0; v < c.nV; ++v) ptr[v + 1] += ptr[v];
-    std::vector<int> fill(ptr.begin(), ptr.end() - 1);
-    for (int I = 0; I < c.nE; ++I)
-        for (int s = 0; s < 2; ++s) inc[fill[c.h_edges[2 * I + s]]++] = I;
+    const std::vector<int> &ptr = c.h_inc_ptr, &inc = c.h_inc;  // (edge, end) pairs at every vertex
     struct Tmp {
         WorkItem w;
         int cost;
@@ -912,8 +906,10 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
             for (int I = t0; I < t0 + nt; ++I)
                 for (int s = 0; s < 2; ++s) {
                     const int v = c.h_edges[2 * I + s];
-                    for (int k = ptr[v]; k < ptr[v + 1]; ++k)
-                        if (inc[k] >= e0 && inc[k] < e1) touch[(inc[k] - e0) / kTile] = 1;
+                    for (int k = ptr[v]; k < ptr[v + 1]; ++k) {
+                        const int J = inc[k] >> 1;
+                        if (J >= e0 && J < e1) touch[(J - e0) / kTile] = 1;
+                    }
                 }
             // tiles with near pairs take longer: they and the super-block itself go first
             int slot = X + 1;
@@ -926,7 +922,7 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
                 tmp.push_back({WorkItem{t0, nt, e0 + s0, e0 + s1, (X << 16) | slot, mask, 0, q},
                                (s1 - s0 + kTile - 1) / kTile + (mask ? kSymMaxTiles : 0)});
             }
-            for (int I = t0; I < t0 + nt; ++I) eslots[I] = sym_row_slots(X, n, span);
+            std::fill_n(eslots.begin() + t0, nt, sym_row_slots(X, n, span));
         }
     }
     std::stable_sort(tmp.begin(), tmp.end(), [](const Tmp &a, const Tmp &b) { return a.cost > b.cost; });

@@ -102,6 +102,7 @@ struct Ctx {
     tp_params prm{};
     KernelParams kp{};
     std::vector<int32_t> h_edges, h_voff, h_eoff;
+    std::vector<int> h_inc_ptr, h_inc;  // per vertex: 2 * edge + end
     std::vector<int32_t> h_prob_v, h_prob_e;  // per-problem vertex / edge offsets [nProb + 1]
     int32_t *d_edges = nullptr;                // [nE][2]
     int32_t *d_inc_ptr = nullptr;              // [nV + 1] incidence CSR
