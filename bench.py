@@ -3,7 +3,7 @@
 
 Workload (default): one closed random Fourier knot with 16 harmonics and 262,144 vertices (262,144
 edges, coefficients N(0, 1/k^2), seed 100), (alpha, beta) = (2, 4.5), barycenter + total-length
-constraints, mixed precision (FP32 pair arithmetic on double-float positions, FP64 near pairs and
+constraints, mixed precision (FP32 pair arithmetic on double-float positions, double-float near pairs, FP64
 reductions), the balancing two-level preconditioner with 8,192 coarse hats, and the constrained
 gradient solved to a TRUE relative residual of 1e-4 (certified by the double-float apply, with residual
 refinement; at this size the FP64-class evaluation floor of the operator is ~2e-5, so 1e-6 is out of
@@ -45,7 +45,17 @@ import numpy as np  # noqa: E402
 FLOP_PER_PAIR = {"energy": 122, "diff": 320, "apply": 255}
 # multi-field apply: the apply's weights (220) once per ordered pair plus 35 / 3 per scalar column, 12 columns
 MULTI_COLS = 12
-FLOP_PER_PAIR["apply_multi"] = 220 + 35 * MULTI_COLS // 3
+
+
+def multi_cols(tuned):
+    """Scalar columns of one multi-field launch: two fields on the symmetric apply, else four."""
+    return MULTI_COLS // 2 if tuned["tpt"].get("apply_symmetric") else MULTI_COLS
+
+
+def flop_per_pair(op, cols=MULTI_COLS):
+    return 220 + 35 * cols // 3 if op == "apply_multi" else FLOP_PER_PAIR[op]
+
+
 MUFU_PER_PAIR = {"energy": 8, "diff": 8, "apply": 8}
 FP32_LANES = 128   # FP32 FMA lanes per SM (Blackwell)
 L2_BYTES = 129 * 2 ** 20
@@ -342,13 +352,14 @@ def pass_throughput_262k(tpe, torch):
     torch.cuda.synchronize()
     pairs = ctx.pairs_per_pass()
     out = {"pairs_per_pass": pairs, "autotune": tuned["tpt"], "autotune_ms": tuned["ms"]}
+    cols = multi_cols(tuned)
     for i, op in [(0, "energy"), (1, "diff"), (2, "apply"), (7, "apply_multi")]:
         ms, n = ctx.profile_read(i)
         out[op] = {"pairs_per_s": pairs * n / (ms / 1e3), "ms_per_launch": ms / n,
-                   "tflops": pairs * FLOP_PER_PAIR[op] * n / (ms / 1e3) / 1e12}
-    # scalar columns served per second: 3 per apply pass, 12 per multi-field pass
+                   "tflops": pairs * flop_per_pair(op, cols) * n / (ms / 1e3) / 1e12}
+    # scalar columns served per second: 3 per apply pass, 6 or 12 per multi-field pass
     out["columns_x_pairs_per_s"] = {"apply": 3 * out["apply"]["pairs_per_s"],
-                                    "apply_multi": MULTI_COLS * out["apply_multi"]["pairs_per_s"]}
+                                    "apply_multi": cols * out["apply_multi"]["pairs_per_s"]}
     ctx.profile(False)
     ctx.close()
     return out
@@ -787,7 +798,8 @@ def run_ours(args, rank, world, local_rank):
     passes["apply"] += prof["apply_cg"][1] / args.steps   # every apply launch (the CG ones may skip converged curves)
     passes["apply_accurate"] = prof["apply_accurate"][1] / args.steps
     passes["coarse_az"] = prof["coarse_az"][1] / args.steps
-    passes["apply_multi"] = prof["apply_multi"][1] / args.steps
+    # in units of the oracle's 12-column applies
+    passes["apply_multi"] = prof["apply_multi"][1] / args.steps * multi_cols(tuned) / MULTI_COLS
     pps = {k: (pairs * prof[k][1] / (prof[k][0] / 1e3) if prof[k][1] else None) for k in prof}
     if not single:
         pps["apply_cg"] = None   # CG applies skip converged problems: their pair count is not a full pass
@@ -807,7 +819,7 @@ def run_ours(args, rank, world, local_rank):
     kernel_share = {k: prof[k][0] / 1e3 / total for k in prof}
     sym_apply = tuned["tpt"].get("apply_symmetric", 0)
     apply_variant = ("symmetric", sym_apply) if sym_apply else ("gather", tuned["tpt"]["apply"])
-    apply_kernel = (f"k_pairs_sym<TPT={sym_apply}> (symmetric Sobolev apply)" if sym_apply
+    apply_kernel = (f"k_sym<PMIX, OP_APPLY, {4 - sym_apply} CTAs per SM> (symmetric Sobolev apply)" if sym_apply
                     else f"k_pairs<PMIX, OP_APPLY, TPT={tuned['tpt']['apply']}> (Sobolev apply)")
     line = {
         "metric": "H^s descent steps/s at 262K edges; pair interactions/s vs FP32 roofline", "value": value,

@@ -1039,8 +1039,9 @@ static bool sym_pays(const Ctx &c, int op)
         for (long long X = 0; X < ns; ++X) items += nb - 2 * X;
         pairs += 0.5 * (double)n * (double)n;
     }
-    const bool fills = items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1)) ||
-                       (c.prm.precision == TP_MIXED && pairs >= (op == OP_ENERGY ? 50e3 : 22e3) * c.sm_count);
+    const bool enough = c.prm.precision == TP_MIXED && pairs >= (op == OP_ENERGY ? 50e3 : 22e3) * c.sm_count;
+    if (!enough && items < c.sm_count) return false;  // no need to load the kernel for its occupancy
+    const bool fills = enough || items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1));
     return fills && sym_part_elems(c, op, 1) * sizeof(double) <= (size_t)1 << 30;
 }
 
