@@ -59,13 +59,13 @@ def flop_per_pair(op, cols=MULTI_COLS):
 MUFU_PER_PAIR = {"energy": 8, "diff": 8, "apply": 8}
 FP32_LANES = 128   # FP32 FMA lanes per SM (Blackwell)
 L2_BYTES = 129 * 2 ** 20
-# DRAM bytes (read + write) of one apply launch on the 8 x 4096 workload, by (pass, targets per thread),
+# DRAM bytes (read + write) of one apply launch on the 8 x 4096 workload, by (pass, variant),
 # from ncu captures of the current kernels (the profiles/ summaries named beside them); others: unknown
 APPLY_TRAFFIC_BYTES = {("knots8x4096", "gather", 2): 5.07e6,                   # apply_pair_kernel_knots8x4096.md
-                      ("knots8x4096", "symmetric", 1): 5.162240e6 + 0.249344e6,  # apply_symmetric_kernel_knots8x4096.md
+                      ("knots8x4096", "symmetric", 1): 13.79e6,  # apply_symmetric_kernel_knots8x4096.md
                       # captured at 65,536 edges and scaled by the pairs (x16):
                       # apply_symmetric_kernel_traffic_knot65536.md
-                      ("knot262144", "symmetric", 1): 16.0 * (19161856 + 1550644736)}
+                      ("knot262144", "symmetric", 1): 16.0 * (15163648 + 551113216)}
 
 
 def parse():
