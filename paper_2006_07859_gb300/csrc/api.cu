@@ -431,11 +431,9 @@ tp_status tp_create(tp_ctx **out, int nV, int nE, const int32_t *edges_host, int
     CK(dalloc(&c.d_counter, 16));
     CK(cudaMemset(c.d_counter, 0, sizeof(int) * 16));
     set_kernel_params(c);
-    make_plans(c);
-    CK(cudaGetLastError());
+    CK(make_plans(c));
     int ms = std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots);
-    c.part_elems = std::max((size_t)ms * std::max(1, nE) * 6, sym_default_elems(c));
-    CK(dalloc(&c.d_part, c.part_elems));
+    CK(part_reserve(c, std::max((size_t)ms * std::max(1, nE) * 6, sym_default_elems(c))));
     CK(sym_defaults(c));
     CK(dalloc(&c.d_rows, nE));
     CK(dalloc(&c.d_esum, 6 * (size_t)nE));
@@ -1428,9 +1426,9 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
     };
     cudaError_t err = cudaSuccess;
     if (c.prm.precision == TP_MIXED && c.kp.fast) {  // the gather passes are timed first
-        CK(sym_select(c, 0));
-        CK(sym_select_energy(c, 0));
-        CK(sym_select_diff(c, 0));
+        err = sym_select(c, 0);
+        if (err == cudaSuccess) err = sym_select_energy(c, 0);
+        if (err == cudaSuccess) err = sym_select_diff(c, 0);
     }
     // a symmetric variant is a candidate while its partial sums fit in 32 GB and in half the free memory
     // (on top of what the partial buffer already holds); the buffer is shrunk to the winners' need below
@@ -1550,11 +1548,8 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (c.energy_sym) need = std::max(need, sym_part_elems(c, OP_ENERGY, c.energy_sym));
         if (c.diff_sym) need = std::max(need, sym_part_elems(c, OP_DIFF, c.diff_sym));
         if (need < c.part_elems) {
-            graphs_reset(c);  // captured blocks hold the old buffer's address
             CK(cudaStreamSynchronize(s));
-            CK(cudaFree(c.d_part));
-            CK(cudaMalloc(&c.d_part, sizeof(double) * need));
-            c.part_elems = need;
+            CK(part_resize(c, need));
         }
     }
     return check_err_word(ctx, s);

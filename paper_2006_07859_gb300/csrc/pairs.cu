@@ -484,11 +484,62 @@ cudaError_t vertices_apply(Ctx &c, const double *esum, double *Au, cudaStream_t 
 
 // ---------------------------------------------------------------------------------- planning
 
+// Resize the buffer of partial sums.  The old one is freed first (on the longest curves both would not fit), so a
+// failed allocation takes the old size back, or holds nothing where even that is gone: part_elems is always
+// what d_part holds, and every pass reserves what it writes before it launches.
+cudaError_t part_resize(Ctx &c, size_t elems)
+{
+    if (c.capturing) return cudaErrorStreamCaptureUnsupported;  // a captured pass reserved its part before
+    graphs_reset(c);  // captured blocks hold the old buffer
+    TPE_CHECK(cudaFree(c.d_part));
+    const size_t old = c.part_elems;
+    c.d_part = nullptr;
+    c.part_elems = 0;
+    cudaError_t e = cudaMalloc(&c.d_part, sizeof(double) * elems);
+    if (e == cudaSuccess) {
+        c.part_elems = elems;
+        return e;
+    }
+    cudaGetLastError();  // reported by the return value
+    c.d_part = nullptr;
+    if (old && old < elems && cudaMalloc(&c.d_part, sizeof(double) * old) == cudaSuccess) {
+        c.part_elems = old;
+    } else {
+        c.d_part = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+
+cudaError_t part_reserve(Ctx &c, size_t elems) { return elems <= c.part_elems ? cudaSuccess : part_resize(c, elems); }
+
+void plan_free(Ctx::Plan &pl)
+{
+    if (pl.d_items) cudaFree(pl.d_items);
+    if (pl.d_eslots) cudaFree(pl.d_eslots);
+    pl = Ctx::Plan{};
+}
+
+// Copy a work list to the device; on failure the plan is empty (d_items NULL).
+cudaError_t plan_upload(Ctx::Plan &pl, const std::vector<WorkItem> &items, const std::vector<int> &eslots)
+{
+    const size_t ni = items.size(), ns = eslots.size();
+    cudaError_t e = cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, ni));
+    if (e == cudaSuccess) e = cudaMalloc(&pl.d_eslots, sizeof(int) * std::max<size_t>(1, ns));
+    if (e == cudaSuccess) e = cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * ni, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * ns, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        plan_free(pl);
+    }
+    return e;
+}
+
 constexpr int kMinChunk = 4;  // sources of the shortest item
 
 // Build the (target block, source chunk) queue of one pass.  Items of big problems come first
 // so the persistent grid ends with the small ones.
-void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
+cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
 {
     const int tb = kThreads * tpt;
     std::vector<WorkItem> items;
@@ -566,10 +617,7 @@ void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
     pl.max_slots = max_slots;
     pl.tpt = tpt;
     pl.grid = std::max(1, std::min(pl.n_items, c.sm_count * std::max(1, occupancy)));
-    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
-    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
-    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
-    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * c.nE, cudaMemcpyHostToDevice);
+    return plan_upload(pl, items, eslots);
 }
 
 constexpr int kTptEnergy = 4, kTptDiff = 2, kTptApply = 2;
@@ -710,32 +758,27 @@ static int occupancy_cls(const Ctx &c, int cls, int tpt)
 
 static Ctx::Plan &plan_of(Ctx &c, int cls) { return cls == 0 ? c.plan_energy : (cls == 1 ? c.plan_diff : c.plan_apply); }
 
-void make_plans(Ctx &c)
+cudaError_t make_plans(Ctx &c)
 {
     // Every slot of an op class shares one layout, so all passes of an op class use the same
     // targets-per-thread (the plan records it and the launch follows the plan).
     for (int cls = 0; cls < 3; ++cls) {
         const int t = tpt_for(c, cls);
-        plan_pass(c, plan_of(c, cls), t, occupancy_cls(c, cls, t));
+        TPE_CHECK(plan_pass(c, plan_of(c, cls), t, occupancy_cls(c, cls, t)));
     }
+    return cudaSuccess;
 }
 
 cudaError_t replan(Ctx &c, int cls)
 {
     graphs_reset(c);
-    Ctx::Plan &pl = plan_of(c, cls);
-    if (pl.d_items) TPE_CHECK(cudaFree(pl.d_items));
-    if (pl.d_eslots) TPE_CHECK(cudaFree(pl.d_eslots));
-    pl = Ctx::Plan{};
+    Ctx::Plan pl;
     const int t = tpt_for(c, cls);
-    plan_pass(c, pl, t, occupancy_cls(c, cls, t));
+    TPE_CHECK(plan_pass(c, pl, t, occupancy_cls(c, cls, t)));  // the old plan stays on failure
+    plan_free(plan_of(c, cls));
+    plan_of(c, cls) = pl;
     const int ms = std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots);
-    const size_t need = (size_t)ms * std::max(1, c.nE) * 6;
-    if (need > c.part_elems) {
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
-    }
+    TPE_CHECK(part_reserve(c, (size_t)ms * std::max(1, c.nE) * 6));
     return cudaGetLastError();
 }
 
@@ -909,6 +952,7 @@ static cudaError_t run_pairs(Ctx &c, int which, const double *gamma, const doubl
 {
     Ctx::Plan &pl = (OP == OP_ENERGY) ? c.plan_energy : (OP == OP_DIFF ? c.plan_diff : c.plan_apply);
     if (pl.n_items == 0) return cudaSuccess;
+    TPE_CHECK(part_reserve(c, (size_t)pl.max_slots * c.nE * 6));
     if (!tunable(c) && pl.tpt != 1 && pl.tpt != tpt_default(c, op_class(OP))) return cudaErrorInvalidValue;  // no such kernel
     constexpr int ctr = OP;
     PairArgs pa;

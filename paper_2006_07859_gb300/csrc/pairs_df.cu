@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_apply_df_general(const DfArgs a
 }
 
 // Edge blocks of 128 per problem; items (b, c >= b) sorted by problem size (large first).
-static void plan_items(Ctx &c, Ctx::Plan &pl, int occupancy)
+static cudaError_t plan_items(Ctx &c, Ctx::Plan &pl, int occupancy)
 {
     const int tb = kThreads;
     std::vector<std::pair<long long, WorkItem>> tmp;
@@ -257,10 +257,7 @@ static void plan_items(Ctx &c, Ctx::Plan &pl, int occupancy)
     pl.max_slots = max_slots;
     pl.tpt = 1;
     pl.grid = std::max(1, std::min(pl.n_items, c.sm_count * std::max(1, occupancy)));
-    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
-    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
-    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
-    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
+    return plan_upload(pl, items, eslots);
 }
 
 static int df_occupancy()
@@ -277,25 +274,14 @@ cudaError_t pair_apply_acc(Ctx &c, const double *gamma_geom, int which, const do
 {
     if (c.prm.precision == TP_FP64) return pair_apply(c, gamma_geom, which, u, Au, s);
     Ctx::Plan &pl = c.plan_df;
-    if (pl.d_items && (pl.tpt == 1) == (c.kp.fast != 0)) {  // the exponents changed since the last call
-        TPE_CHECK(cudaFree(pl.d_items));
-        TPE_CHECK(cudaFree(pl.d_eslots));
-        pl = Ctx::Plan{};
-    }
+    if (pl.d_items && (pl.tpt == 1) == (c.kp.fast != 0)) plan_free(pl);  // the exponents changed since the last call
     TPE_CHECK(build_urecs(c, u, which, s));
     if (c.kp.fast) {
         TPE_CHECK(sym_apply_accurate_pass(c, which, s));
         return vertices_apply(c, c.d_esum, Au, s);
     }
-    if (!pl.d_items) plan_items(c, pl, df_occupancy());
-    // the buffer is shared with the other passes and may have been resized since the last call
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * 6;
-    if (need > c.part_elems) {
-        graphs_reset(c);  // captured blocks hold the old partial buffer
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
-    }
+    if (!pl.d_items) TPE_CHECK(plan_items(c, pl, df_occupancy()));
+    TPE_CHECK(part_reserve(c, (size_t)pl.max_slots * std::max(1, c.nE) * 6));
     if (pl.n_items == 0) return cudaMemsetAsync(Au, 0, sizeof(double) * 3 * c.nV, s);
     TPE_CHECK(cudaMemsetAsync(c.d_counter + 9, 0, sizeof(int), s));
     DfArgs a;

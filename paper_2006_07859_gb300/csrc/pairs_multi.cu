@@ -211,11 +211,11 @@ static cudaError_t multi_init(Ctx &c)
     case TP_MIXED: occ = f ? multi_occupancy<PMIX, true>() : multi_occupancy<PMIX, false>(); break;
     default: occ = f ? multi_occupancy<P32, true>() : multi_occupancy<P32, false>(); break;
     }
-    plan_pass(c, c.plan_multi, 1, occ);
+    if (!c.plan_multi.d_items) TPE_CHECK(plan_pass(c, c.plan_multi, 1, occ));
     const size_t ne = (size_t)std::max(1, c.nE);
-    if (c.prm.precision == TP_FP64)
+    if (c.prm.precision == TP_FP64 && !c.d_urecMD)
         TPE_CHECK(cudaMalloc(&c.d_urecMD, sizeof(URecD) * kMultiG * ne));
-    else if (!c.d_urecMF)
+    if (c.prm.precision != TP_FP64 && !c.d_urecMF)
         TPE_CHECK(cudaMalloc(&c.d_urecMF, sizeof(URecF) * kMultiG * ne));
     TPE_CHECK(cudaMalloc(&c.d_partM, sizeof(double) * (size_t)c.plan_multi.max_slots * ne * 6 * kMultiG));
     c.multi_ready = 1;

@@ -884,7 +884,7 @@ static int sym_max_slots(const Ctx &c, int span)
     return ms;
 }
 
-static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
+static cudaError_t sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
 {
     const int resident = c.sm_count * std::max(1, occupancy);
     const int span = sym_item_span(c, resident);
@@ -932,10 +932,7 @@ static void sym_plan(Ctx &c, Ctx::Plan &pl, int occupancy)
     pl.n_items = (int)items.size();
     pl.max_slots = sym_max_slots(c, span);
     pl.grid = std::max(1, std::min(pl.n_items, resident));
-    cudaMalloc(&pl.d_items, sizeof(WorkItem) * std::max<size_t>(1, items.size()));
-    cudaMemcpy(pl.d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice);
-    cudaMalloc(&pl.d_eslots, sizeof(int) * std::max(1, c.nE));
-    cudaMemcpy(pl.d_eslots, eslots.data(), sizeof(int) * std::max(1, c.nE), cudaMemcpyHostToDevice);
+    return plan_upload(pl, items, eslots);
 }
 
 constexpr int kSymAccurate = 100;  // the apply in double-float
@@ -989,24 +986,28 @@ size_t sym_part_elems(const Ctx &c, int op, int variant)
     return (size_t)sym_max_slots(c, span) * std::max(1, c.nE) * sym_op_width(op);
 }
 
-// Switch one pass to its symmetric form (variant > 0) or back to the gather form; grows the partial buffer.
+// Doubles of partial sums the pass of a built plan writes.
+static size_t plan_elems(const Ctx &c, const Ctx::Plan &pl, int op)
+{
+    return (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(op);
+}
+
+// Switch one pass to its symmetric form (variant > 0) or back to the gather form; grows the partial buffer.  On
+// failure the pass runs in gather form.
 static cudaError_t select_pass(Ctx &c, int op, int variant, int max_variant, Ctx::Plan &pl, int &flag)
 {
     graphs_reset(c);
-    if (pl.d_items) TPE_CHECK(cudaFree(pl.d_items));
-    if (pl.d_eslots) TPE_CHECK(cudaFree(pl.d_eslots));
-    pl = Ctx::Plan{};
+    plan_free(pl);
     flag = 0;
     if (variant <= 0) return cudaSuccess;
     if (!c.kp.fast || variant > max_variant) return cudaErrorInvalidValue;
     if (c.prm.precision != TP_MIXED && !(c.prm.precision == TP_FP32 && op != OP_DIFF)) return cudaErrorInvalidValue;
-    sym_plan(c, pl, sym_occupancy(c, op, variant));
+    TPE_CHECK(sym_plan(c, pl, sym_occupancy(c, op, variant)));
     pl.tpt = variant;
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(op);
-    if (need > c.part_elems) {
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
+    const cudaError_t e = part_reserve(c, plan_elems(c, pl, op));
+    if (e != cudaSuccess) {
+        plan_free(pl);
+        return e;
     }
     flag = variant;
     return cudaGetLastError();
@@ -1068,6 +1069,8 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
                             cudaStream_t s)
 {
     if (pl.n_items == 0) return cudaSuccess;  // no edges: nothing reads the sums
+    // the buffer is shared with the other passes and may have been resized since the last call
+    TPE_CHECK(part_reserve(c, plan_elems(c, pl, op)));
     SymArgs pa;
     pa.items = pl.d_items;
     pa.n_items = pl.n_items;
@@ -1119,16 +1122,8 @@ static cudaError_t lazy_pass(Ctx &c, int op, Ctx::Plan &pl, int variant, int cou
                              double *out, cudaStream_t s)
 {
     if (!pl.d_items) {
-        sym_plan(c, pl, sym_occupancy(c, op, variant));
+        TPE_CHECK(sym_plan(c, pl, sym_occupancy(c, op, variant)));
         pl.tpt = variant;
-    }
-    // the buffer is shared with the other passes and may have been resized since the last call
-    const size_t need = (size_t)pl.max_slots * std::max(1, c.nE) * sym_op_width(op);
-    if (need > c.part_elems) {
-        graphs_reset(c);  // captured blocks hold the old partial buffer
-        TPE_CHECK(cudaFree(c.d_part));
-        TPE_CHECK(cudaMalloc(&c.d_part, sizeof(double) * need));
-        c.part_elems = need;
     }
     return sym_pass(c, op, pl, counter, prof_op, which, skip, out, s);
 }

@@ -154,7 +154,7 @@ struct Ctx {
     double extent = 0.0;  // bounding-box diagonal of the first curve seen
     URecF *d_urecF = nullptr;
     URecD *d_urecD = nullptr;
-    // partial results [max_slots][nE][6] (FP64)
+    // partial results [max_slots][nE][6] (FP64); part_elems doubles, changed by part_resize alone
     double *d_part = nullptr;
     size_t part_elems = 0;
     double *d_rows = nullptr;  // [nE]
@@ -242,7 +242,11 @@ constexpr int kMultiG = 4;
 cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const double *U, double *AU, int m,
                              cudaStream_t s);
 void multi_free(Ctx &c);
-void plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
+cudaError_t part_resize(Ctx &c, size_t elems);
+cudaError_t part_reserve(Ctx &c, size_t elems);
+void plan_free(Ctx::Plan &pl);
+cudaError_t plan_upload(Ctx::Plan &pl, const std::vector<WorkItem> &items, const std::vector<int> &eslots);
+cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
 cudaError_t gather_apply(Ctx &c, const Ctx::Plan &pl, double *Au, cudaStream_t s);
 cudaError_t vertices_apply(Ctx &c, const double *esum, double *Au, cudaStream_t s);  // from per-edge sums
 // symmetric passes (pairs_sym.cu): a variant > 0 or the gather pass (0); the passes write the energy rows
@@ -258,7 +262,7 @@ cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: 
 size_t sym_default_elems(const Ctx &c);
 cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
-void make_plans(Ctx &c);
+cudaError_t make_plans(Ctx &c);
 cudaError_t replan(Ctx &c, int cls);  // rebuild the plan of one op class (0 energy, 1 diff, 2 apply/diag)
 int tpt_default(const Ctx &c, int cls);
 int tpt_candidates(const Ctx &c, int cls, int *out);  // the autotuner's search space; returns the count

@@ -1,0 +1,47 @@
+"""The buffer of partial sums that all pair passes of a context share: passes whose buffer cannot be had are refused
+and leave the context as it was."""
+import numpy as np
+import pytest
+
+import synth as S
+from tests.gpu_util import dev, host, make_ctx, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    return need_gpu()
+
+
+def _knot_among_polygons(n, k, m=256):
+    """One Fourier knot of n edges and k regular polygons of m edges: the knot sets the slots of a row (n / 256), all
+    edges together the size of a slot."""
+    t = 2.0 * np.pi * np.arange(m) / m
+    ring = np.stack([np.cos(t), np.sin(t), 0.1 * np.sin(2 * t)], 1)
+    gamma = np.concatenate([S.fourier_knot(n, 16, 5), np.tile(ring, (k, 1))])
+    edges = np.concatenate([S.closed_edges(n)] +
+                           [np.stack([np.tile(np.arange(m), k), np.tile((np.arange(m) + 1) % m, k)], 1) +
+                            (n + m * np.repeat(np.arange(k), m))[:, None]]).astype(np.int32)
+    off = np.concatenate([[0], n + m * np.arange(k + 1)]).astype(np.int32)
+    return S.Curves(gamma, edges, off, off)
+
+
+def test_refused_partial_sums_leave_the_context_sound(torch):
+    """1,026 slots of 3.9M edges x 10 values: 324 GB of partial sums, more than the device has.  The selection fails and
+    the passes run on in the form, with the buffer and to the bits they had before."""
+    from paper_2006_07859_gb300 import tpe
+    c = _knot_among_polygons(262144, 14400)
+    assert 1026 * c.n_edges * 80 > torch.cuda.get_device_properties(0).total_memory
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI, independent=1)
+    g = dev(c.gamma)
+    rows = torch.empty(c.n_edges, dtype=torch.float64, device="cuda")
+    E = host(tpe.tp_energy(ctx, g, rows=rows))
+    before = host(rows)
+    with pytest.raises(tpe.TpError) as err:
+        tpe.tp_set_diff_variant(ctx, 1)
+    assert err.value.status == tpe.TP_ERR_OOM
+    rows.zero_()
+    assert np.array_equal(host(tpe.tp_energy(ctx, g, rows=rows)), E)
+    assert np.array_equal(host(rows), before)
+    ctx.close()
