@@ -1430,13 +1430,8 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (err == cudaSuccess) err = sym_select_energy(c, 0);
         if (err == cudaSuccess) err = sym_select_diff(c, 0);
     }
-    // a symmetric variant is a candidate while its partial sums fit in 32 GB and in half the free memory
-    // (on top of what the partial buffer already holds); the buffer is shrunk to the winners' need below
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
-    auto fits = [&](size_t bytes) {
-        return bytes <= ((size_t)32 << 30) && bytes <= c.part_elems * sizeof(double) + free_b / 2;
-    };
+    // a symmetric variant is a candidate while its partial sums pass part_fits; the buffer is shrunk to the winners'
+    // need below
     for (int cls = 0; cls < 3 && err == cudaSuccess; ++cls) {
         int cand[4];
         const int nc = tpt_candidates(c, cls, cand);
@@ -1468,7 +1463,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 1 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 4 && err == cudaSuccess; ++t) {
-                if (!fits(sym_part_elems(c, OP_DIFF, t) * sizeof(double))) continue;
+                if (!part_fits(c, sym_part_elems(c, OP_DIFF, t))) continue;
                 if ((err = sym_select_diff(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);
@@ -1491,7 +1486,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 0 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 2 && err == cudaSuccess; ++t) {
-                if (!fits(sym_part_elems(c, OP_ENERGY, t) * sizeof(double))) continue;
+                if (!part_fits(c, sym_part_elems(c, OP_ENERGY, t))) continue;
                 if ((err = sym_select_energy(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);
@@ -1514,7 +1509,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
         if (cls == 2 && nc > 1 && err == cudaSuccess) {
             int best_sym = 0;
             for (int t = 1; t <= 2 && err == cudaSuccess; ++t) {
-                if (!fits(sym_part_elems(c, OP_APPLY, t) * sizeof(double))) continue;
+                if (!part_fits(c, sym_part_elems(c, OP_APPLY, t))) continue;
                 if ((err = sym_select(c, t)) != cudaSuccess) break;
                 if ((err = run(cls)) != cudaSuccess) break;
                 cudaEventRecord(e0, s);

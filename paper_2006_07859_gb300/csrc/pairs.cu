@@ -513,6 +513,18 @@ cudaError_t part_resize(Ctx &c, size_t elems)
 
 cudaError_t part_reserve(Ctx &c, size_t elems) { return elems <= c.part_elems ? cudaSuccess : part_resize(c, elems); }
 
+// Whether partial sums of this size may be taken for a faster form of a pass that has another: at most 32 GB, and
+// half of the free memory on top of what the buffer already holds.
+bool part_fits(const Ctx &c, size_t elems)
+{
+    const size_t bytes = sizeof(double) * elems;
+    if (bytes > (size_t)32 << 30) return false;
+    if (elems <= c.part_elems) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
+    return bytes <= sizeof(double) * c.part_elems + free_b / 2;
+}
+
 void plan_free(Ctx::Plan &pl)
 {
     if (pl.d_items) cudaFree(pl.d_items);

@@ -225,8 +225,8 @@ static cudaError_t multi_init(Ctx &c)
 static cudaError_t apply_multi_sym(Ctx &c, int which, const double *U, double *AU, int m, cudaStream_t s)
 {
     const size_t ne = (size_t)c.nE, nv3 = 3 * (size_t)c.nV;
-    if (!c.d_urecMF) TPE_CHECK(cudaMalloc(&c.d_urecMF, sizeof(URecF) * kMultiG * ne));
-    if (!c.d_esum2) TPE_CHECK(cudaMalloc(&c.d_esum2, sizeof(double) * 12 * ne));
+    if (m > 1 && !c.d_urecMF) TPE_CHECK(cudaMalloc(&c.d_urecMF, sizeof(URecF) * kMultiG * ne));
+    if (m > 1 && !c.d_esum2) TPE_CHECK(cudaMalloc(&c.d_esum2, sizeof(double) * 12 * ne));
     int f = 0;
     for (; f + 2 <= m; f += 2) {
         for (int g = 0; g < 2; ++g) TPE_CHECK(build_urecs_into(c, U + (f + g) * nv3, which, c.d_urecMF + g * ne, nullptr, s));
@@ -246,8 +246,10 @@ cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const 
     }
     // Contexts that run the symmetric apply take the fields two by two through its two-field form (four would
     // not fit in registers): 16,384 edges, four fields 2 x 1,480 us against 3,736 us for the four-field gather pass
-    // below, which evaluates every ordered pair.
-    if (c.apply_sym > 0 && c.prm.precision == TP_MIXED) return apply_multi_sym(c, which, U, AU, m, s);
+    // below, which evaluates every ordered pair.  Its partial sums are twice the apply's (25.8 GB at 262,144 edges, growing
+    // with n^2): where there is no memory for them the gather pass runs, whose slots are at most 64 source chunks.
+    if (c.apply_sym > 0 && c.prm.precision == TP_MIXED && (m == 1 || sym_apply2_ready(c)))
+        return apply_multi_sym(c, which, U, AU, m, s);
     TPE_CHECK(multi_init(c));
     const Ctx::Plan &pl = c.plan_multi;
     const bool p64 = c.prm.precision == TP_FP64;

@@ -1118,26 +1118,32 @@ cudaError_t sym_apply_pass(Ctx &c, int which, cudaStream_t s)
 }
 
 // Passes whose plan is built at the first call.
-static cudaError_t lazy_pass(Ctx &c, int op, Ctx::Plan &pl, int variant, int counter, int prof_op, int which, const int *skip,
-                             double *out, cudaStream_t s)
+static cudaError_t lazy_plan(Ctx &c, int op, Ctx::Plan &pl, int variant)
 {
-    if (!pl.d_items) {
-        TPE_CHECK(sym_plan(c, pl, sym_occupancy(c, op, variant)));
-        pl.tpt = variant;
-    }
-    return sym_pass(c, op, pl, counter, prof_op, which, skip, out, s);
+    if (pl.d_items) return cudaSuccess;
+    TPE_CHECK(sym_plan(c, pl, sym_occupancy(c, op, variant)));
+    pl.tpt = variant;
+    return cudaSuccess;
 }
 
 // The accurate apply: edges' endpoint values into c.d_esum.
 cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s)
 {
-    return lazy_pass(c, OP_APPLY, c.plan_df, kSymAccurate, 7, 5, which, c.d_skip, c.d_esum, s);
+    TPE_CHECK(lazy_plan(c, OP_APPLY, c.plan_df, kSymAccurate));
+    return sym_pass(c, OP_APPLY, c.plan_df, 7, 5, which, c.d_skip, c.d_esum, s);
+}
+
+bool sym_apply2_ready(Ctx &c)
+{
+    Ctx::Plan &pl = c.plan_sym2;
+    const size_t need = pl.d_items ? plan_elems(c, pl, OP_APPLY2) : sym_part_elems(c, OP_APPLY2, 1);
+    return part_fits(c, need) && lazy_plan(c, OP_APPLY2, pl, 1) == cudaSuccess && part_reserve(c, need) == cudaSuccess;
 }
 
 // Two vector fields, the weights once per pair.
 cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s)
 {
-    return lazy_pass(c, OP_APPLY2, c.plan_sym2, 1, 10, 7, which, nullptr, c.d_esum2, s);
+    return sym_pass(c, OP_APPLY2, c.plan_sym2, 10, 7, which, nullptr, c.d_esum2, s);
 }
 
 }  // namespace tpe

@@ -244,6 +244,7 @@ cudaError_t pair_apply_multi(Ctx &c, const double *gamma_geom, int which, const 
 void multi_free(Ctx &c);
 cudaError_t part_resize(Ctx &c, size_t elems);
 cudaError_t part_reserve(Ctx &c, size_t elems);
+bool part_fits(const Ctx &c, size_t elems);
 void plan_free(Ctx::Plan &pl);
 cudaError_t plan_upload(Ctx::Plan &pl, const std::vector<WorkItem> &items, const std::vector<int> &eslots);
 cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy);
@@ -258,7 +259,8 @@ cudaError_t sym_energy_pass(Ctx &c, int which, double *rows, cudaStream_t s);
 cudaError_t sym_select_diff(Ctx &c, int variant);
 cudaError_t sym_diff_pass(Ctx &c, int which, cudaStream_t s);
 cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s);  // specialised powers; grows c.d_part
-cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: c.d_urecMF into c.d_esum2; grows c.d_part
+bool sym_apply2_ready(Ctx &c);  // builds the two-field pass and grows c.d_part; false where there is no memory for it
+cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: c.d_urecMF into c.d_esum2
 size_t sym_default_elems(const Ctx &c);
 cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs

@@ -45,3 +45,25 @@ def test_refused_partial_sums_leave_the_context_sound(torch):
     assert np.array_equal(host(tpe.tp_energy(ctx, g, rows=rows)), E)
     assert np.array_equal(host(rows), before)
     ctx.close()
+
+
+def test_two_fields_without_memory_take_the_gather_pass(torch):
+    """1,026 slots of 364,544 edges: the apply's partial sums take 18 GB and are asked for; those of its two-field form
+    (36 GB) are more than a pass takes unasked, so two fields run the gather pass.  Tolerance of the two forms of the
+    apply: 1e-6 of the largest entry."""
+    from paper_2006_07859_gb300 import tpe
+    c = _knot_among_polygons(262144, 400)
+    ctx = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI, independent=1)
+    tpe.tp_set_apply_variant(ctx, 1)
+    g = dev(c.gamma)
+    U = dev(np.random.default_rng(3).normal(size=(2, c.n_vertices, 3)))
+    one = [tpe.sobolev_apply(ctx, g, U[f]) for f in range(2)]
+    AU = torch.empty_like(U)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    AU = tpe.sobolev_apply_multi(ctx, g, U, AU)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 8e9
+    for f in range(2):
+        assert float((AU[f] - one[f]).abs().max()) <= 1e-6 * float(one[f].abs().max())
+    ctx.close()
