@@ -433,7 +433,8 @@ tp_status tp_create(tp_ctx **out, int nV, int nE, const int32_t *edges_host, int
     set_kernel_params(c);
     CK(make_plans(c));
     int ms = std::max(std::max(c.plan_energy.max_slots, c.plan_diff.max_slots), c.plan_apply.max_slots);
-    CK(part_reserve(c, std::max((size_t)ms * std::max(1, nE) * 6, sym_default_elems(c))));
+    const size_t gather = (size_t)ms * std::max(1, nE) * 6, sym = sym_default_elems(c);
+    if (sym <= gather || part_reserve(c, sym) != cudaSuccess) CK(part_reserve(c, gather));
     CK(sym_defaults(c));
     CK(dalloc(&c.d_rows, nE));
     CK(dalloc(&c.d_esum, 6 * (size_t)nE));

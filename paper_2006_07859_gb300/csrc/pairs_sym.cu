@@ -1017,9 +1017,9 @@ cudaError_t sym_select(Ctx &c, int v) { return select_pass(c, OP_APPLY, v, 2, c.
 cudaError_t sym_select_energy(Ctx &c, int v) { return select_pass(c, OP_ENERGY, v, 2, c.plan_sym_e, c.energy_sym); }
 cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4, c.plan_sym_d, c.diff_sym); }
 
-// Whether a new context runs the pass of `op` in symmetric form: where a work list of whole tiles gives every
+// Whether a context runs the pass of `op` in symmetric form by itself: where a work list of whole tiles gives every
 // resident CTA an item, or (mixed precision) where the unordered pairs per SM reach 22,000, for the energy
-// 50,000; the partial sums stay below 1 GiB.  On smaller graphs the gather pass's short chunks spread the work better
+// 50,000 (sym_default_elems limits the partial sums).  On smaller graphs the gather pass's short chunks spread the work better
 // and the symmetric pass waits for its longest item.  Gather / symmetric in us:
 //   edges      pairs/SM   differential    apply      energy
 //   2,000        13,000     268 / 320     50 / 55    47 / 64
@@ -1042,24 +1042,37 @@ static bool sym_pays(const Ctx &c, int op)
     }
     const bool enough = c.prm.precision == TP_MIXED && pairs >= (op == OP_ENERGY ? 50e3 : 22e3) * c.sm_count;
     if (!enough && items < c.sm_count) return false;  // no need to load the kernel for its occupancy
-    const bool fills = enough || items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1));
-    return fills && sym_part_elems(c, op, 1) * sizeof(double) <= (size_t)1 << 30;
+    return enough || items >= (long long)c.sm_count * std::max(1, sym_occupancy(c, op, 1));
 }
 
-// Doubles of the partial buffer a new context needs for them.
+// Doubles of partial sums the passes that pay may take unasked: 1 GiB a context, and a 64th of the free memory where that
+// is less (a program with many contexts, or one whose other pools hold most of the device, gets the gather passes,
+// which need tens of MB).  Up to 64 MiB the free memory is not looked up.
 size_t sym_default_elems(const Ctx &c)
 {
-    size_t need = 0;
-    for (int op : {OP_ENERGY, OP_DIFF, OP_APPLY})
-        if (sym_pays(c, op)) need = std::max(need, sym_part_elems(c, op, 1));
+    size_t need = 0, limit = (size_t)1 << 30;
+    bool looked_up = false;
+    for (int op : {OP_ENERGY, OP_DIFF, OP_APPLY}) {
+        if (!sym_pays(c, op)) continue;
+        const size_t elems = sym_part_elems(c, op, 1), bytes = sizeof(double) * elems;
+        size_t free_b = 0, total_b = 0;
+        if (bytes > (size_t)64 << 20 && !looked_up) {
+            looked_up = true;
+            if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
+            limit = std::min(limit, std::max((size_t)64 << 20, free_b / 64));
+        }
+        if (bytes <= limit) need = std::max(need, elems);
+    }
     return need;
 }
 
+// Select the passes that pay and whose partial sums fit in the buffer.
 cudaError_t sym_defaults(Ctx &c)
 {
-    if (sym_pays(c, OP_ENERGY)) TPE_CHECK(sym_select_energy(c, 1));
-    if (sym_pays(c, OP_DIFF)) TPE_CHECK(sym_select_diff(c, 1));
-    if (sym_pays(c, OP_APPLY)) TPE_CHECK(sym_select(c, 1));
+    auto takes = [&](int op) { return sym_pays(c, op) && sym_part_elems(c, op, 1) <= c.part_elems; };
+    if (takes(OP_ENERGY)) TPE_CHECK(sym_select_energy(c, 1));
+    if (takes(OP_DIFF)) TPE_CHECK(sym_select_diff(c, 1));
+    if (takes(OP_APPLY)) TPE_CHECK(sym_select(c, 1));
     return cudaSuccess;
 }
 

@@ -262,7 +262,7 @@ cudaError_t sym_apply_accurate_pass(Ctx &c, int which, cudaStream_t s);  // spec
 bool sym_apply2_ready(Ctx &c);  // builds the two-field pass and grows c.d_part; false where there is no memory for it
 cudaError_t sym_apply2_pass(Ctx &c, int which, cudaStream_t s);  // two fields: c.d_urecMF into c.d_esum2
 size_t sym_default_elems(const Ctx &c);
-cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size
+cudaError_t sym_defaults(Ctx &c);  // the choice of a new context, by its size and the memory for it
 size_t sym_part_elems(const Ctx &c, int op, int variant);  // doubles of c.d_part the pass needs
 cudaError_t make_plans(Ctx &c);
 cudaError_t replan(Ctx &c, int cls);  // rebuild the plan of one op class (0 energy, 1 diff, 2 apply/diag)
