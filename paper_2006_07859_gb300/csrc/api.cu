@@ -499,6 +499,7 @@ tp_status tp_set_params(tp_ctx *ctx, const tp_params *p)
     if (p->constraint_set != c.prm.constraint_set) c.constraints_set = 0;
     int indep = c.prm.independent;
     int had_spectral = c.spec != nullptr;
+    const int was_fast = c.kp.fast;
     c.prm = *p;
     c.prm.independent = indep;
     set_kernel_params(c);
@@ -513,6 +514,12 @@ tp_status tp_set_params(tp_ctx *ctx, const tp_params *p)
         CK(sym_select(c, 0));
         CK(sym_select_energy(c, 0));
         CK(sym_select_diff(c, 0));
+    }
+    if (!c.kp.fast)
+        for (int &v : c.sym_choice) v = std::min(v, 0);  // a choice of the gather pass stays
+    if (c.kp.fast && !was_fast) {  // the passes a new context has; without the memory for them the gather passes stay
+        part_reserve(c, sym_default_elems(c));
+        CK(sym_defaults(c));
     }
     if ((p->precond >= TP_PRECOND_SPECTRAL) && !had_spectral) {
         cudaError_t e = spectral_setup(c, 0);
@@ -1378,6 +1385,7 @@ tp_status tp_set_diff_variant(tp_ctx *ctx, int symmetric_tpt)
     if (symmetric_tpt > 0 && !(c.prm.precision == TP_MIXED && c.kp.fast))
         return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric differential exists for TP_MIXED with (alpha, beta) = (2, 4.5)");
     CK(sym_select_diff(c, symmetric_tpt));
+    c.sym_choice[OP_DIFF] = symmetric_tpt;
     return TP_OK;
 }
 
@@ -1389,6 +1397,7 @@ tp_status tp_set_energy_variant(tp_ctx *ctx, int symmetric_tpt)
     if (symmetric_tpt > 0 && !(c.prm.precision == TP_MIXED && c.kp.fast))
         return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric energy exists for TP_MIXED with (alpha, beta) = (2, 4.5)");
     CK(sym_select_energy(c, symmetric_tpt));
+    c.sym_choice[OP_ENERGY] = symmetric_tpt;
     return TP_OK;
 }
 
@@ -1400,6 +1409,7 @@ tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt)
     if (symmetric_tpt > 0 && !(c.prm.precision == TP_MIXED && c.kp.fast))
         return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric apply exists for TP_MIXED with (alpha, beta) = (2, 4.5)");
     CK(sym_select(c, symmetric_tpt));
+    c.sym_choice[OP_APPLY] = symmetric_tpt;
     return TP_OK;
 }
 
@@ -1481,6 +1491,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
                 }
             }
             if (err == cudaSuccess) err = sym_select_diff(c, best_sym);
+            if (err == cudaSuccess) c.sym_choice[OP_DIFF] = best_sym;
             if (tpt) tpt[5] = best_sym;
         }
         // the energy also has the symmetric pass (its rows are one double per edge and slot)
@@ -1504,6 +1515,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
                 }
             }
             if (err == cudaSuccess) err = sym_select_energy(c, best_sym);
+            if (err == cudaSuccess) c.sym_choice[OP_ENERGY] = best_sym;
             if (tpt) tpt[4] = best_sym;
         }
         // the apply also has the symmetric pass (each unordered pair once), if its partial slots fit
@@ -1527,6 +1539,7 @@ tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms
                 }
             }
             if (err == cudaSuccess) err = sym_select(c, best_sym);
+            if (err == cudaSuccess) c.sym_choice[OP_APPLY] = best_sym;
             if (tpt) tpt[3] = best_sym;
         }
     }

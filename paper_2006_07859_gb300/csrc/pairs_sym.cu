@@ -1032,6 +1032,7 @@ cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4
 //   120 x 256    25,800     816 / 524     88 / 76    85 / 93
 static bool sym_pays(const Ctx &c, int op)
 {
+    if (c.sym_choice[op] >= 0) return false;
     if (!c.kp.fast || c.prm.precision == TP_FP64 || (op == OP_DIFF && c.prm.precision != TP_MIXED)) return false;
     long long items = 0;
     double pairs = 0.0;

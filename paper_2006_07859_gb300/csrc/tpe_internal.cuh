@@ -134,6 +134,7 @@ struct Ctx {
     int energy_sym = 0;      // > 0: the energy runs the symmetric pass with this many targets per thread
     Plan plan_sym_d;         // symmetric differential (pairs_sym.cu)
     int diff_sym = 0;        // > 0: the differential runs the symmetric pass
+    int sym_choice[3] = {-1, -1, -1};  // variant asked for (OP_ENERGY, OP_DIFF, OP_APPLY); -1: the default by size
     Plan plan_df;            // double-float apply, built at its first use (tpt 1: general exponents)
     Plan plan_multi;         // multi-field apply (pairs_multi.cu), built at its first use
     URecF *d_urecMF = nullptr;  // multi-field apply: per-edge records of kMultiG fields (FP32 contexts)

@@ -152,3 +152,34 @@ def test_new_context_between_the_passes(torch, n, k):
         out.append([host(rows), host(tpe.tp_differential(ctx, g)), host(tpe.sobolev_apply(ctx, g, u))])
     for new, old in zip(*out):
         assert rel(new, old) <= 1e-5
+
+
+def test_default_passes_return_with_the_exponents(torch):
+    """5,000 edges: a new context runs the symmetric passes.  Other exponents have none; back at (2, 4.5) the context
+    runs them again, to the bit, and a pass that was set to the gather form stays in it."""
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(5000, 5, 17))
+    g, u = dev(c.gamma), dev(np.random.default_rng(5).normal(size=(c.n_vertices, 3)))
+
+    def passes(ctx):
+        rows = torch.empty(c.n_edges, dtype=torch.float64, device="cuda")
+        tpe.tp_energy(ctx, g, rows=rows)
+        return [host(rows), host(tpe.tp_differential(ctx, g)), host(tpe.sobolev_apply(ctx, g, u))]
+
+    def there_and_back(ctx):
+        ctx.set_params(alpha=3.0, beta=6.0)
+        passes(ctx)
+        ctx.set_params(alpha=2.0, beta=4.5)
+
+    new = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    first = passes(new)
+    there_and_back(new)
+    gather = make_ctx(c, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI)
+    tpe.tp_set_energy_variant(gather, 0)
+    tpe.tp_set_diff_variant(gather, 0)
+    tpe.tp_set_apply_variant(gather, 0)
+    ordered = passes(gather)
+    there_and_back(gather)
+    for a, b, c0, c1 in zip(first, passes(new), ordered, passes(gather)):
+        assert np.array_equal(a, b) and np.array_equal(c0, c1)
+        assert not np.array_equal(a, c0)
