@@ -65,7 +65,8 @@ typedef enum {
 
 typedef enum {
     TP_FP64 = 0,  /* pair arithmetic in FP64 */
-    TP_FP32 = 1,  /* pair arithmetic in FP32, per-tile partial sums folded into FP64 */
+    TP_FP32 = 1,  /* pair arithmetic in FP32; sums over at most 512 sources in FP32 (compensated in the symmetric
+                     passes), those partial sums added in FP64 (symmetric passes: double-float) */
     TP_MIXED = 2  /* FP32 pairs on double-float positions, double-float for pairs closer than near_cutoff */
 } tp_precision;
 
@@ -515,17 +516,17 @@ TPE_API tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, do
 
 /* Select the apply pass: symmetric_tpt = 0 the gather pass (every ordered pair), 1 or 2 the symmetric pass
  * (every unordered pair evaluated once, two targets per thread in packed arithmetic; both rows receive their
- * terms; TP_MIXED with (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED), its registers held to three
- * (1) or two (2) resident CTAs per SM.  A new context has the symmetric pass where its work list fills the GPU
+ * terms; TP_MIXED and TP_FP32 with (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED), its registers held to
+ * three (1) or two (2) resident CTAs per SM (TP_FP32: three).  A new context has the symmetric pass where its work list fills the GPU
  * and its partial sums take at most 1 GiB, the gather pass elsewhere.  Both are deterministic and differ
  * only in summation order.  May grow the partial-sum buffer. */
 TPE_API tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt);
 
-/* The same choice for the energy pass (0: gather, 1 or 2: symmetric at three or four resident CTAs per SM; the
- * rows E_I are the same sums in another order). */
+/* The same choice for the energy pass (0: gather, 1 or 2: symmetric at three or four resident CTAs per SM, TP_FP32
+ * four; the rows E_I are the same sums in another order). */
 TPE_API tp_status tp_set_energy_variant(tp_ctx *ctx, int symmetric_tpt);
 
-/* The same choice for the differential pass (0: gather; 1 or 2: symmetric at two resident CTAs per SM, 3 or 4
+/* The same choice for the differential pass, TP_MIXED only (0: gather; 1 or 2: symmetric at two resident CTAs per SM, 3 or 4
  * at three, with spilled registers).  Row J's terms of a pair are the mirror of row I's; near pairs are
  * double-float on both sides). */
 TPE_API tp_status tp_set_diff_variant(tp_ctx *ctx, int symmetric_tpt);

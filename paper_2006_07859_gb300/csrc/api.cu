@@ -1394,8 +1394,8 @@ tp_status tp_set_energy_variant(tp_ctx *ctx, int symmetric_tpt)
     if (!ctx) return TP_ERR_INVALID_ARG;
     Ctx &c = ctx->c;
     if (symmetric_tpt < 0 || symmetric_tpt > 2) return fail(ctx, TP_ERR_INVALID_ARG, "symmetric_tpt must be 0, 1 or 2");
-    if (symmetric_tpt > 0 && !(c.prm.precision == TP_MIXED && c.kp.fast))
-        return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric energy exists for TP_MIXED with (alpha, beta) = (2, 4.5)");
+    if (symmetric_tpt > 0 && !(c.prm.precision != TP_FP64 && c.kp.fast))
+        return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric energy exists for TP_MIXED and TP_FP32 with (alpha, beta) = (2, 4.5)");
     CK(sym_select_energy(c, symmetric_tpt));
     c.sym_choice[OP_ENERGY] = symmetric_tpt;
     return TP_OK;
@@ -1406,8 +1406,8 @@ tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt)
     if (!ctx) return TP_ERR_INVALID_ARG;
     Ctx &c = ctx->c;
     if (symmetric_tpt < 0 || symmetric_tpt > 2) return fail(ctx, TP_ERR_INVALID_ARG, "symmetric_tpt must be 0, 1 or 2");
-    if (symmetric_tpt > 0 && !(c.prm.precision == TP_MIXED && c.kp.fast))
-        return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric apply exists for TP_MIXED with (alpha, beta) = (2, 4.5)");
+    if (symmetric_tpt > 0 && !(c.prm.precision != TP_FP64 && c.kp.fast))
+        return fail(ctx, TP_ERR_UNSUPPORTED, "the symmetric apply exists for TP_MIXED and TP_FP32 with (alpha, beta) = (2, 4.5)");
     CK(sym_select(c, symmetric_tpt));
     c.sym_choice[OP_APPLY] = symmetric_tpt;
     return TP_OK;

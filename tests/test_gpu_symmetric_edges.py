@@ -183,3 +183,20 @@ def test_default_passes_return_with_the_exponents(torch):
     for a, b, c0, c1 in zip(first, passes(new), ordered, passes(gather)):
         assert np.array_equal(a, b) and np.array_equal(c0, c1)
         assert not np.array_equal(a, c0)
+
+
+# plain FP32 positions: the bars of test_new_context_of_many_ragged_curves
+@pytest.mark.parametrize("n", [3, 4, 63, 64, 65, 127, 128, 129, 192, 193, 255, 256, 257, 385])
+@pytest.mark.parametrize("variant", [0, 1, 2])
+def test_fp32_passes_at_block_edges(torch, orc, n, variant):
+    from paper_2006_07859_gb300 import tpe
+    c = S.single(S.fourier_knot(n, 4, 40 + n))
+    ctx = make_ctx(c, precision=tpe.TP_FP32, precond=tpe.TP_PRECOND_JACOBI)
+    tpe.tp_set_energy_variant(ctx, 1)
+    tpe.tp_set_apply_variant(ctx, 1)
+    tpe.tp_set_energy_variant(ctx, variant)
+    tpe.tp_set_apply_variant(ctx, variant)
+    with pytest.raises(tpe.TpError) as err:
+        tpe.tp_set_diff_variant(ctx, 1)
+    assert err.value.status == tpe.TP_ERR_UNSUPPORTED
+    _check(torch, orc, ctx, c, 1, {"energy": 1e-4, "diff": 1.0, "apply": 1e-4})
