@@ -97,6 +97,14 @@ void set_kernel_params(Ctx &c)
     // the differential's near-pair gradient terms are large and cancel between the two sides of a
     // vertex, so they get FP64 over a 4x wider band than the energy
     c.kp.near2f_diff = (float)(16.0 * rn * rn);
+    // the gradient of a pair at distance d goes with d^-2.5 times an edge's length: 2^-56 at the mean edge; the length
+    // times the scale, which every far pair forms, stays above 2^-100
+    c.kp.sum_exp = 0;
+    if (c.kp.fast && c.mean_ell > 0.0 && std::isfinite(c.mean_ell)) {
+        const int e = (int)std::lround(std::log2(c.mean_ell)), s = (int)std::lround(2.5 * std::log2(c.mean_ell)) - 56;
+        c.kp.sum_exp = std::min(std::max(std::max(s, -100 - e), -120), 120);
+    }
+    c.kp.sum_scale = std::ldexp(1.0f, c.kp.sum_exp);
     // tiles closer than far_cutoff x the curve's extent use double-float differences (mixed path)
     double rm = std::max(p.far_cutoff * c.extent, rn);
     c.kp.mid2f = p.far_cutoff >= 10.0 ? 3.0e38f : (float)(rm * rm);

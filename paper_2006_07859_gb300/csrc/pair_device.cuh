@@ -583,6 +583,7 @@ __device__ __forceinline__ void pair_eval(const Tgt<typename RealOf<PREC>::type>
         }
         R L = keep ? s.ell : (R)0;
         if constexpr (PREC == PMIX) {
+            L *= kp.sum_scale;
             // compensated: the vertex gather takes differences of neighbouring edges' rows, which
             // cancel by ~1 / (kappa l), so the rows need more than FP32 summation accuracy
             kahan_add(a.S, a.cS, L * S);
@@ -750,7 +751,7 @@ __device__ __forceinline__ void tile_loop(const Tgt<typename RealOf<PREC>::type>
                     if (keep && dot3(e, e) < pa.kp.near2f_diff) {
                         if constexpr (FAST) {
                             dfl<float> x[10], y[10];
-                            near_diff(pa.recF, pa.recLo, tI[k], s0 + j, x, y);
+                            near_diff(pa.recF, pa.recLo, tI[k], s0 + j, pa.kp.sum_exp, x, y);
                             l_kahan_df(a[k].S, a[k].cS, x[0].hi, x[0].lo);
 #pragma unroll
                             for (int q = 0; q < 3; ++q) {

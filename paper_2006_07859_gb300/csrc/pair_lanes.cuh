@@ -336,11 +336,22 @@ static __device__ __noinline__ void near_energy(const RecF *recF, const RecLo *r
     }
 }
 
-// |d|^-4.5 and |d|^-2 in double-float: r0 = rsqrt(d2.hi) with its residual rho = 1 - d2 r0^2 formed through
+// 2^e, as far as a normal float goes
+__device__ __forceinline__ float near_pow2(int e) { return __int_as_float(min(max(e + 127, 1), 254) << 23); }
+
+// |d|^-4.5 2^sum_exp and |d|^-2 in double-float: r0 = rsqrt(d2.hi) with its residual rho = 1 - d2 r0^2 formed through
 // fma gives |d|^-1 = r0 (1 + eps), and q0 ~ sqrt(r0) from rsqrt(r0) is corrected by (r0 - q0^2) / (2 q0).
-template <class L>
-__device__ __forceinline__ dfl<L> near_pow45(dfl<L> d2, dfl<L> &R2)
+//
+// FP32 exponents hold |d|^-4.5 from 2.7e-9 up only, and the low parts of its double-float up to about 1e7.  So the power
+// is formed at 4^m times the chord's length, between 1 and 4 (a power of four leaves |d|^-4.5 a power of two, so the
+// scaling is exact), and the differential's sums are kept at 2^sum_exp of their value: 2^-56 for the gradient of a pair
+// one mean edge apart, so that they hold pairs down to 1e-12 of an edge, about the resolution of double-float positions.
+__device__ __forceinline__ dfl<float> near_pow45(dfl<float> d2, int sum_exp, dfl<float> &R2)
 {
+    using L = float;
+    const int m = -((__float_as_int(d2.hi) - (127 << 23)) >> 25);
+    const float up = near_pow2(4 * m), back = near_pow2(9 * m + sum_exp);
+    d2 = {l_mul(d2.hi, up), l_mul(d2.lo, up)};
     const L r0 = l_rsqrt(d2.hi);
     const L a = l_mul(r0, r0), b = l_fma(r0, r0, l_neg(a));
     L rho = l_fma(l_neg(d2.hi), a, l_bc<L>(1.f));
@@ -351,14 +362,16 @@ __device__ __forceinline__ dfl<L> near_pow45(dfl<L> d2, dfl<L> &R2)
     const L dq = l_mul(l_fma(l_neg(q0), q0, r0), l_mul(l_bc<L>(0.5f), iq));
     const dfl<L> R = {a, b};  // r0^2
     R2 = l_dfscale(R, l_mul(eps, l_add(l_bc<L>(2.f), eps)));
-    const dfl<L> F = l_dfmul(l_dfsqr(R), dfl<L>{q0, dq});  // r0^4.5
-    return l_dfscale(F, l_mul(eps, l_fma(l_bc<L>(7.875f), eps, l_bc<L>(4.5f))));
+    R2 = {l_mul(R2.hi, up), l_mul(R2.lo, up)};
+    dfl<L> F = l_dfmul(l_dfsqr(R), dfl<L>{q0, dq});  // r0^4.5
+    F = l_dfscale(F, l_mul(eps, l_fma(l_bc<L>(7.875f), eps, l_bc<L>(4.5f))));
+    return {l_mul(F.hi, back), l_mul(F.lo, back)};
 }
 
-// The differential's terms of one near pair, scaled by the other row's length: row I's (S, G1, G2, GT) into x and
-// row J's (S, H1, H2, HT) into y, see pairs_sym.cu.
-static __device__ __noinline__ void near_diff(const RecF *recF, const RecLo *recLo, int I0, int J0, dfl<float> (&x)[10],
-                                              dfl<float> (&y)[10])
+// The differential's terms of one near pair, scaled by the other row's length and 2^sum_exp: row I's (S, G1, G2, GT)
+// into x and row J's (S, H1, H2, HT) into y, see pairs_sym.cu.
+static __device__ __noinline__ void near_diff(const RecF *recF, const RecLo *recLo, int I0, int J0, int sum_exp,
+                                              dfl<float> (&x)[10], dfl<float> (&y)[10])
 {
     using L = float;
     NearEdge<L> I, J;
@@ -391,7 +404,7 @@ static __device__ __noinline__ void near_diff(const RecF *recF, const RecLo *rec
         for (int b = 0; b < 2; ++b) {
             const dfv<L> d = near_chord(I, 0, J, 0);
             dfl<L> r2;
-            const dfl<L> rb = near_pow45(l_dfnorm2(d), r2);
+            const dfl<L> rb = near_pow45(l_dfnorm2(d), sum_exp, r2);
             const dfl<L> fs = l_dfmul(l_dfadd(cI[0], cJ[0]), rb);
             const dfl<L> al = {l_add(rb.hi, rb.hi), l_add(rb.lo, rb.lo)};  // alpha |d|^-beta
             const dfl<L> cb = l_dfneg(l_dfmul(l_dfmulf(fs, 4.5f), r2));

@@ -298,11 +298,12 @@ __global__ void __launch_bounds__(kThreads, (pair_min_blocks<PREC, OP, TPT>())) 
                 const double *T = pa.na.T + 3 * I;
                 double l = pa.na.ell[I];
                 double tg3[3] = {T[0], T[1], T[2]};
+                const double quarter = PREC == PMIX ? 0.25 / (double)pa.kp.sum_scale : 0.25;
                 double gt = tg3[0] * A[k].GT[0] + tg3[1] * A[k].GT[1] + tg3[2] * A[k].GT[2];
                 for (int c = 0; c < 3; ++c) {
                     double pgt = A[k].GT[c] - gt * tg3[c];
-                    o[c] = 0.25 * (-tg3[c] * A[k].S + l * A[k].G1[c] - pgt);
-                    o[3 + c] = 0.25 * (tg3[c] * A[k].S + l * A[k].G2[c] + pgt);
+                    o[c] = quarter * (-tg3[c] * A[k].S + l * A[k].G1[c] - pgt);
+                    o[3 + c] = quarter * (tg3[c] * A[k].S + l * A[k].G2[c] + pgt);
                 }
             } else if constexpr (OP == OP_APPLY) {
                 // h_I / l_I = A1 / 2 (to +i2, -i1) and l_I / 2 = l_I A2 / 8 (to both endpoints)

@@ -65,6 +65,8 @@ struct SymArgs {
     float2 *part;  // [slot][nE][W]
     int nE;
     float near2f, mid2f;
+    int sum_exp;  // OP_DIFF: the sums are kept at 2^sum_exp of their value
+    float sum_scale;
     const int *skip;
 };
 
@@ -438,7 +440,7 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const
             HT[k] = ab == 0 ? l_mul(mJ, dv[k]) : l_fma(mJ, dv[k], HT[k]);
         }
     }
-    const L2 L = l_bc<L2>(s.ell);
+    const L2 L = l_bc<L2>(l_mul(s.ell, pa.sum_scale)), tL = l_mul(t.ell, l_bc<L2>(pa.sum_scale));
     l_kahan_fma(a.s[0], a.c[0], L, S);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -449,7 +451,7 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const
 #pragma unroll
     for (int q = 0; q < 10; ++q) {
         float2 ac = sac[q * kTile];
-        src_add(ac, t.ell, q == 0 ? S : (q < 4 ? H[0][(q + 2) % 3] : (q < 7 ? H[1][(q + 2) % 3] : HT[(q + 2) % 3])));
+        src_add(ac, tL, q == 0 ? S : (q < 4 ? H[0][(q + 2) % 3] : (q < 7 ? H[1][(q + 2) % 3] : HT[(q + 2) % 3])));
         sac[q * kTile] = ac;
     }
 }
@@ -473,7 +475,7 @@ static __device__ __noinline__ void sym_near_flush(SymSmem<PMIX, OP_DIFF> &sm, i
         const int row = v >> 8, at = v & 0xff, loc = kSection * wid + row;
         on = on && loc < ntgt;
         dfl<float> x[10], y[10];
-        near_diff(pa.recF, pa.recLo, tgt0 + min(loc, ntgt - 1), s0 + (((at & 63) << 1) | (at >> 6)), x, y);
+        near_diff(pa.recF, pa.recLo, tgt0 + min(loc, ntgt - 1), s0 + (((at & 63) << 1) | (at >> 6)), pa.sum_exp, x, y);
         const unsigned live = __ballot_sync(0xffffffffu, on);
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
@@ -767,15 +769,16 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
 }
 
 // Row output of the differential from its accumulators (Sec. 5.1 by the chain rule through l_I and T_I):
-// G_i1 = (1/4)[-T S + l G1 - (Id - T T^t) GT],  G_i2 = (1/4)[T S + l G2 + (Id - T T^t) GT]
-__device__ __forceinline__ void diff_row_out(const double *T, double l, const double *v, double *o)
+// G_i1 = (1/4)[-T S + l G1 - (Id - T T^t) GT],  G_i2 = (1/4)[T S + l G2 + (Id - T T^t) GT]; quarter: 1/4 over the scale of
+// the sums
+__device__ __forceinline__ void diff_row_out(const double *T, double l, double quarter, const double *v, double *o)
 {
     const double *G1 = v + 1, *G2 = v + 4, *GT = v + 7;
     const double gt = T[0] * GT[0] + T[1] * GT[1] + T[2] * GT[2];
     for (int c = 0; c < 3; ++c) {
         const double pgt = GT[c] - gt * T[c];
-        o[c] = 0.25 * (-T[c] * v[0] + l * G1[c] - pgt);
-        o[3 + c] = 0.25 * (T[c] * v[0] + l * G2[c] + pgt);
+        o[c] = quarter * (-T[c] * v[0] + l * G1[c] - pgt);
+        o[3 + c] = quarter * (T[c] * v[0] + l * G2[c] + pgt);
     }
 }
 
@@ -785,7 +788,7 @@ __device__ __forceinline__ void diff_row_out(const double *T, double l, const do
 template <int OP, bool D64 = false>
 __global__ void __launch_bounds__(OP == OP_ENERGY ? 256 : 32 * sym_width<OP>())
 k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ part, const double *__restrict__ ell,
-          const double *__restrict__ T, double *__restrict__ out)
+          const double *__restrict__ T, double quarter, double *__restrict__ out)
 {
     constexpr int W = sym_width<OP>(), R = OP == OP_ENERGY ? 256 : 32;  // rows per block
     __shared__ double sh[OP == OP_ENERGY ? 1 : R * W];
@@ -825,7 +828,7 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
         if constexpr (!D64) x = (double)s + (double)lo;
     }
     if constexpr (OP == OP_ENERGY) {
-        if (row < nE) out[row] = 0.25 * ell[row] * x;
+        if (row < nE) out[row] = quarter * ell[row] * x;
     } else {
         sh[threadIdx.x] = x;
         __syncthreads();
@@ -836,7 +839,7 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
         for (int f = 0; f < (OP == OP_APPLY2 ? 2 : 1); ++f, v += 6, out += 6 * (size_t)nE) {
             double o[6];
             if constexpr (OP == OP_DIFF) {
-                diff_row_out(T + 3 * (size_t)I, l, v, o);
+                diff_row_out(T + 3 * (size_t)I, l, quarter, v, o);
             } else {
                 for (int c = 0; c < 3; ++c) {
                     o[c] = 0.5 * v[c];
@@ -1097,21 +1100,23 @@ static cudaError_t sym_pass(Ctx &c, int op, Ctx::Plan &pl, int counter, int prof
     pa.nE = c.nE;
     pa.near2f = op == OP_DIFF ? c.kp.near2f_diff : c.kp.near2f;
     pa.mid2f = c.kp.mid2f;
+    pa.sum_exp = c.kp.sum_exp;
+    pa.sum_scale = c.kp.sum_scale;
     pa.skip = skip;
     const int slot = c.profile ? prof_begin(c, prof_op, s) : -1;
     with_sym_kernel(c.prm.precision, op, pl.tpt, [&](auto kern, size_t smem) { kern<<<pl.grid, kThreads, smem, s>>>(pa); });
     if (slot >= 0 || slot <= -2) prof_end(c, slot, s);
-    const double *ell = c.d_ellw[which], *T = c.d_Tw[which];
+    const double *ell = c.d_ellw[which], *T = c.d_Tw[which], quarter = op == OP_DIFF ? 0.25 / c.kp.sum_scale : 0.25;
     if (op == OP_ENERGY)
-        k_sym_sum<OP_ENERGY><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+        k_sym_sum<OP_ENERGY><<<(c.nE + 255) / 256, 256, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, quarter, out);
     else if (op == OP_DIFF)
-        k_sym_sum<OP_DIFF><<<(c.nE + 31) / 32, 320, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+        k_sym_sum<OP_DIFF><<<(c.nE + 31) / 32, 320, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, quarter, out);
     else if (op == OP_APPLY2)
-        k_sym_sum<OP_APPLY2><<<(c.nE + 31) / 32, 384, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+        k_sym_sum<OP_APPLY2><<<(c.nE + 31) / 32, 384, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, quarter, out);
     else if (pl.tpt == kSymAccurate)
-        k_sym_sum<OP_APPLY, true><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+        k_sym_sum<OP_APPLY, true><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, quarter, out);
     else
-        k_sym_sum<OP_APPLY><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, out);
+        k_sym_sum<OP_APPLY><<<(c.nE + 31) / 32, 192, 0, s>>>(c.nE, pl.d_eslots, pa.part, ell, T, quarter, out);
     c.launches += 2;
     return cudaGetLastError();
 }

@@ -72,6 +72,8 @@ struct KernelParams {
     float near2f;
     float near2f_diff;      // squared near cutoff of the differential (wider: its near terms cancel)
     float mid2f;            // squared distance below which a tile uses double-float differences
+    int sum_exp;            // mixed differential: its FP32 sums are kept at 2^sum_exp of their value (near_diff)
+    float sum_scale;        // 2^sum_exp
 };
 
 // Device-side scalars of one CG solve (all FP64) - one block per problem.
