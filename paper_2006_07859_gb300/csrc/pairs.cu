@@ -169,11 +169,12 @@ __global__ void k_urecs(int nE, const double *__restrict__ u, const int *__restr
 namespace tpe {
 
 // Resident CTAs per SM the register allocation is sized for: the differential and the 4-target
-// apply / diag need more than the 170 registers per thread that 3 CTAs allow, so they get 2.
+// apply / diag need more than the 170 registers per thread that 3 CTAs allow, so they get 2.  The FP64 energy is held to
+// six (80 registers; with 84 it has five, and 3,000 edges take 2,450 us instead of 2,040).
 template <int PREC, int OP, int TPT>
 __host__ __device__ constexpr int pair_min_blocks()
 {
-    return PREC == P64 ? 1 : ((OP == OP_DIFF || (TPT >= 4 && OP != OP_ENERGY)) ? 2 : 3);
+    return PREC == P64 ? (OP == OP_ENERGY ? 6 : 1) : ((OP == OP_DIFF || (TPT >= 4 && OP != OP_ENERGY)) ? 2 : 3);
 }
 
 template <int PREC, int OP, int TPT, bool FAST>
