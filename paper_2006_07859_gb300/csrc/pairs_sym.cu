@@ -214,11 +214,13 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const
     *sac = ac;
 }
 
-// F = |d|^-2.5 and G = |d|^-6.5 in double-float from |d|^2: r0 = rsqrt(d2.hi), its residual rho = 1 - d2 r0^2 formed
-// through fma, |d|^-1 = r0 (1 + eps) with eps = rho / 2 + 3 rho^2 / 8, and sqrt(r0) = q0 + (r0 - q0^2) / (2 q0).
+// F = |d|^-2.5 and G = |d|^-6.5 in double-float from |d|^2: r0 = rsqrt(d2.hi) after a Newton step, its residual rho =
+// 1 - d2 r0^2 formed through fma, |d|^-1 = r0 (1 + eps) with eps = rho / 2 + 3 rho^2 / 8, and sqrt(r0) = q0 +
+// (r0 - q0^2) / (2 q0).  The step makes eps, and with it the low parts whose products l_dfmul drops, four times smaller.
 __device__ __forceinline__ void sym_df_powers(dfl<L2> d2, dfl<L2> &F, dfl<L2> &G)
 {
-    const L2 r0 = l_rsqrt(d2.hi);
+    L2 r0 = l_rsqrt(d2.hi);
+    r0 = l_fma(r0, l_mul(l_bc<L2>(0.5f), l_fma(l_neg(l_mul(d2.hi, r0)), r0, l_bc<L2>(1.f))), r0);
     const L2 a = l_mul(r0, r0), b = l_fma(r0, r0, l_neg(a));
     L2 rho = l_fma(l_neg(d2.hi), a, l_bc<L2>(1.f));
     rho = l_fma(l_neg(d2.hi), b, rho);
@@ -244,17 +246,29 @@ __device__ __forceinline__ dfl<L> l_dfdiff(L ah, L al, L bh, L bl)
     return l_dfnorm(dfl<L>{r.hi, l_add(r.lo, t.lo)});
 }
 
+// A compensated sum acc - c with c at most half an ulp of acc.  Left to itself c takes up the rounding of every
+// addition and the low part of every term, and rounds at its own size each time.
+template <class L>
+__device__ __forceinline__ void l_kahan_norm(L &acc, L &c)
+{
+    const dfl<L> s = l_dfnorm(dfl<L>{acc, l_neg(c)});
+    acc = s.hi;
+    c = l_neg(s.lo);
+}
+
 // source sum += both lanes' double-float terms
 __device__ __forceinline__ void src_add_df(float2 &ac, dfl<L2> v)
 {
     l_kahan_df(ac.x, ac.y, v.hi.x, v.lo.x);
     l_kahan_df(ac.x, ac.y, v.hi.y, v.lo.y);
+    l_kahan_norm(ac.x, ac.y);
 }
 
 // The accurate apply: every quantity of the pair a double-float, about 1,000 operations against the mixed
-// apply's 195; FP32 operand reads bound it (8 x 4,096 edges 2.78 ms; one target per thread in scalar double-float
-// arithmetic took 4.75).  Its error against FP64 stays that of fully renormalised arithmetic (1.5e-13 at 500
-// edges, 8.8e-13 at 4,096, random u) as long as the differences are exact and t is renormalised before t^2.
+// apply's 195; FP32 operand reads bound it (8 x 4,096 edges 2.81 ms; one target per thread in scalar double-float
+// arithmetic took 4.75).  Its error against 64 bits stays that of fully renormalised arithmetic (9.6e-15 on trefoils of
+// 150 edges, 2.7e-14 of 500, 9.0e-13 on knots of 4,096, random u) as long as the differences are exact, d2 and t are
+// renormalised before they are used, and the sums at least every eight terms (1.7e-14 at 150 edges without).
 // Sums are (sum, minus low part) like the compensated ones.
 template <bool CHECK>
 __device__ __forceinline__ void sym_pair_df(const SymTgt &t, const SymTgtU &tu, const SymSmem<PDF, OP_APPLY> &tl,
@@ -281,7 +295,7 @@ __device__ __forceinline__ void sym_pair_df(const SymTgt &t, const SymTgtU &tu, 
 #pragma unroll
     for (int ab = 0; ab < 4; ++ab) {
         const dfv<L2> &d = dd4[ab];
-        d2[ab] = l_dfnorm2(d);
+        d2[ab] = l_dfnorm(l_dfnorm2(d));
         sym_df_powers(d2[ab], F[ab], G[ab]);
         // |T_I x d_ab|^2 depends on b only, |T_J x d_ab|^2 on a only (g_i2 = g_i1 + l_I T_I)
         if (ab < 2) cI[ab] = l_dfnorm(l_dfadd(d2[ab], l_dfneg(l_dfsqr(l_dfnorm(l_dfdot(TI, d))))));
@@ -532,6 +546,10 @@ __device__ __forceinline__ void sym_section(const SymTgt &t, const SymTgtU *tu, 
             }
             sym_pair<PREC, CHECK, MODE>(t, tu, sm, s, at, s0 + j, k0, k1, a, &sm.sac[wid][0][at], pa, n0, n1);
         }
+        if constexpr (PREC == PDF)
+            if ((step & 3) == 3)
+#pragma unroll
+                for (int q = 0; q < 6; ++q) l_kahan_norm(a.s[q], a.c[q]);
         __syncwarp();  // the next step hands this lane's source on
         if constexpr (QUEUE) {
             const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
