@@ -71,8 +71,7 @@ __global__ void k_records(int nE, const double *__restrict__ g, const int *__res
         e[k] = p2[k] - p1[k];
     }
     double l = sqrt(e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
-    bool fin = finite64(l);
-    for (int k = 0; k < 3; ++k) fin = fin && finite64(p1[k]) && finite64(p2[k]);
+    const bool fin = finite64(l) && finite64(p1[0] + p1[1] + p1[2]) && finite64(p2[0] + p2[1] + p2[2]);
     if (!fin) {
         atomicCAS(err, 0, (int)TP_ERR_NONFINITE);
         l = 1.0;
