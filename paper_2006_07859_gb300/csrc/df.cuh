@@ -74,9 +74,6 @@ __device__ __forceinline__ df df_sqr(df x)
     return fast_two_sum(p, e);
 }
 
-// x (1 + f) for a small f (|f| < 1e-5): the correction only touches the low part
-__device__ __forceinline__ df df_scale1p(df x, float f) { return fast_two_sum(x.hi, __fmaf_rn(x.hi, f, x.lo)); }
-
 __device__ __forceinline__ double df_to_double(df x) { return (double)x.hi + (double)x.lo; }
 
 __device__ __forceinline__ df df_from_double(double v)
@@ -84,8 +81,5 @@ __device__ __forceinline__ df df_from_double(double v)
     const float h = (float)v;
     return df{h, (float)(v - (double)h)};
 }
-
-// a - b of two double-float values given as (hi, lo) float pairs
-__device__ __forceinline__ df df_diff(float ah, float al, float bh, float bl) { return df_sub(df{ah, al}, df{bh, bl}); }
 
 }  // namespace tpe

@@ -146,14 +146,6 @@ __device__ __forceinline__ void l_kahan_fma(L &acc, L &c, L a, L b)
     c = l_sub(l_sub(t, acc), y);
     acc = t;
 }
-template <class L>
-__device__ __forceinline__ void l_kahan(L &acc, L &c, L x)
-{
-    const L y = l_sub(x, c);
-    const L t = l_add(acc, y);
-    c = l_sub(l_sub(t, acc), y);
-    acc = t;
-}
 
 // The energy's four-term sums of row I (and of row J): f = sum_ab |T x d_ab|^2 |d_ab|^-4.5 from the two
 // |T x d|^2 that the row needs (they depend on the other edge's endpoint only), each row in its own order
