@@ -505,7 +505,7 @@ __device__ __forceinline__ void pair_eval(const Tgt<typename RealOf<PREC>::type>
         float r[4], r2;
 #pragma unroll
         for (int ab = 0; ab < 4; ++ab) r[ab] = l_pow45(ab == 0 ? d2_11 : l_dot(d[ab], d[ab]), r2);
-        l_kahan_fma(a.s, a.c, s.ell, l_keep(keep, l_energy_sum(c0, c1, r[0], r[1], r[2], r[3])));
+        l_kahan_fma_pos(a.s, a.c, s.ell, l_keep(keep, l_energy_sum(c0, c1, r[0], r[1], r[2], r[3])));
     } else if constexpr (OP == OP_ENERGY) {
         V3<R> dd[4];
         chords<DF>(t, s, dd);
@@ -527,9 +527,10 @@ __device__ __forceinline__ void pair_eval(const Tgt<typename RealOf<PREC>::type>
             f += pow_c<R, FAST>(cI[ab & 1], alpha) * inv_pow<R, FAST, 0>(d2, beta, r2);
         }
         R c = s.ell * f;
-        if constexpr (PREC == PMIX)
+        if constexpr (PREC == PMIX) {
             kahan_add(a.s, a.c, keep ? c : (R)0);
-        else
+            a.c = l_at_most_max(a.c);
+        } else
             a.s += keep ? c : (R)0;
     } else if constexpr (OP == OP_DIFF) {
         // |T_I x d_ab|, its perpendicular d - (T_I.d) T_I depend on b only (T_I . d_2b = T_I . d_1b + l_I);

@@ -147,6 +147,17 @@ __device__ __forceinline__ void l_kahan_fma(L &acc, L &c, L a, L b)
     acc = t;
 }
 
+// The same for the energy, whose terms are positive and overflow below 2.7e-9: an infinite sum stays infinite.  Its
+// compensation would be inf - inf, and the sum NaN with the next term; the smaller of NaN and a number is the number.
+__device__ __forceinline__ float l_at_most_max(float a) { return fminf(a, 3.40282347e38f); }
+__device__ __forceinline__ float2 l_at_most_max(float2 a) { return make_float2(l_at_most_max(a.x), l_at_most_max(a.y)); }
+template <class L>
+__device__ __forceinline__ void l_kahan_fma_pos(L &acc, L &c, L a, L b)
+{
+    l_kahan_fma(acc, c, a, b);
+    c = l_at_most_max(c);
+}
+
 // The energy's four-term sums of row I (and of row J): f = sum_ab |T x d_ab|^2 |d_ab|^-4.5 from the two
 // |T x d|^2 that the row needs (they depend on the other edge's endpoint only), each row in its own order
 // of the endpoints.

@@ -133,7 +133,7 @@ __device__ __forceinline__ void sym_load(SymSrc &s, const SymSmem<PREC, OP> &tl,
 using L2 = float2;
 
 // Two target rows of a thread (rows of invalid lanes repeat the last one with length 0, so that they feed
-// nothing into the sources).
+// nothing into the sources, at a place where no power overflows: 0 x inf would reach the sources as NaN).
 struct SymTgt {
     LV<L2> p, pl, e, T, Tl;  // PDF: el the low part of e
     LV<L2> el;
@@ -174,6 +174,12 @@ __device__ __forceinline__ void src_add(float2 &ac, L2 w, L2 v)
     l_kahan_fma(ac.x, ac.y, w.y, v.y);
 }
 
+__device__ __forceinline__ void src_add_pos(float2 &ac, L2 w, L2 v)
+{
+    l_kahan_fma_pos(ac.x, ac.y, w.x, v.x);
+    l_kahan_fma_pos(ac.x, ac.y, w.y, v.y);
+}
+
 template <int PREC, bool CHECK, int MODE>
 __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const SymSmem<PREC, OP_ENERGY> &, const SymSrc &s,
                                          int, int Jg, bool k0, bool k1, SymAcc<PREC, OP_ENERGY> &a, float2 *sac,
@@ -206,11 +212,11 @@ __device__ __forceinline__ void sym_pair(const SymTgt &t, const SymTgtU *, const
     }
     L2 fI = l_energy_sum(cI[0], cI[1], r[0], r[1], r[2], r[3]);
     if constexpr (CHECK) fI = l_keep(k0, k1, fI);
-    l_kahan_fma(a.s[0], a.c[0], l_bc<L2>(s.ell), fI);
+    l_kahan_fma_pos(a.s[0], a.c[0], l_bc<L2>(s.ell), fI);
     L2 fJ = l_energy_sum(cJ[0], cJ[1], r[0], r[2], r[1], r[3]);
     if constexpr (CHECK) fJ = l_keep(k0, k1, fJ);
     float2 ac = *sac;
-    src_add(ac, t.ell, fJ);
+    src_add_pos(ac, t.ell, fJ);
     *sac = ac;
 }
 
@@ -645,6 +651,8 @@ __global__ void __launch_bounds__(kThreads, MB) k_sym(const SymArgs pa)
 #undef TPE_L2
 #undef TPE_Q2
 #undef TPE_U2
+            if (!valid[0]) t.p.x.x = 1e18f;
+            if (!valid[1]) t.p.x.y = 1e18f;
         }
         if constexpr (MIX) {
 #pragma unroll
@@ -843,7 +851,7 @@ k_sym_sum(int nE, const int *__restrict__ eslots, const float2 *__restrict__ par
             s = r.hi;
             lo = __fadd_rn(lo, __fadd_rn(r.lo, v.y));
         }
-        if constexpr (!D64) x = (double)s + (double)lo;
+        if constexpr (!D64) x = OP == OP_ENERGY && isinf(s) ? (double)s : (double)s + (double)lo;
     }
     if constexpr (OP == OP_ENERGY) {
         if (row < nE) out[row] = quarter * ell[row] * x;
