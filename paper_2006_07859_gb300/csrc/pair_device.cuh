@@ -26,18 +26,18 @@ __device__ __forceinline__ R inv_pow(R d2, R e, R &r2)
             r2 = r * r;
             return WHICH == 0 ? r2 * r2 * sr : r2 * sr;
         } else {
-            // r = |d|^-1 and s = |d|^-1/2 from two hardware approximations (2^-22), each followed by one step of the
-            // series of (1 - e)^-1/2 for its residual e (the cubic term is below 2^-60).  Ten FP64 instructions where
-            // rsqrt() and sqrt() take about twenty: the FP64 passes are bound by their number (2 per clock and SM).
-            // Both roots are within 2.5 units of 2^-53, as rsqrt() and sqrt() of it are, so the powers' errors stay
-            // what they were (one root of order 1/4 raised to the ninth power had twice that).
+            // r = |d|^-1 and y = r^-1/2 from two hardware approximations (2^-22), each followed by one step of the
+            // series of (1 - e)^-1/2 for its residual e (the cubic term is below 2^-60), and s = |d|^-1/2 = r y.  Eleven
+            // FP64 instructions where rsqrt() and sqrt() take about twenty: the FP64 passes are bound by their number (2
+            // per clock and SM).  Both roots are within 2.5 units of 2^-53, as rsqrt() and sqrt() of it are, so the
+            // powers' errors stay what they were (one root of order 1/4 raised to the ninth power had twice that).
             double r0, q0;
             asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d2));
             asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(q0) : "d"(r0));
             const double e = fma(-(d2 * r0), r0, 1.0);
             double r = fma(r0, e * fma(0.375, e, 0.5), r0);
             const double s0 = r * q0, h = fma(-s0, q0, 1.0);
-            double s = fma(s0, h * fma(0.375, h, 0.5), s0);
+            double s = r * fma(q0, h * fma(0.375, h, 0.5), q0);
             // zero and subnormal (infinite powers), infinity (zero) and NaN
             if ((unsigned)(__double2hiint(d2) - 0x00100000) >= 0x7fe00000u) r = s = 1.0 / d2;
             r2 = r * r;
