@@ -550,6 +550,30 @@ cudaError_t plan_upload(Ctx::Plan &pl, const std::vector<WorkItem> &items, const
 
 constexpr int kMinChunk = 4;  // sources of the shortest item
 
+// Source chunks of the gather passes.  Items of at least eight source tiles amortise their targets; where those would
+// leave resident CTAs without an item, one wave of short items is faster: a pass over 256 edges was two CTAs, each
+// walking all 256 sources in turn (energy 284 us, FP64 differential 2,117 us), and is 64 to 128 of them.
+struct Chunking {
+    int tb;              // targets per item
+    long long resident;  // resident CTAs
+    double total;        // squared edges, summed over problems
+    bool small = false;  // the short items
+
+    int blocks(int n) const { return (n + tb - 1) / tb; }
+    int chunks(int n) const
+    {
+        const double share = total > 0 ? (double)n * n / total : 1.0;
+        const double want = std::ceil(share * (double)(small ? resident : 3 * resident) / blocks(n));
+        const int most = std::min(64, small ? n / kMinChunk : n / (8 * kTile));
+        return (int)std::max(1.0, std::min(want, (double)most));
+    }
+    int length(int n) const
+    {
+        const int nch = chunks(n), len = (n + nch - 1) / nch;
+        return small ? len : (len + kTile - 1) / kTile * kTile;
+    }
+};
+
 // Build the (target block, source chunk) queue of one pass.  Items of big problems come first
 // so the persistent grid ends with the small ones.
 cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
@@ -564,33 +588,19 @@ cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
             vmin[v] = std::min(vmin[v], I);
             vmax[v] = std::max(vmax[v], I);
         }
-    const int target_items = std::max(1, 3 * c.sm_count * std::max(1, occupancy));
     // total work estimate to size chunks
     double total = 0.0;
     for (int q = 0; q < c.nProb; ++q) {
         double n = c.h_prob_e[q + 1] - c.h_prob_e[q];
         total += n * n;
     }
-    // Items of at least eight source tiles amortise their targets; where those would leave resident CTAs
-    // without an item, one wave of short items is faster: a pass over 256 edges was two CTAs, each walking
-    // all 256 sources in turn (energy 284 us, FP64 differential 2,117 us), and is 64 to 128 of them.
-    const long long resident = (long long)c.sm_count * std::max(1, occupancy);
-    auto chunks = [&](int n, bool small) {
-        const int nblk = (n + tb - 1) / tb;
-        const double share = total > 0 ? (double)n * n / total : 1.0;
-        const double want = std::ceil(share * (small ? (double)resident : (double)target_items) / nblk);
-        const int most = std::min(64, small ? n / kMinChunk : n / (8 * kTile));
-        return (int)std::max(1.0, std::min(want, (double)most));
-    };
-    auto items_of = [&](bool small) {
-        long long k = 0;
-        for (int q = 0; q < c.nProb; ++q) {
-            const int n = c.h_prob_e[q + 1] - c.h_prob_e[q];
-            k += (long long)((n + tb - 1) / tb) * chunks(n, small);
-        }
-        return k;
-    };
-    const bool small = items_of(false) < resident;
+    Chunking ck{tb, (long long)c.sm_count * std::max(1, occupancy), total};
+    long long whole = 0;
+    for (int q = 0; q < c.nProb; ++q) {
+        const int n = c.h_prob_e[q + 1] - c.h_prob_e[q];
+        if (n > 0) whole += (long long)ck.blocks(n) * ck.chunks(n);
+    }
+    ck.small = whole < ck.resident;
     int max_slots = 1;
     std::vector<int> eslots(c.nE, 1);
     struct Tmp {
@@ -601,11 +611,7 @@ cudaError_t plan_pass(Ctx &c, Ctx::Plan &pl, int tpt, int occupancy)
     for (int q = 0; q < c.nProb; ++q) {
         int e0 = c.h_prob_e[q], e1 = c.h_prob_e[q + 1], n = e1 - e0;
         if (n <= 0) continue;
-        int nblk = (n + tb - 1) / tb;
-        int nch = chunks(n, small);
-        int clen = (n + nch - 1) / nch;
-        if (!small) clen = (clen + kTile - 1) / kTile * kTile;
-        nch = (n + clen - 1) / clen;
+        const int nblk = ck.blocks(n), clen = ck.length(n), nch = (n + clen - 1) / clen;
         max_slots = std::max(max_slots, nch);
         for (int b = 0; b < nblk; ++b) {
             int t0 = e0 + b * tb, nt = std::min(tb, e1 - t0);
@@ -667,13 +673,14 @@ int tpt_candidates(const Ctx &c, int cls, int *out)
 
 // Too few edges to give every SM two items of tpt targets per thread and eight source tiles: one target
 // per thread then doubles or quadruples the items (256 edges: energy with four targets 16 items, with one 64).
+static long long long_items(long long n, int tpt)
+{
+    return ((n + kThreads * tpt - 1) / (kThreads * tpt)) * std::max(1LL, n / (8 * kTile));
+}
 static bool small_graph(const Ctx &c, int tpt)
 {
     long long items = 0;
-    for (int q = 0; q < c.nProb; ++q) {
-        const long long n = c.h_prob_e[q + 1] - c.h_prob_e[q];
-        items += ((n + kThreads * tpt - 1) / (kThreads * tpt)) * std::max(1LL, n / (8 * kTile));
-    }
+    for (int q = 0; q < c.nProb; ++q) items += long_items(c.h_prob_e[q + 1] - c.h_prob_e[q], tpt);
     return items < 2LL * c.sm_count;
 }
 
@@ -847,7 +854,7 @@ __global__ void k_static_stats(int nV, int nE, const double *__restrict__ g, con
 cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, int nE, double alpha, double beta,
                                  double near_cutoff, RecF *recF, RecLo *recLo, double *ell, double *T, double *x,
                                  WorkItem *items, int *eslots, double *part, double *rows, int *counter, int *err,
-                                 double *scal, int *off, int max_items, int max_slots, double *E, cudaStream_t s,
+                                 double *scal, int *off, int max_items, long long max_part, double *E, cudaStream_t s,
                                  int *status)
 {
     *status = 0;
@@ -876,23 +883,30 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
     kp.near2f = (float)(rn * rn);
     kp.near2f_diff = (float)(16.0 * rn * rn);
     kp.mid2f = 3.0e38f;  // double-float positions in every tile (the context's default)
-    // blocking: targets per item = kThreads * kTptEnergy, at least 8 source tiles per item
+    // the blocking of a context's gather pass over the same graph, so that the sums are the same to the bit wherever the
+    // scratch holds as many slots
     int dev = 0, sms = 0, occ = 0;
     TPE_CHECK(cudaGetDevice(&dev));
     TPE_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (kp.fast)
-        TPE_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs<PMIX, OP_ENERGY, kTptEnergy, true>, kThreads, 0));
-    else
-        TPE_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs<PMIX, OP_ENERGY, kTptEnergy, false>, kThreads, 0));
-    const int tb = kThreads * kTptEnergy;
-    const int nblk = (nE + tb - 1) / tb;
-    int want = (3 * sms * std::max(1, occ) + nblk - 1) / nblk;
-    int nch = std::min(std::min(std::max(1, want), std::max(1, nE / (8 * kTile))), max_slots);
-    int clen = ((nE + nch - 1) / nch + kTile - 1) / kTile * kTile;
-    nch = (nE + clen - 1) / clen;
-    if (nblk * nch > max_items || nch > max_slots) return cudaErrorInvalidValue;
-    const int nit = nblk * nch;
-    k_static_items<<<(std::max(nit, nE) + 255) / 256, 256, 0, s>>>(nE, tb, clen, nch, items, eslots, off);
+    const int tpt = long_items(nE, kTptEnergy) < 2LL * sms ? 1 : kTptEnergy;
+    auto with_kernel = [&](auto f) {
+        if (kp.fast)
+            with_pair_kernel<PMIX, OP_ENERGY, true>(tpt, f);
+        else
+            with_pair_kernel<PMIX, OP_ENERGY, false>(tpt, f);
+    };
+    with_kernel([&](auto kern) { cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0); });
+    Chunking ck{kThreads * tpt, (long long)sms * std::max(1, occ), (double)nE * nE};
+    ck.small = (long long)ck.blocks(nE) * ck.chunks(nE) < ck.resident;
+    int clen = ck.length(nE), nch = (nE + clen - 1) / clen;
+    if ((long long)nch * nE > max_part) {  // longer chunks, as many as the scratch holds partial sums for
+        clen = (nE + (int)(max_part / nE) - 1) / (int)(max_part / nE);
+        clen = (clen + kTile - 1) / kTile * kTile;
+        nch = (nE + clen - 1) / clen;
+    }
+    const int nit = ck.blocks(nE) * nch;
+    if (nit > max_items) return cudaErrorInvalidValue;
+    k_static_items<<<(std::max(nit, nE) + 255) / 256, 256, 0, s>>>(nE, ck.tb, clen, nch, items, eslots, off);
     TPE_CHECK(cudaMemsetAsync(counter, 0, sizeof(int), s));
     PairArgs pa;
     pa.items = items;
@@ -909,10 +923,7 @@ cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, 
     pa.kp = kp;
     pa.skip = nullptr;
     const int grid = std::max(1, std::min(nit, sms * std::max(1, occ)));
-    if (kp.fast)
-        k_pairs<PMIX, OP_ENERGY, kTptEnergy, true><<<grid, kThreads, 0, s>>>(pa);
-    else
-        k_pairs<PMIX, OP_ENERGY, kTptEnergy, false><<<grid, kThreads, 0, s>>>(pa);
+    with_kernel([&](auto kern) { kern<<<grid, kThreads, 0, s>>>(pa); });
     k_energy_rows<<<(nE + 31) / 32, 256, 0, s>>>(nE, eslots, part, ell, rows);
     k_segment_sum<<<1, kSegThreads, 0, s>>>(off, rows, E);
     return cudaGetLastError();

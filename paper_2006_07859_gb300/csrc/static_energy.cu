@@ -19,7 +19,7 @@ namespace tpe {
 cudaError_t static_energy_launch(const double *gamma, const int *edges, int nV, int nE, double alpha, double beta,
                                  double near_cutoff, RecF *recF, RecLo *recLo, double *ell, double *T, double *x,
                                  WorkItem *items, int *eslots, double *part, double *rows, int *counter, int *err,
-                                 double *scal, int *off, int max_items, int max_slots, double *E, cudaStream_t s,
+                                 double *scal, int *off, int max_items, long long max_part, double *E, cudaStream_t s,
                                  int *status);
 }  // namespace tpe
 
@@ -28,7 +28,7 @@ namespace {
 // Scratch of the no-allocation energy, shared by every call on a device.
 constexpr int kStaticMaxEdges = 65536;  // largest graph tp_energy_static accepts
 constexpr int kStaticMaxItems = 8192;
-constexpr int kStaticSlots = 16;
+constexpr int kStaticSlots = 16;  // of the largest graph; smaller ones have up to 64
 
 __device__ __align__(256) tpe::RecF g_recF[kStaticMaxEdges];
 __device__ __align__(256) tpe::RecLo g_recLo[kStaticMaxEdges];
@@ -110,7 +110,7 @@ extern "C" TPE_API tp_status tp_energy_static(const double *gamma, const int32_t
     int status = 0;
     e = tpe::static_energy_launch(gamma, edges, n_vertices, n_edges, alpha, beta, 4.0, p->recF, p->recLo, p->ell, p->T,
                                   p->x, p->items, p->eslots, p->part, p->rows, p->counter, p->err, p->scal, p->off,
-                                  kStaticMaxItems, kStaticSlots, E, (cudaStream_t)stream, &status);
+                                  kStaticMaxItems, (long long)kStaticSlots * kStaticMaxEdges, E, (cudaStream_t)stream, &status);
     if (e != cudaSuccess) return TP_ERR_CUDA;
     if (status) return (tp_status)status;  // TP_ERR_DEGENERATE_EDGE or TP_ERR_NONFINITE
     return TP_OK;
