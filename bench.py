@@ -56,6 +56,9 @@ def flop_per_pair(op, cols=MULTI_COLS):
     return 220 + 35 * cols // 3 if op == "apply_multi" else FLOP_PER_PAIR[op]
 
 
+# What the symmetric apply executes per unordered pair on the FP32 pipe (an FMA is one operation): both directions of
+# the pair share chords, powers and cross products, so it is less than the canonical count of two ordered pairs
+SYM_APPLY_OPS = 195
 MUFU_PER_PAIR = {"energy": 8, "diff": 8, "apply": 8}
 FP32_LANES = 128   # FP32 FMA lanes per SM (Blackwell)
 L2_BYTES = 129 * 2 ** 20
@@ -101,13 +104,13 @@ def parse():
                     help="hat functions per curve of the coarse space (0: 1024 on the 262,144-edge knot, 128 on "
                          "the 4,096-vertex knots)")
     ap.add_argument("--apply-variant", type=int, default=-1,
-                    help="bench mode: after the autotuner, pin the apply pass (0 gather, 1 or 2 the symmetric "
-                         "pass with that many targets per thread); for launch lists taken under a profiler")
+                    help="bench mode: after the autotuner, pin the apply pass (0 gather, 1 or 2 a variant of the "
+                         "symmetric pass); for launch lists taken under a profiler")
     ap.add_argument("--accurate", action="store_true",
                     help="passes mode: also two double-float applies (sobolev_apply_accurate)")
     ap.add_argument("--sym-tpt", type=int, default=0,
-                    help="passes mode: run the symmetric energy / differential / apply passes with this many "
-                         "targets per thread (0: the gather passes)")
+                    help="passes mode: variant of the symmetric energy / differential / apply passes "
+                         "(0: the gather passes)")
     ap.add_argument("--rows", type=int, default=1024, help="precision mode: sampled rows / vertices")
     ap.add_argument("--with-fp64", action="store_true", help="precision mode: also run the FP64 GPU passes")
     ap.add_argument("--train-steps", type=int, default=300, help="learned mode: Adam steps")
@@ -373,10 +376,10 @@ def run_passes(args):
     from paper_2006_07859_gb300 import tpe
     curves, cfg, indep = workload(args.workload)
     ctx = tpe.Context.from_curves(curves, precision=tpe.TP_MIXED, precond=tpe.TP_PRECOND_JACOBI, independent=indep)
-    if args.sym_tpt:
-        tpe.tp_set_energy_variant(ctx, args.sym_tpt)
-        tpe.tp_set_diff_variant(ctx, args.sym_tpt)
-        tpe.tp_set_apply_variant(ctx, args.sym_tpt)
+    # 0 too: a new context of these sizes runs the symmetric passes by default
+    tpe.tp_set_energy_variant(ctx, args.sym_tpt)
+    tpe.tp_set_diff_variant(ctx, args.sym_tpt)
+    tpe.tp_set_apply_variant(ctx, args.sym_tpt)
     g = torch.as_tensor(curves.gamma).cuda()
     u = torch.as_tensor(np.random.default_rng(1).normal(size=(curves.n_vertices, 3))).cuda()
     tpe.tp_energy(ctx, g)
@@ -853,7 +856,10 @@ def run_ours(args, rank, world, local_rank):
                      "frac": achieved / peak if achieved else None,
                      "traffic": APPLY_TRAFFIC_BYTES.get((args.workload,) + apply_variant),
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
-                     "flop_per_pair": FLOP_PER_PAIR["apply"], "launches": n_a, "avg_launch_ms": avg_s * 1e3,
+                     "flop_per_pair": FLOP_PER_PAIR["apply"],
+                     "executed_ops_per_unordered_pair": SYM_APPLY_OPS if sym_apply else None,
+                     "executed_frac": pairs / 2 * SYM_APPLY_OPS * 2 / avg_s / peak if sym_apply and n_a else None,
+                     "launches": n_a, "avg_launch_ms": avg_s * 1e3,
                      "peak_note": f"{sms} SMs (device attribute) x {FP32_LANES} FP32 lanes x 2 x {mhz:.0f} MHz "
                                   f"(median SM clock sampled during the timed steps)",
                      "measured_fp32_peak_tflops": peaks["fp32_flops"] / 1e12,

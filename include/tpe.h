@@ -21,11 +21,14 @@
  *     asynchronous unless it says otherwise.  Calls that return host-side info structs
  *     synchronise the stream before returning.
  *   - The caller owns every pointer it passes; the context owns its own scratch memory,
- *     allocated once in tp_create and sized for the graph it was created with.  Only
- *     tp_set_params (switching a preconditioner, a constraint set or the line search on),
- *     tp_autotune (a larger work queue), the first tp_set_penalties, the first tp_set_pins,
- *     tp_set_tangents or tp_set_surface (and one that needs more solves than any before) and the
- *     first tp_collision_time allocate device memory after tp_create.
+ *     allocated in tp_create and sized for the graph it was created with.  Only
+ *     tp_set_params (switching a preconditioner, a constraint set, the line search or the specialised
+ *     exponents on), tp_autotune and tp_set_*_variant (work lists, and the partial sums the pair passes
+ *     share), the first sobolev_apply_multi and sobolev_apply_accurate and the first preconditioner set-up or
+ *     refined solve that runs one (the same), the first tp_set_penalties, the first tp_set_pins,
+ *     tp_set_tangents or tp_set_surface (and one that needs more solves than any before), the
+ *     Barnes-Hut passes and the first tp_collision_time allocate device memory after tp_create.  Where the
+ *     pair passes' partial sums cannot be had, the call returns TP_ERR_OOM and the context stays as it was.
  *   - Every call returns a tp_status; nothing aborts or traps.  tp_last_error() gives a
  *     human-readable message for the last failing call on a context.
  *   - A context is not thread-safe; use one context per host thread.
@@ -59,7 +62,7 @@ typedef enum {
     TP_ERR_BREAKDOWN = 6,       /* CG found p^T A p <= 0 (operator not SPD on range(P)) */
     TP_ERR_LINESEARCH = 7,      /* no step size passed Armijo + projection within max_halvings */
     TP_ERR_PROJECTION = 8,      /* constraint projection did not reach proj_tol */
-    TP_ERR_OOM = 9,             /* device allocation failed in tp_create */
+    TP_ERR_OOM = 9,             /* a device allocation failed */
     TP_ERR_UNSUPPORTED = 10     /* option not available for this graph (e.g. spectral on open curves) */
 } tp_status;
 
@@ -67,7 +70,7 @@ typedef enum {
     TP_FP64 = 0,  /* pair arithmetic in FP64 */
     TP_FP32 = 1,  /* pair arithmetic in FP32; sums over at most 512 sources in FP32 (compensated in the symmetric
                      passes), those partial sums added in FP64 (symmetric passes: double-float) */
-    TP_MIXED = 2  /* FP32 pairs on double-float positions, double-float for pairs closer than near_cutoff */
+    TP_MIXED = 2  /* FP32 pairs on double-float positions, compensated sums; closer pairs see near_cutoff */
 } tp_precision;
 
 typedef enum {
@@ -131,7 +134,9 @@ typedef struct {
     double alpha, beta;   /* kernel exponents of Eq. 3; Lemma 1 needs alpha > 1, beta in [alpha+2, 2 alpha+1) */
     double sigma;         /* fractional order of B, B0; NaN => (beta - 1)/alpha - 1 (Sec. 4.2.2) */
     int precision;        /* tp_precision */
-    double near_cutoff;   /* TP_MIXED: |x_I - x_J| < near_cutoff * mean edge length => FP64 pair */
+    double near_cutoff;   /* TP_MIXED: pairs with |g_i1 - g_j1| < near_cutoff * mean edge length form |T x d|^2 of the
+                             energy in double-float; the differential evaluates pairs within 4 times that wholly in
+                             double-float (other exponents than (2, 4.5): in FP64) */
     double cg_rtol;       /* stop when ||P(a - A-bar x)|| <= cg_rtol ||P a|| */
     int cg_maxit;
     int cg_check_every;   /* host polls the device-side convergence flag every k iterations */
@@ -226,9 +231,12 @@ TPE_API tp_status sobolev_apply(tp_ctx *ctx, const double *gamma, const double *
 /* AU_f = A-bar U_f for m vector fields at once (Secs. 5.2.2-5.2.3, Eq. 19 per field): U, AU device
  * double [m][nV][3] (field-major: field f starts at U + 3 nV f); m >= 0 (m = 0 does nothing).  Every
  * pair's Gram weights and tangent gap (about 220 of the 255 canonical FLOP of an apply) are computed
- * once per pass and applied to 4 fields (12 scalar columns); the per-column arithmetic is
- * sobolev_apply's (same precision mode).  Builds its work list, per-field records and partial sums at
- * the first call (about 4 nE records and slots x nE x 24 doubles).  U and AU must not overlap.
+ * once per pass and applied to several fields; the per-column arithmetic is sobolev_apply's (same precision mode).
+ * Contexts on the gather apply take four fields per pass (12 scalar columns); their first call builds a work
+ * list, 4 nE records and slots x nE x 24 doubles of partial sums (slots: source chunks, at most 64).  TP_MIXED
+ * contexts on the symmetric apply take two fields per pass and grow the shared partial sums to slots x nE x 12
+ * doubles (slots: nE / 256 of the longest problem and up to three more; 25.8 GB at 262,144 edges), unless that
+ * is more than 32 GB or half of the free memory: then they take the gather pass.  U and AU must not overlap.
  * Errors: TP_ERR_INVALID_ARG (NULL pointers with m > 0, m < 0), TP_ERR_CUDA. */
 TPE_API tp_status sobolev_apply_multi(tp_ctx *ctx, const double *gamma, const double *U, double *AU, int m,
                                       tp_stream stream);
@@ -236,8 +244,8 @@ TPE_API tp_status sobolev_apply_multi(tp_ctx *ctx, const double *gamma, const do
 /* The same product A-bar u in double-float arithmetic (every pair term as an unevaluated sum of two
  * floats, ~48 bits, from the FP64 positions, tangents, lengths and u): the accurate operator with which
  * the solves of TP_FP32 and TP_MIXED contexts judge their true residuals (FP64 contexts run their
- * FP64 pass).  About an order of magnitude slower than sobolev_apply.  Builds its own work list at the
- * first call (the only allocation, and it may grow the context's partial-sum buffer). */
+ * FP64 pass).  About five times slower than sobolev_apply.  Builds its own work list at the first call and may
+ * grow the context's partial-sum buffer (12.9 GB at 262,144 edges). */
 TPE_API tp_status sobolev_apply_accurate(tp_ctx *ctx, const double *gamma, const double *u, double *Au,
                                          tp_stream stream);
 
@@ -377,7 +385,7 @@ TPE_API int64_t tp_pairs_per_pass(const tp_ctx *ctx);
  * 3 diag, 4 apply inside CG solves (items of already converged problems skipped), 5 double-float
  * apply (tp_sobolev_apply_accurate and the refined solves' residuals), 6 the coarse-space pass that
  * assembles A Z for the two-level preconditioners, 7 the multi-field apply (sobolev_apply_multi and
- * the Rayleigh-quotient probes of the spectral set-up), one launch per 4 fields.
+ * the Rayleigh-quotient probes of the spectral set-up), one launch per 4 fields (symmetric form: 2).
  * tp_profile_read synchronises the recorded events and returns the summed device time (ms) and
  * the number of launches of that pair kernel since profiling was enabled. */
 TPE_API tp_status tp_profile(tp_ctx *ctx, int enable);
@@ -510,16 +518,19 @@ TPE_API tp_status tp_gnn_train_step(tp_ctx *ctx, const double *gamma, int n, con
  *       [0..2], differential [3..5] and apply [6..8] gather passes, then the variants 1, 2 of the symmetric
  *       apply [9..10] and energy [11..12] and the variants 1, 2 [13..14] and 3, 4 [15..16] of the symmetric
  *       differential (0 where not a candidate).
- * May reallocate the context's partial-sum buffer (the only allocation after tp_create).
+ * May reallocate the context's partial-sum buffer.  Variants 1 and 2 of the differential run the same kernel, as do
+ * 3 and 4.
  * Synchronises the stream.  Errors: TP_ERR_INVALID_ARG, TP_ERR_CUDA, TP_ERR_DEGENERATE_EDGE. */
 TPE_API tp_status tp_autotune(tp_ctx *ctx, const double *gamma, int32_t *tpt, double *ms, tp_stream stream);
 
 /* Select the apply pass: symmetric_tpt = 0 the gather pass (every ordered pair), 1 or 2 the symmetric pass
  * (every unordered pair evaluated once, two targets per thread in packed arithmetic; both rows receive their
  * terms; TP_MIXED and TP_FP32 with (alpha, beta) = (2, 4.5) only, else TP_ERR_UNSUPPORTED), its registers held to
- * three (1) or two (2) resident CTAs per SM (TP_FP32: three).  A new context has the symmetric pass where its work list fills the GPU
- * and its partial sums take at most 1 GiB, the gather pass elsewhere.  Both are deterministic and differ
- * only in summation order.  May grow the partial-sum buffer. */
+ * three (1) or two (2) resident CTAs per SM (TP_FP32: three).  A new context has the symmetric pass where its
+ * work list fills the GPU and its partial sums take at most 1 GiB and, above 64 MiB, at most a 64th of the free
+ * memory; the gather pass elsewhere.  tp_set_params to other exponents drops the symmetric passes; back at
+ * (2, 4.5) a context has those of a new one, except a pass that was set to 0.  Both forms are deterministic and
+ * differ only in summation order.  May grow the partial-sum buffer. */
 TPE_API tp_status tp_set_apply_variant(tp_ctx *ctx, int symmetric_tpt);
 
 /* The same choice for the energy pass (0: gather, 1 or 2: symmetric at three or four resident CTAs per SM, TP_FP32

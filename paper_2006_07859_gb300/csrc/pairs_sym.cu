@@ -270,7 +270,7 @@ __device__ __forceinline__ void src_add_df(float2 &ac, dfl<L2> v)
     l_kahan_norm(ac.x, ac.y);
 }
 
-// The accurate apply: every quantity of the pair a double-float, about 1,000 operations against the mixed
+// The accurate apply: every quantity of the pair a double-float, about 1,100 operations against the mixed
 // apply's 195; FP32 operand reads bound it (8 x 4,096 edges 2.81 ms; one target per thread in scalar double-float
 // arithmetic took 4.75).  Its error against 64 bits stays that of fully renormalised arithmetic (9.6e-15 on trefoils of
 // 150 edges, 2.7e-14 of 500, 9.0e-13 on knots of 4,096, random u) as long as the differences are exact, d2 and t are
@@ -1059,6 +1059,8 @@ cudaError_t sym_select_diff(Ctx &c, int v) { return select_pass(c, OP_DIFF, v, 4
 //   20 x 500     16,400     439 / 353     67 / 73    57 / 73
 //   12 x 1,000   39,400     550 / 398    114 / 91    89 / 100
 //   120 x 256    25,800     816 / 524     88 / 76    85 / 93
+// The rule separates single curves.  A batch of short ones just below it stays on the gather differential although the
+// symmetric one is faster there (20 x 500).
 static bool sym_pays(const Ctx &c, int op)
 {
     if (c.sym_choice[op] >= 0) return false;

@@ -102,8 +102,8 @@ __device__ __forceinline__ bool sine_leads(int k) { return (unsigned)(k - kMaxFF
 // where the sine is the larger part (the factor i is a swap of b's components).  v rounds once, so a transform's error is
 // the smallest of the forms tried (1,024 points, relative norm: 1.69e-16; complex product and two sums, eight
 // instructions, 1.88e-16; 2 u - (u + w b) for the difference, six, 2.01e-16).  Iteration of a solve of two curves of 2,497
-// vertices, whose Bluestein transforms run on six SMs: 0.71, 0.87 and 0.72 ms.  Signs are turned in the high word: the
-// negation of a selected double is an FP64 instruction (0.78 ms).
+// vertices, whose Bluestein transforms run on six SMs: 0.71, 0.87 and 0.72 ms.  Signs are turned in the high word
+// (0.78 ms with a floating-point negation of the selected component).
 __device__ void fft_batch(double2 *a, int G, int M, int logM, const double2 *__restrict__ tw, bool inv)
 {
     const int total = G * M;
@@ -246,7 +246,7 @@ __device__ __forceinline__ double2 lane_butterfly(double2 a, int bit, int lane)
 // a column is Hermitian: N2 real values take an N2/2-point complex transform, and only k2 = 0..N2/2 pass the middle
 // step, one lane per (k2, m1) with the 8-point DFTs across lanes (all four schedulers work, where a thread per
 // k2 with 64 twiddled products kept one busy).  Twice the even part of the symbol is used, which is all that reaches
-// the real part of the result.  8 curves of 4,096: 27.7 us, before 46.7.
+// the real part of the result.  8 curves of 4,096: 29 us, before 47.
 __global__ void __cluster_dims__(kClusterFFT, 1, 1) __launch_bounds__(kClusterThreads)
     k_spec_cluster(const SpecCurve *__restrict__ curves, const int *__restrict__ idx, const double *__restrict__ r,
                    double *__restrict__ z, const double *__restrict__ dinv, const double2 *__restrict__ tw,

@@ -130,12 +130,12 @@ struct Ctx {
     };
     Plan plan_energy, plan_diff, plan_apply;
     int tpt[3] = {0, 0, 0};  // targets per thread chosen by tp_autotune (energy, diff, apply + diag); 0: default
-    Plan plan_sym;           // symmetric apply (pairs_sym.cu): items over edge-block pairs (b, c >= b)
-    int apply_sym = 0;       // > 0: the apply runs the symmetric pass with this many targets per thread
+    Plan plan_sym;           // symmetric apply (pairs_sym.cu): items of a super-block and sources beyond or inside it
+    int apply_sym = 0;       // > 0: the apply runs this variant of the symmetric pass
     Plan plan_sym_e;         // symmetric energy (pairs_sym.cu)
-    int energy_sym = 0;      // > 0: the energy runs the symmetric pass with this many targets per thread
+    int energy_sym = 0;      // > 0: the energy runs this variant of the symmetric pass
     Plan plan_sym_d;         // symmetric differential (pairs_sym.cu)
-    int diff_sym = 0;        // > 0: the differential runs the symmetric pass
+    int diff_sym = 0;        // > 0: the differential runs this variant of the symmetric pass
     int sym_choice[3] = {-1, -1, -1};  // variant asked for (OP_ENERGY, OP_DIFF, OP_APPLY); -1: the default by size
     Plan plan_df;            // double-float apply, built at its first use (tpt 1: general exponents)
     Plan plan_multi;         // multi-field apply (pairs_multi.cu), built at its first use

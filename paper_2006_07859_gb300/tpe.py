@@ -529,8 +529,8 @@ def tp_gnn_train_step(ctx: Context, gamma, R, B, AB, ER, lr: float, grad=None, I
 
 
 def tp_autotune(ctx: Context, gamma) -> dict:
-    """Pick the fastest targets-per-thread of each pair pass on `gamma` (mixed precision, alpha = 2,
-    beta = 4.5); returns the choices and the measured ms per pass."""
+    """Pick the fastest form of each pair pass on `gamma` (mixed precision, alpha = 2, beta = 4.5): targets per thread of
+    the gather passes, variants of the symmetric ones; returns the choices and the measured ms per pass."""
     t = (ctypes.c_int32 * 6)()
     ms = (ctypes.c_double * 17)()
     ctx._check(library().tp_autotune(ctx.handle, _ptr(gamma), t, ms, _stream()))
@@ -548,12 +548,14 @@ def tp_autotune(ctx: Context, gamma) -> dict:
 
 
 def tp_set_apply_variant(ctx: Context, symmetric_tpt: int):
-    """0: gather apply (every ordered pair); 1 or 2: symmetric apply with that many targets per thread."""
+    """0: gather apply (every ordered pair); 1 or 2: symmetric apply (every unordered pair once; 1 holds it to three
+    resident CTAs per SM, 2 to two).  Mixed and FP32 contexts with (alpha, beta) = (2, 4.5)."""
     ctx._check(library().tp_set_apply_variant(ctx.handle, int(symmetric_tpt)))
 
 
 def tp_set_energy_variant(ctx: Context, symmetric_tpt: int):
-    """0: gather energy pass (every ordered pair); 1 or 2: symmetric pass with that many targets per thread."""
+    """0: gather energy pass (every ordered pair); 1 or 2: symmetric pass (three or four resident CTAs per SM).
+    Mixed and FP32 contexts with (alpha, beta) = (2, 4.5)."""
     ctx._check(library().tp_set_energy_variant(ctx.handle, int(symmetric_tpt)))
 
 
@@ -566,5 +568,6 @@ def tp_last_solve(ctx: Context):
 
 
 def tp_set_diff_variant(ctx: Context, symmetric_tpt: int):
-    """0: gather differential (every ordered pair); 1 or 2: symmetric pass with that many targets per thread."""
+    """0: gather differential (every ordered pair); 1 or 2: symmetric pass at two resident CTAs per SM, 3 or 4 at three.
+    Mixed contexts with (alpha, beta) = (2, 4.5)."""
     ctx._check(library().tp_set_diff_variant(ctx.handle, int(symmetric_tpt)))
